@@ -82,9 +82,12 @@ typedef struct {
 /* Heads and element type.  Supported: head_dim 64 or 128; Hq % Hkv == 0;
  * ISM_BF16 (fp32 accumulation) or ISM_FP32 (fp32 CUDA-core path); ISM_E4M3
  * (fp8 inputs, head_dim 128) only for the e4m3 entry points and their
- * workspace queries.  The tensor-core kernels serve bf16 and e4m3 at
- * head_dim 128; bf16 at head_dim 64 runs the CUDA-core kernels (correct, but
- * far from the tensor-core rate), as does fp32.  softmax_scale multiplies q.k before the softmax (the paper omits
+ * workspace queries.  The tensor-core kernels serve bf16 at head_dim 64 and
+ * 128 and e4m3 at head_dim 128; fp32 runs the CUDA-core kernels, and so does a
+ * single-token step at head_dim 64.  At head_dim 64 P and dS are kept to 16
+ * mantissa bits (two bf16 parts), at 128 to bf16.  As at head_dim 128, a key
+ * tile of 128 rows is read whole: NaN or Inf in K, V, Q or dO rows of a tile
+ * reaches the results of other rows of that tile.  softmax_scale multiplies q.k before the softmax (the paper omits
  * the factor, Section 2.1; 1/sqrt(head_dim) is the usual choice). */
 typedef struct {
   int32_t num_heads_q;

@@ -277,7 +277,7 @@ bool force_cuda_cores() { return knobs().force_cuda_cores; }
 uint32_t tc_flags() { return knobs().drain_tmem_reuse ? kFlagDrainTmemReuse : 0u; }
 
 bool use_tc(const ism_attn_shape_t* sh) {
-  return sh->dtype == ISM_BF16 && sh->head_dim == 128 && tc_available() && !force_cuda_cores();
+  return sh->dtype == ISM_BF16 && tc_available() && !force_cuda_cores();
 }
 bool use_tc_bwd(const ism_attn_shape_t* sh) { return use_tc(sh) && tc_bwd_available(); }
 
@@ -287,15 +287,25 @@ bool use_tc_bwd(const ism_attn_shape_t* sh) { return use_tc(sh) && tc_bwd_availa
 bool fwd_tile_pairs(const ism_attn_shape_t* sh) {
   if ((sh->num_heads_q / sh->num_heads_kv) % 2 == 0) return false;
   if (sh->dtype == ISM_E4M3) return true;  // the e4m3 forward runs only the paired kernel
-  if (!use_tc(sh)) return false;
+  if (!use_tc(sh) || sh->head_dim != 128) return false;
   return !knobs().fwd_one_head;
 }
 
+// Whether the metadata pass puts the query-tile pair heads at the front of
+// q_order: an odd group without a pair list of its own.  The head_dim 64
+// forward pairs tiles from there, so its workspaces and plans are those of the
+// CUDA-core kernels (which take any order), in size and in use: a plan built
+// for fp32 or under ISM_FORCE_CUDA_CORES=1 serves it and the other way round.
+bool pairs_first(const ism_attn_shape_t* sh) {
+  return (sh->num_heads_q / sh->num_heads_kv) % 2 != 0 && !fwd_tile_pairs(sh);
+}
+
 // dS tile slots of the stored-dS backward (pairs x query heads), or 0 where
-// that path does not apply: CUDA-core backward, ISM_BWD_RECOMPUTE_DQ=1, or
-// more pairs than the 32-bit pair offsets hold.
+// that path does not apply: CUDA-core backward, head_dim 64 (the tile is as
+// large as at 128 and saves half the work), ISM_BWD_RECOMPUTE_DQ=1, or more
+// pairs than the 32-bit pair offsets hold.
 int64_t stored_ds_slots(const ism_segments_t* s, const ism_attn_shape_t* sh) {
-  if (!use_tc_bwd(sh)) return 0;
+  if (!use_tc_bwd(sh) || sh->head_dim != 128) return 0;
   if (knobs().bwd_recompute_dq) return 0;
   const int64_t pairs = count_pairs(s);
   if (pairs >= (int64_t(1) << 31)) return 0;
@@ -310,13 +320,13 @@ ism_status_t check_ws(void* ws, size_t have, size_t need) {
 }
 
 ism_status_t build_pass_meta(const ism_segments_t* s, const Counts& c, const PassLayout& L, bool bwd,
-                             cudaStream_t st) {
+                             cudaStream_t st, bool heads_first = false) {
   SegsDev d = dev_view(s);
   timer_begin(ISM_KERNEL_META, st);
   ISM_TRY_CUDA(launch_pass_meta(d, L.kv_end, kTile, kTile, c.nq, bwd ? c.nk : 0, L.qtiles, bwd ? L.ktiles : nullptr,
                                 c.max_cost, L.q_order, bwd ? L.k_order : nullptr, L.pair_order, L.kpair_off,
                                 L.counters, L.counters ? kPassCounters : 0, st,
-                                knobs().dkdv_pair ? L.kp_order : nullptr),
+                                knobs().dkdv_pair ? L.kp_order : nullptr, heads_first),
                "metadata launch");
   timer_end(ISM_KERNEL_META, st);
   count_launch(1);
@@ -543,7 +553,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     q = q_rot;
     k = k_rot;
   }
-  if (!pre && (r = build_pass_meta(segs, c, L, false, st)) != ISM_OK) return r;
+  if (!pre && (r = build_pass_meta(segs, c, L, false, st, pairs_first(shape))) != ISM_OK) return r;
 
   AttnArgs a{};
   a.q = q; a.k = k; a.v = v; a.out = o; a.lse = lse;
@@ -552,6 +562,10 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.qk_descale = qk_descale; a.v_descale = v_descale;
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
   a.pair_order = L.pair_order; a.npairs = L.pair_order ? c.npairs : 0;
+  if (use_tc(shape) && shape->head_dim == 64 && pairs_first(shape)) {
+    a.pair_order = L.q_order;
+    a.npairs = c.npairs;
+  }
   a.status = status;
   a.flags = tc_flags();
   timer_begin(ISM_KERNEL_FWD, st);
@@ -736,7 +750,7 @@ ism_status_t ism_attn_plan_build(const ism_segments_t* segs, const ism_attn_shap
   if ((r = check_ws(plan, plan_bytes, L.bytes)) != ISM_OK) return r;
   if (info.total_tokens > 0) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if ((r = build_pass_meta(segs, c, L, true, st)) != ISM_OK) return r;
+    if ((r = build_pass_meta(segs, c, L, true, st, pairs_first(shape))) != ISM_OK) return r;
   }
   plan_info->fingerprint = plan_fingerprint(segs, shape, tile_pairs);
   plan_info->bytes = L.bytes;
@@ -1047,14 +1061,12 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order;
   a.nq = (int64_t)batch * ((l_new + kTile - 1) / kTile);
   a.pages = cg.pages;
-  if (shape->dtype == ISM_E4M3) {
-    // the e4m3 forward is the paired kernel: neighbouring q-tiles for an odd group
-    a.qk_descale = qk_descale;
-    a.v_descale = v_descale;
-    if ((hq / hkv) % 2) {
-      a.pair_order = L.pair_order;
-      a.npairs = L.npairs;
-    }
+  a.qk_descale = qk_descale;
+  a.v_descale = v_descale;
+  if ((shape->dtype == ISM_E4M3 || d == 64) && (hq / hkv) % 2) {
+    // e4m3 and head_dim 64 run only the paired kernel: neighbouring q-tiles for an odd group
+    a.pair_order = L.pair_order;
+    a.npairs = L.npairs;
   }
   a.status = status;
   a.flags = tc_flags();

@@ -11,6 +11,11 @@
 //                  dP^T = V dO^T (TMEM), P^T and dS^T back into TMEM (A operands
 //                  of the next MMAs), dV += P^T dO, dK += dS^T Q (TMEM
 //                  accumulators); dK = scale * dK.
+// Each kernel is a template over head_dim 128 and 64.  At 64 the recompute
+// schedule always runs; one layer of 16 heads over three dialogues (6001
+// tokens): dq_kernel 86 us, dkdv_kernel 118 us, against 78.8 and 79.9 ms of the
+// CUDA-core kernels they replace there.  An iteration is then 2 x 4 MMA steps
+// over the head dimension and 16 a contraction with a split operand.
 // Warp roles in both MMA kernels: warps 0..7 compute (two warpgroups, each
 // owning 64 of the 128 columns of a tile; thread = TMEM lane = tile row),
 // warp 8 loads (TMA), warp 9 owns TMEM and issues the MMAs.
@@ -32,27 +37,55 @@ __device__ __forceinline__ void ld64(uint32_t taddr, uint32_t (&a)[32], uint32_t
   ptx::tmem_ld32(taddr + 32, b);
 }
 
+// One 128 x kHD tile: 64-column boxes of 128 rows.
+template <int kHD>
+__device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int32_t x, int32_t y) {
+  ptx::tma_load_2d(dst, map, bar, x, y);
+  if constexpr (kHD == 128) ptx::tma_load_2d(dst + kHalfBytes, map, bar, x + 64, y);
+}
+// D = A B^T over the head dimension (both operands K-major in shared memory).
+template <int kHD>
+__device__ __forceinline__ void mma_head_dim(uint32_t d, uint32_t sA, uint32_t sB, uint32_t idesc) {
+  if constexpr (kHD == 128)
+    ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(d, desc_kmajor(sA, 0), desc_kmajor(sB, 0), idesc, 0u);
+  else
+    ptx::mma4_bf16_ss_warp<2, 2>(d, desc_kmajor(sA, 0), desc_kmajor(sB, 0), idesc, 0u);
+}
+// D += A B with A (128 x 128, bf16 pairs in tensor memory, 64 elements at
+// columns [0, 32) and 64 at [64, 96)) and B MN-major in shared memory.  At
+// head_dim 64 A also has a low part 32 columns on: P and dS keep 16 mantissa
+// bits there (hi = bf16(x), lo = bf16(x - hi)), because the results of that
+// head size are to be those of fp32 P and dS to within the output rounding.
+template <int kHD>
+__device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t sB, uint32_t idesc, uint32_t acc) {
+  ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(d, tA, desc_mnmajor(sB, 0), idesc, acc);
+  if constexpr (kHD == 64)
+    ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(d, tA + 32, desc_mnmajor(sB, 0), idesc, 1u);
+}
+
 // ------------------------------------------------------------------ delta
-// One 16-lane group per (row, head): 8 bf16 per lane, D = 128.  A group takes
+// One group of kHD / 8 lanes per (row, head): 8 bf16 per lane.  A group takes
 // four (row, head) pairs per round with all eight loads issued before any
 // use (more bytes in flight per thread: the kernel only streams O and dO).
-// The reductions shuffle within the group's own 16 lanes, so the two groups
-// of a warp may run different numbers of rounds.
+// The reductions shuffle within the group's own lanes, so the groups of a
+// warp may run different numbers of rounds.
+template <int kHD>
 __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
                              float* __restrict__ delta, int64_t rows, int hq) {
   constexpr int kUnroll = 4;
   const int64_t n = rows * hq;
-  const int sub = threadIdx.x & 15;
-  const uint32_t group_mask = 0xFFFFu << (threadIdx.x & 16);
-  const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 4;
-  for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4; i0 < n; i0 += groups * kUnroll) {
+  constexpr int kLanes = kHD / 8;
+  const int sub = threadIdx.x % kLanes;
+  const uint32_t group_mask = ((1u << kLanes) - 1u) << (threadIdx.x & 31 & ~(kLanes - 1));
+  const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / kLanes;
+  for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes; i0 < n; i0 += groups * kUnroll) {
     uint4 a[kUnroll], b[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int64_t i = i0 + u * groups;
       if (i < n) {
-        a[u] = reinterpret_cast<const uint4*>(O + i * kD)[sub];
-        b[u] = reinterpret_cast<const uint4*>(dO + i * kD)[sub];
+        a[u] = reinterpret_cast<const uint4*>(O + i * kHD)[sub];
+        b[u] = reinterpret_cast<const uint4*>(dO + i * kHD)[sub];
       }
     }
 #pragma unroll
@@ -68,7 +101,7 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
         acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
       }
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(group_mask, acc, o);
+      for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(group_mask, acc, o);
       if (sub == 0) {
         const int64_t row = i / hq;
         const int h = (int)(i % hq);
@@ -86,9 +119,12 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
 // scores are turned into dS.
 namespace dq {
 constexpr int kKStages = 3;
-constexpr uint32_t OFF_Q = 0, OFF_DO = kTileBytes, OFF_K = 2 * kTileBytes, OFF_V = 5 * kTileBytes,
-                   OFF_BAR = 7 * kTileBytes;
-constexpr uint32_t kSmemBytes = OFF_BAR + 256 + 1024;
+template <int kHD>
+struct Layout {
+  static constexpr uint32_t TB = kHD / 64 * kHalfBytes;
+  static constexpr uint32_t Q = 0, DO = TB, K = 2 * TB, V = 5 * TB, BAR = 7 * TB;
+  static constexpr uint32_t kSmemBytes = BAR + 256 + 1024;
+};
 constexpr uint32_t TM_S = 0, TM_DP = 256, TM_DQ = 384;  // S regions at 0 and 128
 
 struct Bars {
@@ -106,13 +142,15 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
+template <int kHD>
 __global__ void __launch_bounds__(kThreads, 1)
     dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
               const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
   using namespace dq;
+  using L = Layout<kHD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  Bars* bar = reinterpret_cast<Bars*>(smem + OFF_BAR);
+  Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t tpos;
   int h;
@@ -156,11 +194,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::tma_prefetch_desc(&tmK);
         ptx::tma_prefetch_desc(&tmV);
         const int32_t qy = w.q_base + w.tile * kRows;
-        ptx::mbar_expect_tx(&bar->qdo_full, 2 * kTileBytes);
-        ptx::tma_load_2d(smem + OFF_Q, &tmQ, &bar->qdo_full, h * kD, qy);
-        ptx::tma_load_2d(smem + OFF_Q + kHalfBytes, &tmQ, &bar->qdo_full, h * kD + 64, qy);
-        ptx::tma_load_2d(smem + OFF_DO, &tmdO, &bar->qdo_full, h * kD, qy);
-        ptx::tma_load_2d(smem + OFF_DO + kHalfBytes, &tmdO, &bar->qdo_full, h * kD + 64, qy);
+        ptx::mbar_expect_tx(&bar->qdo_full, 2 * L::TB);
+        load_tile<kHD>(smem + L::Q, &tmQ, &bar->qdo_full, h * kHD, qy);
+        load_tile<kHD>(smem + L::DO, &tmdO, &bar->qdo_full, h * kHD, qy);
       }
       __syncwarp();
       uint32_t nk[kKStages] = {0, 0, 0}, nv[2] = {0, 0};
@@ -173,9 +209,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         if (lane == 0) {
-          ptx::mbar_expect_tx(&bar->k_full[sk], kTileBytes);
-          ptx::tma_load_2d(smem + OFF_K + sk * kTileBytes, &tmK, &bar->k_full[sk], g * kD, ky);
-          ptx::tma_load_2d(smem + OFF_K + sk * kTileBytes + kHalfBytes, &tmK, &bar->k_full[sk], g * kD + 64, ky);
+          ptx::mbar_expect_tx(&bar->k_full[sk], L::TB);
+          load_tile<kHD>(smem + L::K + sk * L::TB, &tmK, &bar->k_full[sk], g * kHD, ky);
         }
         __syncwarp();
         ++nk[sk];
@@ -184,9 +219,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         if (lane == 0) {
-          ptx::mbar_expect_tx(&bar->v_full[sv], kTileBytes);
-          ptx::tma_load_2d(smem + OFF_V + sv * kTileBytes, &tmV, &bar->v_full[sv], g * kD, ky);
-          ptx::tma_load_2d(smem + OFF_V + sv * kTileBytes + kHalfBytes, &tmV, &bar->v_full[sv], g * kD + 64, ky);
+          ptx::mbar_expect_tx(&bar->v_full[sv], L::TB);
+          load_tile<kHD>(smem + L::V + sv * L::TB, &tmV, &bar->v_full[sv], g * kHD, ky);
         }
         __syncwarp();
         ++nv[sv];
@@ -203,29 +237,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the whole warp runs the loop, one elected lane issues each instruction
     if (nkb > 0) {
       constexpr uint32_t idesc_nt = ptx::idesc_bf16_f32(128, 128, 0, 0);  // A K-major, B K-major
-      constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, 128, 0, 1);  // A K-major, B MN-major
-      const uint32_t sQ = ptx::smem_u32(smem + OFF_Q), sdO = ptx::smem_u32(smem + OFF_DO);
+      constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, kHD, 0, 1);  // A K-major, B MN-major
+      const uint32_t sQ = ptx::smem_u32(smem + L::Q), sdO = ptx::smem_u32(smem + L::DO);
       auto issue_s = [&](int c) {
-        const uint32_t sK = ptx::smem_u32(smem + OFF_K + (c % kKStages) * kTileBytes);
-        ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tmem + TM_S + 128u * (c & 1), desc_kmajor(sQ, 0),
-                                                                  desc_kmajor(sK, 0), idesc_nt, 0u);
+        const uint32_t sK = ptx::smem_u32(smem + L::K + (c % kKStages) * L::TB);
+        mma_head_dim<kHD>(tmem + TM_S + 128u * (c & 1), sQ, sK, idesc_nt);
         ptx::mma_commit_warp(&bar->s_full[c & 1]);
       };
       auto issue_dp = [&](int c) {
         const int sv = c & 1;
-        const uint32_t sV = ptx::smem_u32(smem + OFF_V + sv * kTileBytes);
-        ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tmem + TM_DP, desc_kmajor(sdO, 0), desc_kmajor(sV, 0),
-                                                                  idesc_nt, 0u);
+        const uint32_t sV = ptx::smem_u32(smem + L::V + sv * L::TB);
+        mma_head_dim<kHD>(tmem + TM_DP, sdO, sV, idesc_nt);
         ptx::mma_commit_warp(&bar->dp_full);
         ptx::mma_commit_warp(&bar->v_empty[sv]);
       };
       auto issue_dq = [&](int c) {
         const int R = c & 1;
-        const uint32_t sK = ptx::smem_u32(smem + OFF_K + (c % kKStages) * kTileBytes);
+        const uint32_t sK = ptx::smem_u32(smem + L::K + (c % kKStages) * L::TB);
         // dQ += dS K_c: dS (bf16, keys packed two per column) in S region R, keys [0,64) at
         // columns [0,32) and [64,128) at columns [64,96)
-        ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(tmem + TM_DQ, tmem + TM_S + 128u * R,
-                                                                      desc_mnmajor(sK, 0), idesc_nn, c > 0 ? 1u : 0u);
+        mma_tile_rows<kHD>(tmem + TM_DQ, tmem + TM_S + 128u * R, sK, idesc_nn, c > 0 ? 1u : 0u);
         ptx::mma_commit_warp(&bar->dq_done[R]);
         ptx::mma_commit_warp(&bar->k_empty[c % kKStages]);
       };
@@ -316,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::tc_fence_before();
       ptx::mbar_arrive(&bar->dp_read);
       const int lim = (c < kfull) ? 128 : ke - c * kRows - wg * 64;  // visible columns of this half
-      uint32_t pk[32];  // pk[k] holds columns 2k and 2k+1 of this half
+      uint32_t pk[32], plo[kHD == 64 ? 32 : 1];  // pk[k] holds columns 2k and 2k+1 of this half
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         float v[2];
@@ -329,9 +360,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           v[e] = p * (dv - dl);
         }
         pk[k] = pack_bf16(v[0], v[1]);
+        if constexpr (kHD == 64) plo[k] = pack_bf16_rest(v[0], v[1], pk[k]);
       }
       // dS over the first 32 columns of this half of S (already read)
       ptx::tmem_st32(tS, pk);
+      if constexpr (kHD == 64) ptx::tmem_st32(tS + 32, plo);
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
       ptx::mbar_arrive(&bar->p_full[R]);
@@ -339,20 +372,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     // rotary encoding: this warpgroup's 32 pairs of the row's tables, loaded
     // while the last dQ MMAs run
     float rc[32], rs[32];
-    if (valid && a.rope_cos) {
+    if (valid && a.rope_cos && wg < kHD / 64) {
       const int64_t pos = (int64_t)w.tile * kRows + r;
-      rope_row<32>(a.rope_cos + pos * 64 + wg * 32, a.rope_sin + pos * 64 + wg * 32, rc, rs);
+      rope_row<32>(a.rope_cos + pos * (kHD / 2) + wg * 32, a.rope_sin + pos * (kHD / 2) + wg * 32, rc, rs);
     }
     if (ok) ok = wait(&bar->final_mma, 0, a.status);
     if (!ok) {
       set_abort(&bar->abort);
-    } else {
+    } else if (wg < kHD / 64) {  // (64 columns: warpgroup 0 alone)
       ptx::tc_fence_after();
       uint32_t q0[32], q1[32];
       if (a.rope_cos) {
-        // rotary encoding: warpgroup wg takes columns wg*32.. and 64 + wg*32.., which pair up
+        // rotary encoding: warpgroup wg takes columns wg*32.. and kHD/2 + wg*32.., which pair up
         ptx::tmem_ld32(tmem + lane_addr + TM_DQ + wg * 32, q0);
-        ptx::tmem_ld32(tmem + lane_addr + TM_DQ + 64 + wg * 32, q1);
+        ptx::tmem_ld32(tmem + lane_addr + TM_DQ + kHD / 2 + wg * 32, q1);
       } else {
         ld64(tmem + lane_addr + TM_DQ + wg * 64, q0, q1);
       }
@@ -360,8 +393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::reg_fence(q0);
       ptx::reg_fence(q1);
       // rows are stored by groups of four lanes (store_slice32)
-      const int64_t rstride = (int64_t)a.hq * kD;
-      __nv_bfloat16* const g0 = reinterpret_cast<__nv_bfloat16*>(a.dq) + (grow - (lane & 3)) * rstride + h * kD;
+      const int64_t rstride = (int64_t)a.hq * kHD;
+      __nv_bfloat16* const g0 = reinterpret_cast<__nv_bfloat16*>(a.dq) + (grow - (lane & 3)) * rstride + h * kHD;
       const int g_rows = w.q_len - (row - (lane & 3));
       uint32_t w0[16], w1[16];
       if (a.rope_cos) {
@@ -371,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         rope_back_pack(q0, q1, a.scale, rc, rs, w0, w1);
         store_slice32(w0, g0 + 32 * wg, rstride, g_rows);
-        store_slice32(w1, g0 + 64 + 32 * wg, rstride, g_rows);
+        store_slice32(w1, g0 + kHD / 2 + 32 * wg, rstride, g_rows);
       } else {
         pack_scaled32(q0, a.scale, w0);
         pack_scaled32(q1, a.scale, w1);
@@ -395,12 +428,15 @@ namespace dkv {
 // memory over the S^T it came from and dS^T over the dP^T it came from, so dV
 // can start as soon as P is written and dP^T of the next tile only waits for dK.
 constexpr int kQStages = 3;
-constexpr uint32_t OFF_K = 0, OFF_V = kTileBytes, OFF_Q = 2 * kTileBytes, OFF_DO = 5 * kTileBytes,
-                   OFF_META = 7 * kTileBytes;
 // per stage: lse2[128] f32, delta[128] f32, visible-key count[128] u8
 constexpr uint32_t kMetaStage = 128 * 4 + 128 * 4 + 128;
-constexpr uint32_t OFF_BAR = OFF_META + 2 * kMetaStage;
-constexpr uint32_t kSmemBytes = OFF_BAR + 512;  // needs a 1024-aligned dynamic shared base
+template <int kHD>
+struct Layout {
+  static constexpr uint32_t TB = kHD / 64 * kHalfBytes;
+  static constexpr uint32_t K = 0, V = TB, Q = 2 * TB, DO = 5 * TB, META = 7 * TB;
+  static constexpr uint32_t BAR = META + 2 * kMetaStage;
+  static constexpr uint32_t kSmemBytes = BAR + 512;  // needs a 1024-aligned dynamic shared base
+};
 constexpr uint32_t TM_S = 0, TM_DP = 128, TM_DV = 256, TM_DK = 384;
 // warps 0-7 compute, 8 work items + TMA loads, 9 TMEM + MMA issue, 10 per-query metadata
 constexpr int kLoadWarp = 8, kMmaWarp = 9, kMetaWarp = 10;
@@ -418,16 +454,18 @@ struct Bars {
   int32_t items[kItemSlots];
 };
 static_assert(sizeof(Bars) <= 512, "barrier block");
-static_assert(kSmemBytes <= 232448, "shared memory per CTA");
+static_assert(Layout<128>::kSmemBytes <= 232448, "shared memory per CTA");
 }  // namespace dkv
 
+template <int kHD>
 __global__ void __launch_bounds__(dkv::kThreads, 1)
     dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
                 const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
   using namespace dkv;
+  using L = Layout<kHD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
-  Bars* bar = reinterpret_cast<Bars*>(smem + OFF_BAR);
+  Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (ptx::smem_u32(smem) & 1023u) {  // the swizzled tiles need 1024-byte alignment
     if (threadIdx.x == 0) atomicOr(a.status, kStatusSmemAlign);
@@ -524,10 +562,10 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           for (int rr = lane; rr < kRows; rr += 32) {
             const int key = x.c * kRows + rr;
             if (key >= x.w.k_len) break;
-            const int64_t off = ((int64_t)x.w.k_base + key) * a.hkv * kD + x.g * kD;
+            const int64_t off = ((int64_t)x.w.k_base + key) * a.hkv * kHD + x.g * kHD;
             uint4* dk = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.dk) + off);
             uint4* dv = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.dv) + off);
-            for (int k = 0; k < kD / 8; ++k) dk[k] = dv[k] = make_uint4(0u, 0u, 0u, 0u);
+            for (int k = 0; k < kHD / 8; ++k) dk[k] = dv[k] = make_uint4(0u, 0u, 0u, 0u);
           }
           continue;
         }
@@ -551,11 +589,9 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
       }
       const int32_t ky = x.w.k_base + x.c * kRows;
       if (lane == 0) {
-        ptx::mbar_expect_tx(&bar->kv_full, 2 * kTileBytes);
-        ptx::tma_load_2d(smem + OFF_K, &tmK, &bar->kv_full, x.g * kD, ky);
-        ptx::tma_load_2d(smem + OFF_K + kHalfBytes, &tmK, &bar->kv_full, x.g * kD + 64, ky);
-        ptx::tma_load_2d(smem + OFF_V, &tmV, &bar->kv_full, x.g * kD, ky);
-        ptx::tma_load_2d(smem + OFF_V + kHalfBytes, &tmV, &bar->kv_full, x.g * kD + 64, ky);
+        ptx::mbar_expect_tx(&bar->kv_full, 2 * L::TB);
+        load_tile<kHD>(smem + L::K, &tmK, &bar->kv_full, x.g * kHD, ky);
+        load_tile<kHD>(smem + L::V, &tmV, &bar->kv_full, x.g * kHD, ky);
       }
       __syncwarp();
       ++nkv;
@@ -567,9 +603,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         bool okq = I < kQStages || wait_warp(&bar->q_empty[sq], (I / kQStages - 1) & 1, a.status);
         if (okq) {
           if (lane == 0) {
-            ptx::mbar_expect_tx(&bar->q_full[sq], kTileBytes);
-            ptx::tma_load_2d(smem + OFF_Q + sq * kTileBytes, &tmQ, &bar->q_full[sq], h * kD, qy);
-            ptx::tma_load_2d(smem + OFF_Q + sq * kTileBytes + kHalfBytes, &tmQ, &bar->q_full[sq], h * kD + 64, qy);
+            ptx::mbar_expect_tx(&bar->q_full[sq], L::TB);
+            load_tile<kHD>(smem + L::Q + sq * L::TB, &tmQ, &bar->q_full[sq], h * kHD, qy);
           }
           __syncwarp();
           ++nq[sq];
@@ -577,9 +612,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         }
         if (okq) {
           if (lane == 0) {
-            ptx::mbar_expect_tx(&bar->do_full[s], kTileBytes);
-            ptx::tma_load_2d(smem + OFF_DO + s * kTileBytes, &tmdO, &bar->do_full[s], h * kD, qy);
-            ptx::tma_load_2d(smem + OFF_DO + s * kTileBytes + kHalfBytes, &tmdO, &bar->do_full[s], h * kD + 64, qy);
+            ptx::mbar_expect_tx(&bar->do_full[s], L::TB);
+            load_tile<kHD>(smem + L::DO + s * L::TB, &tmdO, &bar->do_full[s], h * kHD, qy);
           }
           __syncwarp();
           ++ndo[s];
@@ -611,7 +645,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         const int h = x.g * group + hh;
         if (aborted(&bar->abort)) break;
         if (I >= 2 && !wait(&bar->meta_empty[s], ((I >> 1) - 1) & 1, a.status)) { set_abort(&bar->abort); break; }
-        uint8_t* meta = smem + OFF_META + s * kMetaStage;
+        uint8_t* meta = smem + L::META + s * kMetaStage;
         float* mlse = reinterpret_cast<float*>(meta);
         float* mdel = mlse + 128;
         uint8_t* mlim = reinterpret_cast<uint8_t*>(mdel + 128);
@@ -642,33 +676,33 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
     // ------------------------------------------------ MMA issue (the whole warp runs the
     // loop, one elected lane issues each instruction)
     constexpr uint32_t idesc_nt = ptx::idesc_bf16_f32(128, 128, 0, 0);
-    constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, 128, 0, 1);
-    const uint32_t sK = ptx::smem_u32(smem + OFF_K), sV = ptx::smem_u32(smem + OFF_V);
+    constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, kHD, 0, 1);
+    const uint32_t sK = ptx::smem_u32(smem + L::K), sV = ptx::smem_u32(smem + L::V);
     uint32_t I0 = 0, nkv = 0;  // iterations of earlier items; items with K / V loaded
     bool ok = true;
     auto issue_s = [&](uint32_t gi) {
-      const uint32_t sQ = ptx::smem_u32(smem + OFF_Q + (gi % kQStages) * kTileBytes);
-      ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tmem + TM_S, desc_kmajor(sK, 0), desc_kmajor(sQ, 0), idesc_nt, 0u);
+      const uint32_t sQ = ptx::smem_u32(smem + L::Q + (gi % kQStages) * L::TB);
+      mma_head_dim<kHD>(tmem + TM_S, sK, sQ, idesc_nt);
       ptx::mma_commit_warp(&bar->s_full);
     };
     auto issue_dp = [&](uint32_t gi) {
-      const uint32_t sdO = ptx::smem_u32(smem + OFF_DO + (gi & 1) * kTileBytes);
-      ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tmem + TM_DP, desc_kmajor(sV, 0), desc_kmajor(sdO, 0), idesc_nt, 0u);
+      const uint32_t sdO = ptx::smem_u32(smem + L::DO + (gi & 1) * L::TB);
+      mma_head_dim<kHD>(tmem + TM_DP, sV, sdO, idesc_nt);
       ptx::mma_commit_warp(&bar->dp_full);
     };
     // P^T (bf16, two queries per column) sits in the S^T columns and dS^T in the dP^T
     // columns: warpgroup wg's queries [64 wg, 64 wg + 64) at column 64 wg + [0, 32)
     auto issue_dv = [&](uint32_t gi, bool first) {
       const uint32_t s = gi & 1;
-      const uint32_t sdO = ptx::smem_u32(smem + OFF_DO + s * kTileBytes);
-      ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(tmem + TM_DV, tmem + TM_S, desc_mnmajor(sdO, 0), idesc_nn, first ? 0u : 1u);
+      const uint32_t sdO = ptx::smem_u32(smem + L::DO + s * L::TB);
+      mma_tile_rows<kHD>(tmem + TM_DV, tmem + TM_S, sdO, idesc_nn, first ? 0u : 1u);
       ptx::mma_commit_warp(&bar->do_empty[s]);
       ptx::mma_commit_warp(&bar->dv_done);
     };
     auto issue_dk = [&](uint32_t gi, bool first) {
       const uint32_t sq = gi % kQStages;
-      const uint32_t sQ = ptx::smem_u32(smem + OFF_Q + sq * kTileBytes);
-      ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(tmem + TM_DK, tmem + TM_DP, desc_mnmajor(sQ, 0), idesc_nn, first ? 0u : 1u);
+      const uint32_t sQ = ptx::smem_u32(smem + L::Q + sq * L::TB);
+      mma_tile_rows<kHD>(tmem + TM_DK, tmem + TM_DP, sQ, idesc_nn, first ? 0u : 1u);
       ptx::mma_commit_warp(&bar->q_empty[sq]);
       ptx::mma_commit_warp(&bar->dk_done);
     };
@@ -774,12 +808,13 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           break;
         }
         ptx::tc_fence_after();
-        const uint8_t* meta = smem + OFF_META + s * kMetaStage;
+        const uint8_t* meta = smem + L::META + s * kMetaStage;
         const float4* mlse4 = reinterpret_cast<const float4*>(meta) + wg * 16;
         const float4* mdel4 = reinterpret_cast<const float4*>(meta + 512) + wg * 16;
         const uint32_t* mlim4 = reinterpret_cast<const uint32_t*>(meta + 1024) + wg * 16;
         // phase 1: P from S^T (dP^T may still be in flight)
         uint32_t pp[32];  // pp[k]: queries 64 wg + 2k, 64 wg + 2k + 1 (bf16)
+        float pf[kHD == 64 ? 64 : 1];  // P itself (head_dim 64)
         {
           uint32_t sv[2][32];
           ld64(tS, sv[0], sv[1]);
@@ -797,8 +832,12 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
                                       make_float2(-l4.x, -l4.y));
               const float2 a23 = fma2(make_float2(__uint_as_float(sq[2]), __uint_as_float(sq[3])), sl2x2,
                                       make_float2(-l4.z, -l4.w));
-              pp[q4 * 2] = pack_bf16(ex2(a01.x), ex2(a01.y));
-              pp[q4 * 2 + 1] = pack_bf16(ex2(a23.x), ex2(a23.y));
+              const float p[4] = {ex2(a01.x), ex2(a01.y), ex2(a23.x), ex2(a23.y)};
+              pp[q4 * 2] = pack_bf16(p[0], p[1]);
+              pp[q4 * 2 + 1] = pack_bf16(p[2], p[3]);
+              if constexpr (kHD == 64)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) pf[q4 * 4 + e] = p[e];
             }
           } else {
 #pragma unroll
@@ -814,11 +853,20 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
               }
               pp[q4 * 2] = pack_bf16(p[0], p[1]);
               pp[q4 * 2 + 1] = pack_bf16(p[2], p[3]);
+              if constexpr (kHD == 64)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) pf[q4 * 4 + e] = p[e];
             }
           }
         }
         // P^T over this warpgroup's (already read) S^T columns; dV may start
         ptx::tmem_st32(tS, pp);
+        if constexpr (kHD == 64) {
+          uint32_t lo[32];
+#pragma unroll
+          for (int k = 0; k < 32; ++k) lo[k] = pack_bf16_rest(pf[2 * k], pf[2 * k + 1], pp[k]);
+          ptx::tmem_st32(tS + 32, lo);
+        }
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
         ptx::mbar_arrive(&bar->pt_full);
@@ -833,7 +881,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         // phase 2: dS from dP^T
         if (!wait(&bar->dp_full, I & 1, a.status)) { ok = false; break; }
         ptx::tc_fence_after();
-        uint32_t pd[32];
+        uint32_t pd[32], pdl[kHD == 64 ? 32 : 1];
         {
           uint32_t dv[2][32];
           ld64(tP, dv[0], dv[1]);
@@ -843,25 +891,38 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
 #pragma unroll
           for (int q4 = 0; q4 < 16; ++q4) {
             const float4 d4 = mdel4[q4];
-            const uint32_t w0 = pp[q4 * 2], w1 = pp[q4 * 2 + 1];
             const int b = (q4 & 7) * 4, hv = q4 >> 3;
-            const float2 v01 = mul2(make_float2(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u)),
+            float2 p01, p23;
+            if constexpr (kHD == 64) {
+              p01 = make_float2(pf[q4 * 4], pf[q4 * 4 + 1]);
+              p23 = make_float2(pf[q4 * 4 + 2], pf[q4 * 4 + 3]);
+            } else {
+              const uint32_t w0 = pp[q4 * 2], w1 = pp[q4 * 2 + 1];
+              p01 = make_float2(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u));
+              p23 = make_float2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xFFFF0000u));
+            }
+            const float2 v01 = mul2(p01,
                                     add2(make_float2(__uint_as_float(dv[hv][b + 0]), __uint_as_float(dv[hv][b + 1])),
                                          make_float2(-d4.x, -d4.y)));
-            const float2 v23 = mul2(make_float2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xFFFF0000u)),
+            const float2 v23 = mul2(p23,
                                     add2(make_float2(__uint_as_float(dv[hv][b + 2]), __uint_as_float(dv[hv][b + 3])),
                                          make_float2(-d4.z, -d4.w)));
             pd[q4 * 2] = pack_bf16(v01.x, v01.y);
             pd[q4 * 2 + 1] = pack_bf16(v23.x, v23.y);
+            if constexpr (kHD == 64) {
+              pdl[q4 * 2] = pack_bf16_rest(v01.x, v01.y, pd[q4 * 2]);
+              pdl[q4 * 2 + 1] = pack_bf16_rest(v23.x, v23.y, pd[q4 * 2 + 1]);
+            }
           }
         }
         ptx::mbar_arrive(&bar->meta_empty[s]);
         // dS^T over this warpgroup's (already read) dP^T columns
         ptx::tmem_st32(tP, pd);
+        if constexpr (kHD == 64) ptx::tmem_st32(tP + 32, pdl);
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
         ptx::mbar_arrive(&bar->p_full);
-        if (a.ds) {
+        if (kHD == 128 && a.ds) {
           // keep dS^T row r, queries [64 wg, 64 wg + 64), for the dQ GEMM, in
           // the 8-interleaved layout (16-byte unit (query group, key)): the 32
           // lanes of a warp store 512 contiguous bytes per instruction.  Issued
@@ -895,23 +956,23 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
       ptx::tc_fence_after();
       // rows are stored by groups of four lanes (store_slice32): the group of
       // this lane starts at key - (lane & 3)
-      const int64_t rstride = (int64_t)a.hkv * kD;
+      const int64_t rstride = (int64_t)a.hkv * kHD;
       const int64_t grow = (int64_t)x.w.k_base + key - (lane & 3);
       const int g_rows = x.w.k_len - (key - (lane & 3));
-      __nv_bfloat16* const dvg = reinterpret_cast<__nv_bfloat16*>(a.dv) + grow * rstride + x.g * kD;
-      __nv_bfloat16* const dkg = reinterpret_cast<__nv_bfloat16*>(a.dk) + grow * rstride + x.g * kD;
+      __nv_bfloat16* const dvg = reinterpret_cast<__nv_bfloat16*>(a.dv) + grow * rstride + x.g * kHD;
+      __nv_bfloat16* const dkg = reinterpret_cast<__nv_bfloat16*>(a.dk) + grow * rstride + x.g * kHD;
       if (wg == 1 && a.rope_cos) {
 #pragma unroll 1
-        for (int q2 = 0; q2 < 2; ++q2) {
+        for (int q2 = 0; q2 < kHD / 64; ++q2) {
           uint32_t lo[32], hi[32];
           ptx::tmem_ld32(tmem + lane_addr + TM_DK + q2 * 32, lo);
-          ptx::tmem_ld32(tmem + lane_addr + TM_DK + 64 + q2 * 32, hi);
+          ptx::tmem_ld32(tmem + lane_addr + TM_DK + kHD / 2 + q2 * 32, hi);
           ptx::tmem_ld_wait();
           ptx::reg_fence(lo);
           ptx::reg_fence(hi);
           float rc[32], rs[32];
           if (kvalid) {
-            rope_row<32>(a.rope_cos + (int64_t)key * 64 + 32 * q2, a.rope_sin + (int64_t)key * 64 + 32 * q2, rc, rs);
+            rope_row<32>(a.rope_cos + (int64_t)key * (kHD / 2) + 32 * q2, a.rope_sin + (int64_t)key * (kHD / 2) + 32 * q2, rc, rs);
           } else {
 #pragma unroll
             for (int k = 0; k < 32; ++k) rc[k] = rs[k] = 0.f;
@@ -919,14 +980,14 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           uint32_t wl[16], wh[16];
           rope_back_pack(lo, hi, a.scale, rc, rs, wl, wh);
           store_slice32(wl, dkg + q2 * 32, rstride, g_rows);
-          store_slice32(wh, dkg + 64 + q2 * 32, rstride, g_rows);
+          store_slice32(wh, dkg + kHD / 2 + q2 * 32, rstride, g_rows);
         }
         ptx::tc_fence_before();
         continue;
       }
       // warpgroup 0 writes dV, warpgroup 1 writes dK (scaled)
 #pragma unroll 1
-      for (int q4 = 0; q4 < 4; ++q4) {
+      for (int q4 = 0; q4 < kHD / 32; ++q4) {
         uint32_t v[32], w[16];
         ptx::tmem_ld32(tmem + lane_addr + (wg == 0 ? TM_DV : TM_DK) + 32 * q4, v);
         ptx::tmem_ld_wait();
@@ -950,52 +1011,54 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
 
 cudaError_t launch_dkdv_pair(const AttnArgs& a, const CUtensorMap& tk, const CUtensorMap& tv, cudaStream_t st);
 
-cudaError_t launch_bwd(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
+template <int kHD>
+cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
   cudaError_t e;
   if (a.q_rows > 0) {
     int64_t groups = a.q_rows * a.hq;
-    int grid = (int)((groups * 16 + 255) / 256);
+    int grid = (int)((groups * (kHD / 8) + 255) / 256);
     if (grid > 152 * 16) grid = 152 * 16;
     timer_begin(ISM_KERNEL_BWD_PRE, st);
-    delta_kernel<<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows,
+    delta_kernel<kHD><<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows,
                                        a.hq);
     timer_end(ISM_KERNEL_BWD_PRE, st);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   CUtensorMap tq, tdo, tk, tv;
-  if ((e = make_tmap_bf16(&tq, a.q, (uint64_t)a.hq * kD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&tdo, a.dout, (uint64_t)a.hq * kD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&tk, a.k, (uint64_t)a.hkv * kD, (uint64_t)k_rows)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&tv, a.v, (uint64_t)a.hkv * kD, (uint64_t)k_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tq, a.q, (uint64_t)a.hq * kHD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tdo, a.dout, (uint64_t)a.hq * kHD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tk, a.k, (uint64_t)a.hkv * kHD, (uint64_t)k_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tv, a.v, (uint64_t)a.hkv * kHD, (uint64_t)k_rows)) != cudaSuccess) return e;
   // Recompute path: dQ recomputes S, P and dP itself and runs before dK/dV.
   // Stored-dS path: dK/dV writes the dS^T tiles, then dQ is a GEMM over them.
   if (a.nq && !a.ds) {
-    if ((e = cudaFuncSetAttribute(dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dq::kSmemBytes)) !=
+    if ((e = cudaFuncSetAttribute(dq_kernel<kHD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)dq::Layout<kHD>::kSmemBytes)) !=
         cudaSuccess)
       return e;
     timer_begin(ISM_KERNEL_BWD_DQ, st);
-    dq_kernel<<<(unsigned)(a.nq * a.hq), kThreads, dq::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
+    dq_kernel<kHD><<<(unsigned)(a.nq * a.hq), kThreads, dq::Layout<kHD>::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
     timer_end(ISM_KERNEL_BWD_DQ, st);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (a.nk && knobs().dkdv_pair && a.kp_order) {
+  if (kHD == 128 && a.nk && knobs().dkdv_pair && a.kp_order) {
     // the CTA-pair kernel (ism_dkdv2_tc.cu)
     timer_begin(ISM_KERNEL_BWD_DKDV, st);
     if ((e = launch_dkdv_pair(a, tk, tv, st)) != cudaSuccess) return e;
     timer_end(ISM_KERNEL_BWD_DKDV, st);
     count_launch();
   } else if (a.nk) {
-    if ((e = cudaFuncSetAttribute(dkdv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)dkv::kSmemBytes)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(dkdv_kernel<kHD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)dkv::Layout<kHD>::kSmemBytes)) != cudaSuccess)
       return e;
     // persistent: one CTA per SM takes (k-tile, KV head) items from the work counter
     int64_t grid = knobs().dkdv_grid > 0 ? knobs().dkdv_grid : sm_count();
     if (grid > a.nk * a.hkv) grid = a.nk * a.hkv;
     if (!a.work_counter) return cudaErrorInvalidValue;
     timer_begin(ISM_KERNEL_BWD_DKDV, st);
-    dkdv_kernel<<<(unsigned)grid, dkv::kThreads, dkv::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
+    dkdv_kernel<kHD><<<(unsigned)grid, dkv::kThreads, dkv::Layout<kHD>::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
     timer_end(ISM_KERNEL_BWD_DKDV, st);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1007,6 +1070,10 @@ cudaError_t launch_bwd(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
     count_launch();
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_bwd(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
+  return a.d == 64 ? launch_bwd_t<64>(a, k_rows, st) : launch_bwd_t<128>(a, k_rows, st);
 }
 
 }  // namespace tc

@@ -557,10 +557,10 @@ cudaError_t launch_fwd(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
     if ((e = make_tmap_e4m3(&tv, a.v, (uint64_t)a.hkv * kD, (uint64_t)k_rows)) != cudaSuccess) return e;
     return launch_fwd_pair(a, tq, tk, tv, st);
   }
-  if ((e = make_tmap_bf16(&tq, a.q, (uint64_t)a.hq * kD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&tk, a.k, (uint64_t)a.hkv * kD, (uint64_t)k_rows)) != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&tv, a.v, (uint64_t)a.hkv * kD, (uint64_t)k_rows)) != cudaSuccess) return e;
-  if (((a.hq / a.hkv) % 2 == 0 || a.pair_order) && !knobs().fwd_one_head)
+  if ((e = make_tmap_bf16(&tq, a.q, (uint64_t)a.hq * a.d, (uint64_t)a.q_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tk, a.k, (uint64_t)a.hkv * a.d, (uint64_t)k_rows)) != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&tv, a.v, (uint64_t)a.hkv * a.d, (uint64_t)k_rows)) != cudaSuccess) return e;
+  if (a.d == 64 || (((a.hq / a.hkv) % 2 == 0 || a.pair_order) && !knobs().fwd_one_head))
     return launch_fwd_pair(a, tq, tk, tv, st);
   if ((e = cudaFuncSetAttribute(fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) !=
       cudaSuccess)

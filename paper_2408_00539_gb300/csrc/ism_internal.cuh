@@ -83,11 +83,12 @@ cudaError_t launch_order(const Tile* qtiles, int64_t nq, const Tile* ktiles, int
                          int32_t* q_order, int32_t* k_order, cudaStream_t st, int32_t* pair_order = nullptr);
 cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_off, cudaStream_t st);
 // kv_end, tiles, work lists (and pair offsets when kpair_off is set, the
-// k-tile pair list when kp_order is set) in one launch.
+// k-tile pair list when kp_order is set) in one launch.  pairs_first: q_order
+// starts with the even-indexed q-tiles (pair heads, in the pair list's order).
 cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, int64_t nq, int64_t nk,
                              Tile* qtiles, Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order,
                              int32_t* pair_order, int32_t* kpair_off, int32_t* counters, int n_counters,
-                             cudaStream_t st, int32_t* kp_order = nullptr);
+                             cudaStream_t st, int32_t* kp_order = nullptr, bool pairs_first = false);
 // k_base of sequence b's tiles = b * kbase_stride (the cache capacity, or 1 for a paged cache)
 cudaError_t launch_append_plan(const AppendSegs& segs, int batch, int64_t kbase_stride, int bm, int bn,
                                int32_t* cache_len, int32_t* c_snap, int32_t* kv_end, Tile* qtiles,

@@ -185,27 +185,38 @@ __device__ __forceinline__ bool pair_head(const Tile* qtiles, int64_t nq, int64_
   return true;
 }
 
+// pairs_first: q_order lists the pair heads of the third list first (in its
+// order), then the odd-indexed q-tiles; the forward of an odd group at
+// head_dim 64 reads its pairs from there.
 __device__ void order_body(const Tile* __restrict__ qtiles, int64_t nq, const Tile* __restrict__ ktiles, int64_t nk,
                            int max_cost, int32_t* q_order, int32_t* k_order, int32_t* pair_order, int32_t* hist,
-                           int32_t* kp_order = nullptr) {
-  for (int pass = 0; pass < 4; ++pass) {
-    const Tile* items = pass == 1 || pass == 3 ? ktiles : qtiles;
-    int64_t n = pass == 1 || pass == 3 ? nk : nq;
-    int32_t* order = pass == 0 ? q_order : pass == 1 ? k_order : pass == 2 ? pair_order : kp_order;
+                           int32_t* kp_order = nullptr, bool pairs_first = false) {
+  int32_t heads = 0;  // pair heads listed at the front of q_order (pairs_first)
+  for (int pass = 0; pass < 5; ++pass) {
+    const bool keys = pass == 1 || pass == 3;
+    const Tile* items = keys ? ktiles : qtiles;
+    const int64_t n = keys ? nk : nq;
+    int32_t* order = pass == 0 ? q_order : pass == 1 ? k_order : pass == 2 ? pair_order : pass == 3 ? kp_order
+                     : pairs_first && q_order ? q_order + heads : nullptr;
     if (items == nullptr || order == nullptr || n == 0) continue;
+    // cost of item i in this pass (false: not listed in it)
+    auto cost_of = [&](int64_t i, int* cost) -> bool {
+      if (pass == 2 || (pass == 0 && pairs_first)) {
+        if (!pair_head(items, n, i, cost)) return false;
+      } else {
+        const Tile w = items[i];
+        if (pass == 3 && (w.tile & 1)) return false;   // k-tile pairs: the even tile, costed by its query tiles
+        if (pass == 4 && !(w.tile & 1)) return false;  // the odd q-tiles
+        *cost = keys ? w.a1 - w.a0 : w.a1;
+      }
+      *cost = min(max(*cost, 0), max_cost);
+      return true;
+    };
     for (int i = threadIdx.x; i <= max_cost; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
       int cost;
-      if (pass == 2) {
-        if (!pair_head(items, n, i, &cost)) continue;
-      } else {
-        const Tile w = items[i];
-        if (pass == 3 && (w.tile & 1)) continue;  // k-tile pairs: the even tile, costed by its query tiles
-        cost = pass == 0 ? w.a1 : w.a1 - w.a0;
-      }
-      cost = min(max(cost, 0), max_cost);
-      atomicAdd(&hist[cost], 1);
+      if (cost_of(i, &cost)) atomicAdd(&hist[cost], 1);
     }
     __syncthreads();
     // exclusive scan from the highest cost down (each thread rewrites the
@@ -219,18 +230,11 @@ __device__ void order_body(const Tile* __restrict__ qtiles, int64_t nq, const Ti
       if (c >= 0) hist[c] = run + incl - h;
       run += tot;
     }
+    if (pass == 0) heads = run;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
       int cost;
-      if (pass == 2) {
-        if (!pair_head(items, n, i, &cost)) continue;
-      } else {
-        const Tile w = items[i];
-        if (pass == 3 && (w.tile & 1)) continue;  // k-tile pairs: the even tile, costed by its query tiles
-        cost = pass == 0 ? w.a1 : w.a1 - w.a0;
-      }
-      cost = min(max(cost, 0), max_cost);
-      order[atomicAdd(&hist[cost], 1)] = (int32_t)i;
+      if (cost_of(i, &cost)) order[atomicAdd(&hist[cost], 1)] = (int32_t)i;
     }
     __syncthreads();
   }
@@ -272,7 +276,7 @@ __global__ void pair_offsets_kernel(const Tile* __restrict__ ktiles, int64_t nk,
 __global__ void __launch_bounds__(1024)
     pass_meta_kernel(SegsDev s, int32_t* kv_end, int bm, int bn, int64_t nq, int64_t nk, Tile* qtiles,
                      Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order, int32_t* pair_order,
-                     int32_t* kpair_off, int32_t* counters, int n_counters, int32_t* kp_order) {
+                     int32_t* kpair_off, int32_t* counters, int n_counters, int32_t* kp_order, bool pairs_first) {
   extern __shared__ __align__(16) unsigned char dyn[];
   if ((int)threadIdx.x < n_counters) counters[threadIdx.x] = 0;  // work counters of the kernels that follow
   // kv_end: one warp per segment, lanes over its tokens
@@ -289,7 +293,7 @@ __global__ void __launch_bounds__(1024)
   tiles_body(s, bm, bn, kv_end, nq, nk, qtiles, ktiles, nullptr, nullptr, nullptr, nullptr, dyn);
   __syncthreads();
   order_body(qtiles, nq, ktiles, nk, max_cost, q_order, k_order, pair_order, reinterpret_cast<int32_t*>(dyn),
-             kp_order);
+             kp_order, pairs_first);
   if (kpair_off) pair_offsets_body(ktiles, nk, kpair_off);
 }
 
@@ -560,7 +564,7 @@ cudaError_t launch_order(const Tile* qtiles, int64_t nq, const Tile* ktiles, int
 cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, int64_t nq, int64_t nk,
                              Tile* qtiles, Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order,
                              int32_t* pair_order, int32_t* kpair_off, int32_t* counters, int n_counters,
-                             cudaStream_t st, int32_t* kp_order) {
+                             cudaStream_t st, int32_t* kp_order, bool pairs_first) {
   size_t a = (size_t)(s.num_seqs + 1) * (sizeof(int64_t) + 2 * sizeof(int32_t));
   size_t b = sizeof(int32_t) * (size_t)(max_cost + 1);
   size_t smem = a > b ? a : b;
@@ -572,7 +576,7 @@ cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, 
     if (e != cudaSuccess) return e;
   }
   pass_meta_kernel<<<1, 1024, smem, st>>>(s, kv_end, bm, bn, nq, nk, qtiles, ktiles, max_cost, q_order, k_order,
-                                          pair_order, kpair_off, counters, n_counters, kp_order);
+                                          pair_order, kpair_off, counters, n_counters, kp_order, pairs_first);
   return cudaGetLastError();
 }
 

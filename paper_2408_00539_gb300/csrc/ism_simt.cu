@@ -1,5 +1,5 @@
-// CUDA-core attention under the ISM mask: the fp32 path (and the fallback
-// for head sizes the tensor-core kernels do not take).  fp32 arithmetic with
+// CUDA-core attention under the ISM mask: the fp32 path (and bf16 under
+// ISM_FORCE_CUDA_CORES=1).  fp32 arithmetic with
 // natural-base exponentials throughout.
 //
 // Forward (Eq. e_ISM with softmax): one warp per query row, lanes over keys

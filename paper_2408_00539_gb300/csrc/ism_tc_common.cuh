@@ -98,6 +98,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
+// The part of (lo, hi) that the bf16 pair `packed` = pack_bf16(lo, hi) leaves
+// out, itself rounded to bf16: packed + rest carries 16 mantissa bits.  The
+// differences are exact in fp32.
+__device__ __forceinline__ uint32_t pack_bf16_rest(float lo, float hi, uint32_t packed) {
+  return pack_bf16(lo - __uint_as_float(packed << 16), hi - __uint_as_float(packed & 0xFFFF0000u));
+}
 // Four values as e4m3 (round to nearest, saturating), x0 in the lowest byte.
 __device__ __forceinline__ uint32_t pack_e4m3x4(float x0, float x1, float x2, float x3) {
   uint32_t r;

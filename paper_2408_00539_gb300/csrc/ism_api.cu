@@ -842,15 +842,22 @@ struct AppendLayout {
   float* part_o;
   float* part_ml;
   void* q_rot;  // rotated queries of a RoPE append (bf16 [batch * l_new, Hq, D]), else null
-  // partials of the forward's key-range split (prefill): up to split_cap items
-  float* part_fo;
-  float* part_fml;
-  int64_t split_cap;
-  size_t bytes;
+  // partials of the forward's key-range split (prefill), the last region: as
+  // many units as the caller's workspace holds
+  size_t part_off;
+  int32_t part_rows;   // rows of a unit's half
+  size_t bytes;        // what the call requires
+  size_t full_bytes;   // what the size query reports: partials for as many units as a split can use
 };
 
-// Forward items (query tile, head pair) that may run as two key-range halves.
-constexpr int64_t kMaxSplitItems = 256;
+// Key-range units of a split forward that the reported workspace holds, at most.
+constexpr int64_t kMaxSplitUnits = 512;
+
+// One-head items (query tile, head pair), or (query-tile pair, head) for an odd group.
+int64_t append_items(const ism_attn_shape_t* sh, int batch, int l_new, bool tile_pairs) {
+  const int64_t nqt = (l_new + kTile - 1) / kTile;
+  return batch * (tile_pairs ? (nqt + 1) / 2 * sh->num_heads_q : nqt * (sh->num_heads_q / 2));
+}
 
 AppendLayout append_layout(void* ws, const ism_attn_shape_t* sh, int batch, int l_new, bool rope = false) {
   Carve cv(ws);
@@ -870,17 +877,58 @@ AppendLayout append_layout(void* ws, const ism_attn_shape_t* sh, int batch, int 
     L.part_o = L.part_ml = nullptr;
   }
   L.q_rot = rope ? (void*)cv.take<__nv_bfloat16>((int64_t)batch * l_new * sh->num_heads_q * sh->head_dim) : nullptr;
+  L.part_off = (cv.off + 255) & ~size_t(255);
+  L.part_rows = l_new < kTile ? l_new : kTile;
+  // required: two halves of up to 256 head-pair items with whole tiles
   if (l_new > 1 && sh->num_heads_q % 2 == 0) {
-    const int64_t items = nqt * (sh->num_heads_q / 2);
-    L.split_cap = items < kMaxSplitItems ? items : kMaxSplitItems;
-    L.part_fo = cv.take<float>(L.split_cap * 2 * 2 * kTile * 128);
-    L.part_fml = cv.take<float>(L.split_cap * 2 * 2 * kTile * 2);
-  } else {
-    L.split_cap = 0;
-    L.part_fo = L.part_fml = nullptr;
+    int64_t items = nqt * (sh->num_heads_q / 2);
+    if (items > 256) items = 256;
+    cv.take<float>(items * 2 * 2 * kTile * 128);
+    cv.take<float>(items * 2 * 2 * kTile * 2);
   }
   L.bytes = ((cv.off + 255) & ~size_t(255)) + 256;
+  L.full_bytes = L.bytes;
+  if (l_new > 1 && sh->dtype != ISM_FP32) {
+    int64_t units = 32 * append_items(sh, batch, l_new, (sh->num_heads_q / sh->num_heads_kv) % 2 != 0);
+    if (units > kMaxSplitUnits) units = kMaxSplitUnits;
+    const size_t full = L.part_off + (size_t)units * 2 * L.part_rows * (sh->head_dim + 2) * sizeof(float) + 512;
+    if (full > L.full_bytes) L.full_bytes = full;
+  }
   return L;
+}
+
+// How a prefill's items are split over their key range.  All items cost about
+// the same (every row sees the whole cache), so with `items` below the SM
+// count every item is split, else those of the last, partial round; into the
+// number of parts that minimises the rounds of that part of the launch, at
+// ceil(tiles / parts) key tiles and about two tiles' time of start-up and
+// epilogue each, plus the merge (a dependent launch and the partials written
+// and read once, together at about 3 TB/s).  In units of a key tile, 1.46 us.
+// Measured: one 40-token query over 3000 keys (16 items of 24 tiles) forward
+// 51 us whole, 30 in two halves, 14 in eight parts, and a 6 us merge; 8 x 512
+// queries over 16384 keys (512 items of 132 tiles) 826 us a call whole, 770
+// with the last 56 split; 20 x 100 over 8000 keys 392 whole, 311 split.
+struct KeySplit {
+  int64_t items = 0;  // split items (the last ones); 0: none
+  int32_t parts = 1;
+};
+KeySplit plan_key_split(int64_t items, int64_t tiles, int rows, int head_dim, int64_t cap_units) {
+  const int64_t sms = sm_count();
+  KeySplit best;
+  const int64_t n = items < sms ? items : items % sms;
+  if (n == 0) return best;
+  double best_cost = 0;
+  for (int p = 1; p <= 32 && p <= tiles; ++p) {
+    if (p > 1 && n * p > cap_units) break;
+    double cost = (double)((n * p + sms - 1) / sms) * (double)((tiles + p - 1) / p + 2);
+    if (p > 1) cost += 2.0 + (double)(n * p) * rows * head_dim * 16.0 / 3.0e6 / 1.46;
+    if (p == 1 || cost < best_cost) {
+      best_cost = cost;
+      best.items = p > 1 ? n : 0;
+      best.parts = p;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -891,7 +939,7 @@ ism_status_t ism_attn_prefill_append_workspace_size(const ism_attn_shape_t* shap
   if (r != ISM_OK) return r;
   if (batch < 0 || l_new < 0) return fail(ISM_ERR_INVALID_ARG, "batch and l_new must be >= 0");
   if (!bytes) return fail(ISM_ERR_INVALID_ARG, "bytes is NULL");
-  *bytes = append_layout(nullptr, shape, batch, l_new).bytes;  // (e4m3 shapes included)
+  *bytes = append_layout(nullptr, shape, batch, l_new).full_bytes;  // (e4m3 shapes included)
   return ISM_OK;
 }
 
@@ -901,7 +949,7 @@ ism_status_t ism_attn_prefill_append_rope_workspace_size(const ism_attn_shape_t*
   if (r != ISM_OK) return r;
   if (batch < 0 || l_new < 0) return fail(ISM_ERR_INVALID_ARG, "batch and l_new must be >= 0");
   if (!bytes) return fail(ISM_ERR_INVALID_ARG, "bytes is NULL");
-  *bytes = append_layout(nullptr, shape, batch, l_new, true).bytes;
+  *bytes = append_layout(nullptr, shape, batch, l_new, true).full_bytes;
   return ISM_OK;
 }
 
@@ -975,28 +1023,30 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
   // groups take the forward kernels (one query row per tile)
   const bool decode = l_new == 1 && (shape->dtype == ISM_BF16 || shape->dtype == ISM_E4M3) && !force_cuda_cores() &&
                       hq / hkv <= kMaxDecodeGroup;
-  // A single-token step needs no tile plan: the cache write reads the cache
-  // lengths and snapshots them, and the decode's combine kernel advances them.
+  // The cache write lays out the chunk's plan (a single-token step needs none,
+  // but a copy of the cache lengths); the attention kernels advance the lengths.
+  AppendPlan plan{};
+  if (!decode) {
+    plan.segs = sg;
+    plan.kbase_stride = paged ? 1 : cg.cap;
+    plan.bm = plan.bn = kTile;
+    plan.kv_end = L.kv_end; plan.qtiles = L.qtiles; plan.q_order = L.q_order; plan.pair_order = L.pair_order;
+  }
   timer_begin(ISM_KERNEL_META, st);
-  if (!decode)
-    ISM_TRY_CUDA(launch_append_plan(sg, batch, paged ? 1 : cg.cap, kTile, kTile, cache_len, L.c_snap, L.kv_end,
-                                    L.qtiles, L.q_order, L.pair_order, st),
-                 "append plan launch");
-  const int32_t* c_src = decode ? cache_len : L.c_snap;
   int32_t* snap_out = decode ? L.c_snap : nullptr;
   if (rope) {
-    ISM_TRY_CUDA(launch_rope_cache_write(shape->dtype, batch, l_new, hq, hkv, d, cg.cap, cg.pages, c_src, q_new,
+    ISM_TRY_CUDA(launch_rope_cache_write(shape->dtype, batch, l_new, hq, hkv, d, cg.cap, cg.pages, cache_len, q_new,
                                          k_new, v_new, rope->cos, rope->sin, q_descale, k_descale, v_descale,
-                                         L.q_rot, k_cache, v_cache, st, snap_out),
+                                         L.q_rot, k_cache, v_cache, plan, st, snap_out),
                  "rope cache write launch");
     q_new = L.q_rot;  // the attention below reads the rotated queries
   } else {
-    ISM_TRY_CUDA(launch_cache_write(shape->dtype, batch, l_new, hkv, d, cg.cap, cg.pages, c_src, k_new, v_new,
-                                    k_cache, v_cache, st, snap_out),
+    ISM_TRY_CUDA(launch_cache_write(shape->dtype, batch, l_new, hkv, d, cg.cap, cg.pages, cache_len, k_new, v_new,
+                                    k_cache, v_cache, plan, st, snap_out),
                  "cache write launch");
   }
   timer_end(ISM_KERNEL_META, st);
-  count_launch(decode ? 1 : 2);
+  count_launch(1);
   if (decode) {
     DecodeArgs a{};
     a.cache_len = cache_len;
@@ -1063,37 +1113,44 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
   a.pages = cg.pages;
   a.qk_descale = qk_descale;
   a.v_descale = v_descale;
-  if ((shape->dtype == ISM_E4M3 || d == 64) && (hq / hkv) % 2) {
-    // e4m3 and head_dim 64 run only the paired kernel: neighbouring q-tiles for an odd group
-    a.pair_order = L.pair_order;
-    a.npairs = L.npairs;
-  }
+  a.adv_cache_len = cache_len;
+  a.adv_batch = batch;
+  a.adv_len = l_new;
   a.status = status;
   a.flags = tc_flags();
-  // The items of the paired forward (query tile, head pair) all cost about the
-  // same in a prefill; those that would leave a last round with idle SMs run
-  // as two halves of their key range instead, when the items are long enough
-  // (at least 64 key tiles) for the halves to outweigh the merge.  Measured
-  // on the 8 x 16K prefill with the persistent forward: bf16 0.795 -> 0.719
-  // ms, e4m3 0.668 -> 0.595 ms; 40-token chunks over 4000 keys stay whole.
-  // ISM_PREFILL_SPLIT=n forces n split items.
-  if ((use_tc(shape) || shape->dtype == ISM_E4M3) && d == 128 && (hq / hkv) % 2 == 0 && !a.pair_order &&
-      L.split_cap > 0) {
-    const int64_t items = a.nq * (hq / 2);
-    int64_t n_split = 0;
-    if (knobs().prefill_split >= 0) {
-      n_split = knobs().prefill_split;
-    } else {
-      const int sms = sm_count();
-      const int64_t key_tiles = ((int64_t)max_c + l_new + kTile - 1) / kTile;
-      if (items > sms && key_tiles >= 64) n_split = items % sms;
+  if (use_tc(shape) || shape->dtype == ISM_E4M3) {
+    const bool odd = (hq / hkv) % 2 != 0;
+    const int64_t tiles = ((int64_t)max_c + l_new + kTile - 1) / kTile;
+    const int64_t items = append_items(shape, batch, l_new, odd);
+    const int64_t cap_units = (int64_t)((workspace_bytes - L.part_off) /
+                                        ((size_t)2 * L.part_rows * (d + 2) * sizeof(float)));
+    KeySplit sp = plan_key_split(items, tiles, L.part_rows, d, cap_units);
+    if (knobs().prefill_split >= 0) {  // ISM_PREFILL_SPLIT=n: n items as two halves
+      sp.items = knobs().prefill_split < items ? knobs().prefill_split : items;
+      sp.parts = 2;
+      if (sp.items * 2 > cap_units) sp.items = cap_units / 2;
     }
-    if (n_split > L.split_cap) n_split = L.split_cap;
-    if (n_split > 0) {
-      a.split_items = n_split;
-      a.split_whole = items - n_split;
-      a.part_o = L.part_fo;
-      a.part_ml = L.part_fml;
+    // An odd group pairs neighbouring q-tiles of a head.  e4m3 and head_dim 64
+    // have only the paired kernel; bf16 at 128 takes the one-head kernel
+    // instead when no tile has a neighbour (half of a paired CTA would idle),
+    // unless its rounds leave a quarter of the SMs idle and the items split:
+    // 32 heads over 16 x 4000 keys (512 items, 0.84 of four rounds) one-head
+    // 212 us, split pairs 227; over 6 x 16000 keys (192, 0.63) 366 and 314.
+    const int64_t rounds = (items + sm_count() - 1) / sm_count();
+    const bool one_head = d == 128 && shape->dtype == ISM_BF16 &&
+                          (knobs().fwd_one_head ||
+                           (odd && l_new <= kTile && (sp.items == 0 || items * 4 > rounds * sm_count() * 3)));
+    if (odd && !one_head) {
+      a.pair_order = L.pair_order;
+      a.npairs = L.npairs;
+    }
+    if (!one_head && sp.items > 0) {
+      a.split_items = sp.items;
+      a.split_whole = items - sp.items;
+      a.split_parts = sp.parts;
+      a.part_rows = L.part_rows;
+      a.part_o = reinterpret_cast<float*>(reinterpret_cast<uintptr_t>(workspace) + L.part_off);
+      a.part_ml = a.part_o + sp.items * sp.parts * 2 * L.part_rows * d;
     }
   }
   timer_begin(ISM_KERNEL_FWD, st);

@@ -16,6 +16,8 @@
 // Warps 0-3 softmax of head A, 4-7 of head B, 8 TMA producer, 9 MMA issuer.
 // The mask and the lazy-rescale online softmax are those of the one-head
 // kernel (Eq. e_ISM with the bound of Eq. fj; full tiles unmasked).
+#include <cfloat>
+
 #include "ism_tc_common.cuh"
 
 namespace ism {
@@ -54,40 +56,25 @@ __device__ __forceinline__ void set_abort(int32_t* f) { *reinterpret_cast<volati
 struct Unit {
   Tile w0, w1;
   int h0, h1, nkb0, nkb1;
-  int jb, half;     // first key tile; half of a split item (-1: the whole item)
-  int64_t split_k;  // index of a split item among the split ones
+  int jb;  // first key tile
+  int pu;  // index of a part among all parts of the split items (-1: a whole item)
   __device__ int nkb() const { return nkb0 > nkb1 ? nkb0 : nkb1; }
 };
 
-template <bool kTilePairs, bool kSplit>
-__device__ __forceinline__ Unit decode_unit(const AttnArgs& a, int64_t u) {
-  Unit x;
-  x.jb = 0;
-  x.half = -1;
-  x.split_k = 0;
+// Item `item` of the launch: tiles and heads of its two halves.
+template <bool kTilePairs>
+__device__ __forceinline__ void decode_item(const AttnArgs& a, int64_t item, Unit& x) {
   if constexpr (!kTilePairs) {
-    const int npairs = a.hq >> 1;
-    int64_t item = u;
-    if (kSplit && item >= a.split_whole) {
-      x.split_k = (item - a.split_whole) >> 1;
-      x.half = (int)((item - a.split_whole) & 1);
-      item = a.split_whole + x.split_k;
-    }
     int64_t tpos;
     int hp;
-    bucket_item(item, a.nq, npairs, tpos, hp, false);  // head pairs of a tile share K / V
+    bucket_item(item, a.nq, a.hq >> 1, tpos, hp, false);  // head pairs of a tile share K / V
     x.w0 = x.w1 = a.qtiles[a.q_order[tpos]];
     x.h0 = 2 * hp;
     x.h1 = x.h0 + 1;
     x.nkb0 = x.nkb1 = x.w0.a1;
-    if (x.half >= 0) {  // key tiles [0, mid) or [mid, a1)
-      const int mid = x.w0.a1 / 2;
-      x.jb = x.half ? mid : 0;
-      x.nkb0 = x.nkb1 = x.half ? x.w0.a1 - mid : mid;
-    }
   } else {
     int64_t ppos;
-    bucket_item(u, a.npairs, a.hq, ppos, x.h0, a.hq == a.hkv);  // one query head per KV head: bucketed
+    bucket_item(item, a.npairs, a.hq, ppos, x.h0, a.hq == a.hkv);  // one query head per KV head: bucketed
     x.h1 = x.h0;
     const int gq = a.pair_order[ppos];
     x.w0 = a.qtiles[gq];
@@ -99,6 +86,26 @@ __device__ __forceinline__ Unit decode_unit(const AttnArgs& a, int64_t u) {
     if (!second) x.w1 = x.w0;
     x.nkb0 = x.w0.a1;
     x.nkb1 = second ? x.w1.a1 : 0;
+  }
+}
+
+template <bool kTilePairs, bool kSplit>
+__device__ __forceinline__ Unit decode_unit(const AttnArgs& a, int64_t u) {
+  Unit x;
+  x.jb = 0;
+  x.pu = -1;
+  int64_t item = u;
+  if (kSplit && u >= a.split_whole) {
+    x.pu = (int)(u - a.split_whole);
+    item = a.split_whole + x.pu / a.split_parts;
+  }
+  decode_item<kTilePairs>(a, item, x);
+  if (kSplit && x.pu >= 0) {  // an equal share of the key tiles (the second tile sees at least the first's)
+    const int top = x.nkb(), part = x.pu % a.split_parts;
+    const int lo = top * part / a.split_parts, hi = top * (part + 1) / a.split_parts;
+    x.jb = lo;
+    x.nkb0 = max(min(x.nkb0, hi) - lo, 0);
+    x.nkb1 = max(min(x.nkb1, hi) - lo, 0);
   }
   return x;
 }
@@ -115,8 +122,8 @@ __device__ __forceinline__ int64_t unit_of(int64_t k, int64_t n_units) {
 // kE4M3: Q, K, V in e4m3 (kind::f8f6f4 MMAs, K = 32 a step); the scores are
 // scaled by qk_descale, P is rounded to e4m3 for O += P V and O is scaled by
 // v_descale (per-tensor dequantisation factors of the inputs).
-// kSplit: the launch runs items past a.split_whole as two key-range halves
-// (head pairs only); the instantiation without it is the plain kernel.
+// kSplit: the launch runs items past a.split_whole as a.split_parts key-range
+// parts each; the instantiation without it is the plain kernel.
 // Persistent: each CTA walks its units (unit_of) with one set of barriers
 // whose phases run on across units.  The next unit's Q is loaded as soon as
 // the last score MMA of the current unit has read Q, and its first score MMAs
@@ -169,6 +176,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  if constexpr (kSplit) {
+    // launched as a programmatic dependent of the append's cache write: the
+    // set-up above overlaps it
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
+  advance_cache_len(a);
 
   if (warp == 8) {
     // ------------------------------------------------------------ producer (the warp waits
@@ -366,15 +379,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int64_t k = 0; ok; ++k) {
       const int64_t u = unit_of(k, n_units);
       if (u < 0) break;
-      const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
-      const int h = xh ? x.h1 : x.h0;
-      const Tile wm = xh ? x.w1 : x.w0;
-      const int nkbm = xh ? x.nkb1 : x.nkb0, kfull = wm.a0 - x.jb;  // key tiles counted from the unit's first
-      const int k_first = x.jb * kRows;
-      const int row = wm.tile * kRows + r;
-      const bool valid = row < wm.q_len;
-      const int ke = a.kv_end[wm.kv_base + (valid ? row : wm.q_len - 1)] - k_first;
-      float m_use = -INFINITY, l = 0.f;
+      int nkbm, kfull, ke;  // key tiles and bounds counted from the unit's first key tile
+      {
+        const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
+        const Tile& wm = xh ? x.w1 : x.w0;
+        nkbm = xh ? x.nkb1 : x.nkb0;
+        kfull = wm.a0 - x.jb;
+        ke = a.kv_end[wm.kv_base + min(wm.tile * kRows + r, wm.q_len - 1)] - x.jb * kRows;
+      }
+      // a part of a split item may hold no key that this row sees: its maximum
+      // stays finite, so that P = 2^(-inf) = 0 and not NaN
+      float m_use = kSplit ? -FLT_MAX : -INFINITY, l = 0.f;
       for (int j = 0; ok && j < nkbm; ++j) {
         const uint32_t blk = nb + (uint32_t)j;
         if (!wait(&bar->s_full[xh], blk & 1, a.status)) { ok = false; break; }
@@ -477,18 +492,27 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::mbar_arrive(&bar->p_full[xh]);
       }
       if (!ok) break;
+      // the unit once more for the epilogue: held across the blocks, its fields
+      // would not fit the registers beside a row of scores
+      const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
+      const int h = xh ? x.h1 : x.h0;
+      const Tile wm = xh ? x.w1 : x.w0;
+      const int row = wm.tile * kRows + r;
+      const bool valid = row < wm.q_len;
       if (nkbm > 0) {
         nb += (uint32_t)nkbm;
         // one decision for the whole warp: the epilogue's loads and shuffles are warp-wide
         if (!__all_sync(0xffffffffu, wait(&bar->pv_done[xh], (nb - 1) & 1, a.status))) { ok = false; break; }
         ptx::tc_fence_after();
       }
-      if (kSplit && x.half >= 0) {
-        // half of a split item: unnormalised O and (max, sum) for the merge; a
-        // half without key tiles leaves max -inf (weight 0, its O is not read)
-        const int64_t pu = ((x.split_k * 2 + x.half) * 2 + xh) * kRows + r;
-        a.part_ml[pu * 2] = nkbm > 0 ? m_use : -INFINITY;
-        a.part_ml[pu * 2 + 1] = nkbm > 0 ? l : 0.f;
+      if (kSplit && x.pu >= 0) {
+        // part of a split item: unnormalised O and (max, sum) for the merge; a
+        // part without key tiles leaves max -inf (weight 0, its O is not read)
+        const int64_t pu = ((int64_t)x.pu * 2 + xh) * a.part_rows + (valid ? r : 0);
+        if (valid) {
+          a.part_ml[pu * 2] = nkbm > 0 ? m_use : -INFINITY;
+          a.part_ml[pu * 2 + 1] = nkbm > 0 ? l : 0.f;
+        }
         if (nkbm > 0) {
           const float f = kE4M3 ? a.v_descale : 1.f;
           float4* dst = reinterpret_cast<float4*>(a.part_o + pu * kHD);
@@ -498,10 +522,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::tmem_ld32(tO + c * 32, o);
             ptx::tmem_ld_wait();
             ptx::reg_fence(o);
+            if (valid)
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dst[c * 8 + i] = make_float4(__uint_as_float(o[4 * i]) * f, __uint_as_float(o[4 * i + 1]) * f,
-                                           __uint_as_float(o[4 * i + 2]) * f, __uint_as_float(o[4 * i + 3]) * f);
+              for (int i = 0; i < 8; ++i)
+                dst[c * 8 + i] = make_float4(__uint_as_float(o[4 * i]) * f, __uint_as_float(o[4 * i + 1]) * f,
+                                             __uint_as_float(o[4 * i + 2]) * f, __uint_as_float(o[4 * i + 3]) * f);
           }
         }
       } else if (nkbm > 0) {
@@ -525,6 +550,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!ok) set_abort(&bar->abort);
   }
+  // the merge may be launched once every CTA is done (its blocks would take
+  // issue slots and registers of the running ones otherwise)
+  if constexpr (kSplit) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 9) {
@@ -533,67 +561,117 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Merge of the two halves of each split item: block (split item k, head x,
-// row r) of 128 threads (dimensions).  m in the base-2 scaled units of the
-// forward, so O = (w0 O0 + w1 O1) / (w0 l0 + w1 l1) with w = 2^(m - M), and
-// LSE = (M + log2 L) ln 2, as the whole-item epilogue writes them.
+// Merge of the parts of each split item: a warp per (split item, half x, row),
+// lanes first over the parts, then over the dimensions.  m in the base-2
+// scaled units of the forward, so O = sum_p w_p O_p / sum_p w_p l_p with
+// w_p = 2^(m_p - M), and LSE = (M + log2 L) ln 2, as the whole-item epilogue
+// writes them.  Bound by reading the partials once; with a block of 128
+// threads a row and two scalar loads a thread it took 12.3 us on two halves of
+// the 8 x 16K prefill's last 56 items, 8.6 us now.
+constexpr int kMaxParts = 32;
+template <bool kTilePairs, int kHD>
 __global__ void __launch_bounds__(128) fwd_split_merge_kernel(const AttnArgs a) {
-  const int64_t b = blockIdx.x;
-  const int r = (int)(b % kRows), x = (int)((b / kRows) & 1);
-  const int64_t k = b / (2 * kRows);
-  const int npairs = a.hq >> 1;
-  const int64_t item = a.split_whole + k;
-  int64_t tpos;
-  int hp;
-  bucket_item(item, a.nq, npairs, tpos, hp, false);  // as fwd_pair_kernel decodes its items
-  const Tile w = a.qtiles[a.q_order[tpos]];
-  const int h = 2 * hp + x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int r = (int)(i % a.part_rows), x = (int)((i / a.part_rows) & 1);
+  const int64_t k = i / (2 * (int64_t)a.part_rows);
+  if (k >= a.split_items) return;
+  Unit un;
+  decode_item<kTilePairs>(a, a.split_whole + k, un);
+  if ((x ? un.nkb1 : un.nkb0) == 0) return;  // a tile pair without its second tile
+  const Tile w = x ? un.w1 : un.w0;
+  const int h = x ? un.h1 : un.h0;
   const int row = w.tile * kRows + r;
   if (row >= w.q_len) return;
-  const int d = threadIdx.x;
-  const int64_t p0 = ((k * 2 + 0) * 2 + x) * kRows + r, p1 = ((k * 2 + 1) * 2 + x) * kRows + r;
-  const float m0 = a.part_ml[p0 * 2], l0 = a.part_ml[p0 * 2 + 1];
-  const float m1 = a.part_ml[p1 * 2], l1 = a.part_ml[p1 * 2 + 1];
-  const float M = fmaxf(m0, m1);
-  const float f0 = m0 == -INFINITY ? 0.f : exp2f(m0 - M), f1 = m1 == -INFINITY ? 0.f : exp2f(m1 - M);
-  const float o0 = f0 != 0.f ? a.part_o[p0 * kD + d] : 0.f, o1 = f1 != 0.f ? a.part_o[p1 * kD + d] : 0.f;
-  const float L = (f0 != 0.f ? f0 * l0 : 0.f) + (f1 != 0.f ? f1 * l1 : 0.f);
+  const int parts = a.split_parts;
+  const int64_t stride = 2 * (int64_t)a.part_rows;                        // partial rows from part to part
+  const int64_t p0 = (k * parts * 2 + x) * (int64_t)a.part_rows + r;      // part 0's
+  float m = -INFINITY, l = 0.f;
+  if (lane < parts) {
+    const float2 ml = *reinterpret_cast<const float2*>(a.part_ml + (p0 + lane * stride) * 2);
+    m = ml.x;
+    l = ml.y;
+  }
+  float M = m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  const float f = m == -INFINITY ? 0.f : exp2f(m - M);
+  float L = f * l;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+  constexpr int kPer = kHD / 32;  // dimensions a lane
+  float acc[kPer] = {};
+#pragma unroll 4
+  for (int p = 0; p < parts; ++p) {
+    const float fp = __shfl_sync(0xffffffffu, f, p);
+    if (fp == 0.f) continue;  // no key tile: O not written
+    const float* src = a.part_o + (p0 + p * stride) * kHD + lane * kPer;
+#pragma unroll
+    for (int d = 0; d < kPer; ++d) acc[d] = fmaf(fp, src[d], acc[d]);
+  }
   const int64_t orow = (int64_t)w.q_base + row;
-  reinterpret_cast<__nv_bfloat16*>(a.out)[(orow * a.hq + h) * kD + d] = __float2bfloat16_rn((f0 * o0 + f1 * o1) / L);
-  if (d == 0 && a.lse) a.lse[(int64_t)h * a.q_rows + orow] = (M + log2f(L)) * kLn2;
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + (orow * a.hq + h) * kHD + lane * kPer;
+#pragma unroll
+  for (int d = 0; d < kPer; d += 2)
+    *reinterpret_cast<__nv_bfloat162*>(out + d) = __floats2bfloat162_rn(acc[d] / L, acc[d + 1] / L);
+  if (lane == 0 && a.lse) a.lse[(int64_t)h * a.q_rows + orow] = (M + log2f(L)) * kLn2;
 }
 
-template <bool kE4M3, int kHD = 128>
+// Launch as a programmatic dependent of the kernel before it on the stream.
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), int64_t grid, int threads, uint32_t smem, cudaStream_t st,
+                             Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <bool kE4M3, int kHD, bool kTilePairs>
 cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                               cudaStream_t st) {
   cudaError_t e;
-  const bool tile_pairs = a.pair_order != nullptr;
-  const bool split_launch = !tile_pairs && a.split_items > 0;
-  auto kern = tile_pairs ? fwd_pair_kernel<true, kE4M3, false, kHD>
-                         : (split_launch ? fwd_pair_kernel<false, kE4M3, true, kHD>
-                                         : fwd_pair_kernel<false, kE4M3, false, kHD>);
+  const bool split = a.split_items > 0;
+  auto kern = split ? fwd_pair_kernel<kTilePairs, kE4M3, true, kHD> : fwd_pair_kernel<kTilePairs, kE4M3, false, kHD>;
   constexpr uint32_t smem = PairLayout<kE4M3, kHD>::SMEM;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
-  const int64_t items = tile_pairs ? a.npairs * a.hq : a.nq * (a.hq / 2);
+  const int64_t items = kTilePairs ? a.npairs * a.hq : a.nq * (a.hq / 2);
   if (items == 0) return cudaSuccess;
-  const bool split = !tile_pairs && a.split_items > 0;
-  if (split && (a.split_whole + a.split_items != items || !a.part_o || !a.part_ml)) return cudaErrorInvalidValue;
-  const int64_t n_units = split ? a.split_whole + 2 * a.split_items : items;
+  if (split && (a.split_whole + a.split_items != items || !a.part_o || !a.part_ml || a.split_parts < 1 ||
+                a.split_parts > kMaxParts))
+    return cudaErrorInvalidValue;
+  const int64_t n_units = split ? a.split_whole + a.split_parts * a.split_items : items;
   // persistent: one CTA per SM walks its share of the units
   const int64_t grid = n_units < sm_count() ? n_units : sm_count();
-  kern<<<(unsigned)grid, kThreads, smem, st>>>(tq, tk, tv, a, n_units);
-  if ((e = cudaGetLastError()) != cudaSuccess || !split) return e;
-  fwd_split_merge_kernel<<<(unsigned)(a.split_items * 2 * kRows), 128, 0, st>>>(a);
-  return cudaGetLastError();
+  if (!split) {
+    kern<<<(unsigned)grid, kThreads, smem, st>>>(tq, tk, tv, a, n_units);
+    return cudaGetLastError();
+  }
+  if ((e = launch_dependent(kern, grid, kThreads, smem, st, tq, tk, tv, a, n_units)) != cudaSuccess) return e;
+  const int64_t rows = a.split_items * 2 * a.part_rows;
+  return launch_dependent(fwd_split_merge_kernel<kTilePairs, kHD>, (rows + 3) / 4, 128, 0, st, a);
 }
 
 }  // namespace
 
 cudaError_t launch_fwd_pair(const AttnArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                             cudaStream_t st) {
-  if (a.d == 64) return launch_fwd_pair_t<false, 64>(a, tq, tk, tv, st);
-  return a.dtype == ISM_E4M3 ? launch_fwd_pair_t<true>(a, tq, tk, tv, st) : launch_fwd_pair_t<false>(a, tq, tk, tv, st);
+  if (a.pair_order)
+    return a.dtype == ISM_E4M3 ? launch_fwd_pair_t<true, 128, true>(a, tq, tk, tv, st)
+           : a.d == 64         ? launch_fwd_pair_t<false, 64, true>(a, tq, tk, tv, st)
+                               : launch_fwd_pair_t<false, 128, true>(a, tq, tk, tv, st);
+  return a.dtype == ISM_E4M3 ? launch_fwd_pair_t<true, 128, false>(a, tq, tk, tv, st)
+         : a.d == 64         ? launch_fwd_pair_t<false, 64, false>(a, tq, tk, tv, st)
+                             : launch_fwd_pair_t<false, 128, false>(a, tq, tk, tv, st);
 }
 
 }  // namespace tc

@@ -94,6 +94,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
 
+  advance_cache_len(a);
+
   if (warp == 4) {
     // ------------------------------------------------------------ producer (the warp waits
     // converged, lane 0 issues the copies)

@@ -89,24 +89,36 @@ cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, 
                              Tile* qtiles, Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order,
                              int32_t* pair_order, int32_t* kpair_off, int32_t* counters, int n_counters,
                              cudaStream_t st, int32_t* kp_order = nullptr, bool pairs_first = false);
-// k_base of sequence b's tiles = b * kbase_stride (the cache capacity, or 1 for a paged cache)
-cudaError_t launch_append_plan(const AppendSegs& segs, int batch, int64_t kbase_stride, int bm, int bn,
-                               int32_t* cache_len, int32_t* c_snap, int32_t* kv_end, Tile* qtiles,
-                               int32_t* q_order, int32_t* pair_order, cudaStream_t st);
-// c_snap: cache lengths before the append.  snap_out (nullable): receives a
-// copy of them (single-token steps pass cache_len itself as c_snap).
+// What the forward over an appended chunk reads, written by the cache-write
+// kernels along with the cache: the absolute key bound of every new row (all
+// cached keys plus Eq. fj within the chunk), one descriptor per (sequence,
+// chunk tile) in order, and the pair heads.  kbase_stride: k_base of sequence
+// b's tiles is b times it (the cache capacity, or 1 for a paged cache).
+// qtiles == nullptr (single-token steps): nothing of it.
+struct AppendPlan {
+  AppendSegs segs;
+  int64_t kbase_stride;
+  int32_t bm, bn;
+  int32_t* kv_end;
+  Tile* qtiles;
+  int32_t* q_order;
+  int32_t* pair_order;
+};
+// cache_len: lengths before the append (read only; the attention kernels
+// advance them).  snap_out (nullable): receives a copy of them.
 cudaError_t launch_cache_write(int dtype, int batch, int l_new, int hkv, int d, int64_t cap, const KvPages& pages,
-                               const int32_t* c_snap, const void* k_new, const void* v_new,
-                               void* k_cache, void* v_cache, cudaStream_t st, int32_t* snap_out = nullptr);
+                               const int32_t* cache_len, const void* k_new, const void* v_new,
+                               void* k_cache, void* v_cache, const AppendPlan& plan, cudaStream_t st,
+                               int32_t* snap_out);
 // Cache write with the rotary encoding of the new queries and keys (bf16
 // inputs, head_dim a multiple of 16): rotated keys and plain values into the
 // cache, rotated queries into q_rot [batch * l_new, hq, d], all in the cache's
 // type: bf16, or e4m3 (dtype ISM_E4M3) after division by the descales.
 cudaError_t launch_rope_cache_write(int dtype, int batch, int l_new, int hq, int hkv, int d, int64_t cap,
-                                   const KvPages& pages, const int32_t* c_snap, const void* q_new,
+                                   const KvPages& pages, const int32_t* cache_len, const void* q_new,
                                    const void* k_new, const void* v_new, const float* cos_t, const float* sin_t,
                                    float q_descale, float k_descale, float v_descale, void* q_rot, void* k_cache,
-                                   void* v_cache, cudaStream_t st, int32_t* snap_out = nullptr);
+                                   void* v_cache, const AppendPlan& plan, cudaStream_t st, int32_t* snap_out);
 
 // Rotary encoding of the one-pass path (ism_rope.cu): rotates every query and
 // key head row of a packed batch by its position inside its sequence (pairs
@@ -154,14 +166,18 @@ struct AttnArgs {
   // e4m3 forward: per-tensor dequantisation factors (scores scaled by
   // q_descale * k_descale, the output by v_descale).
   float qk_descale, v_descale;
-  // Key-range split of the paired forward (head pairs only): launch items
-  // [0, split_whole) run whole; each later item runs as two CTAs over the
-  // first and the second half of its key tiles, writing unnormalised O and
-  // (max, sum) to part_o / part_ml, merged by a second kernel.  Off when
-  // split_items == 0.
+  // Key-range split of the paired forward: launch items [0, split_whole) run
+  // whole; each later item runs as split_parts units over equal shares of its
+  // key tiles, writing unnormalised O and (max, sum) to part_o / part_ml,
+  // merged by a second kernel.  Off when split_items == 0.
   int64_t split_whole, split_items;
-  float* part_o;    // [split_items][2 halves][2 heads][128 rows][128] fp32
-  float* part_ml;   // [split_items][2 halves][2 heads][128 rows][2] fp32
+  int32_t split_parts, part_rows;  // part_rows: the most rows of a query tile
+  float* part_o;    // [split_items][split_parts][2][part_rows][d] fp32
+  float* part_ml;   // [split_items][split_parts][2][part_rows][2] fp32
+  // Append-prefill: the cache lengths [adv_batch], advanced by adv_len by the
+  // forward kernel (the kernels before it read them; it does not).
+  int32_t* adv_cache_len;
+  int32_t adv_batch, adv_len;
   // Rotary encoding (tensor-core backward only): when rope_cos is set, the dQ
   // and dK epilogues store the gradients of the unrotated queries and keys,
   // applying the transposed rotation of the row's position in its sequence
@@ -174,6 +190,11 @@ struct AttnArgs {
   uint32_t flags;
 };
 enum : uint32_t { kFlagDrainTmemReuse = 1u };
+// Called by every thread of every block of a forward kernel.
+__device__ __forceinline__ void advance_cache_len(const AttnArgs& a) {
+  if (a.adv_cache_len && blockIdx.x == 0)
+    for (int b = threadIdx.x; b < a.adv_batch; b += blockDim.x) a.adv_cache_len[b] += a.adv_len;
+}
 cudaError_t launch_simt_fwd(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_simt_bwd(const AttnArgs& a, cudaStream_t st);
 

@@ -307,52 +307,28 @@ __device__ __forceinline__ int32_t chunk_kv_end(const AppendSegs& sg, int32_t j)
   return j + 1;
 }
 
-// Append plan (one block): snapshot cache_len, advance it by l_new, write the
-// absolute key bound of every new row (all cached keys plus Eq. fj within
-// the chunk) and one q-tile descriptor per (sequence, chunk tile).
-__global__ void append_plan_kernel(AppendSegs sg, int batch, int64_t kbase_stride, int bm, int bn,
-                                   int32_t* cache_len, int32_t* c_snap, int32_t* kv_end,
-                                   Tile* qtiles, int32_t* q_order, int32_t* pair_order) {
-  __shared__ int32_t cs[1024];
+// The append plan's share of one thread (grid-stride; see AppendPlan).
+__device__ __forceinline__ void append_plan_part(const AppendPlan& p, int batch, const int32_t* __restrict__ cache_len) {
+  if (!p.qtiles) return;
+  const AppendSegs& sg = p.segs;
   const int32_t Ln = sg.l_new;
-  for (int base = 0; base < batch; base += 1024) {
-    // (batch > 1024 is handled in chunks; every thread sees its own chunk)
-    int b = base + threadIdx.x;
-    if (threadIdx.x < 1024 && b < batch) cs[threadIdx.x] = cache_len[b];
-    __syncthreads();
-    int nb = min(1024, batch - base);
-    for (int i = threadIdx.x; i < nb * Ln; i += blockDim.x) {
-      int bl = i / Ln, j = i % Ln;
-      kv_end[(int64_t)(base + bl) * Ln + j] = cs[bl] + chunk_kv_end(sg, j);
-    }
-    int nqt = (Ln + bm - 1) / bm;
-    for (int i = threadIdx.x; i < nb * nqt; i += blockDim.x) {
-      int bl = i / nqt, t = i % nqt;
-      int32_t c = cs[bl];
-      int32_t r0 = t * bm, rl = min(Ln, r0 + bm) - 1;
-      Tile w;
-      w.q_base = (base + bl) * Ln; w.k_base = (int32_t)((base + bl) * kbase_stride);
-      w.q_len = Ln; w.k_len = c + Ln; w.tile = t;
-      w.a0 = (r0 + bm <= Ln) ? (c + chunk_kv_end(sg, r0)) / bn : 0;
-      w.a1 = (c + chunk_kv_end(sg, rl) + bn - 1) / bn;
-      w.kv_base = (base + bl) * Ln;
-      int64_t g = (int64_t)(base + bl) * nqt + t;
-      qtiles[g] = w;
-      q_order[g] = (int32_t)g;
-    }
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = t0; i < (int64_t)batch * Ln; i += stride)
+    p.kv_end[i] = cache_len[i / Ln] + chunk_kv_end(sg, (int32_t)(i % Ln));
+  const int nqt = (Ln + p.bm - 1) / p.bm, npt = (nqt + 1) / 2;
+  for (int64_t g = t0; g < (int64_t)batch * nqt; g += stride) {
+    const int b = (int)(g / nqt), t = (int)(g % nqt);
+    const int32_t c = cache_len[b], r0 = t * p.bm, rl = min(Ln, r0 + p.bm) - 1;
+    Tile w;
+    w.q_base = b * Ln; w.k_base = (int32_t)(b * p.kbase_stride);
+    w.q_len = Ln; w.k_len = c + Ln; w.tile = t;
+    w.a0 = (r0 + p.bm <= Ln) ? (c + chunk_kv_end(sg, r0)) / p.bn : 0;
+    w.a1 = (c + chunk_kv_end(sg, rl) + p.bn - 1) / p.bn;
+    w.kv_base = b * Ln;
+    p.qtiles[g] = w;
+    p.q_order[g] = (int32_t)g;
     // q-tile pairs (2i, 2i + 1) of each sequence's chunk for the paired forward
-    const int npt = (nqt + 1) / 2;
-    if (pair_order)
-      for (int i = threadIdx.x; i < nb * npt; i += blockDim.x) {
-        const int bl = i / npt, p = i % npt;
-        pair_order[(int64_t)(base + bl) * npt + p] = (int32_t)((int64_t)(base + bl) * nqt + 2 * p);
-      }
-    __syncthreads();
-    if (threadIdx.x < nb) {
-      c_snap[base + threadIdx.x] = cs[threadIdx.x];
-      cache_len[base + threadIdx.x] = cs[threadIdx.x] + Ln;
-    }
-    __syncthreads();
+    if (p.pair_order && !(t & 1)) p.pair_order[(int64_t)b * npt + t / 2] = (int32_t)g;
   }
 }
 
@@ -366,9 +342,11 @@ __global__ void append_plan_kernel(AppendSegs sg, int batch, int64_t kbase_strid
 // cache write (clipped to the capacity of a contiguous cache; a paged tile
 // lies within one page).  Keys need no such care: masked scores are replaced,
 // not multiplied.
-// Single-token steps run without the plan kernel: the cache write reads the
-// cache lengths itself (c_snap = cache_len, unchanged until the decode's
-// combine kernel advances it) and records them in snap_out for the decode.
+// The cache write also lays out the chunk's plan (one launch less: 3.4 us of
+// the 60 us of a 40-token append over 3000 keys were a one-block plan kernel).
+// It reads the cache lengths themselves (c_snap = cache_len): they stay as
+// they are until the attention kernel after it advances them, and single-token
+// steps find a copy in snap_out.
 __device__ __forceinline__ void copy_snapshot(int batch, const int32_t* __restrict__ c_snap, int32_t* snap_out) {
   if (!snap_out) return;
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += (int64_t)gridDim.x * blockDim.x)
@@ -397,9 +375,10 @@ __device__ __forceinline__ void zero_value_tail(int batch, int l_new, int vec_pe
 __global__ void cache_write_kernel(int batch, int l_new, int row_bytes, int64_t cap, KvPages pages,
                                    const int32_t* __restrict__ c_snap, const uint4* __restrict__ k_new,
                                    const uint4* __restrict__ v_new, uint4* k_cache, uint4* v_cache,
-                                   int32_t* snap_out) {
-  // a decode kernel launched as a programmatic dependent may start its set-up now
+                                   const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
+  // a kernel launched as a programmatic dependent may start its set-up now
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  append_plan_part(plan, batch, c_snap);
   const int vec_per_row = row_bytes / 16;
   copy_snapshot(batch, c_snap, snap_out);
   const int64_t total = (int64_t)batch * l_new * vec_per_row;
@@ -464,8 +443,9 @@ __global__ void rope_cache_write_kernel(int batch, int l_new, int hq, int hkv, i
                                         const __nv_bfloat16* __restrict__ v_new, const float* __restrict__ cos_t,
                                         const float* __restrict__ sin_t, float q_descale, float k_descale,
                                         float v_descale, void* q_rot, void* k_cache, void* v_cache,
-                                        int32_t* snap_out) {
+                                        const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  append_plan_part(plan, batch, c_snap);
   copy_snapshot(batch, c_snap, snap_out);
   const int half = d / 2;
   const int units = half / 8;  // 8-coordinate units in one half of a head row
@@ -586,17 +566,10 @@ cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_o
   return cudaGetLastError();
 }
 
-cudaError_t launch_append_plan(const AppendSegs& segs, int batch, int64_t kbase_stride, int bm, int bn,
-                               int32_t* cache_len, int32_t* c_snap, int32_t* kv_end, Tile* qtiles,
-                               int32_t* q_order, int32_t* pair_order, cudaStream_t st) {
-  append_plan_kernel<<<1, 1024, 0, st>>>(segs, batch, kbase_stride, bm, bn, cache_len, c_snap, kv_end, qtiles,
-                                         q_order, pair_order);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_cache_write(int dtype, int batch, int l_new, int hkv, int d, int64_t cap, const KvPages& pages,
                                const int32_t* c_snap, const void* k_new, const void* v_new,
-                               void* k_cache, void* v_cache, cudaStream_t st, int32_t* snap_out) {
+                               void* k_cache, void* v_cache, const AppendPlan& plan, cudaStream_t st,
+                               int32_t* snap_out) {
   int elem = dtype == ISM_BF16 ? 2 : dtype == ISM_E4M3 ? 1 : 4;
   int row_bytes = hkv * d * elem;
   int64_t total = (int64_t)batch * l_new * (row_bytes / 16);
@@ -606,7 +579,7 @@ cudaError_t launch_cache_write(int dtype, int batch, int l_new, int hkv, int d, 
   int grid = (int)((total + 255) / 256);
   if (grid > 152 * 16) grid = 152 * 16;
   cache_write_kernel<<<grid, 256, 0, st>>>(batch, l_new, row_bytes, cap, pages, c_snap, (const uint4*)k_new,
-                                           (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, snap_out);
+                                           (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, plan, snap_out);
   return cudaGetLastError();
 }
 
@@ -614,7 +587,7 @@ cudaError_t launch_rope_cache_write(int dtype, int batch, int l_new, int hq, int
                                    const KvPages& pages, const int32_t* c_snap, const void* q_new,
                                    const void* k_new, const void* v_new, const float* cos_t, const float* sin_t,
                                    float q_descale, float k_descale, float v_descale, void* q_rot, void* k_cache,
-                                   void* v_cache, cudaStream_t st, int32_t* snap_out) {
+                                   void* v_cache, const AppendPlan& plan, cudaStream_t st, int32_t* snap_out) {
   int64_t total = (int64_t)batch * l_new * (hq + 2 * hkv) * (d / 16);
   if (total == 0) return cudaSuccess;
   const bool e4m3 = dtype == ISM_E4M3;
@@ -625,7 +598,7 @@ cudaError_t launch_rope_cache_write(int dtype, int batch, int l_new, int hq, int
   auto kern = e4m3 ? rope_cache_write_kernel<true> : rope_cache_write_kernel<false>;
   kern<<<grid, 256, 0, st>>>(batch, l_new, hq, hkv, d, cap, pages, c_snap, (const __nv_bfloat16*)q_new,
                              (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, cos_t, sin_t, q_descale,
-                             k_descale, v_descale, q_rot, k_cache, v_cache, snap_out);
+                             k_descale, v_descale, q_rot, k_cache, v_cache, plan, snap_out);
   return cudaGetLastError();
 }
 

@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(C::TH) simt_fwd_kernel(const AttnArgs a) {
   float *own = sm, *kt = own + C::OWN, *vt = kt + C::TILE, *wt = vt + C::TILE;
   int h, row0;
   const Tile w = own_rows<C>(a.qtiles, a.q_order, a.hq, &h, &row0);
+  advance_cache_len(a);
   if (row0 >= w.q_len) return;
   const int g = h / (a.hq / a.hkv);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rw = warp % C::W, sw = warp / C::W;

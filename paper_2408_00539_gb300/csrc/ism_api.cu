@@ -912,11 +912,23 @@ struct KeySplit {
   int64_t items = 0;  // split items (the last ones); 0: none
   int32_t parts = 1;
 };
-KeySplit plan_key_split(int64_t items, int64_t tiles, int rows, int head_dim, int64_t cap_units) {
+// e4m3: P is rounded to three mantissa bits relative to its part's maximum, so
+// another split gives other roundings (3.5 % of the output between two equally
+// exact results); it keeps two halves of the last round's items, from 64 key
+// tiles on.
+KeySplit plan_key_split(const ism_attn_shape_t* sh, int64_t items, int64_t tiles, int rows, int64_t cap_units) {
   const int64_t sms = sm_count();
+  const int head_dim = sh->head_dim;
   KeySplit best;
   const int64_t n = items < sms ? items : items % sms;
   if (n == 0) return best;
+  if (sh->dtype == ISM_E4M3) {
+    if ((sh->num_heads_q / sh->num_heads_kv) % 2 == 0 && items > sms && tiles >= 64) {
+      best.items = n * 2 > cap_units ? cap_units / 2 : n;
+      best.parts = 2;
+    }
+    return best;
+  }
   double best_cost = 0;
   for (int p = 1; p <= 32 && p <= tiles; ++p) {
     if (p > 1 && n * p > cap_units) break;
@@ -1124,7 +1136,7 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
     const int64_t items = append_items(shape, batch, l_new, odd);
     const int64_t cap_units = (int64_t)((workspace_bytes - L.part_off) /
                                         ((size_t)2 * L.part_rows * (d + 2) * sizeof(float)));
-    KeySplit sp = plan_key_split(items, tiles, L.part_rows, d, cap_units);
+    KeySplit sp = plan_key_split(shape, items, tiles, L.part_rows, cap_units);
     if (knobs().prefill_split >= 0) {  // ISM_PREFILL_SPLIT=n: n items as two halves
       sp.items = knobs().prefill_split < items ? knobs().prefill_split : items;
       sp.parts = 2;

@@ -13,7 +13,8 @@
 //
 // Tensor memory (512 columns): S_A [0,128) O_A [128,256) S_B [256,384)
 // O_B [384,512).  Shared memory: Q_A, Q_B, and a 2-stage K / V ring.
-// Warps 0-3 softmax of head A, 4-7 of head B, 8 TMA producer, 9 MMA issuer.
+// Warps 0-3 softmax of head A, 4-7 of head B, 8 TMA producer, 9 MMA issuer, 10
+// and 11 idle.
 // The mask and the lazy-rescale online softmax are those of the one-head
 // kernel (Eq. e_ISM with the bound of Eq. fj; full tiles unmasked).
 #include <cfloat>
@@ -24,7 +25,16 @@ namespace ism {
 namespace tc {
 namespace {
 
-constexpr int kThreads = 320;
+// three warpgroups: two of softmax warps, one with the producer, the MMA issuer
+// and two idle warps, so that registers can move between them (setmaxnreg acts
+// on whole warpgroups): 168 a thread at launch, 80 + 2 * 208 <= 3 * 168 after.
+// A softmax thread holds a row of 128 scores beside its state; at 168 registers
+// it spilled 88 bytes in the block loop (480 at head_dim 64).  Forward of 2 x
+// 8192 grouped-query 690 -> 663 us, 4 x 4096 multi-head 453 -> 412, head_dim 64
+// (16 heads, 6001 tokens) 124 -> 102, e4m3 2 x 8192 567 -> 560.
+constexpr int kThreads = 384;
+constexpr int kRegsService = 80, kRegsSoftmax = 208;
+static_assert(kRegsService + 2 * kRegsSoftmax <= 3 * 168, "the block's registers at launch");
 constexpr uint32_t kTmemCols = 512;
 // Shared memory: Q_A, Q_B, K ring (2), V ring (2), barriers.  A 128 x 128 tile
 // is 32 KB in bf16 (two 64-column swizzled halves) and 16 KB in e4m3 (one); a
@@ -138,7 +148,7 @@ __device__ __forceinline__ int64_t unit_of(int64_t k, int64_t n_units) {
 // rounding (measured error against 64 bits 0.0017 relative, all of it the bf16
 // output's).  A block of two heads is 2 x (4 + 16) MMA steps; the tensor pipe
 // still waits for the softmax warps.  One layer of 16 heads over three
-// dialogues (6001 tokens): 132 us, against 44.3 ms of the CUDA-core kernel.
+// dialogues (6001 tokens): 102 us, against 44.3 ms of the CUDA-core kernel.
 template <bool kTilePairs, bool kE4M3, bool kSplit = false, int kHD = 128>
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -183,192 +193,196 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   advance_cache_len(a);
 
-  if (warp == 8) {
-    // ------------------------------------------------------------ producer (the warp waits
-    // converged, lane 0 issues the copies)
-    // one 128 x 128 tile: two 64-column boxes in bf16, one 128-column box in e4m3
-    auto load_tile = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* b, int32_t x, int32_t y) {
-      ptx::tma_load_2d(dst, map, b, x, y);
-      if (!kE4M3 && kHD == 128) ptx::tma_load_2d(dst + kHalfBytes, map, b, x + 64, y);
-    };
-    if (lane == 0) {
-      ptx::tma_prefetch_desc(&tmQ);
-      ptx::tma_prefetch_desc(&tmK);
-      ptx::tma_prefetch_desc(&tmV);
-    }
-    uint32_t nq = 0, it = 0;           // Q loads and K / V blocks so far (all units)
-    uint32_t nk[2] = {0, 0}, nv[2] = {0, 0};
-    bool ok = true;
-    for (int64_t k = 0; ok; ++k) {
-      const int64_t u = unit_of(k, n_units);
-      if (u < 0) break;
-      const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
-      const int nkb = x.nkb();
-      if (nkb == 0) continue;
-      const int g = x.h0 / (a.hq / a.hkv);
-      const int k_first = x.jb * kRows;
-      // the previous unit's score MMAs have read its Q
-      if (nq > 0 && !wait_warp(&bar->q_empty, (nq - 1) & 1, a.status)) {
-        if (lane == 0) set_abort(&bar->abort);
-        ok = false;
-        break;
-      }
+  if (warp >= 8) {
+    ptx::setmaxnreg_dec<kRegsService>();
+    if (warp == 8) {
+      // ------------------------------------------------------------ producer (the warp waits
+      // converged, lane 0 issues the copies)
+      // one 128 x 128 tile: two 64-column boxes in bf16, one 128-column box in e4m3
+      auto load_tile = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* b, int32_t x, int32_t y) {
+        ptx::tma_load_2d(dst, map, b, x, y);
+        if (!kE4M3 && kHD == 128) ptx::tma_load_2d(dst + kHalfBytes, map, b, x + 64, y);
+      };
       if (lane == 0) {
-        const int32_t qy0 = x.w0.q_base + x.w0.tile * kRows, qy1 = x.w1.q_base + x.w1.tile * kRows;
-        ptx::mbar_expect_tx(&bar->q_full, (x.nkb1 > 0 ? 2 : 1) * kTB);
-        load_tile(smem + L::QA, &tmQ, &bar->q_full, x.h0 * kHD, qy0);
-        if (x.nkb1 > 0) load_tile(smem + L::QB, &tmQ, &bar->q_full, x.h1 * kHD, qy1);
+        ptx::tma_prefetch_desc(&tmQ);
+        ptx::tma_prefetch_desc(&tmK);
+        ptx::tma_prefetch_desc(&tmV);
       }
-      __syncwarp();
-      ++nq;
-      for (int j = 0; j < nkb; ++j, ++it) {
-        const int s = it & 1;
-        const uint32_t n = it >> 1;
-        if (__any_sync(0xffffffffu, aborted(&bar->abort))) { ok = false; break; }
-        const int32_t ky = a.pages.table
-                               ? (int32_t)paged_row(a.pages, x.w0.k_base, (int64_t)k_first + j * kRows)
-                               : x.w0.k_base + k_first + j * kRows;
-        if (it >= 2 && !wait_warp(&bar->k_empty[s], (n - 1) & 1, a.status)) {
+      uint32_t nq = 0, it = 0;           // Q loads and K / V blocks so far (all units)
+      uint32_t nk[2] = {0, 0}, nv[2] = {0, 0};
+      bool ok = true;
+      for (int64_t k = 0; ok; ++k) {
+        const int64_t u = unit_of(k, n_units);
+        if (u < 0) break;
+        const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
+        const int nkb = x.nkb();
+        if (nkb == 0) continue;
+        const int g = x.h0 / (a.hq / a.hkv);
+        const int k_first = x.jb * kRows;
+        // the previous unit's score MMAs have read its Q
+        if (nq > 0 && !wait_warp(&bar->q_empty, (nq - 1) & 1, a.status)) {
           if (lane == 0) set_abort(&bar->abort);
           ok = false;
           break;
         }
         if (lane == 0) {
-          ptx::mbar_expect_tx(&bar->k_full[s], kTB);
-          load_tile(smem + L::K + s * kTB, &tmK, &bar->k_full[s], g * kHD, ky);
+          const int32_t qy0 = x.w0.q_base + x.w0.tile * kRows, qy1 = x.w1.q_base + x.w1.tile * kRows;
+          ptx::mbar_expect_tx(&bar->q_full, (x.nkb1 > 0 ? 2 : 1) * kTB);
+          load_tile(smem + L::QA, &tmQ, &bar->q_full, x.h0 * kHD, qy0);
+          if (x.nkb1 > 0) load_tile(smem + L::QB, &tmQ, &bar->q_full, x.h1 * kHD, qy1);
         }
         __syncwarp();
-        ++nk[s];
-        if (it >= 2 && !wait_warp(&bar->v_empty[s], (n - 1) & 1, a.status)) {
-          if (lane == 0) set_abort(&bar->abort);
+        ++nq;
+        for (int j = 0; j < nkb; ++j, ++it) {
+          const int s = it & 1;
+          const uint32_t n = it >> 1;
+          if (__any_sync(0xffffffffu, aborted(&bar->abort))) { ok = false; break; }
+          const int32_t ky = a.pages.table
+                                 ? (int32_t)paged_row(a.pages, x.w0.k_base, (int64_t)k_first + j * kRows)
+                                 : x.w0.k_base + k_first + j * kRows;
+          if (it >= 2 && !wait_warp(&bar->k_empty[s], (n - 1) & 1, a.status)) {
+            if (lane == 0) set_abort(&bar->abort);
+            ok = false;
+            break;
+          }
+          if (lane == 0) {
+            ptx::mbar_expect_tx(&bar->k_full[s], kTB);
+            load_tile(smem + L::K + s * kTB, &tmK, &bar->k_full[s], g * kHD, ky);
+          }
+          __syncwarp();
+          ++nk[s];
+          if (it >= 2 && !wait_warp(&bar->v_empty[s], (n - 1) & 1, a.status)) {
+            if (lane == 0) set_abort(&bar->abort);
+            ok = false;
+            break;
+          }
+          if (lane == 0) {
+            ptx::mbar_expect_tx(&bar->v_full[s], kTB);
+            load_tile(smem + L::V + s * kTB, &tmV, &bar->v_full[s], g * kHD, ky);
+          }
+          __syncwarp();
+          ++nv[s];
+        }
+      }
+      if (!ok || __any_sync(0xffffffffu, aborted(&bar->abort))) {
+        // let the copies in flight land before the CTA exits
+        if (nq) wait_warp(&bar->q_full, (nq - 1) & 1, a.status);
+        for (int s = 0; s < 2; ++s) {
+          if (nk[s]) wait_warp(&bar->k_full[s], (nk[s] - 1) & 1, a.status);
+          if (nv[s]) wait_warp(&bar->v_full[s], (nv[s] - 1) & 1, a.status);
+        }
+      }
+    } else if (warp == 9) {
+      // ------------------------------------------------------------ MMA issuer (the whole
+      // warp runs the loop, one elected lane issues each instruction)
+      constexpr uint32_t idesc_qk = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 0, 0) : ptx::idesc_bf16_f32(128, 128, 0, 0);
+      constexpr uint32_t idesc_pv = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 0, 1) : ptx::idesc_bf16_f32(128, kHD, 0, 1);
+      const uint32_t sQ0 = ptx::smem_u32(smem + L::QA);
+      uint32_t nq = 0, it = 0;       // units with key blocks, K / V blocks (all units)
+      uint32_t nb[2] = {0, 0};       // blocks of unit x so far (P hand-offs)
+      // head x: Q at sQ0 + x * kTB, S at tmem + 256 x, O at tmem + 128 + 256 x
+      auto issue_s = [&](int x, uint32_t blk) {
+        const uint32_t sK = ptx::smem_u32(smem + L::K + (blk & 1) * kTB);
+        const uint32_t sQ = sQ0 + (uint32_t)x * kTB, tS = tmem + 256u * (uint32_t)x;
+        if constexpr (kE4M3)  // 128-byte rows: k-steps of 32 bytes
+          ptx::mma4_e4m3_ss_warp<2, 2>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0), idesc_qk, 0u);
+        else if constexpr (kHD == 64)
+          ptx::mma4_bf16_ss_warp<2, 2>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0), idesc_qk, 0u);
+        else
+          ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0),
+                                                                    idesc_qk, 0u);
+        ptx::mma_commit_warp(&bar->s_full[x]);
+      };
+      // P V in two halves of 64 keys for bf16: the first as soon as the softmax
+      // warps have written P of keys [0, 64) (p_half), the second after p_full
+      auto issue_pv = [&](int x, uint32_t blk, bool first) -> bool {
+        const uint32_t sV = ptx::smem_u32(smem + L::V + (blk & 1) * kTB);
+        const uint32_t tS = tmem + 256u * (uint32_t)x, tO = tS + 128u;
+        if (!wait_warp(&bar->p_half[x], nb[x] & 1, a.status)) return false;
+        ptx::tc_fence_after();
+        if constexpr (!kE4M3) ptx::mma4_bf16_ts_warp<8, 128>(tO, tS, desc_mnmajor(sV, 0), idesc_pv, first ? 0u : 1u);
+        if constexpr (kHD == 64)  // the low parts of P
+          ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 64, desc_mnmajor(sV, 0), idesc_pv, 1u);
+        if (!wait_warp(&bar->p_full[x], nb[x] & 1, a.status)) return false;
+        ptx::tc_fence_after();
+        if constexpr (kE4M3)  // P: four e4m3 a column; V MN-major, 32 rows of 128 bytes a k-step
+          ptx::mma4_e4m3_ts_warp<8, 256>(tO, tS, desc_kmajor(sV, 0), idesc_pv, first ? 0u : 1u);
+        else  // keys [64, 128): P columns 32 + 8 kk, V rows 64 + 16 kk
+          ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 32, desc_mnmajor(sV, 4), idesc_pv, 1u);
+        if constexpr (kHD == 64) ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 96, desc_mnmajor(sV, 4), idesc_pv, 1u);
+        ptx::mma_commit_warp(&bar->pv_done[x]);
+        ++nb[x];
+        return true;
+      };
+      bool ok = true;
+      for (int64_t k = 0; ok; ++k) {
+        const int64_t u = unit_of(k, n_units);
+        if (u < 0) break;
+        const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
+        const int nkb = x.nkb();
+        if (nkb == 0) continue;
+        // unit y runs key blocks [0, nkb_y); the last unit reading block j
+        // releases its K / V stages (unit 1 whenever it has the block: nkb1 is
+        // either equal to nkb0, at least nkb0, or 0)
+        auto last_user = [&](int j) { return j < x.nkb1 ? 1 : 0; };
+        if (__shfl_sync(0xffffffffu, aborted(&bar->abort) ? 1 : 0, 0) ||
+            !wait_warp(&bar->q_full, nq & 1, a.status) || !wait_warp(&bar->k_full[it & 1], (it >> 1) & 1, a.status)) {
           ok = false;
           break;
         }
-        if (lane == 0) {
-          ptx::mbar_expect_tx(&bar->v_full[s], kTB);
-          load_tile(smem + L::V + s * kTB, &tmV, &bar->v_full[s], g * kHD, ky);
-        }
-        __syncwarp();
-        ++nv[s];
-      }
-    }
-    if (!ok || __any_sync(0xffffffffu, aborted(&bar->abort))) {
-      // let the copies in flight land before the CTA exits
-      if (nq) wait_warp(&bar->q_full, (nq - 1) & 1, a.status);
-      for (int s = 0; s < 2; ++s) {
-        if (nk[s]) wait_warp(&bar->k_full[s], (nk[s] - 1) & 1, a.status);
-        if (nv[s]) wait_warp(&bar->v_full[s], (nv[s] - 1) & 1, a.status);
-      }
-    }
-  } else if (warp == 9) {
-    // ------------------------------------------------------------ MMA issuer (the whole
-    // warp runs the loop, one elected lane issues each instruction)
-    constexpr uint32_t idesc_qk = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 0, 0) : ptx::idesc_bf16_f32(128, 128, 0, 0);
-    constexpr uint32_t idesc_pv = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 0, 1) : ptx::idesc_bf16_f32(128, kHD, 0, 1);
-    const uint32_t sQ0 = ptx::smem_u32(smem + L::QA);
-    uint32_t nq = 0, it = 0;       // units with key blocks, K / V blocks (all units)
-    uint32_t nb[2] = {0, 0};       // blocks of unit x so far (P hand-offs)
-    // head x: Q at sQ0 + x * kTB, S at tmem + 256 x, O at tmem + 128 + 256 x
-    auto issue_s = [&](int x, uint32_t blk) {
-      const uint32_t sK = ptx::smem_u32(smem + L::K + (blk & 1) * kTB);
-      const uint32_t sQ = sQ0 + (uint32_t)x * kTB, tS = tmem + 256u * (uint32_t)x;
-      if constexpr (kE4M3)  // 128-byte rows: k-steps of 32 bytes
-        ptx::mma4_e4m3_ss_warp<2, 2>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0), idesc_qk, 0u);
-      else if constexpr (kHD == 64)
-        ptx::mma4_bf16_ss_warp<2, 2>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0), idesc_qk, 0u);
-      else
-        ptx::mma8_bf16_ss_warp<ptx::KMajorSw128, ptx::KMajorSw128>(tS, desc_kmajor(sQ, 0), desc_kmajor(sK, 0),
-                                                                  idesc_qk, 0u);
-      ptx::mma_commit_warp(&bar->s_full[x]);
-    };
-    // P V in two halves of 64 keys for bf16: the first as soon as the softmax
-    // warps have written P of keys [0, 64) (p_half), the second after p_full
-    auto issue_pv = [&](int x, uint32_t blk, bool first) -> bool {
-      const uint32_t sV = ptx::smem_u32(smem + L::V + (blk & 1) * kTB);
-      const uint32_t tS = tmem + 256u * (uint32_t)x, tO = tS + 128u;
-      if (!wait_warp(&bar->p_half[x], nb[x] & 1, a.status)) return false;
-      ptx::tc_fence_after();
-      if constexpr (!kE4M3) ptx::mma4_bf16_ts_warp<8, 128>(tO, tS, desc_mnmajor(sV, 0), idesc_pv, first ? 0u : 1u);
-      if constexpr (kHD == 64)  // the low parts of P
-        ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 64, desc_mnmajor(sV, 0), idesc_pv, 1u);
-      if (!wait_warp(&bar->p_full[x], nb[x] & 1, a.status)) return false;
-      ptx::tc_fence_after();
-      if constexpr (kE4M3)  // P: four e4m3 a column; V MN-major, 32 rows of 128 bytes a k-step
-        ptx::mma4_e4m3_ts_warp<8, 256>(tO, tS, desc_kmajor(sV, 0), idesc_pv, first ? 0u : 1u);
-      else  // keys [64, 128): P columns 32 + 8 kk, V rows 64 + 16 kk
-        ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 32, desc_mnmajor(sV, 4), idesc_pv, 1u);
-      if constexpr (kHD == 64) ptx::mma4_bf16_ts_warp<8, 128>(tO, tS + 96, desc_mnmajor(sV, 4), idesc_pv, 1u);
-      ptx::mma_commit_warp(&bar->pv_done[x]);
-      ++nb[x];
-      return true;
-    };
-    bool ok = true;
-    for (int64_t k = 0; ok; ++k) {
-      const int64_t u = unit_of(k, n_units);
-      if (u < 0) break;
-      const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
-      const int nkb = x.nkb();
-      if (nkb == 0) continue;
-      // unit y runs key blocks [0, nkb_y); the last unit reading block j
-      // releases its K / V stages (unit 1 whenever it has the block: nkb1 is
-      // either equal to nkb0, at least nkb0, or 0)
-      auto last_user = [&](int j) { return j < x.nkb1 ? 1 : 0; };
-      if (__shfl_sync(0xffffffffu, aborted(&bar->abort) ? 1 : 0, 0) ||
-          !wait_warp(&bar->q_full, nq & 1, a.status) || !wait_warp(&bar->k_full[it & 1], (it >> 1) & 1, a.status)) {
-        ok = false;
-        break;
-      }
-      ++nq;
-      // S of block 0 overwrites the previous unit's last P: issued after that
-      // unit's last P V (in issue order; the drained variant waits for it)
-      if (a.flags & kFlagDrainTmemReuse)
-        for (int y = 0; ok && y < 2; ++y)
-          if (nb[y] > 0 && !wait_warp(&bar->pv_done[y], (nb[y] - 1) & 1, a.status)) ok = false;
-      if (!ok) break;
-      ptx::tc_fence_after();
-      if (x.nkb0 > 0) issue_s(0, it);
-      if (x.nkb1 > 0) issue_s(1, it);
-      ptx::mma_commit_warp(&bar->k_empty[it & 1]);
-      if (nkb == 1) ptx::mma_commit_warp(&bar->q_empty);  // every score MMA of the unit is issued
-      // Per block: PV_A(j), S_A(j+1), PV_B(j), S_B(j+1).  S_x(j+1) overwrites
-      // the P_x(j) that PV_x(j) reads; MMAs issued by this thread execute in
-      // order, so S_x(j+1) follows PV_x(j) without a wait (kFlagDrainTmemReuse
-      // makes it wait for PV_x(j) to complete instead).
-      for (int j = 0; ok && j < nkb; ++j) {
-        const uint32_t blk = it + (uint32_t)j;
-        const int s = blk & 1, s1 = (blk + 1) & 1;
-        const bool more = j + 1 < nkb;
-        if (__shfl_sync(0xffffffffu, aborted(&bar->abort) ? 1 : 0, 0)) { ok = false; break; }
-        if (!wait_warp(&bar->v_full[s], (blk >> 1) & 1, a.status)) { ok = false; break; }
-        if (more && !wait_warp(&bar->k_full[s1], ((blk + 1) >> 1) & 1, a.status)) { ok = false; break; }
-        for (int y = 0; y < 2; ++y) {
-          const int nkby = y ? x.nkb1 : x.nkb0;
-          if (j >= nkby) continue;
-          if (!issue_pv(y, blk, j == 0)) { ok = false; break; }
-          if (y == last_user(j)) ptx::mma_commit_warp(&bar->v_empty[s]);
-          if (j + 1 < nkby) {
-            if ((a.flags & kFlagDrainTmemReuse) && !wait_warp(&bar->pv_done[y], (nb[y] - 1) & 1, a.status)) {
-              ok = false;
-              break;
-            }
-            ptx::tc_fence_after();
-            issue_s(y, blk + 1);
-            if (y == last_user(j + 1)) {
-              ptx::mma_commit_warp(&bar->k_empty[s1]);
-              if (j + 2 == nkb) ptx::mma_commit_warp(&bar->q_empty);  // the unit's last score MMA
+        ++nq;
+        // S of block 0 overwrites the previous unit's last P: issued after that
+        // unit's last P V (in issue order; the drained variant waits for it)
+        if (a.flags & kFlagDrainTmemReuse)
+          for (int y = 0; ok && y < 2; ++y)
+            if (nb[y] > 0 && !wait_warp(&bar->pv_done[y], (nb[y] - 1) & 1, a.status)) ok = false;
+        if (!ok) break;
+        ptx::tc_fence_after();
+        if (x.nkb0 > 0) issue_s(0, it);
+        if (x.nkb1 > 0) issue_s(1, it);
+        ptx::mma_commit_warp(&bar->k_empty[it & 1]);
+        if (nkb == 1) ptx::mma_commit_warp(&bar->q_empty);  // every score MMA of the unit is issued
+        // Per block: PV_A(j), S_A(j+1), PV_B(j), S_B(j+1).  S_x(j+1) overwrites
+        // the P_x(j) that PV_x(j) reads; MMAs issued by this thread execute in
+        // order, so S_x(j+1) follows PV_x(j) without a wait (kFlagDrainTmemReuse
+        // makes it wait for PV_x(j) to complete instead).
+        for (int j = 0; ok && j < nkb; ++j) {
+          const uint32_t blk = it + (uint32_t)j;
+          const int s = blk & 1, s1 = (blk + 1) & 1;
+          const bool more = j + 1 < nkb;
+          if (__shfl_sync(0xffffffffu, aborted(&bar->abort) ? 1 : 0, 0)) { ok = false; break; }
+          if (!wait_warp(&bar->v_full[s], (blk >> 1) & 1, a.status)) { ok = false; break; }
+          if (more && !wait_warp(&bar->k_full[s1], ((blk + 1) >> 1) & 1, a.status)) { ok = false; break; }
+          for (int y = 0; y < 2; ++y) {
+            const int nkby = y ? x.nkb1 : x.nkb0;
+            if (j >= nkby) continue;
+            if (!issue_pv(y, blk, j == 0)) { ok = false; break; }
+            if (y == last_user(j)) ptx::mma_commit_warp(&bar->v_empty[s]);
+            if (j + 1 < nkby) {
+              if ((a.flags & kFlagDrainTmemReuse) && !wait_warp(&bar->pv_done[y], (nb[y] - 1) & 1, a.status)) {
+                ok = false;
+                break;
+              }
+              ptx::tc_fence_after();
+              issue_s(y, blk + 1);
+              if (y == last_user(j + 1)) {
+                ptx::mma_commit_warp(&bar->k_empty[s1]);
+                if (j + 2 == nkb) ptx::mma_commit_warp(&bar->q_empty);  // the unit's last score MMA
+              }
             }
           }
         }
+        it += (uint32_t)nkb;
       }
-      it += (uint32_t)nkb;
+      if (!ok && lane == 0) set_abort(&bar->abort);
+      __syncwarp();
+      ptx::mma_commit_warp(&bar->final_mma);
+      wait_warp(&bar->final_mma, 0, a.status);
+      __syncwarp();
     }
-    if (!ok && lane == 0) set_abort(&bar->abort);
-    __syncwarp();
-    ptx::mma_commit_warp(&bar->final_mma);
-    wait_warp(&bar->final_mma, 0, a.status);
-    __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax of head x
+    ptx::setmaxnreg_inc<kRegsSoftmax>();
     const int xh = warp >> 2;
     const int r = threadIdx.x & 127;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;

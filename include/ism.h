@@ -547,6 +547,67 @@ const char* ism_last_error(void);
 /* 1 if the library was built with the sm_103a tensor-core kernels. */
 int32_t ism_has_tensor_cores(void);
 
+/* ---------------------------------------------------------------------------
+ * The same calls with their arguments in one struct, for bindings where each
+ * argument of a foreign call costs time.  Every field means what the argument
+ * of its name means above; shapes are given as heads, head_dim, dtype and a
+ * softmax_scale that is rounded to float.  No state, no checks of their own.
+ * `form` names the call: the sum of ISM_CALL_E4M3, ISM_CALL_ROPE, ISM_CALL_PAGED.
+ *   ism_call_fwd: ism_attn_fwd, ISM_CALL_E4M3: ism_attn_fwd_e4m3, ISM_CALL_ROPE:
+ *     ism_attn_fwd_rope; with plan (not e4m3) the planned forms.
+ *   ism_call_bwd: ism_attn_bwd, ISM_CALL_ROPE: ism_attn_bwd_rope (q, k the
+ *     rotated ones); with plan the planned forms.
+ *   ism_call_pass_sizes: bytes[0] = ism_attn_fwd_workspace_size, or
+ *     backward != 0: bytes[0], bytes[1] = ism_attn_bwd_workspace_size, _min.
+ *   ism_call_append: ism_attn_prefill_append, ISM_CALL_PAGED: the paged form,
+ *     ISM_CALL_E4M3: the e4m3 form (not paged), with ISM_CALL_ROPE their rotary
+ *     forms.
+ * ------------------------------------------------------------------------- */
+enum { ISM_CALL_E4M3 = 1, ISM_CALL_ROPE = 2, ISM_CALL_PAGED = 4 };
+
+typedef struct {
+  ism_segments_t segs;
+  int32_t num_heads_q, num_heads_kv, head_dim, dtype, form;
+  double softmax_scale, q_descale, k_descale, v_descale;
+  ism_rope_t rope;
+  void* plan;
+  ism_attn_plan_info_t plan_info;
+  const void *q, *k, *v;
+  void* o;
+  float* lse;
+  const void* dout;
+  void *dq, *dk, *dv, *q_rot, *k_rot;
+  void* workspace;
+  size_t workspace_bytes;
+  ism_stream_t stream;
+} ism_pass_call_t;
+
+ism_status_t ism_call_fwd(const ism_pass_call_t* call);
+ism_status_t ism_call_bwd(const ism_pass_call_t* call);
+ism_status_t ism_call_pass_sizes(const ism_pass_call_t* call, int32_t backward, size_t* bytes);
+
+typedef struct {
+  int32_t num_heads_q, num_heads_kv, head_dim, dtype, form;
+  double softmax_scale, q_descale, k_descale, v_descale;
+  ism_rope_t rope;
+  int32_t batch, l_new, n_new_segs, num_pages, page_size, max_pages;
+  const int32_t* new_seg_end_host;
+  const uint8_t* new_seg_type_host;
+  const void *q_new, *k_new, *v_new;
+  void *k_cache, *v_cache;
+  int64_t cache_capacity;
+  const int32_t *block_table, *block_table_host;
+  int32_t* cache_len;
+  const int32_t* cache_len_host;
+  void* o_new;
+  float* lse_new;
+  void* workspace;
+  size_t workspace_bytes;
+  ism_stream_t stream;
+} ism_append_call_t;
+
+ism_status_t ism_call_append(const ism_append_call_t* call);
+
 #ifdef __cplusplus
 }
 #endif

@@ -8,7 +8,10 @@ is raised.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
+import struct
+from array import array
 from dataclasses import dataclass
 from typing import Optional
 
@@ -110,7 +113,22 @@ EXPORTS = {
     "ism_attn_bwd_planned": (C.c_int, [C.c_void_p] * 14 + [C.c_size_t, C.c_void_p]),
     "ism_attn_fwd_rope_planned": (C.c_int, [C.c_void_p] * 13),
     "ism_attn_bwd_rope_planned": (C.c_int, [C.c_void_p] * 15 + [C.c_size_t, C.c_void_p]),
+    "ism_call_fwd": (C.c_int, [C.c_char_p]),
+    "ism_call_bwd": (C.c_int, [C.c_char_p]),
+    "ism_call_pass_sizes": (C.c_int, [C.c_char_p, C.c_int32, C.c_void_p]),
+    "ism_call_append": (C.c_int, [C.c_char_p]),
 }
+
+# The argument structs of ism_call_* (ism_pass_call_t, ism_append_call_t) as
+# packed bytes: one pointer to marshal instead of some twenty arguments.
+#   segments; heads, head_dim, dtype, form; scale, descales; rope; plan, fingerprint, bytes;
+#   q, k, v, o, lse, dout, dq, dk, dv, q_rot, k_rot; workspace, its bytes; stream
+_PASS = struct.Struct("@2i8P5i4d2PiPQN11PPNP")
+#   heads, head_dim, dtype, form; scale, descales; rope; batch, l_new, n_new_segs, num_pages, page_size,
+#   max_pages; segments; q, k, v, caches; capacity; block tables; cache lengths; o, lse; workspace, its bytes; stream
+_APPEND = struct.Struct("@5i4d2Pi4x6i2P5Pq2P2P2PPNP")
+_NO_ROPE, _NO_PLAN = (0, 0, 0), (0, 0, 0)
+_FORM_E4M3, _FORM_ROPE, _FORM_PAGED = 1, 2, 4
 
 KERNEL_FWD, KERNEL_BWD_DKDV, KERNEL_BWD_DQ, KERNEL_BWD_PRE, KERNEL_DECODE, KERNEL_META, KERNEL_ROPE = 1, 2, 3, 4, 5, 6, 7
 
@@ -153,6 +171,29 @@ def _stream(device=None):
     return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
 
 
+def _raw_stream(t: torch.Tensor) -> int:
+    """The current stream of the tensor's device, as an integer."""
+    i = t.get_device()
+    return torch._C._cuda_getCurrentRawStream(i) if i >= 0 else torch.cuda.current_stream(t.device).cuda_stream
+
+
+def _addr(a: np.ndarray) -> int:
+    return a.__array_interface__["data"][0]
+
+
+def _host_array(x, dtype, code):
+    """(address, length, owner) of a host array of the given element type; the
+    owner must outlive the call."""
+    if type(x) is list:
+        try:
+            x = array(code, x)
+            return (*x.buffer_info(), x)
+        except TypeError:  # other numbers: as numpy converts them
+            pass
+    x = np.ascontiguousarray(x, dtype=dtype)
+    return _addr(x), x.shape[0], x
+
+
 def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.bfloat16:
         return ISM_BF16
@@ -164,9 +205,12 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _workspace(nbytes: int, device) -> torch.Tensor:
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    if ws.data_ptr() % 256 == 0:  # as the caching allocator hands it out
+        return ws
     ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
     off = (-ws.data_ptr()) % 256
-    return ws[off:off + nbytes] if nbytes else ws[off:off]
+    return ws[off:off + nbytes]
 
 
 @dataclass
@@ -196,6 +240,13 @@ class Segments:
     @property
     def total_tokens(self) -> int:
         return int(self.cu_seqlens_host[-1])
+
+    def fields(self):
+        """The values of ism_segments_t, in order."""
+        return (self.cu_seqlens_host.shape[0] - 1, self.seg_end_host.shape[0],
+                self.cu_seqlens.data_ptr(), _addr(self.cu_seqlens_host), self.cu_segs.data_ptr(),
+                _addr(self.cu_segs_host), self.seg_end.data_ptr(), _addr(self.seg_end_host),
+                self.seg_type.data_ptr(), _addr(self.seg_type_host))
 
     def struct(self) -> _Segments:
         s = _Segments()
@@ -270,33 +321,54 @@ class Plan:
         return self
 
 
+def _pass_head(segs: Segments, q, k, softmax_scale: float, form: int, descales=(0.0, 0.0, 0.0)):
+    """The leading values of ism_pass_call_t."""
+    return (*segs.fields(), q.shape[-2], k.shape[-2], q.shape[-1], _dtype_code(q), form, float(softmax_scale),
+            *descales)
+
+
+_NO_TENSORS = (0,) * 14
+
+
+def _pass_sizes(head, backward: bool):
+    """Workspace bytes of the forward, or (full, minimum) of the backward."""
+    out = (C.c_size_t * 2)()
+    _check(load().ism_call_pass_sizes(_PASS.pack(*head, *_NO_ROPE, *_NO_PLAN, *_NO_TENSORS), backward, out),
+           "ism_attn_bwd_workspace_size" if backward else "ism_attn_fwd_workspace_size")
+    return (out[0], out[1]) if backward else out[0]
+
+
+def _plan_fields(plan: "Plan"):
+    return (plan.buffer.data_ptr(), plan.info.fingerprint, plan.info.bytes) if plan is not None else _NO_PLAN
+
+
+def _run_fwd(name, head, rope, plan, q, k, v, out, lse, q_rot, k_rot, workspace):
+    """The forward of ism_call_fwd on given outputs; allocates the workspace
+    where one is needed and none (or too small a one) is given."""
+    ws = (0, 0)
+    if plan is None:
+        nbytes = _pass_sizes(head, False)
+        if workspace is None or workspace.numel() < nbytes:
+            workspace = _workspace(nbytes, q.device)
+        ws = (workspace.data_ptr(), workspace.numel())
+    _check(load().ism_call_fwd(_PASS.pack(
+        *head, *rope, *_plan_fields(plan), q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr(),
+        0, 0, 0, 0, 0 if q_rot is None else q_rot.data_ptr(), 0 if k_rot is None else k_rot.data_ptr(), *ws,
+        _raw_stream(q))), name + ("" if plan is None else "_planned"))
+
+
 def fwd(segs: Segments, q, k, v, softmax_scale: float, out=None, lse=None, workspace=None, plan: Plan = None):
     """Forward over packed dialogues.  q [T,Hq,D], k/v [T,Hkv,D] -> (o, lse [Hq,T]).
     With a plan of these segments the metadata pass is not run again (and no
     workspace is needed)."""
-    lib = load()
     _contig(q, k, v)
     T, hq, D = q.shape
-    s, sh = segs.struct(), _shape(q, k, softmax_scale)
-    if plan is not None:
-        if out is None:
-            out = torch.empty_like(q)
-        if lse is None:
-            lse = torch.empty((hq, T), dtype=torch.float32, device=q.device)
-        _check(lib.ism_attn_fwd_planned(C.byref(s), C.byref(sh), _ptr(plan.buffer), C.byref(plan.info), _ptr(q),
-                                        _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _stream(q.device)),
-               "ism_attn_fwd_planned")
-        return out, lse
-    nbytes = C.c_size_t()
-    _check(lib.ism_attn_fwd_workspace_size(C.byref(s), C.byref(sh), C.byref(nbytes)), "ism_attn_fwd_workspace_size")
     if out is None:
         out = torch.empty_like(q)
     if lse is None:
         lse = torch.empty((hq, T), dtype=torch.float32, device=q.device)
-    if workspace is None or workspace.numel() < nbytes.value:
-        workspace = _workspace(nbytes.value, q.device)
-    _check(lib.ism_attn_fwd(C.byref(s), C.byref(sh), _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse),
-                            _ptr(workspace), workspace.numel(), _stream(q.device)), "ism_attn_fwd")
+    _run_fwd("ism_attn_fwd", _pass_head(segs, q, k, softmax_scale, 0), _NO_ROPE, plan, q, k, v, out, lse, None, None,
+             workspace)
     return out, lse
 
 
@@ -305,21 +377,14 @@ def fwd_e4m3(segs: Segments, q, k, v, q_descale: float, k_descale: float, v_desc
     """Forward with e4m3 inputs (torch.float8_e4m3fn; head_dim 128): the
     attention of q * q_descale, k * k_descale, v * v_descale.  Returns
     (o bf16 [T,Hq,D], lse [Hq,T])."""
-    lib = load()
     _contig(q, k, v)
     T, hq, D = q.shape
-    s, sh = segs.struct(), _shape(q, k, softmax_scale)
-    nbytes = C.c_size_t()
-    _check(lib.ism_attn_fwd_workspace_size(C.byref(s), C.byref(sh), C.byref(nbytes)), "ism_attn_fwd_workspace_size")
     if out is None:
         out = torch.empty(q.shape, dtype=torch.bfloat16, device=q.device)
     if lse is None:
         lse = torch.empty((hq, T), dtype=torch.float32, device=q.device)
-    if workspace is None or workspace.numel() < nbytes.value:
-        workspace = _workspace(nbytes.value, q.device)
-    _check(lib.ism_attn_fwd_e4m3(C.byref(s), C.byref(sh), _ptr(q), _ptr(k), _ptr(v), q_descale, k_descale, v_descale,
-                                 _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel(), _stream(q.device)),
-           "ism_attn_fwd_e4m3")
+    _run_fwd("ism_attn_fwd_e4m3", _pass_head(segs, q, k, softmax_scale, _FORM_E4M3, (q_descale, k_descale, v_descale)),
+             _NO_ROPE, None, q, k, v, out, lse, None, None, workspace)
     return out, lse
 
 
@@ -329,28 +394,38 @@ def fwd_rope(segs: Segments, q, k, v, rope_cos, rope_sin, softmax_scale: float, 
     are rotated at their positions inside their sequences (tables rope_cos /
     rope_sin float32 [rows, D/2]) into q_rot / k_rot, then attended.
     Returns (o, lse, q_rot, k_rot); the backward takes q_rot and k_rot."""
-    lib = load()
     _contig(q, k, v)
     T, hq, D = q.shape
-    s, sh = segs.struct(), _shape(q, k, softmax_scale)
-    rope = _rope_struct(rope_cos, rope_sin)
-    nbytes = C.c_size_t()
-    _check(lib.ism_attn_fwd_workspace_size(C.byref(s), C.byref(sh), C.byref(nbytes)), "ism_attn_fwd_workspace_size")
+    rope = _rope_fields(rope_cos, rope_sin)
     q_rot = torch.empty_like(q) if q_rot is None else q_rot
     k_rot = torch.empty_like(k) if k_rot is None else k_rot
     out = torch.empty_like(q) if out is None else out
     lse = torch.empty((hq, T), dtype=torch.float32, device=q.device) if lse is None else lse
-    if plan is not None:  # the plan's metadata instead of a metadata pass
-        _check(lib.ism_attn_fwd_rope_planned(C.byref(s), C.byref(sh), _ptr(plan.buffer), C.byref(plan.info),
-                                             _ptr(q), _ptr(k), _ptr(v), C.byref(rope), _ptr(q_rot), _ptr(k_rot),
-                                             _ptr(out), _ptr(lse), _stream(q.device)), "ism_attn_fwd_rope_planned")
-        return out, lse, q_rot, k_rot
-    if workspace is None or workspace.numel() < nbytes.value:
-        workspace = _workspace(nbytes.value, q.device)
-    _check(lib.ism_attn_fwd_rope(C.byref(s), C.byref(sh), _ptr(q), _ptr(k), _ptr(v), C.byref(rope), _ptr(q_rot),
-                                 _ptr(k_rot), _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel(),
-                                 _stream(q.device)), "ism_attn_fwd_rope")
+    _run_fwd("ism_attn_fwd_rope", _pass_head(segs, q, k, softmax_scale, _FORM_ROPE), rope, plan, q, k, v, out, lse,
+             q_rot, k_rot, workspace)
     return out, lse, q_rot, k_rot
+
+
+def _run_bwd(name, head, rope, plan, q, k, v, o, lse, dout, dq, dk, dv, workspace, minimal, fall_back):
+    """The backward of ism_call_bwd.  Without a workspace (or with one below
+    the minimum) it allocates the full one, or the minimum: with `minimal`, or
+    with `fall_back` when the full one does not fit."""
+    full, low = _pass_sizes(head, True)
+    dq = torch.empty_like(q) if dq is None else dq
+    dk = torch.empty_like(k) if dk is None else dk
+    dv = torch.empty_like(v) if dv is None else dv
+    if workspace is None or workspace.numel() < low:
+        try:
+            workspace = _workspace(low if minimal else full, q.device)
+        except torch.cuda.OutOfMemoryError:
+            if minimal or not fall_back:
+                raise
+            workspace = _workspace(low, q.device)
+    _check(load().ism_call_bwd(_PASS.pack(
+        *head, *rope, *_plan_fields(plan), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+        dout.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), 0, 0, workspace.data_ptr(), workspace.numel(),
+        _raw_stream(q))), name + ("" if plan is None else "_planned"))
+    return dq, dk, dv
 
 
 def bwd_rope(segs: Segments, q_rot, k_rot, v, o, lse, dout, rope_cos, rope_sin, softmax_scale: float, dq=None,
@@ -358,29 +433,10 @@ def bwd_rope(segs: Segments, q_rot, k_rot, v, o, lse, dout, rope_cos, rope_sin, 
     """Backward of ``fwd_rope``: takes the rotated q_rot / k_rot the forward
     wrote and returns (dq, dk, dv) with dq, dk the gradients of the UNROTATED
     queries and keys.  Workspace as for ``bwd``."""
-    lib = load()
     _contig(q_rot, k_rot, v, o, lse, dout)
-    s, sh = segs.struct(), _shape(q_rot, k_rot, softmax_scale)
-    rope = _rope_struct(rope_cos, rope_sin)
-    full, low = C.c_size_t(), C.c_size_t()
-    _check(lib.ism_attn_bwd_workspace_size(C.byref(s), C.byref(sh), C.byref(full)), "ism_attn_bwd_workspace_size")
-    _check(lib.ism_attn_bwd_workspace_size_min(C.byref(s), C.byref(sh), C.byref(low)),
-           "ism_attn_bwd_workspace_size_min")
-    dq = torch.empty_like(q_rot) if dq is None else dq
-    dk = torch.empty_like(k_rot) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    if workspace is None or workspace.numel() < low.value:
-        workspace = _workspace(low.value if minimal_workspace else full.value, q_rot.device)
-    if plan is not None:  # the plan's metadata instead of a metadata pass
-        _check(lib.ism_attn_bwd_rope_planned(C.byref(s), C.byref(sh), _ptr(plan.buffer), C.byref(plan.info),
-                                             _ptr(q_rot), _ptr(k_rot), _ptr(v), _ptr(o), _ptr(lse), _ptr(dout),
-                                             C.byref(rope), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace),
-                                             workspace.numel(), _stream(q_rot.device)), "ism_attn_bwd_rope_planned")
-        return dq, dk, dv
-    _check(lib.ism_attn_bwd_rope(C.byref(s), C.byref(sh), _ptr(q_rot), _ptr(k_rot), _ptr(v), _ptr(o), _ptr(lse),
-                                 _ptr(dout), C.byref(rope), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace),
-                                 workspace.numel(), _stream(q_rot.device)), "ism_attn_bwd_rope")
-    return dq, dk, dv
+    return _run_bwd("ism_attn_bwd_rope", _pass_head(segs, q_rot, k_rot, softmax_scale, _FORM_ROPE),
+                    _rope_fields(rope_cos, rope_sin), plan, q_rot, k_rot, v, o, lse, dout, dq, dk, dv, workspace,
+                    minimal_workspace, False)
 
 
 def bwd_workspace_size(segs: Segments, q, k, softmax_scale: float, minimal: bool = False) -> int:
@@ -402,53 +458,65 @@ def bwd(segs: Segments, q, k, v, o, lse, dout, softmax_scale: float, dq=None, dk
     least the minimum); without one, a workspace of the stored-dS size is
     allocated (the minimum with minimal_workspace=True, or when the larger
     one does not fit in device memory)."""
-    lib = load()
     _contig(q, k, v, o, lse, dout)
-    s, sh = segs.struct(), _shape(q, k, softmax_scale)
-    full, low = C.c_size_t(), C.c_size_t()
-    _check(lib.ism_attn_bwd_workspace_size(C.byref(s), C.byref(sh), C.byref(full)), "ism_attn_bwd_workspace_size")
-    _check(lib.ism_attn_bwd_workspace_size_min(C.byref(s), C.byref(sh), C.byref(low)),
-           "ism_attn_bwd_workspace_size_min")
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    if workspace is None or workspace.numel() < low.value:
-        if minimal_workspace:
-            workspace = _workspace(low.value, q.device)
-        else:
-            try:
-                workspace = _workspace(full.value, q.device)
-            except torch.cuda.OutOfMemoryError:
-                workspace = _workspace(low.value, q.device)
-    if plan is not None:  # the plan's metadata instead of a metadata pass
-        _check(lib.ism_attn_bwd_planned(C.byref(s), C.byref(sh), _ptr(plan.buffer), C.byref(plan.info), _ptr(q),
-                                        _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(dout), _ptr(dq), _ptr(dk),
-                                        _ptr(dv), _ptr(workspace), workspace.numel(), _stream(q.device)),
-               "ism_attn_bwd_planned")
-        return dq, dk, dv
-    _check(lib.ism_attn_bwd(C.byref(s), C.byref(sh), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(dout),
-                            _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace), workspace.numel(), _stream(q.device)),
-           "ism_attn_bwd")
-    return dq, dk, dv
+    return _run_bwd("ism_attn_bwd", _pass_head(segs, q, k, softmax_scale, 0), _NO_ROPE, plan, q, k, v, o, lse, dout,
+                    dq, dk, dv, workspace, minimal_workspace, True)
+
+
+@functools.lru_cache(maxsize=256)
+def _append_size(hq: int, hkv: int, D: int, dtype: int, batch: int, l_new: int, rope: bool) -> int:
+    """Workspace bytes of an append, a function of these numbers alone."""
+    sh = _Shape(hq, hkv, D, dtype, 1.0)
+    nbytes = C.c_size_t()
+    name = "ism_attn_prefill_append_rope_workspace_size" if rope else "ism_attn_prefill_append_workspace_size"
+    _check(getattr(load(), name)(C.byref(sh), batch, l_new, C.byref(nbytes)), name)
+    return nbytes.value
 
 
 def append_workspace_size(q_new, k_new, softmax_scale: float, rope: bool = False) -> int:
     """Workspace bytes ``prefill_append`` (``prefill_append_rope`` when rope is
     set) needs for this batch and chunk length."""
-    lib = load()
-    B, Ln = q_new.shape[0], q_new.shape[1]
-    sh = _shape(q_new, k_new, softmax_scale)
-    nbytes = C.c_size_t()
-    name = "ism_attn_prefill_append_rope_workspace_size" if rope else "ism_attn_prefill_append_workspace_size"
-    _check(getattr(lib, name)(C.byref(sh), B, Ln, C.byref(nbytes)), name)
-    return nbytes.value
+    B, Ln, hq, D = q_new.shape
+    return _append_size(hq, k_new.shape[-2], D, _dtype_code(q_new), B, Ln, rope)
 
 
-def _rope_struct(cos, sin) -> _Rope:
+def _rope_fields(cos, sin):
+    """The values of ism_rope_t."""
     _contig(cos, sin)
     if cos.dtype != torch.float32 or sin.dtype != torch.float32 or cos.shape != sin.shape or cos.dim() != 2:
         raise ValueError("rope tables must be float32 [rows, head_dim/2] tensors of one shape")
-    return _Rope(_ptr(cos), _ptr(sin), cos.shape[0])
+    return cos.data_ptr(), sin.data_ptr(), cos.shape[0]
+
+
+def _append(name, form, dtype, q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_host, new_seg_end,
+            new_seg_type, softmax_scale, out, lse, workspace, rope=_NO_ROPE, descales=(1.0, 1.0, 1.0), capacity=0,
+            pages=(0, 0, 0), tables=(0, 0), keep_small=False, prepare=False):
+    """One append call (ism_append_call_t); allocates what is not given (a given
+    workspace that is too small is replaced unless keep_small).  pages:
+    num_pages, page_size, max_pages.  prepare: returns the packed call and what
+    its addresses point to instead of running it."""
+    B, Ln, hq, D = q_new.shape
+    hkv = k_new.shape[-2]
+    if out is None:
+        out = torch.empty(q_new.shape, dtype=torch.bfloat16 if dtype == ISM_E4M3 else q_new.dtype, device=q_new.device)
+    if lse is None:
+        lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device)
+    nbytes = _append_size(hq, hkv, D, dtype, B, Ln, form & _FORM_ROPE)
+    if workspace is None or (not keep_small and workspace.numel() < nbytes):
+        workspace = _workspace(nbytes, q_new.device)
+    end_addr, n_segs, end = _host_array(new_seg_end, np.int32, "i")
+    type_addr, _, types = _host_array(new_seg_type, np.uint8, "B")
+    len_addr, _, lens = _host_array(cache_len_host, np.int32, "i")
+    call = _APPEND.pack(hq, hkv, D, dtype, form, softmax_scale, *descales, *rope, B, Ln, n_segs, *pages, end_addr,
+                        type_addr, q_new.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), k_cache.data_ptr(),
+                        v_cache.data_ptr(), capacity, *tables, cache_len.data_ptr(), len_addr, out.data_ptr(),
+                        lse.data_ptr(), workspace.data_ptr(), workspace.numel(), _raw_stream(q_new))
+    if prepare:
+        return out, lse, call, (end, types, lens, workspace)
+    code = load().ism_call_append(call)
+    if code:
+        _check(code, name)
+    return out, lse
 
 
 def prefill_append_rope(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_host, new_seg_end, new_seg_type,
@@ -457,28 +525,10 @@ def prefill_append_rope(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_
     positions cache_len[b] + j (rotate-half pairs, angles given by the fp32
     tables rope_cos / rope_sin [rows, D/2]); the caches receive the rotated
     keys.  Returns (o_new, lse [Hq,B,Ln])."""
-    lib = load()
     _contig(q_new, k_new, v_new, k_cache, v_cache, cache_len)
-    B, Ln, hq, D = q_new.shape
-    sh = _shape(q_new, k_new, softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    rope = _rope_struct(rope_cos, rope_sin)
-    nbytes = append_workspace_size(q_new, k_new, softmax_scale, rope=True)
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device)
-    if workspace is None or workspace.numel() < nbytes:
-        workspace = _workspace(nbytes, q_new.device)
-    _check(lib.ism_attn_prefill_append_rope(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                            C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data), se.shape[0],
-                                            _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(cache_len),
-                                            C.c_void_p(ch.ctypes.data), C.byref(rope), _ptr(out), _ptr(lse),
-                                            _ptr(workspace), workspace.numel(), _stream(q_new.device)),
-           "ism_attn_prefill_append_rope")
-    return out, lse
+    return _append("ism_attn_prefill_append_rope", _FORM_ROPE, _dtype_code(q_new), q_new, k_new, v_new, k_cache, v_cache,
+                   cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace,
+                   _rope_fields(rope_cos, rope_sin), capacity=k_cache.shape[1])
 
 
 def prefill_append(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_host, new_seg_end, new_seg_type,
@@ -487,30 +537,10 @@ def prefill_append(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_h
     q_new [B,Ln,Hq,D], k_new/v_new [B,Ln,Hkv,D], caches [B,cap,Hkv,D],
     cache_len int32 [B] on the device (advanced by Ln), cache_len_host its
     host mirror (the caller advances it).  Returns (o_new, lse [Hq,B,Ln])."""
-    lib = load()
     _contig(q_new, k_new, v_new, k_cache, v_cache, cache_len)
-    B, Ln, hq, D = q_new.shape
-    cap = k_cache.shape[1]
-    sh = _shape(q_new, k_new, softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    nbytes = C.c_size_t()
-    _check(lib.ism_attn_prefill_append_workspace_size(C.byref(sh), B, Ln, C.byref(nbytes)),
-           "ism_attn_prefill_append_workspace_size")
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device)
-    if workspace is None or workspace.numel() < nbytes.value:
-        workspace = _workspace(nbytes.value, q_new.device)
-    _check(lib.ism_attn_prefill_append(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                       C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data), se.shape[0],
-                                       _ptr(k_cache), _ptr(v_cache), cap, _ptr(cache_len), C.c_void_p(ch.ctypes.data),
-                                       _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel(),
-                                       _stream(q_new.device)),
-           "ism_attn_prefill_append")
-    return out, lse
+    return _append("ism_attn_prefill_append", 0, _dtype_code(q_new), q_new, k_new, v_new, k_cache, v_cache, cache_len,
+                   cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace,
+                   capacity=k_cache.shape[1])
 
 
 class AppendStep:
@@ -527,33 +557,19 @@ class AppendStep:
         if not (isinstance(cache_len_host, np.ndarray) and cache_len_host.dtype == np.int32 and
                 cache_len_host.flags["C_CONTIGUOUS"]):
             raise TypeError("cache_len_host must be a contiguous int32 numpy array (advanced in place)")
-        B, Ln, hq, D = q_new.shape
-        self._sh = _shape(q_new, k_new, softmax_scale)
-        self._se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-        self._st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-        self._host = cache_len_host
-        self.out = torch.empty_like(q_new) if out is None else out
-        self.lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device) if lse is None else lse
-        if workspace is None:
-            workspace = _workspace(append_workspace_size(q_new, k_new, softmax_scale, rope=rope is not None),
-                                   q_new.device)
-        self._keep = (q_new, k_new, v_new, k_cache, v_cache, cache_len, workspace, rope)
-        head = (C.byref(self._sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                C.c_void_p(self._se.ctypes.data), C.c_void_p(self._st.ctypes.data), self._se.shape[0],
-                _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(cache_len),
-                C.c_void_p(cache_len_host.ctypes.data))
-        tail = (_ptr(self.out), _ptr(self.lse), _ptr(workspace), workspace.numel(), _stream(q_new.device))
-        if rope is None:
-            self._name = "ism_attn_prefill_append"
-            self._args = head + tail
-        else:
-            self._rope = _rope_struct(*rope)
-            self._name = "ism_attn_prefill_append_rope"
-            self._args = head + (C.byref(self._rope),) + tail
-        self._fn = getattr(lib, self._name)
+        self._name = "ism_attn_prefill_append" if rope is None else "ism_attn_prefill_append_rope"
+        self.out, self.lse, self._call, kept = _append(
+            self._name, 0 if rope is None else _FORM_ROPE, _dtype_code(q_new), q_new, k_new, v_new, k_cache, v_cache,
+            cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace,
+            _NO_ROPE if rope is None else _rope_fields(*rope), capacity=k_cache.shape[1], keep_small=True, prepare=True)
+        # what the packed addresses point to
+        self._keep = (q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_host, rope, kept)
+        self._fn = lib.ism_call_append
 
     def __call__(self):
-        _check(self._fn(*self._args), self._name)
+        code = self._fn(self._call)
+        if code:
+            _check(code, self._name)
         return self.out, self.lse
 
 
@@ -562,27 +578,23 @@ def prefill_append_e4m3(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_
                         workspace=None):
     """``prefill_append`` with e4m3 (torch.float8_e4m3fn) q_new, k_new, v_new and
     caches, dequantised by the per-tensor factors; returns (o bf16, lse)."""
-    lib = load()
     _contig(q_new, k_new, v_new, k_cache, v_cache, cache_len)
-    B, Ln, hq, D = q_new.shape
-    cap = k_cache.shape[1]
-    sh = _shape(q_new, k_new, softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    if out is None:
-        out = torch.empty(q_new.shape, dtype=torch.bfloat16, device=q_new.device)
-    if lse is None:
-        lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device)
-    if workspace is None:
-        workspace = _workspace(append_workspace_size(q_new, k_new, softmax_scale), q_new.device)
-    _check(lib.ism_attn_prefill_append_e4m3(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                            C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data), se.shape[0],
-                                            _ptr(k_cache), _ptr(v_cache), cap, _ptr(cache_len),
-                                            C.c_void_p(ch.ctypes.data), q_descale, k_descale, v_descale, _ptr(out),
-                                            _ptr(lse), _ptr(workspace), workspace.numel(), _stream(q_new.device)),
-           "ism_attn_prefill_append_e4m3")
-    return out, lse
+    return _append("ism_attn_prefill_append_e4m3", _FORM_E4M3, _dtype_code(q_new), q_new, k_new, v_new, k_cache, v_cache,
+                   cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace,
+                   keep_small=True, descales=(q_descale, k_descale, v_descale), capacity=k_cache.shape[1])
+
+
+def _paged(name, form, q_new, k_new, v_new, k_pool, v_pool, page_size, block_table, block_table_host, cache_len,
+           cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace, rope=_NO_ROPE):
+    _contig(q_new, k_new, v_new, k_pool, v_pool, cache_len, block_table)
+    rows = k_pool.shape[0]
+    if rows % page_size:
+        raise ValueError("pool rows must be a whole number of pages")
+    bt = np.ascontiguousarray(block_table_host, dtype=np.int32)
+    return _append(name, form | _FORM_PAGED, _dtype_code(q_new), q_new, k_new, v_new, k_pool, v_pool, cache_len,
+                   cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace, rope, keep_small=True,
+                   pages=(rows // page_size, page_size, block_table.shape[1]),
+                   tables=(block_table.data_ptr(), _addr(bt)))
 
 
 def prefill_append_paged(q_new, k_new, v_new, k_pool, v_pool, page_size: int, block_table, block_table_host,
@@ -593,31 +605,9 @@ def prefill_append_paged(q_new, k_new, v_new, k_pool, v_pool, page_size: int, bl
     block_table[b, p // page_size] * page_size + p % page_size.  block_table
     int32 [B, max_pages] on the device, block_table_host its host mirror
     (numpy); cache_len / cache_len_host as for ``prefill_append``."""
-    lib = load()
-    _contig(q_new, k_new, v_new, k_pool, v_pool, cache_len, block_table)
-    B, Ln, hq, D = q_new.shape
-    rows = k_pool.shape[0]
-    if rows % page_size:
-        raise ValueError("pool rows must be a whole number of pages")
-    sh = _shape(q_new, k_new, softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    bt = np.ascontiguousarray(block_table_host, dtype=np.int32)
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device)
-    if workspace is None:
-        workspace = _workspace(append_workspace_size(q_new, k_new, softmax_scale), q_new.device)
-    _check(lib.ism_attn_prefill_append_paged(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                             C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data), se.shape[0],
-                                             _ptr(k_pool), _ptr(v_pool), rows // page_size, page_size,
-                                             _ptr(block_table), C.c_void_p(bt.ctypes.data), block_table.shape[1],
-                                             _ptr(cache_len), C.c_void_p(ch.ctypes.data), _ptr(out), _ptr(lse),
-                                             _ptr(workspace), workspace.numel(), _stream(q_new.device)),
-           "ism_attn_prefill_append_paged")
-    return out, lse
+    return _paged("ism_attn_prefill_append_paged", 0, q_new, k_new, v_new, k_pool, v_pool, page_size, block_table,
+                  block_table_host, cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse,
+                  workspace)
 
 
 def prefill_append_paged_rope(q_new, k_new, v_new, k_pool, v_pool, page_size: int, block_table, block_table_host,
@@ -625,31 +615,9 @@ def prefill_append_paged_rope(q_new, k_new, v_new, k_pool, v_pool, page_size: in
                               softmax_scale: float, out=None, lse=None, workspace=None):
     """``prefill_append_paged`` with rotary encoding of the new queries and
     keys at positions cache_len[b] + j (as ``prefill_append_rope``)."""
-    lib = load()
-    _contig(q_new, k_new, v_new, k_pool, v_pool, cache_len, block_table)
-    B, Ln, hq, D = q_new.shape
-    rows = k_pool.shape[0]
-    if rows % page_size:
-        raise ValueError("pool rows must be a whole number of pages")
-    sh = _shape(q_new, k_new, softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    bt = np.ascontiguousarray(block_table_host, dtype=np.int32)
-    rope = _rope_struct(rope_cos, rope_sin)
-    out = torch.empty_like(q_new) if out is None else out
-    lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device) if lse is None else lse
-    if workspace is None:
-        workspace = _workspace(append_workspace_size(q_new, k_new, softmax_scale, rope=True), q_new.device)
-    _check(lib.ism_attn_prefill_append_paged_rope(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                                  C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data),
-                                                  se.shape[0], _ptr(k_pool), _ptr(v_pool), rows // page_size,
-                                                  page_size, _ptr(block_table), C.c_void_p(bt.ctypes.data),
-                                                  block_table.shape[1], _ptr(cache_len), C.c_void_p(ch.ctypes.data),
-                                                  C.byref(rope), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                  workspace.numel(), _stream(q_new.device)),
-           "ism_attn_prefill_append_paged_rope")
-    return out, lse
+    return _paged("ism_attn_prefill_append_paged_rope", _FORM_ROPE, q_new, k_new, v_new, k_pool, v_pool, page_size,
+                  block_table, block_table_host, cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale,
+                  out, lse, workspace, _rope_fields(rope_cos, rope_sin))
 
 
 def prefill_append_e4m3_rope(q_new, k_new, v_new, k_cache, v_cache, cache_len, cache_len_host, new_seg_end,
@@ -659,31 +627,11 @@ def prefill_append_e4m3_rope(q_new, k_new, v_new, k_cache, v_cache, cache_len, c
     unrotated; queries and keys are rotated at positions cache_len[b] + j,
     then quantised with the factors (keys and values into the caches).
     Returns (o bf16, lse [Hq,B,Ln])."""
-    lib = load()
     _contig(q_new, k_new, v_new, k_cache, v_cache, cache_len)
-    B, Ln, hq, D = q_new.shape
-    sh = _Shape()
-    sh.num_heads_q, sh.num_heads_kv, sh.head_dim = hq, k_new.shape[2], D
-    sh.dtype, sh.softmax_scale = ISM_E4M3, float(softmax_scale)
-    se = np.ascontiguousarray(new_seg_end, dtype=np.int32)
-    st = np.ascontiguousarray(new_seg_type, dtype=np.uint8)
-    ch = np.ascontiguousarray(cache_len_host, dtype=np.int32)
-    rope = _rope_struct(rope_cos, rope_sin)
-    out = torch.empty(q_new.shape, dtype=torch.bfloat16, device=q_new.device) if out is None else out
-    lse = torch.empty((hq, B, Ln), dtype=torch.float32, device=q_new.device) if lse is None else lse
-    if workspace is None:
-        nbytes = C.c_size_t()
-        _check(lib.ism_attn_prefill_append_rope_workspace_size(C.byref(sh), B, Ln, C.byref(nbytes)),
-               "ism_attn_prefill_append_rope_workspace_size")
-        workspace = _workspace(nbytes.value, q_new.device)
-    _check(lib.ism_attn_prefill_append_e4m3_rope(C.byref(sh), B, _ptr(q_new), _ptr(k_new), _ptr(v_new), Ln,
-                                                 C.c_void_p(se.ctypes.data), C.c_void_p(st.ctypes.data), se.shape[0],
-                                                 _ptr(k_cache), _ptr(v_cache), k_cache.shape[1], _ptr(cache_len),
-                                                 C.c_void_p(ch.ctypes.data), q_descale, k_descale, v_descale,
-                                                 C.byref(rope), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                 workspace.numel(), _stream(q_new.device)),
-           "ism_attn_prefill_append_e4m3_rope")
-    return out, lse
+    return _append("ism_attn_prefill_append_e4m3_rope", _FORM_E4M3 | _FORM_ROPE, ISM_E4M3, q_new, k_new, v_new, k_cache,
+                   v_cache, cache_len, cache_len_host, new_seg_end, new_seg_type, softmax_scale, out, lse, workspace,
+                   _rope_fields(rope_cos, rope_sin), keep_small=True, descales=(q_descale, k_descale, v_descale),
+                   capacity=k_cache.shape[1])
 
 
 def debug_mma_tile_e4m3(a: torch.Tensor, b: torch.Tensor, mode: int) -> torch.Tensor:

@@ -979,6 +979,40 @@ struct CacheGeom {
   KvPages pages;     // table == nullptr: contiguous
 };
 
+// The bf16 tensor-core decode's work split (DecodeArgs): tiles per CTA so that one
+// CTA per SM covers the row, and room for the partials of any (sequence, KV
+// head): the CTAs that its tiles touch, times the items of a CTA's share.
+// Where that exceeds kMaxSplits (a few very long caches), every cache starts at
+// a CTA's share of kDecTcTiles tiles instead.  false: more tiles than 32 bits hold.
+bool decode_row(DecodeArgs& a, const int32_t* cache_len_host, int32_t batch, int32_t hkv, int sms) {
+  int64_t sum = 0;
+  int32_t most = 0, least = INT32_MAX;
+  for (int b = 0; b < batch; ++b) {
+    const int32_t n = dec_tiles(cache_len_host[b]);
+    sum += n;
+    if (n > most) most = n;
+    if (n < least) least = n;
+  }
+  a.align = 1;
+  int64_t row = sum * hkv, tpc = (row + sms - 1) / sms;
+  const int64_t per_cta = (tpc + kDecTcTiles - 1) / kDecTcTiles;
+  int64_t slots = ((most + tpc - 1) / tpc + 1) * per_cta;
+  if (slots > kMaxSplits) {
+    tpc = a.align = kDecTcTiles;
+    row = 0;
+    for (int b = 0; b < batch; ++b) row += dec_alloc_tiles(a, dec_tiles(cache_len_host[b]));
+    row *= hkv;
+    slots = (most + tpc - 1) / tpc;
+  }
+  if (row >= (int64_t(1) << 31) - kDecTcTiles || slots > kMaxSplits) return false;
+  a.uniform = most == least ? most : 0;
+  a.tpc = (int32_t)tpc;
+  a.row_tiles = (int32_t)row;
+  a.splits = (int32_t)slots;
+  a.chunk = 0;
+  return true;
+}
+
 ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const void* q_new, const void* k_new,
                          const void* v_new, int32_t l_new, const int32_t* new_seg_end_host,
                          const uint8_t* new_seg_type_host, int32_t n_new_segs, void* k_cache, void* v_cache,
@@ -1069,24 +1103,18 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
     a.qk_descale = qk_descale; a.v_descale = v_descale;
     a.kv_rows = cg.kv_rows;
     a.scale = shape->softmax_scale;
-    // chunks of a multiple of 64 keys, as many as fill whole waves of resident
-    // CTAs: 4 per SM for the register kernel (one wave), 2 per SM for the TMA
-    // kernel (four waves, so each CTA's ring runs several tiles)
     int64_t kv_max = (int64_t)max_c + 1;
     int64_t pairs = (int64_t)batch * hkv;
     const int sms = sm_count();
     a.tma = (d == 128 && tc_available() && !knobs().decode_no_tma) ? 1 : 0;
-    a.tc = (a.tma && !knobs().decode_no_tc &&
-            kv_max <= (int64_t)kMaxSplits * kDecTcMaxKeys)
-               ? 1
-               : 0;
-    int64_t splits, chunk;
-    if (a.tc) {
-      // persistent tensor-core kernel: the split count that minimises the
-      // busiest CTA's work, (items per CTA) x (128-key tiles per item + 1 for
-      // the item's hand-offs), over chunks of whole tiles up to kDecTcMaxKeys
+    const bool e4m3 = shape->dtype == ISM_E4M3;
+    a.tc = a.tma && !knobs().decode_no_tc && kv_max <= (int64_t)kMaxSplits * kDecTcMaxKeys &&
+           (e4m3 || decode_row(a, cache_len_host, batch, hkv, sms));
+    if (a.tc && e4m3) {
+      // persistent tensor-core kernel on equal chunks: the split count that
+      // minimises the busiest CTA's work, (items per CTA) x (128-key tiles per
+      // item + 1 for the item's hand-offs), over whole tiles up to kDecTcMaxKeys
       int64_t best = -1;
-      splits = chunk = 0;
       for (int64_t sp = 1; sp <= kMaxSplits; ++sp) {
         const int64_t ch = ((kv_max + sp - 1) / sp + 127) / 128 * 128;
         if (ch > kDecTcMaxKeys) continue;
@@ -1095,19 +1123,23 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
         const int64_t cost = per_cta * (ch / 128 + 1);
         if (best < 0 || cost < best) {
           best = cost;
-          splits = used;
-          chunk = ch;
+          a.splits = (int32_t)used;
+          a.chunk = (int32_t)ch;
         }
       }
+    } else if (a.tc) {
+      a.start = L.kv_end;  // (a single-token step has no plan there)
     } else {
+      // chunks of a multiple of 64 keys, as many as fill whole waves of resident
+      // CTAs: 4 per SM for the register kernel (one wave), 2 per SM for the TMA
+      // kernel (four waves, so each CTA's ring runs several tiles)
       int64_t want = (a.tma ? 8 * (int64_t)sms : 4 * (int64_t)sms) / pairs;
-      splits = want < 1 ? 1 : want > kMaxSplits ? kMaxSplits : want;
-      chunk = (kv_max + splits - 1) / splits;
+      int64_t splits = want < 1 ? 1 : want > kMaxSplits ? kMaxSplits : want;
+      int64_t chunk = (kv_max + splits - 1) / splits;
       chunk = (chunk + 63) / 64 * 64;
-      splits = (kv_max + chunk - 1) / chunk;
+      a.splits = (int32_t)((kv_max + chunk - 1) / chunk);
+      a.chunk = (int32_t)chunk;
     }
-    a.splits = (int32_t)splits;
-    a.chunk = (int32_t)chunk;
     a.part_o = L.part_o; a.part_ml = L.part_ml;
     a.status = status;
     timer_begin(ISM_KERNEL_DECODE, st);

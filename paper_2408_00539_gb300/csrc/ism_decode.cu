@@ -417,37 +417,58 @@ __global__ void __launch_bounds__(160) decode_tma_kernel(const __grid_constant__
 
 // grid B*Hq, block D threads.  Launched as a programmatic dependent of the
 // split kernel: it may start while that kernel runs and waits for it (and
-// its memory) before reading the partials.
-template <int D>
+// its memory) before reading the partials.  kRow: the partials of the
+// tensor-core kernel, whose CTAs share out one row of tiles (DecodeArgs); else
+// one for each of a.splits chunks, those without keys marked by a maximum of -inf.
+template <int D, bool kRow>
 __global__ void decode_combine_kernel(DecodeArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int bh = blockIdx.x;
   const int d = threadIdx.x;
+  const int b = bh / a.hq, h = bh % a.hq;
+  int n_slots = a.splits;
+  int s = 0, end = 0, per_cta = 1, c0 = 0;
+  if constexpr (kRow) {
+    const int n = dec_tiles(a.c_snap[b]), alloc = dec_alloc_tiles(a, n);
+    s = (a.uniform ? b * a.hkv * alloc : a.start[b]) + h / a.group * alloc;
+    end = s + n;
+    per_cta = (a.tpc + kDecTcTiles - 1) / kDecTcTiles;
+    c0 = s / a.tpc;
+    n_slots = min(((end - 1) / a.tpc - c0 + 1) * per_cta, a.splits);
+  }
+  // whether CTA c0 + slot / per_cta has a (slot % per_cta)-th item here
+  auto used = [&](int slot) -> bool {
+    if (slot >= n_slots) return false;
+    if (!kRow || per_cta == 1) return true;
+    const int c = c0 + slot / per_cta;
+    return max(s, c * a.tpc) + slot % per_cta * kDecTcTiles < min(end, (c + 1) * a.tpc);
+  };
   const float* pml = a.part_ml + (int64_t)bh * a.splits * 2;
-  // splits in chunks of eight with every load of a chunk issued before any
-  // use (a split count below eight is one chunk); a split without keys (max
-  // -inf) has weight 0 and its partial O, never written, is replaced by 0
+  // slots in chunks of eight with every load of a chunk issued before any use
+  // (up to eight slots are one chunk)
   const float* po = a.part_o + (int64_t)bh * a.splits * D + d;
   float M = -INFINITY;
-  for (int s0 = 0; s0 < a.splits; s0 += 8) {
+  for (int s0 = 0; s0 < n_slots; s0 += 8) {
     float ms[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) ms[u] = s0 + u < a.splits ? pml[2 * (s0 + u)] : -INFINITY;
+    for (int u = 0; u < 8; ++u) ms[u] = used(s0 + u) ? pml[2 * (s0 + u)] : -INFINITY;
 #pragma unroll
     for (int u = 0; u < 8; ++u) M = fmaxf(M, ms[u]);
   }
   float acc = 0.f, L = 0.f;
-  for (int s0 = 0; s0 < a.splits; s0 += 8) {
+  for (int s0 = 0; s0 < n_slots; s0 += 8) {
     float ms[8], ls[8], v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const bool in = s0 + u < a.splits;
+      const bool in = used(s0 + u);
       ms[u] = in ? pml[2 * (s0 + u)] : -INFINITY;
       ls[u] = in ? pml[2 * (s0 + u) + 1] : 0.f;
       v[u] = in ? po[(int64_t)(s0 + u) * D] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
+      // weight 0 without keys (max -inf; O was never written)
       const bool live = ms[u] != -INFINITY;
       const float f = live ? exp2f(ms[u] - M) : 0.f;
       acc = fmaf(live ? v[u] : 0.f, f, acc);
@@ -455,14 +476,13 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
     }
   }
   ((__nv_bfloat16*)a.out)[(int64_t)bh * D + d] = __float2bfloat16_rn(acc / L);
-  const int b = bh / a.hq, h = bh % a.hq;
   if (a.lse && d == 0) a.lse[(int64_t)h * a.batch + b] = (M + log2f(L)) * 0.6931471805599453f;
   // the attention of this step has read the cache lengths: advance them
   if (a.cache_len && h == 0 && d == 0) a.cache_len[b] = a.c_snap[b] + 1;
 }
 
 // The combine as a programmatic dependent launch of the kernel before it.
-template <int D>
+template <int D, bool kRow = false>
 cudaError_t launch_combine(const DecodeArgs& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.batch * a.hq));
@@ -473,7 +493,7 @@ cudaError_t launch_combine(const DecodeArgs& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_combine_kernel<D>, a);
+  return cudaLaunchKernelEx(&cfg, decode_combine_kernel<D, kRow>, a);
 }
 
 template <int D, int G>
@@ -534,7 +554,7 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st) {
   if (a.tc) {
     cudaError_t e = tc::launch_decode_tc(a, st);
     if (e != cudaSuccess) return e;
-    return launch_combine<128>(a, st);
+    return a.dtype == ISM_E4M3 ? launch_combine<128>(a, st) : launch_combine<128, true>(a, st);
   }
   return a.d == 64 ? run_d<64>(a, st) : run_d<128>(a, st);
 }

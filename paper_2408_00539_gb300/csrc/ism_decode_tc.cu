@@ -6,8 +6,15 @@
 // slots on dot products and the reductions that assemble them; here both
 // contractions run on the tensor cores and the threads only do the softmax.
 //
-// Work item: (sequence b, KV head g, split) = keys [k0, k1) of the cache, in
-// tiles of 128 keys.  A persistent CTA per SM walks the items; per item
+// Work split: the 128-key tiles of all (sequence b, KV head g) caches stand in
+// one row, b outermost, and CTA c takes tiles [c * tpc, (c + 1) * tpc) of it,
+// tpc = tiles / SMs rounded up, so every CTA reads the same number of bytes
+// whatever the cache lengths are.  A work item is what a CTA's share has of one
+// (b, g), at most kMaxTiles tiles: keys [k0, k1).  Equal chunks of the longest
+// cache, dealt out in turn, took 64.4 us on 40 ragged caches (250 to 4000
+// keys, 341 MB) and this split takes 59.  (e4m3 keeps equal chunks, splits of
+// the longest cache: P is rounded to three mantissa bits relative to its
+// item's maximum, so other items would move its results by 3.5 %.)  Per item
 //   pass 1: S^T_t = K_t Q^T for every tile t (M = 128 keys, N = 16 query
 //           heads of the group, zero or foreign rows past the group), all
 //           tiles kept in tensor memory (16 columns each); the softmax
@@ -88,28 +95,141 @@ __device__ __forceinline__ bool aborted(const int32_t* f) { return *reinterpret_
 __device__ __forceinline__ void set_abort(int32_t* f) { *reinterpret_cast<volatile int32_t*>(f) = 1; }
 
 struct DecItem {
-  int b, g, split, k0, k1;
+  int b, g, k0, k1;
+  int slot;  // of the partial result among those of (b, g)
   int nt;    // ring tiles (kSub sub-tiles of 128 keys each, the last possibly short)
   int nsub;  // 128-key sub-tiles
+  bool first;  // the first tile of sequence b's first KV head: `s0` is its place in the row
+  int s0;
 };
-// item = (split * batch + b) * hkv + g: consecutive CTAs take the KV heads of
-// one (sequence, split), whose rows lie side by side in the cache
-// ([B, cap, Hkv, D]): CTAs that start together read neighbouring pieces of
-// the same cache rows, which keeps DRAM pages open across their requests
-// (an e4m3 head row is only 128 bytes of a 1 KB cache row)
-template <int kSub>
-__device__ __forceinline__ DecItem dec_item(const DecodeArgs& a, int64_t item) {
-  DecItem x;
-  x.g = (int)(item % a.hkv);
-  const int64_t rest = item / a.hkv;
-  x.b = (int)(rest % a.batch);
-  x.split = (int)(rest / a.batch);
-  const int kv_len = a.c_snap[x.b] + 1;
-  x.k0 = x.split * a.chunk;
-  x.k1 = min(kv_len, x.k0 + a.chunk);
-  x.nsub = x.k1 > x.k0 ? (x.k1 - x.k0 + 127) / 128 : 0;
-  x.nt = (x.nsub + kSub - 1) / kSub;
-  return x;
+
+// The items of this CTA, one after the other; every role walks them alike.
+struct DecWalk {
+  int t, end;    // tiles of the row left to this CTA
+  int b, g, s;   // current (b, g) and its first tile in the row
+  int len;       // keys of sequence b, the new one included
+  int64_t item;  // (equal chunks) the next item
+};
+// The whole warp: finds the (b, g) of the CTA's first tile.
+template <bool kRow>
+__device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
+  DecWalk w;
+  if constexpr (!kRow) {
+    w.item = blockIdx.x;
+    return w;
+  }
+  w.t = (int)blockIdx.x * a.tpc;
+  w.end = min(w.t + a.tpc, a.row_tiles);
+  w.b = 0;
+  int sb = 0;  // first tile of sequence w.b
+  if (a.uniform) {
+    const int per = dec_alloc_tiles(a, a.uniform) * a.hkv;
+    w.b = w.t / per;
+    sb = w.b * per;
+  } else {
+    const int lane = threadIdx.x & 31;
+    for (int base = 0; base < a.batch; base += 128) {
+      // four sequences a lane, in order
+      int n[4], sum = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int b = base + lane * 4 + i;
+        n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.c_snap[b])) * a.hkv : 0;
+        sum += n[i];
+      }
+      int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      if (w.t >= sb + total && base + 128 < a.batch) {
+        sb += total;
+        continue;
+      }
+      int at = sb + incl - sum, found = -1, start = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (w.t >= at && w.t < at + n[i]) {
+          found = base + lane * 4 + i;
+          start = at;
+        }
+        at += n[i];
+      }
+      const uint32_t who = __ballot_sync(0xffffffffu, found >= 0);
+      if (!who) {
+        w.end = w.t;  // past the last tile: nothing to do
+        break;
+      }
+      const int src = __ffs(who) - 1;
+      w.b = __shfl_sync(0xffffffffu, found, src);
+      sb = __shfl_sync(0xffffffffu, start, src);
+      break;
+    }
+  }
+  if (w.b >= a.batch) {
+    w.b = 0;
+    w.end = w.t;
+  }
+  w.len = a.c_snap[w.b] + 1;
+  const int per_head = dec_alloc_tiles(a, (w.len + 127) / 128);
+  w.g = w.t < w.end ? (w.t - sb) / per_head : 0;
+  w.s = sb + w.g * per_head;
+  return w;
+}
+template <bool kRow, int kSub>
+__device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecItem& x) {
+  if constexpr (!kRow) {
+    // item = (split * batch + b) * hkv + g: consecutive CTAs take the KV heads of
+    // one (sequence, split), whose rows lie side by side in the cache
+    // ([B, cap, Hkv, D]): CTAs that start together read neighbouring pieces of
+    // the same cache rows, which keeps DRAM pages open across their requests
+    // (an e4m3 head row is only 128 bytes of a 1 KB cache row)
+    if (w.item >= (int64_t)a.batch * a.hkv * a.splits) return false;
+    x.g = (int)(w.item % a.hkv);
+    const int64_t rest = w.item / a.hkv;
+    x.b = (int)(rest % a.batch);
+    x.slot = (int)(rest / a.batch);
+    x.k0 = x.slot * a.chunk;
+    x.k1 = min(a.c_snap[x.b] + 1, x.k0 + a.chunk);
+    x.nsub = x.k1 > x.k0 ? (x.k1 - x.k0 + 127) / 128 : 0;
+    x.nt = (x.nsub + kSub - 1) / kSub;
+    x.first = false;
+    w.item += gridDim.x;
+    return true;
+  } else {
+    while (w.t < w.end) {
+      const int n = (w.len + 127) / 128, alloc = dec_alloc_tiles(a, n), local = w.t - w.s;
+      if (local >= alloc) {  // the next (b, g)
+        w.s += alloc;
+        if (++w.g == a.hkv) {
+          w.g = 0;
+          if (++w.b >= a.batch) return false;
+          w.len = a.c_snap[w.b] + 1;
+        }
+        continue;
+      }
+      if (local >= n) {  // padding of the row
+        w.t = w.s + alloc;
+        continue;
+      }
+      const int cnt = min(min(n - local, w.end - w.t), kMaxTiles);
+      const int begin = (int)blockIdx.x * a.tpc;
+      x.b = w.b;
+      x.g = w.g;
+      x.k0 = local * 128;
+      x.k1 = min(w.len, x.k0 + cnt * 128);
+      x.nsub = cnt;
+      x.nt = (cnt + kSub - 1) / kSub;
+      x.slot = min(dec_slot(a, w.s, (int)blockIdx.x, (w.t - max(w.s, begin)) / kMaxTiles), a.splits - 1);
+      x.first = w.g == 0 && local == 0;
+      x.s0 = w.s;
+      w.t += cnt;
+      return true;
+    }
+    return false;
+  }
 }
 
 // The P operand is stored MN-major (128-byte swizzled rows = keys, the heads
@@ -135,9 +255,10 @@ __device__ __forceinline__ void ld_scores(uint32_t taddr, uint32_t (&v)[G]) {
 template <bool kE4M3, int kG>
 __global__ void __launch_bounds__(kThreads, 1)
     decode_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                     const __grid_constant__ CUtensorMap tmV, const DecodeArgs a, int64_t n_items) {
+                     const __grid_constant__ CUtensorMap tmV, const DecodeArgs a) {
   using Cfg = DecCfg<kE4M3>;
   constexpr int kStages = Cfg::kStages, kSub = Cfg::kSub;
+  constexpr bool kRow = !kE4M3;
   constexpr uint32_t kTile = Cfg::kTile, kSubBytes = Cfg::kSubBytes, kQHalf = Cfg::kQHalf, kQBytes = Cfg::kQBytes;
   constexpr uint32_t OFF_RING = Cfg::OFF_RING, OFF_P = Cfg::OFF_P, OFF_Q = Cfg::OFF_Q, OFF_BAR = Cfg::OFF_BAR;
   extern __shared__ uint8_t smem_raw[];
@@ -194,9 +315,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::tma_prefetch_desc(&tmK);
       ptx::tma_prefetch_desc(&tmV);
     }
-    for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-      const DecItem x = dec_item<Cfg::kSub>(a, item);
-      if (x.nt == 0) continue;
+    DecWalk walk = dec_walk<kRow>(a);
+    DecItem x;
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+      if (!kRow && x.nt == 0) continue;
       const uint32_t qb = nu & 1;
       if (__any_sync(0xffffffffu, aborted(&bar->abort)) ||
           (nu >= 2 && !wait_warp(&bar->q_empty[qb], ((nu >> 1) - 1) & 1, a.status))) {
@@ -259,9 +381,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t idesc_pv = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 1, 1) : ptx::idesc_bf16_f32(128, 128, 1, 1);
     uint32_t nl = 0, nu = 0, T = 0, TS = 0;  // ring tiles consumed; non-empty items; P tiles; S tiles
     bool ok = true;
-    for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-      const DecItem x = dec_item<Cfg::kSub>(a, item);
-      if (x.nt == 0) continue;
+    DecWalk walk = dec_walk<kRow>(a);
+    DecItem x;
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+      if (!kRow && x.nt == 0) continue;
       const uint32_t qb = nu & 1;
       // Q landed; the softmax warps have read the previous item's S
       if (!wait_warp(&bar->q_full[qb], (nu >> 1) & 1, a.status) ||
@@ -347,10 +470,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int group = a.group;
     uint32_t nu = 0, T = 0, TS = 0;
     bool ok = true;
-    for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-      const DecItem x = dec_item<Cfg::kSub>(a, item);
-      const int64_t pbase = ((int64_t)x.b * a.hq + (int64_t)x.g * group) * a.splits + x.split;
-      if (x.nt == 0) {
+    DecWalk walk = dec_walk<kRow>(a);
+    DecItem x;
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+      const int64_t pbase = ((int64_t)x.b * a.hq + (int64_t)x.g * group) * a.splits + x.slot;
+      if (!kRow && x.nt == 0) {
         // a split past the sequence's keys: a partial the combine skips
         if (warp == 0 && lane < group) {
           a.part_ml[(pbase + (int64_t)lane * a.splits) * 2] = -INFINITY;
@@ -358,6 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         continue;
       }
+      if (kRow && x.first && r == 0) a.start[x.b] = x.s0;  // where the combine finds the sequence's parts
       // pass 1: maximum of the scaled scores per head over the item's keys,
       // ring tile by ring tile as the score MMAs complete
       static_assert(kG == 4 || kG == 8 || kG == kHeadsPad, "heads per softmax pass");
@@ -545,9 +670,13 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
   if ((e = cudaFuncSetAttribute(decode_tc_kernel<kE4M3, kG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Cfg::kSmemBytes)) != cudaSuccess)
     return e;
-  const int64_t sms = sm_count();
-  const int64_t n_items = (int64_t)a.batch * a.hkv * a.splits;
-  int64_t grid = sms < n_items ? sms : n_items;
+  int64_t grid;
+  if constexpr (kE4M3) {
+    const int64_t sms = sm_count(), n_items = (int64_t)a.batch * a.hkv * a.splits;
+    grid = sms < n_items ? sms : n_items;
+  } else {
+    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc;
+  }
   if (grid <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -559,14 +688,15 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_tc_kernel<kE4M3, kG>, tq, tk, tv, a, n_items);
+  return cudaLaunchKernelEx(&cfg, decode_tc_kernel<kE4M3, kG>, tq, tk, tv, a);
 }
 
 }  // namespace
 
 cudaError_t launch_decode_tc(const DecodeArgs& a, cudaStream_t st) {
-  if (a.d != kD || (a.dtype != ISM_BF16 && a.dtype != ISM_E4M3) || a.group > kHeadsPad || a.chunk % 128 != 0 ||
-      a.chunk > kDecTcMaxKeys)
+  if (a.d != kD || (a.dtype != ISM_BF16 && a.dtype != ISM_E4M3) || a.group > kHeadsPad)
+    return cudaErrorInvalidValue;
+  if (a.dtype == ISM_E4M3 ? a.chunk % 128 != 0 || a.chunk > kDecTcMaxKeys : a.tpc < 1 || !a.start)
     return cudaErrorInvalidValue;
   // the softmax warps process the group's heads rounded up to 4, 8 or 16
   if (a.dtype == ISM_E4M3)

@@ -217,13 +217,30 @@ struct DecodeArgs {
   float* part_o;         // [B, Hq, splits, D]
   float* part_ml;        // [B, Hq, splits, 2]
   int32_t tma;           // stream the cache with TMA (head_dim 128, sm_103)
-  int32_t tc;            // tensor-core kernel (bf16 or e4m3, head_dim 128, group <= 16; chunk a multiple of 128)
+  int32_t tc;            // tensor-core kernel (bf16 or e4m3, head_dim 128, group <= 16)
+  // e4m3: equal chunks of a multiple of 128 keys (splits, chunk).  bf16: the 128-key tiles of all (sequence, KV head) caches in one
+  // row of row_tiles, tpc of them per CTA, an item at most kDecTcTiles; splits =
+  // room for partials per (sequence, KV head).  uniform: tiles of every cache
+  // when all are equal, else 0.  align: each cache's tiles are padded to a
+  // multiple of it in the row (1: not).  start [B]: written with the first tile
+  // of each sequence in the row.
+  int32_t tpc, row_tiles, uniform, align;
+  int32_t* start;
   uint32_t* status;      // device status word (bounded waits)
   int32_t* cache_len;    // nullable: the combine kernel advances it by one (single-token steps)
 };
 // Keys one work item of the tensor-core decode covers at most (its scores of
 // 24 tiles of 128 keys stay in tensor memory).
-constexpr int kDecTcMaxKeys = 24 * 128;
+constexpr int kDecTcTiles = 24;
+constexpr int kDecTcMaxKeys = kDecTcTiles * 128;
+__host__ __device__ __forceinline__ int32_t dec_tiles(int32_t cached) { return (cached + 1 + 127) / 128; }
+__host__ __device__ __forceinline__ int32_t dec_alloc_tiles(const DecodeArgs& a, int32_t tiles) {
+  return a.align == 1 ? tiles : (tiles + a.align - 1) / a.align * a.align;
+}
+// Slot of the j-th item that CTA c has of the (sequence, KV head) whose tiles start at s.
+__host__ __device__ __forceinline__ int32_t dec_slot(const DecodeArgs& a, int32_t s, int32_t c, int32_t j) {
+  return (c - s / a.tpc) * ((a.tpc + kDecTcTiles - 1) / kDecTcTiles) + j;
+}
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st);
 
 // Tensor-core kernels (ism_fwd_tc.cu / ism_bwd_tc.cu), bf16 only.

@@ -1096,6 +1096,7 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
   if (decode) {
     DecodeArgs a{};
     a.cache_len = cache_len;
+    a.q_written = rope != nullptr;
     a.q = q_new; a.k_cache = k_cache; a.v_cache = v_cache; a.pages = cg.pages; a.out = o_new; a.lse = lse_new;
     a.c_snap = L.c_snap;
     a.batch = batch; a.hq = hq; a.hkv = hkv; a.d = d; a.dtype = shape->dtype; a.cap = cg.cap;

@@ -478,7 +478,7 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
   ((__nv_bfloat16*)a.out)[(int64_t)bh * D + d] = __float2bfloat16_rn(acc / L);
   if (a.lse && d == 0) a.lse[(int64_t)h * a.batch + b] = (M + log2f(L)) * 0.6931471805599453f;
   // the attention of this step has read the cache lengths: advance them
-  if (a.cache_len && h == 0 && d == 0) a.cache_len[b] = a.c_snap[b] + 1;
+  if (h == 0 && d == 0) a.cache_len[b] = a.c_snap[b] + 1;
 }
 
 // The combine as a programmatic dependent launch of the kernel before it.

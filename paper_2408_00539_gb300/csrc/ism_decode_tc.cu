@@ -134,7 +134,7 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int b = base + lane * 4 + i;
-        n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.c_snap[b])) * a.hkv : 0;
+        n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * a.hkv : 0;
         sum += n[i];
       }
       int incl = sum;
@@ -172,7 +172,7 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
     w.b = 0;
     w.end = w.t;
   }
-  w.len = a.c_snap[w.b] + 1;
+  w.len = a.cache_len[w.b] + 1;
   const int per_head = dec_alloc_tiles(a, (w.len + 127) / 128);
   w.g = w.t < w.end ? (w.t - sb) / per_head : 0;
   w.s = sb + w.g * per_head;
@@ -192,7 +192,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
     x.b = (int)(rest % a.batch);
     x.slot = (int)(rest / a.batch);
     x.k0 = x.slot * a.chunk;
-    x.k1 = min(a.c_snap[x.b] + 1, x.k0 + a.chunk);
+    x.k1 = min(a.cache_len[x.b] + 1, x.k0 + a.chunk);
     x.nsub = x.k1 > x.k0 ? (x.k1 - x.k0 + 127) / 128 : 0;
     x.nt = (x.nsub + kSub - 1) / kSub;
     x.first = false;
@@ -206,7 +206,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
         if (++w.g == a.hkv) {
           w.g = 0;
           if (++w.b >= a.batch) return false;
-          w.len = a.c_snap[w.b] + 1;
+          w.len = a.cache_len[w.b] + 1;
         }
         continue;
       }
@@ -298,16 +298,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
-  // launched as a programmatic dependent of the cache write: the set-up above
-  // overlaps it; the cache lengths and the new rows are read only after it
-  // has completed.  The combine kernel after this one may start early and
-  // waits for this grid in turn.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Launched as a programmatic dependent of the cache write, which lets this
+  // grid start once its own predecessors are complete: everything but what the
+  // write itself brings may be read at once.  The cache lengths stay until the
+  // combine advances them; only the copies of a cache's last tile (the new
+  // row, and the values zeroed after it) and of rotated queries wait for the
+  // write (every cache has a last tile, so this grid does not end before it).
+  // The combine after this grid may start early and waits for it in turn.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == kLoadWarp) {
     // ------------------------------------------------ TMA loads (the warp waits converged, lane 0 issues)
     uint32_t nl = 0, nu = 0;  // ring tiles issued; non-empty items
+    bool written = false;     // the cache write has been waited for
     uint32_t nf[kStages] = {}, nq[2] = {0, 0};
     bool ok = true;
     const uint64_t pol = ptx::l2_policy_evict_first();  // the cache is streamed once per step
@@ -325,22 +328,34 @@ __global__ void __launch_bounds__(kThreads, 1)
         ok = false;
         break;
       }
-      if (lane == 0) {
-        // the 16 query rows from the group's first head (rows past the group
-        // are other heads' queries or zero fill; their outputs are not used)
-        const int32_t qy = x.b * a.hq + x.g * a.group;
-        uint8_t* dq = smem + OFF_Q + qb * kQBytes;
-        ptx::mbar_expect_tx(&bar->q_full[qb], kQBytes);
-        ptx::tma_load_2d(dq, &tmQ, &bar->q_full[qb], 0, qy);
-        if (!kE4M3) ptx::tma_load_2d(dq + kQHalf, &tmQ, &bar->q_full[qb], 64, qy);
-      }
-      __syncwarp();
-      ++nq[qb];
+      const bool last_item = x.k1 == a.cache_len[x.b] + 1;  // it has the cache's last tile
+      auto load_q = [&] {
+        if (lane == 0) {
+          // the 16 query rows from the group's first head (rows past the group
+          // are other heads' queries or zero fill; their outputs are not used)
+          const int32_t qy = x.b * a.hq + x.g * a.group;
+          uint8_t* dq = smem + OFF_Q + qb * kQBytes;
+          ptx::mbar_expect_tx(&bar->q_full[qb], kQBytes);
+          ptx::tma_load_2d(dq, &tmQ, &bar->q_full[qb], 0, qy);
+          if (!kE4M3) ptx::tma_load_2d(dq + kQHalf, &tmQ, &bar->q_full[qb], 64, qy);
+        }
+        __syncwarp();
+        ++nq[qb];
+      };
+      // rotated queries of the first item: after as many K tiles as the ring
+      // takes (a full ring needs Q to drain)
+      const int q_after = a.q_written && !written ? min(x.nt - 1, kStages) : 0;
       ++nu;
       for (int pass = 0; ok && pass < 2; ++pass) {
         const CUtensorMap* map = pass ? &tmV : &tmK;
         for (int t = 0; t < x.nt; ++t, ++nl) {
           const uint32_t s = nl % kStages;
+          const bool needs_q = pass == 0 && t == q_after;
+          if (!written && ((last_item && t == x.nt - 1) || (needs_q && a.q_written))) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            written = true;
+          }
+          if (needs_q) load_q();
           if (__any_sync(0xffffffffu, aborted(&bar->abort)) ||
               (nl >= kStages && !wait_warp(&bar->empty[s], ((nl / kStages) - 1) & 1, a.status))) {
             ok = false;

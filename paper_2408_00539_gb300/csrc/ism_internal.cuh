@@ -225,9 +225,10 @@ struct DecodeArgs {
   // multiple of it in the row (1: not).  start [B]: written with the first tile
   // of each sequence in the row.
   int32_t tpc, row_tiles, uniform, align;
+  int32_t q_written;     // the queries come from the cache write (rotated)
   int32_t* start;
   uint32_t* status;      // device status word (bounded waits)
-  int32_t* cache_len;    // nullable: the combine kernel advances it by one (single-token steps)
+  int32_t* cache_len;    // [B] equal to c_snap until the combine kernel advances it by one
 };
 // Keys one work item of the tensor-core decode covers at most (its scores of
 // 24 tiles of 128 keys stay in tensor memory).

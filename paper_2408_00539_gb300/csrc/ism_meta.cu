@@ -308,7 +308,7 @@ __device__ __forceinline__ int32_t chunk_kv_end(const AppendSegs& sg, int32_t j)
 }
 
 // The append plan's share of one thread (grid-stride; see AppendPlan).
-__device__ __forceinline__ void append_plan_part(const AppendPlan& p, int batch, const int32_t* __restrict__ cache_len) {
+__device__ __forceinline__ void append_plan_part(const AppendPlan& p, int batch, const int32_t* cache_len) {
   if (!p.qtiles) return;
   const AppendSegs& sg = p.segs;
   const int32_t Ln = sg.l_new;
@@ -347,14 +347,14 @@ __device__ __forceinline__ void append_plan_part(const AppendPlan& p, int batch,
 // It reads the cache lengths themselves (c_snap = cache_len): they stay as
 // they are until the attention kernel after it advances them, and single-token
 // steps find a copy in snap_out.
-__device__ __forceinline__ void copy_snapshot(int batch, const int32_t* __restrict__ c_snap, int32_t* snap_out) {
+__device__ __forceinline__ void copy_snapshot(int batch, const int32_t* c_snap, int32_t* snap_out) {
   if (!snap_out) return;
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += (int64_t)gridDim.x * blockDim.x)
     snap_out[b] = c_snap[b];
 }
 
 __device__ __forceinline__ void zero_value_tail(int batch, int l_new, int vec_per_row, int64_t cap,
-                                                const KvPages& pages, const int32_t* __restrict__ c_snap,
+                                                const KvPages& pages, const int32_t* c_snap,
                                                 uint4* v_cache) {
   const int64_t total = (int64_t)batch * 128 * vec_per_row;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -372,12 +372,24 @@ __device__ __forceinline__ void zero_value_tail(int batch, int l_new, int vec_pe
   }
 }
 
-__global__ void cache_write_kernel(int batch, int l_new, int row_bytes, int64_t cap, KvPages pages,
-                                   const int32_t* __restrict__ c_snap, const uint4* __restrict__ k_new,
-                                   const uint4* __restrict__ v_new, uint4* k_cache, uint4* v_cache,
-                                   const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
-  // a kernel launched as a programmatic dependent may start its set-up now
+// Both cache-write kernels are launched as programmatic dependents, so that
+// their launch overlaps the end of whatever runs before (the combine of the
+// step before, in a generation loop), and let the attention kernel start as
+// soon as that is complete: what it reads beside the new rows is then in place.
+// A rotary decode step over 3000 keys 13.1 -> 10.6 us, 40 ragged caches 70 -> 67,
+// e4m3 8 x 16384 keys 50.7 -> 48 (with the decode reading the old keys while
+// the new row is written).  Inputs are not __restrict__: nothing may be loaded
+// before the wait.
+__device__ __forceinline__ void write_prologue() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__global__ void cache_write_kernel(int batch, int l_new, int row_bytes, int64_t cap, KvPages pages,
+                                   const int32_t* c_snap, const uint4* k_new,
+                                   const uint4* v_new, uint4* k_cache, uint4* v_cache,
+                                   const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
+  write_prologue();
   append_plan_part(plan, batch, c_snap);
   const int vec_per_row = row_bytes / 16;
   copy_snapshot(batch, c_snap, snap_out);
@@ -438,13 +450,13 @@ __device__ __forceinline__ void store8(void* base, int64_t elem, const float (&x
 
 template <bool kE4M3>
 __global__ void rope_cache_write_kernel(int batch, int l_new, int hq, int hkv, int d, int64_t cap, KvPages pages,
-                                        const int32_t* __restrict__ c_snap, const __nv_bfloat16* __restrict__ q_new,
-                                        const __nv_bfloat16* __restrict__ k_new,
-                                        const __nv_bfloat16* __restrict__ v_new, const float* __restrict__ cos_t,
+                                        const int32_t* c_snap, const __nv_bfloat16* q_new,
+                                        const __nv_bfloat16* k_new,
+                                        const __nv_bfloat16* v_new, const float* __restrict__ cos_t,
                                         const float* __restrict__ sin_t, float q_descale, float k_descale,
                                         float v_descale, void* q_rot, void* k_cache, void* v_cache,
                                         const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  write_prologue();
   append_plan_part(plan, batch, c_snap);
   copy_snapshot(batch, c_snap, snap_out);
   const int half = d / 2;
@@ -566,6 +578,25 @@ cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_o
   return cudaGetLastError();
 }
 
+namespace {
+// A cache-write kernel over `total` threads, as a programmatic dependent.
+template <class... Params, class... Args>
+cudaError_t launch_write(void (*kern)(Params...), int64_t total, cudaStream_t st, Args... args) {
+  int64_t grid = (total + 255) / 256;
+  if (grid > 152 * 16) grid = 152 * 16;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+}  // namespace
+
 cudaError_t launch_cache_write(int dtype, int batch, int l_new, int hkv, int d, int64_t cap, const KvPages& pages,
                                const int32_t* c_snap, const void* k_new, const void* v_new,
                                void* k_cache, void* v_cache, const AppendPlan& plan, cudaStream_t st,
@@ -576,11 +607,8 @@ cudaError_t launch_cache_write(int dtype, int batch, int l_new, int hkv, int d, 
   if (total == 0) return cudaSuccess;
   const int64_t tail = (int64_t)batch * 128 * (row_bytes / 16);  // value rows zeroed past the new end
   if (tail > total) total = tail;
-  int grid = (int)((total + 255) / 256);
-  if (grid > 152 * 16) grid = 152 * 16;
-  cache_write_kernel<<<grid, 256, 0, st>>>(batch, l_new, row_bytes, cap, pages, c_snap, (const uint4*)k_new,
-                                           (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, plan, snap_out);
-  return cudaGetLastError();
+  return launch_write(cache_write_kernel, total, st, batch, l_new, row_bytes, cap, pages, c_snap, (const uint4*)k_new,
+                      (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, plan, snap_out);
 }
 
 cudaError_t launch_rope_cache_write(int dtype, int batch, int l_new, int hq, int hkv, int d, int64_t cap,
@@ -593,13 +621,10 @@ cudaError_t launch_rope_cache_write(int dtype, int batch, int l_new, int hq, int
   const bool e4m3 = dtype == ISM_E4M3;
   const int64_t tail = (int64_t)batch * 128 * (hkv * d * (e4m3 ? 1 : 2) / 16);  // value rows zeroed past the new end
   if (tail > total) total = tail;
-  int grid = (int)((total + 255) / 256);
-  if (grid > 152 * 16) grid = 152 * 16;
-  auto kern = e4m3 ? rope_cache_write_kernel<true> : rope_cache_write_kernel<false>;
-  kern<<<grid, 256, 0, st>>>(batch, l_new, hq, hkv, d, cap, pages, c_snap, (const __nv_bfloat16*)q_new,
-                             (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, cos_t, sin_t, q_descale,
-                             k_descale, v_descale, q_rot, k_cache, v_cache, plan, snap_out);
-  return cudaGetLastError();
+  return launch_write(e4m3 ? rope_cache_write_kernel<true> : rope_cache_write_kernel<false>, total, st, batch, l_new, hq,
+                      hkv, d, cap, pages, c_snap, (const __nv_bfloat16*)q_new, (const __nv_bfloat16*)k_new,
+                      (const __nv_bfloat16*)v_new, cos_t, sin_t, q_descale, k_descale, v_descale, q_rot, k_cache,
+                      v_cache, plan, snap_out);
 }
 
 }  // namespace ism

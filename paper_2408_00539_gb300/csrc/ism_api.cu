@@ -208,10 +208,11 @@ struct PassLayout {
   void* ds;
   int32_t* pair_order;
   int32_t* kp_order;  // k-tile pairs in cost order (backward only)
-  int32_t* counters;  // work counters of the persistent backward kernels (backward only)
+  int32_t* counters;  // work counters: of dK/dV (backward), of the forward's query-tile pairs
   size_t bytes;
 };
 constexpr int kPassCounters = 2;
+constexpr int kBwdCounter = 0, kFwdCounter = 1;
 
 PassLayout pass_layout(void* ws, const ism_segments_t* s, const Counts& c, int64_t T, int hq, bool bwd,
                        int64_t ds_slots = 0, bool tile_pairs = false) {
@@ -227,8 +228,10 @@ PassLayout pass_layout(void* ws, const ism_segments_t* s, const Counts& c, int64
   L.ds = ds_slots > 0 ? static_cast<void*>(cv.take<uint16_t>(ds_slots * kTile * kTile)) : nullptr;
   L.pair_order = tile_pairs ? cv.take<int32_t>(c.npairs) : nullptr;
   L.kp_order = bwd ? cv.take<int32_t>(c.npairs) : nullptr;  // k-tile pairs number as q-tile pairs here
-  L.counters = bwd ? cv.take<int32_t>(kPassCounters) : nullptr;
+  if (bwd) L.counters = cv.take<int32_t>(kPassCounters);
   L.bytes = ((cv.off + 255) & ~size_t(255)) + 256;
+  // the forward's lie in the 256 bytes that every layout ends with
+  if (!bwd) L.counters = reinterpret_cast<int32_t*>(reinterpret_cast<uintptr_t>(ws) + L.bytes - 256);
   return L;
 }
 
@@ -553,7 +556,16 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     q = q_rot;
     k = k_rot;
   }
-  if (!pre && (r = build_pass_meta(segs, c, L, false, st, pairs_first(shape))) != ISM_OK) return r;
+  // query-tile pairs: an odd group
+  const bool tile_pairs = L.pair_order || (use_tc(shape) && shape->head_dim == 64 && pairs_first(shape));
+  const bool dynamic = (use_tc(shape) || e4m3) &&
+                       fwd_dynamic(tile_pairs ? c.npairs * shape->num_heads_q : c.nq * (shape->num_heads_q / 2),
+                                   tile_pairs);
+  if (!pre) {
+    if ((r = build_pass_meta(segs, c, L, false, st, pairs_first(shape))) != ISM_OK) return r;
+  } else if (dynamic) {
+    ISM_TRY_CUDA(cudaMemsetAsync(L.counters + kFwdCounter, 0, sizeof(int32_t), st), "work counter reset");
+  }
 
   AttnArgs a{};
   a.q = q; a.k = k; a.v = v; a.out = o; a.lse = lse;
@@ -562,10 +574,11 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.qk_descale = qk_descale; a.v_descale = v_descale;
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
   a.pair_order = L.pair_order; a.npairs = L.pair_order ? c.npairs : 0;
-  if (use_tc(shape) && shape->head_dim == 64 && pairs_first(shape)) {
+  if (tile_pairs && !a.pair_order) {
     a.pair_order = L.q_order;
     a.npairs = c.npairs;
   }
+  a.work_counter = dynamic ? L.counters + kFwdCounter : nullptr;
   a.status = status;
   a.flags = tc_flags();
   timer_begin(ISM_KERNEL_FWD, st);
@@ -663,8 +676,8 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   if ((r = status_ptr(&status)) != ISM_OK) return r;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (pre) {
-    // the plan's work counters start at zero for this call
-    ISM_TRY_CUDA(cudaMemsetAsync(L.counters, 0, kPassCounters * sizeof(int32_t), st), "work counter reset");
+    // the plan's work counter starts at zero for this call
+    ISM_TRY_CUDA(cudaMemsetAsync(L.counters + kBwdCounter, 0, sizeof(int32_t), st), "work counter reset");
   } else if ((r = build_pass_meta(segs, c, L, true, st)) != ISM_OK) {
     return r;
   }
@@ -677,7 +690,7 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
   a.ktiles = L.ktiles; a.k_order = L.k_order; a.nk = c.nk;
   a.ds = L.ds; a.kpair_off = L.kpair_off; a.ds_slots = L.ds ? slots : 0;
-  a.work_counter = L.counters;
+  a.work_counter = L.counters + kBwdCounter;
   // the k-tile pair list exists only when the CTA-pair dK/dV kernel will run
   // (and a plan holds none)
   a.kp_order = knobs().dkdv_pair && !pre ? L.kp_order : nullptr;
@@ -1077,6 +1090,7 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
     plan.kbase_stride = paged ? 1 : cg.cap;
     plan.bm = plan.bn = kTile;
     plan.kv_end = L.kv_end; plan.qtiles = L.qtiles; plan.q_order = L.q_order; plan.pair_order = L.pair_order;
+    plan.counter = L.c_snap;  // (only single-token steps have lengths there)
   }
   timer_begin(ISM_KERNEL_META, st);
   int32_t* snap_out = decode ? L.c_snap : nullptr;
@@ -1185,6 +1199,7 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
     const bool one_head = d == 128 && shape->dtype == ISM_BF16 &&
                           (knobs().fwd_one_head ||
                            (odd && l_new <= kTile && (sp.items == 0 || items * 4 > rounds * sm_count() * 3)));
+    if (fwd_dynamic(items, odd)) a.work_counter = L.c_snap;
     if (odd && !one_head) {
       a.pair_order = L.pair_order;
       a.npairs = L.npairs;

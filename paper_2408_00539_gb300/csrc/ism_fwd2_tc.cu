@@ -46,14 +46,19 @@ struct PairLayout {
   static constexpr uint32_t SMEM = BAR + 256 + 1024;
 };
 
+constexpr int kUnitSlots = 4;  // units published ahead of the roles that follow them (kDyn)
+
 struct Bars {
   uint64_t q_full, q_empty;
   uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];
   uint64_t s_full[2], p_half[2], p_full[2], pv_done[2];  // per head of the pair
   uint64_t final_mma;
+  uint64_t unit_full[kUnitSlots], unit_read[kUnitSlots];
+  int32_t units[kUnitSlots];
   uint32_t tmem_base;
   int32_t abort;
 };
+static_assert(sizeof(Bars) <= 256, "barrier block");
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
@@ -84,7 +89,7 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, int64_t item, Uni
     x.nkb0 = x.nkb1 = x.w0.a1;
   } else {
     int64_t ppos;
-    bucket_item(item, a.npairs, a.hq, ppos, x.h0, a.hq == a.hkv);  // one query head per KV head: bucketed
+    bucket_item(item, a.npairs, a.hq, ppos, x.h0, false);
     x.h1 = x.h0;
     const int gq = a.pair_order[ppos];
     x.w0 = a.qtiles[gq];
@@ -149,11 +154,14 @@ __device__ __forceinline__ int64_t unit_of(int64_t k, int64_t n_units) {
 // output's).  A block of two heads is 2 x (4 + 16) MMA steps; the tensor pipe
 // still waits for the softmax warps.  One layer of 16 heads over three
 // dialogues (6001 tokens): 102 us, against 44.3 ms of the CUDA-core kernel.
-template <bool kTilePairs, bool kE4M3, bool kSplit = false, int kHD = 128>
+// kDyn: the units come from a work counter (see fwd_dynamic) instead of the
+// static walk.
+template <bool kTilePairs, bool kE4M3, bool kSplit, int kHD, bool kDyn>
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const AttnArgs a, int64_t n_units) {
   static_assert(kHD == 128 || (kHD == 64 && !kE4M3), "head sizes of the paired forward");
+  static_assert(!(kSplit && kDyn), "split launches walk statically");
   using L = PairLayout<kE4M3, kHD>;
   constexpr uint32_t kTB = L::TB;
   extern __shared__ uint8_t smem_raw[];
@@ -175,6 +183,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::mbar_init(&bar->pv_done[s], 1);
     }
     ptx::mbar_init(&bar->final_mma, 1);
+    for (int s = 0; s < kUnitSlots; ++s) {
+      ptx::mbar_init(&bar->unit_full[s], 1);
+      ptx::mbar_init(&bar->unit_read[s], 9);  // the softmax warps and the MMA warp
+    }
     bar->abort = 0;
     ptx::fence_mbar_init();
   }
@@ -192,6 +204,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   advance_cache_len(a);
+
+  // the k-th unit of this CTA for the warps that follow the producer (-1: none left)
+  auto next_unit = [&](int k) -> int64_t {
+    if constexpr (!kDyn) return unit_of(k, n_units);
+    const int slot = k % kUnitSlots;
+    int u = -1;
+    if (wait(&bar->unit_full[slot], (k / kUnitSlots) & 1, a.status))
+      u = *reinterpret_cast<volatile int32_t*>(&bar->units[slot]);
+    u = __reduce_min_sync(0xffffffffu, u);  // one answer for the warp (a wait may give up)
+    if (lane == 0) ptx::mbar_arrive(&bar->unit_read[slot]);
+    return u;
+  };
 
   if (warp >= 8) {
     ptx::setmaxnreg_dec<kRegsService>();
@@ -211,8 +235,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t nq = 0, it = 0;           // Q loads and K / V blocks so far (all units)
       uint32_t nk[2] = {0, 0}, nv[2] = {0, 0};
       bool ok = true;
-      for (int64_t k = 0; ok; ++k) {
-        const int64_t u = unit_of(k, n_units);
+      for (int k = 0; ok; ++k) {
+        int64_t u;
+        if constexpr (kDyn) {
+          // the first unit is the block's, the others come from the counter
+          if (k >= kUnitSlots &&
+              !wait_warp(&bar->unit_read[k % kUnitSlots], (k / kUnitSlots - 1) & 1, a.status)) {
+            if (lane == 0) set_abort(&bar->abort);
+            ok = false;
+            break;
+          }
+          int v = 0;
+          if (lane == 0) {
+            v = k == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(a.work_counter, 1);
+            if (v >= n_units) v = -1;
+            bar->units[k % kUnitSlots] = v;
+            ptx::mbar_arrive(&bar->unit_full[k % kUnitSlots]);  // release: the entry is visible to the waiters
+          }
+          u = __shfl_sync(0xffffffffu, v, 0);
+        } else {
+          u = unit_of(k, n_units);
+        }
         if (u < 0) break;
         const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
         const int nkb = x.nkb();
@@ -318,8 +361,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         return true;
       };
       bool ok = true;
-      for (int64_t k = 0; ok; ++k) {
-        const int64_t u = unit_of(k, n_units);
+      for (int k = 0; ok; ++k) {
+        const int64_t u = next_unit(k);
         if (u < 0) break;
         const Unit x = decode_unit<kTilePairs, kSplit>(a, u);
         const int nkb = x.nkb();
@@ -393,8 +436,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float sl2 = a.scale * kLog2e * (kE4M3 ? a.qk_descale : 1.f);
     uint32_t nb = 0;  // blocks of this head so far (all units)
     bool ok = true;
-    for (int64_t k = 0; ok; ++k) {
-      const int64_t u = unit_of(k, n_units);
+    for (int k = 0; ok; ++k) {
+      const int64_t u = next_unit(k);
       if (u < 0) break;
       int nkbm, kfull, ke;  // key tiles and bounds counted from the unit's first key tile
       {
@@ -658,7 +701,9 @@ cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CU
                               cudaStream_t st) {
   cudaError_t e;
   const bool split = a.split_items > 0;
-  auto kern = split ? fwd_pair_kernel<kTilePairs, kE4M3, true, kHD> : fwd_pair_kernel<kTilePairs, kE4M3, false, kHD>;
+  auto kern = split ? fwd_pair_kernel<kTilePairs, kE4M3, true, kHD, false>
+              : a.work_counter ? fwd_pair_kernel<kTilePairs, kE4M3, false, kHD, true>
+                               : fwd_pair_kernel<kTilePairs, kE4M3, false, kHD, kTilePairs>;
   constexpr uint32_t smem = PairLayout<kE4M3, kHD>::SMEM;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
@@ -668,6 +713,7 @@ cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CU
                 a.split_parts > kMaxParts))
     return cudaErrorInvalidValue;
   const int64_t n_units = split ? a.split_whole + a.split_parts * a.split_items : items;
+  if (!split && (a.work_counter ? n_units >= (int64_t(1) << 30) : kTilePairs)) return cudaErrorInvalidValue;
   // persistent: one CTA per SM walks its share of the units
   const int64_t grid = n_units < sm_count() ? n_units : sm_count();
   if (!split) {

@@ -103,6 +103,7 @@ struct AppendPlan {
   Tile* qtiles;
   int32_t* q_order;
   int32_t* pair_order;
+  int32_t* counter;  // set to zero (the forward's work counter)
 };
 // cache_len: lengths before the append (read only; the attention kernels
 // advance them).  snap_out (nullable): receives a copy of them.
@@ -130,6 +131,9 @@ cudaError_t launch_rope_rows(const int32_t* cu_seqlens, int num_seqs, int64_t T,
                              const float* sin_t, float sin_sign, cudaStream_t st);
 
 // CUDA-core attention (ism_simt.cu), fp32 or bf16 storage, fp32 math.
+// Multiprocessor count of the current device (looked up once per device).
+int sm_count();
+
 struct AttnArgs {
   const void* q; const void* k; const void* v; const void* o; const void* dout;
   void* out; float* lse; const float* lse_in;
@@ -154,7 +158,8 @@ struct AttnArgs {
   // the next q-tile of its sequence, when there is one) in cost order.
   const int32_t* pair_order;
   int64_t npairs;
-  // Work counter of the persistent dK/dV kernel (zeroed by the metadata pass).
+  // Work counter, at zero: of the persistent dK/dV kernel, or of the paired
+  // forward on query-tile pairs.
   int32_t* work_counter;
   // dK/dV on CTA pairs: kp_order lists the even-indexed k-tiles (each with the
   // next k-tile of its sequence, when there is one) in cost order; nkp of them.
@@ -190,6 +195,16 @@ struct AttnArgs {
   uint32_t flags;
 };
 enum : uint32_t { kFlagDrainTmemReuse = 1u };
+// Whether the paired forward takes its units (whole items) from a work counter
+// in cost order, or walks them statically.  The counter evens out CTAs that get
+// few or unequal units; the static walk starts a unit a little sooner.  Query-
+// tile pairs always gain (units of one or two long tiles of many sizes): 4 x 4096
+// multi-head 414 -> 387 us, 6 ragged dialogues of 32 heads 692 -> 575, head_dim
+// 64 with 16 heads over 6001 tokens 98 -> 67.  Head pairs gain below eight units
+// a CTA (16 / 4 heads over 5000 ragged tokens, 2 units a CTA: 46 -> 39) and lose
+// on many even ones (2 x 8192, 13 a CTA: 654 -> 662; one dialogue of 32768 4881
+// -> 4951).
+inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || items < 8 * (int64_t)sm_count(); }
 // Called by every thread of every block of a forward kernel.
 __device__ __forceinline__ void advance_cache_len(const AttnArgs& a) {
   if (a.adv_cache_len && blockIdx.x == 0)
@@ -273,8 +288,6 @@ struct Knobs {
 };
 const Knobs& knobs();
 void reload_knobs();
-// Multiprocessor count of the current device (looked up once per device).
-int sm_count();
 
 // Measurement hooks (ism_api.cu): events recorded around launches of one
 // kernel kind on the calling host thread, and a count of every launch.

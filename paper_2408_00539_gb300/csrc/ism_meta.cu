@@ -313,6 +313,7 @@ __device__ __forceinline__ void append_plan_part(const AppendPlan& p, int batch,
   const AppendSegs& sg = p.segs;
   const int32_t Ln = sg.l_new;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  if (t0 == 0) *p.counter = 0;
   for (int64_t i = t0; i < (int64_t)batch * Ln; i += stride)
     p.kv_end[i] = cache_len[i / Ln] + chunk_kv_end(sg, (int32_t)(i % Ln));
   const int nqt = (Ln + p.bm - 1) / p.bm, npt = (nqt + 1) / 2;

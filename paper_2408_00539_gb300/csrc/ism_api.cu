@@ -323,13 +323,13 @@ ism_status_t check_ws(void* ws, size_t have, size_t need) {
 }
 
 ism_status_t build_pass_meta(const ism_segments_t* s, const Counts& c, const PassLayout& L, bool bwd,
-                             cudaStream_t st, bool heads_first = false) {
+                             cudaStream_t st, int heads, bool heads_first = false) {
   SegsDev d = dev_view(s);
   timer_begin(ISM_KERNEL_META, st);
   ISM_TRY_CUDA(launch_pass_meta(d, L.kv_end, kTile, kTile, c.nq, bwd ? c.nk : 0, L.qtiles, bwd ? L.ktiles : nullptr,
                                 c.max_cost, L.q_order, bwd ? L.k_order : nullptr, L.pair_order, L.kpair_off,
                                 L.counters, L.counters ? kPassCounters : 0, st,
-                                knobs().dkdv_pair ? L.kp_order : nullptr, heads_first),
+                                knobs().dkdv_pair ? L.kp_order : nullptr, heads_first, dependent_pass(c.nq, heads)),
                "metadata launch");
   timer_end(ISM_KERNEL_META, st);
   count_launch(1);
@@ -549,7 +549,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     timer_begin(ISM_KERNEL_ROPE, st);
     ISM_TRY_CUDA(launch_rope_rows(segs->cu_seqlens, segs->num_seqs, info.total_tokens, shape->num_heads_q,
                                   shape->num_heads_kv, shape->head_dim, shape->dtype, q, k, q_rot, k_rot, rope->cos,
-                                  rope->sin, 1.f, st),
+                                  rope->sin, 1.f, st, dependent_pass(c.nq, shape->num_heads_q)),
                  "rope launch");
     timer_end(ISM_KERNEL_ROPE, st);
     count_launch(1);
@@ -562,7 +562,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
                        fwd_dynamic(tile_pairs ? c.npairs * shape->num_heads_q : c.nq * (shape->num_heads_q / 2),
                                    tile_pairs);
   if (!pre) {
-    if ((r = build_pass_meta(segs, c, L, false, st, pairs_first(shape))) != ISM_OK) return r;
+    if ((r = build_pass_meta(segs, c, L, false, st, shape->num_heads_q, pairs_first(shape))) != ISM_OK) return r;
   } else if (dynamic) {
     ISM_TRY_CUDA(cudaMemsetAsync(L.counters + kFwdCounter, 0, sizeof(int32_t), st), "work counter reset");
   }
@@ -571,6 +571,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.q = q; a.k = k; a.v = v; a.out = o; a.lse = lse;
   a.hq = shape->num_heads_q; a.hkv = shape->num_heads_kv; a.d = shape->head_dim; a.dtype = shape->dtype;
   a.q_rows = info.total_tokens; a.scale = shape->softmax_scale;
+  a.dependent = dependent_pass(c.nq, shape->num_heads_q);
   a.qk_descale = qk_descale; a.v_descale = v_descale;
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
   a.pair_order = L.pair_order; a.npairs = L.pair_order ? c.npairs : 0;
@@ -678,7 +679,7 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   if (pre) {
     // the plan's work counter starts at zero for this call
     ISM_TRY_CUDA(cudaMemsetAsync(L.counters + kBwdCounter, 0, sizeof(int32_t), st), "work counter reset");
-  } else if ((r = build_pass_meta(segs, c, L, true, st)) != ISM_OK) {
+  } else if ((r = build_pass_meta(segs, c, L, true, st, shape->num_heads_q)) != ISM_OK) {
     return r;
   }
 
@@ -687,6 +688,7 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.dq = dq; a.dk = dk; a.dv = dv; a.delta = L.delta;
   a.hq = shape->num_heads_q; a.hkv = shape->num_heads_kv; a.d = shape->head_dim; a.dtype = shape->dtype;
   a.q_rows = info.total_tokens; a.scale = shape->softmax_scale;
+  a.dependent = dependent_pass(c.nq, shape->num_heads_q);
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
   a.ktiles = L.ktiles; a.k_order = L.k_order; a.nk = c.nk;
   a.ds = L.ds; a.kpair_off = L.kpair_off; a.ds_slots = L.ds ? slots : 0;
@@ -709,7 +711,7 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
       timer_begin(ISM_KERNEL_ROPE, st);
       ISM_TRY_CUDA(launch_rope_rows(segs->cu_seqlens, segs->num_seqs, info.total_tokens, shape->num_heads_q,
                                     shape->num_heads_kv, shape->head_dim, shape->dtype, dq, dk, dq, dk, rope->cos,
-                                    rope->sin, -1.f, st),
+                                    rope->sin, -1.f, st, a.dependent),
                    "rope launch");
       timer_end(ISM_KERNEL_ROPE, st);
       count_launch(1);
@@ -763,7 +765,7 @@ ism_status_t ism_attn_plan_build(const ism_segments_t* segs, const ism_attn_shap
   if ((r = check_ws(plan, plan_bytes, L.bytes)) != ISM_OK) return r;
   if (info.total_tokens > 0) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if ((r = build_pass_meta(segs, c, L, true, st, pairs_first(shape))) != ISM_OK) return r;
+    if ((r = build_pass_meta(segs, c, L, true, st, shape->num_heads_q, pairs_first(shape))) != ISM_OK) return r;
   }
   plan_info->fingerprint = plan_fingerprint(segs, shape, tile_pairs);
   plan_info->bytes = L.bytes;
@@ -1167,6 +1169,7 @@ ism_status_t append_impl(const ism_attn_shape_t* shape, int32_t batch, const voi
   a.q = q_new; a.k = k_cache; a.v = v_cache; a.out = o_new; a.lse = lse_new;
   a.hq = hq; a.hkv = hkv; a.d = d; a.dtype = shape->dtype;
   a.q_rows = (int64_t)batch * l_new; a.scale = shape->softmax_scale;
+  a.dependent = dependent_pass((int64_t)batch * ((l_new + kTile - 1) / kTile), hq);
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order;
   a.nq = (int64_t)batch * ((l_new + kTile - 1) / kTile);
   a.pages = cg.pages;

@@ -69,9 +69,14 @@ __device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t 
 // use (more bytes in flight per thread: the kernel only streams O and dO).
 // The reductions shuffle within the group's own lanes, so the groups of a
 // warp may run different numbers of rounds.
-template <int kHD>
+template <int kHD, bool kDependent>
 __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
                              float* __restrict__ delta, int64_t rows, int hq) {
+  // O and dO are in place when this kernel runs at all: its direct predecessor
+  // is the metadata pass (or a reset of its counter), which it does not depend on
+  // and runs beside as a dependent launch.  The wait at the end makes this
+  // kernel's completion imply that one's.  (It costs 4 of 48 us on 2 x 8192
+  // tokens of 32 heads, which are launched plainly.)
   constexpr int kUnroll = 4;
   const int64_t n = rows * hq;
   constexpr int kLanes = kHD / 8;
@@ -109,6 +114,7 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
       }
     }
   }
+  if constexpr (kDependent) pdl_wait();
 }
 
 // ------------------------------------------------------------------ dQ
@@ -152,6 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   int64_t tpos;
   int h;
   bucket_item(blockIdx.x, a.nq, a.hq, tpos, h, a.hq == a.hkv);  // blocks start roughly in index order
@@ -468,6 +475,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
   Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (ptx::smem_u32(smem) & 1023u) {  // the swizzled tiles need 1024-byte alignment
+    pdl_wait();
     if (threadIdx.x == 0) atomicOr(a.status, kStatusSmemAlign);
     return;
   }
@@ -507,6 +515,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  pdl_wait();  // the set-up above overlaps the kernel before
 
   // Work items (k-tile k_order[item / hkv], KV head item % hkv) come from a
   // global counter, most expensive first; the load warp takes them and
@@ -1019,11 +1028,11 @@ cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
     int grid = (int)((groups * (kHD / 8) + 255) / 256);
     if (grid > 152 * 16) grid = 152 * 16;
     timer_begin(ISM_KERNEL_BWD_PRE, st);
-    delta_kernel<kHD><<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows,
-                                       a.hq);
+    e = launch(a.dependent, a.dependent ? delta_kernel<kHD, true> : delta_kernel<kHD, false>, grid, 256, 0, st, (const __nv_bfloat16*)a.o,
+                         (const __nv_bfloat16*)a.dout, a.delta, a.q_rows, a.hq);
     timer_end(ISM_KERNEL_BWD_PRE, st);
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   CUtensorMap tq, tdo, tk, tv;
   if ((e = make_tmap_bf16(&tq, a.q, (uint64_t)a.hq * kHD, (uint64_t)a.q_rows)) != cudaSuccess) return e;
@@ -1038,10 +1047,11 @@ cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
         cudaSuccess)
       return e;
     timer_begin(ISM_KERNEL_BWD_DQ, st);
-    dq_kernel<kHD><<<(unsigned)(a.nq * a.hq), kThreads, dq::Layout<kHD>::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
+    e = launch(a.dependent, dq_kernel<kHD>, a.nq * a.hq, kThreads, dq::Layout<kHD>::kSmemBytes, st, tq,
+                         tdo, tk, tv, a);
     timer_end(ISM_KERNEL_BWD_DQ, st);
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   if (kHD == 128 && a.nk && knobs().dkdv_pair && a.kp_order) {
     // the CTA-pair kernel (ism_dkdv2_tc.cu)
@@ -1058,10 +1068,11 @@ cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
     if (grid > a.nk * a.hkv) grid = a.nk * a.hkv;
     if (!a.work_counter) return cudaErrorInvalidValue;
     timer_begin(ISM_KERNEL_BWD_DKDV, st);
-    dkdv_kernel<kHD><<<(unsigned)grid, dkv::kThreads, dkv::Layout<kHD>::kSmemBytes, st>>>(tq, tdo, tk, tv, a);
+    e = launch(a.dependent, dkdv_kernel<kHD>, grid, dkv::kThreads, dkv::Layout<kHD>::kSmemBytes, st, tq, tdo,
+                         tk, tv, a);
     timer_end(ISM_KERNEL_BWD_DKDV, st);
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   if (a.nq && a.ds) {
     timer_begin(ISM_KERNEL_BWD_DQ, st);

@@ -422,6 +422,7 @@ __global__ void __launch_bounds__(160) decode_tma_kernel(const __grid_constant__
 // one for each of a.splits chunks, those without keys marked by a maximum of -inf.
 template <int D, bool kRow>
 __global__ void decode_combine_kernel(DecodeArgs a) {
+  // the next step's cache write, which waits for this kernel, may be launched at once
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int bh = blockIdx.x;
@@ -484,16 +485,7 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
 // The combine as a programmatic dependent launch of the kernel before it.
 template <int D, bool kRow = false>
 cudaError_t launch_combine(const DecodeArgs& a, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.batch * a.hq));
-  cfg.blockDim = dim3(D);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_combine_kernel<D, kRow>, a);
+  return launch(true, decode_combine_kernel<D, kRow>, (int64_t)a.batch * a.hq, D, 0, st, a);
 }
 
 template <int D, int G>

@@ -693,17 +693,7 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc;
   }
   if (grid <= 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg::kSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_tc_kernel<kE4M3, kG>, tq, tk, tv, a);
+  return launch(true, decode_tc_kernel<kE4M3, kG>, grid, kThreads, Cfg::kSmemBytes, st, tq, tk, tv, a);
 }
 
 }  // namespace

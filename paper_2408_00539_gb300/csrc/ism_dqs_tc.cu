@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  pdl_wait();  // the set-up above overlaps the kernel before
 
   if (warp == 4) {
     // ------------------------------------------------ copies (the warp waits converged, lane 0 issues)
@@ -252,8 +253,7 @@ cudaError_t launch_dq_gemm(const AttnArgs& a, const CUtensorMap& tk, cudaStream_
   int grid = knobs().dq_grid > 0 ? knobs().dq_grid : sm_count();
   if (grid > n_items) grid = (int)n_items;
   if (grid <= 0) return cudaSuccess;
-  dq_gemm_kernel<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tk, a, n_items);
-  return cudaGetLastError();
+  return launch(a.dependent, dq_gemm_kernel, grid, kThreads, kSmemBytes, st, tk, a, n_items);
 }
 
 }  // namespace tc

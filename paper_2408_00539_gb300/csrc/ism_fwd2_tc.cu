@@ -198,11 +198,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
-  if constexpr (kSplit) {
-    // launched as a programmatic dependent of the append's cache write: the
-    // set-up above overlaps it
+  // the set-up above overlaps the kernel before (a split launch lets the merge
+  // start only once every CTA is done: its blocks would take issue slots and
+  // registers of the running ones)
+  if constexpr (kSplit)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-  }
+  else
+    pdl_wait();
   advance_cache_len(a);
 
   // the k-th unit of this CTA for the warps that follow the producer (-1: none left)
@@ -611,8 +613,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!ok) set_abort(&bar->abort);
   }
-  // the merge may be launched once every CTA is done (its blocks would take
-  // issue slots and registers of the running ones otherwise)
   if constexpr (kSplit) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   ptx::tc_fence_before();
   __syncthreads();
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 constexpr int kMaxParts = 32;
 template <bool kTilePairs, int kHD>
 __global__ void __launch_bounds__(128) fwd_split_merge_kernel(const AttnArgs a) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   const int r = (int)(i % a.part_rows), x = (int)((i / a.part_rows) & 1);
@@ -679,23 +679,6 @@ __global__ void __launch_bounds__(128) fwd_split_merge_kernel(const AttnArgs a) 
   if (lane == 0 && a.lse) a.lse[(int64_t)h * a.q_rows + orow] = (M + log2f(L)) * kLn2;
 }
 
-// Launch as a programmatic dependent of the kernel before it on the stream.
-template <class... Params, class... Args>
-cudaError_t launch_dependent(void (*kern)(Params...), int64_t grid, int threads, uint32_t smem, cudaStream_t st,
-                             Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 template <bool kE4M3, int kHD, bool kTilePairs>
 cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                               cudaStream_t st) {
@@ -716,13 +699,11 @@ cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CU
   if (!split && (a.work_counter ? n_units >= (int64_t(1) << 30) : kTilePairs)) return cudaErrorInvalidValue;
   // persistent: one CTA per SM walks its share of the units
   const int64_t grid = n_units < sm_count() ? n_units : sm_count();
-  if (!split) {
-    kern<<<(unsigned)grid, kThreads, smem, st>>>(tq, tk, tv, a, n_units);
-    return cudaGetLastError();
-  }
-  if ((e = launch_dependent(kern, grid, kThreads, smem, st, tq, tk, tv, a, n_units)) != cudaSuccess) return e;
+  if ((e = launch(split || a.dependent, kern, grid, kThreads, smem, st, tq, tk, tv, a, n_units)) != cudaSuccess ||
+      !split)
+    return e;
   const int64_t rows = a.split_items * 2 * a.part_rows;
-  return launch_dependent(fwd_split_merge_kernel<kTilePairs, kHD>, (rows + 3) / 4, 128, 0, st, a);
+  return launch(true, fwd_split_merge_kernel<kTilePairs, kHD>, (rows + 3) / 4, 128, 0, st, a);
 }
 
 }  // namespace

@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   Bars* bar = reinterpret_cast<Bars*>(smem + OFF_BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   const int h = blockIdx.x % a.hq;
   const Tile w = a.qtiles[a.q_order[blockIdx.x / a.hq]];
   const int g = h / (a.hq / a.hkv);
@@ -567,8 +568,7 @@ cudaError_t launch_fwd(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
   if ((e = cudaFuncSetAttribute(fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) !=
       cudaSuccess)
     return e;
-  fwd_kernel<<<(unsigned)(a.nq * a.hq), kThreads, kSmemBytes, st>>>(tq, tk, tv, a);
-  return cudaGetLastError();
+  return launch(a.dependent, fwd_kernel, a.nq * a.hq, kThreads, kSmemBytes, st, tq, tk, tv, a);
 }
 
 cudaError_t launch_mma_tile(const void* A, const void* B, float* C, int mode, uint32_t* status, cudaStream_t st) {

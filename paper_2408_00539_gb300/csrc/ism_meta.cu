@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(1024)
                      Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order, int32_t* pair_order,
                      int32_t* kpair_off, int32_t* counters, int n_counters, int32_t* kp_order, bool pairs_first) {
   extern __shared__ __align__(16) unsigned char dyn[];
+  pdl_wait();
   if ((int)threadIdx.x < n_counters) counters[threadIdx.x] = 0;  // work counters of the kernels that follow
   // kv_end: one warp per segment, lanes over its tokens
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -295,6 +296,114 @@ __global__ void __launch_bounds__(1024)
   order_body(qtiles, nq, ktiles, nk, max_cost, q_order, k_order, pair_order, reinterpret_cast<int32_t*>(dyn),
              kp_order, pairs_first);
   if (kpair_off) pair_offsets_body(ktiles, nk, kpair_off);
+}
+
+// The same for a small batch (at most kSmallTiles tiles and sequences and
+// kSmallSegs segments, bm == bn): the segments are read into shared memory
+// once, every bound, descriptor, rank and offset is computed there and in
+// registers, one thread a tile, and the results are written at the end.  The
+// ranks are counted by comparing every pair of tiles.  The general pass goes
+// through global memory and some twenty block barriers of 1024 threads: one
+// dialogue of 256 tokens 8.0 us, this one 5.0; 2 x 8192 tokens 11.5 and 10.
+constexpr int kSmallTiles = 256, kSmallSegs = 1024, kSmallThreads = 512;
+
+// How many of the n costs come before cost c of item i in the list (higher
+// first, equal ones by index); costs below zero are not listed.
+__device__ __forceinline__ int rank_of(const int32_t* costs, int n, int32_t c, int i) {
+  int r = 0;
+  for (int j = 0; j < n; j += 4) {  // (n rounded up: the padding is negative)
+    const int4 v = *reinterpret_cast<const int4*>(costs + j);
+    r += (v.x > c || (v.x == c && j < i)) + (v.y > c || (v.y == c && j + 1 < i)) +
+         (v.z > c || (v.z == c && j + 2 < i)) + (v.w > c || (v.w == c && j + 3 < i));
+  }
+  return r;
+}
+
+__global__ void __launch_bounds__(kSmallThreads)
+    pass_meta_small_kernel(SegsDev s, int32_t* kv_end, int bm, int nq, Tile* qtiles, Tile* ktiles, int32_t* q_order,
+                           int32_t* k_order, int32_t* pair_order, int32_t* kpair_off, int32_t* counters,
+                           int n_counters, bool pairs_first) {
+  __shared__ int32_t cu[kSmallTiles + 1], cseg[kSmallTiles + 1], off[kSmallTiles + 1], ends[kSmallSegs];
+  __shared__ uint8_t types[kSmallSegs];
+  // per list: q-tiles, k-tiles, pair heads, odd q-tiles; -1 where not listed
+  __shared__ __align__(16) int32_t cost[4][kSmallTiles + 4];
+  const int tid = threadIdx.x;
+  pdl_wait();
+  for (int i = tid; i <= s.num_seqs; i += kSmallThreads) {
+    cu[i] = s.cu_seqlens[i];
+    cseg[i] = s.cu_segs[i];
+  }
+  for (int i = tid; i < s.num_segs; i += kSmallThreads) {
+    ends[i] = s.seg_end[i];
+    types[i] = s.seg_type[i];
+  }
+  for (int i = tid; i < 4 * (kSmallTiles + 4); i += kSmallThreads) (&cost[0][0])[i] = -1;
+  __syncthreads();
+  int32_t total;
+  const int32_t n_b = tid < s.num_seqs ? (cu[tid + 1] - cu[tid] + bm - 1) / bm : 0;
+  const int32_t incl = block_inclusive_scan<int32_t>(n_b, &total);
+  if (tid < s.num_seqs) off[tid + 1] = incl;
+  if (tid == 0) off[0] = 0;
+  __syncthreads();
+  // segment of row (or key) x of sequence b, and the row's key bound (Eq. fj)
+  auto seg_of = [&](int b, int x) { return cseg[b] + upper_bound_i32(ends + cseg[b], cseg[b + 1] - cseg[b], x); };
+  auto bound = [&](int b, int row) {
+    const int g = seg_of(b, row);
+    return types[g] == ISM_SEG_QUERY ? ends[g] : row + 1;
+  };
+  Tile q{}, k{};
+  if (tid < nq) {
+    const int b = upper_bound_i32(off, s.num_seqs + 1, tid) - 1;
+    const int t = tid - off[b], L = cu[b + 1] - cu[b], r0 = t * bm;
+    q.q_base = q.k_base = q.kv_base = cu[b];
+    q.q_len = q.k_len = L;
+    q.tile = t;
+    k = q;
+    q.a0 = r0 + bm <= L ? bound(b, r0) / bm : 0;
+    q.a1 = (bound(b, min(L, r0 + bm) - 1) + bm - 1) / bm;
+    // first row that sees key r0 (as in tiles_body)
+    const int g = seg_of(b, r0), start = g > cseg[b] ? ends[g - 1] : 0;
+    k.a0 = (types[g] == ISM_SEG_QUERY ? start : max(r0, start)) / bm;
+    k.a1 = (L + bm - 1) / bm;
+    cost[0][tid] = q.a1;
+    cost[1][tid] = max(k.a1 - k.a0, 0);
+  }
+  __syncthreads();
+  const bool odd = q.tile & 1;
+  if (tid < nq) {
+    // a pair costs what its second tile does (the first, when it has none)
+    const bool second = tid + 1 < nq && !odd && (q.tile + 1) * bm < q.q_len;
+    cost[odd ? 3 : 2][tid] = odd ? q.a1 : max(q.a1, second ? cost[0][tid + 1] : 0);
+  }
+  __syncthreads();
+  int32_t pairs;
+  const int32_t before = block_inclusive_scan<int32_t>(tid < nq ? cost[1][tid] : 0, &pairs);
+  int rq = 0, rk = 0, rp = 0;
+  int32_t heads = 0;
+  if (pairs_first) block_inclusive_scan<int32_t>(tid < nq && !odd ? 1 : 0, &heads);
+  if (tid < nq) {
+    if (!odd && (pair_order || pairs_first)) rp = rank_of(cost[2], nq, cost[2][tid], tid);
+    rq = !pairs_first ? rank_of(cost[0], nq, cost[0][tid], tid)
+         : odd        ? heads + rank_of(cost[3], nq, cost[3][tid], tid)
+                      : rp;
+    if (k_order) rk = rank_of(cost[1], nq, cost[1][tid], tid);
+  }
+  if (tid < n_counters) counters[tid] = 0;
+  if (tid < nq) {
+    qtiles[tid] = q;
+    q_order[rq] = tid;
+    if (ktiles) ktiles[tid] = k;
+    if (k_order) k_order[rk] = tid;
+    if (pair_order && !odd) pair_order[rp] = tid;
+    if (kpair_off) kpair_off[tid] = before - cost[1][tid];
+  }
+  const int warp = tid >> 5, lane = tid & 31;
+  for (int seg = warp; seg < s.num_segs; seg += kSmallThreads / 32) {
+    const int b = upper_bound_i32(cseg, s.num_seqs + 1, seg) - 1;
+    const int start = seg > cseg[b] ? ends[seg - 1] : 0, end = ends[seg];
+    const bool query = types[seg] == ISM_SEG_QUERY;
+    for (int j = start + lane; j < end; j += 32) kv_end[cu[b] + j] = query ? end : j + 1;
+  }
 }
 
 __device__ __forceinline__ int32_t chunk_kv_end(const AppendSegs& sg, int32_t j) {
@@ -373,24 +482,17 @@ __device__ __forceinline__ void zero_value_tail(int batch, int l_new, int vec_pe
   }
 }
 
-// Both cache-write kernels are launched as programmatic dependents, so that
-// their launch overlaps the end of whatever runs before (the combine of the
-// step before, in a generation loop), and let the attention kernel start as
-// soon as that is complete: what it reads beside the new rows is then in place.
+// The cache-write kernels let the attention kernel start as soon as what ran
+// before them is complete: what it reads beside the new rows is then in place.
 // A rotary decode step over 3000 keys 13.1 -> 10.6 us, 40 ragged caches 70 -> 67,
 // e4m3 8 x 16384 keys 50.7 -> 48 (with the decode reading the old keys while
 // the new row is written).  Inputs are not __restrict__: nothing may be loaded
 // before the wait.
-__device__ __forceinline__ void write_prologue() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 __global__ void cache_write_kernel(int batch, int l_new, int row_bytes, int64_t cap, KvPages pages,
                                    const int32_t* c_snap, const uint4* k_new,
                                    const uint4* v_new, uint4* k_cache, uint4* v_cache,
                                    const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
-  write_prologue();
+  pdl_wait();
   append_plan_part(plan, batch, c_snap);
   const int vec_per_row = row_bytes / 16;
   copy_snapshot(batch, c_snap, snap_out);
@@ -457,7 +559,7 @@ __global__ void rope_cache_write_kernel(int batch, int l_new, int hq, int hkv, i
                                         const float* __restrict__ sin_t, float q_descale, float k_descale,
                                         float v_descale, void* q_rot, void* k_cache, void* v_cache,
                                         const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
-  write_prologue();
+  pdl_wait();
   append_plan_part(plan, batch, c_snap);
   copy_snapshot(batch, c_snap, snap_out);
   const int half = d / 2;
@@ -557,7 +659,10 @@ cudaError_t launch_order(const Tile* qtiles, int64_t nq, const Tile* ktiles, int
 cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, int64_t nq, int64_t nk,
                              Tile* qtiles, Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order,
                              int32_t* pair_order, int32_t* kpair_off, int32_t* counters, int n_counters,
-                             cudaStream_t st, int32_t* kp_order, bool pairs_first) {
+                             cudaStream_t st, int32_t* kp_order, bool pairs_first, bool dependent) {
+  if (bm == bn && nq <= kSmallTiles && s.num_seqs <= kSmallTiles && s.num_segs <= kSmallSegs && !kp_order)
+    return launch(dependent, pass_meta_small_kernel, 1, kSmallThreads, 0, st, s, kv_end, bm, (int)nq, qtiles,
+                            ktiles, q_order, k_order, pair_order, kpair_off, counters, n_counters, pairs_first);
   size_t a = (size_t)(s.num_seqs + 1) * (sizeof(int64_t) + 2 * sizeof(int32_t));
   size_t b = sizeof(int32_t) * (size_t)(max_cost + 1);
   size_t smem = a > b ? a : b;
@@ -568,9 +673,8 @@ cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, 
     cudaError_t e = cudaFuncSetAttribute(pass_meta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  pass_meta_kernel<<<1, 1024, smem, st>>>(s, kv_end, bm, bn, nq, nk, qtiles, ktiles, max_cost, q_order, k_order,
-                                          pair_order, kpair_off, counters, n_counters, kp_order, pairs_first);
-  return cudaGetLastError();
+  return launch(dependent, pass_meta_kernel, 1, 1024, smem, st, s, kv_end, bm, bn, nq, nk, qtiles, ktiles, max_cost,
+                          q_order, k_order, pair_order, kpair_off, counters, n_counters, kp_order, pairs_first);
 }
 
 cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_off, cudaStream_t st) {
@@ -580,21 +684,12 @@ cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_o
 }
 
 namespace {
-// A cache-write kernel over `total` threads, as a programmatic dependent.
+// A cache-write kernel over `total` threads.
 template <class... Params, class... Args>
 cudaError_t launch_write(void (*kern)(Params...), int64_t total, cudaStream_t st, Args... args) {
   int64_t grid = (total + 255) / 256;
   if (grid > 152 * 16) grid = 152 * 16;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(256);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  return launch(true, kern, grid, 256, 0, st, args...);
 }
 }  // namespace
 

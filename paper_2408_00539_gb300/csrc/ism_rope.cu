@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* __restric
                                                         const E* k_src, E* q_dst, E* k_dst,
                                                         const float* __restrict__ cos_t,
                                                         const float* __restrict__ sin_t, float sin_sign) {
+  pdl_wait();
   constexpr int N = Vec<E>::N;
   const int half = d / 2;
   const int units = half / N;
@@ -119,26 +120,21 @@ __global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* __restric
 
 cudaError_t launch_rope_rows(const int32_t* cu_seqlens, int num_seqs, int64_t T, int hq, int hkv, int d, int dtype,
                              const void* q_src, const void* k_src, void* q_dst, void* k_dst, const float* cos_t,
-                             const float* sin_t, float sin_sign, cudaStream_t st) {
+                             const float* sin_t, float sin_sign, cudaStream_t st, bool dependent) {
   const int elems = dtype == ISM_BF16 ? 8 : 4;
   const int64_t total = T * (hq + hkv) * (d / 2 / elems);
   if (total == 0) return cudaSuccess;
   int64_t grid = (total + 255) / 256;
   const int64_t cap = (int64_t)sm_count() * 16;
   if (grid > cap) grid = cap;
-  if (dtype == ISM_BF16) {
-    rope_rows_kernel<__nv_bfloat16><<<(unsigned)grid, 256, 0, st>>>(
-        cu_seqlens, num_seqs, T, hq, hkv, d, static_cast<const __nv_bfloat16*>(q_src),
-        static_cast<const __nv_bfloat16*>(k_src), static_cast<__nv_bfloat16*>(q_dst),
-        static_cast<__nv_bfloat16*>(k_dst), cos_t, sin_t, sin_sign);
-  } else {
-    rope_rows_kernel<float><<<(unsigned)grid, 256, 0, st>>>(cu_seqlens, num_seqs, T, hq, hkv, d,
-                                                            static_cast<const float*>(q_src),
-                                                            static_cast<const float*>(k_src),
-                                                            static_cast<float*>(q_dst), static_cast<float*>(k_dst),
-                                                            cos_t, sin_t, sin_sign);
-  }
-  return cudaGetLastError();
+  if (dtype == ISM_BF16)
+    return launch(dependent, rope_rows_kernel<__nv_bfloat16>, grid, 256, 0, st, cu_seqlens, num_seqs, T, hq,
+                            hkv, d, static_cast<const __nv_bfloat16*>(q_src), static_cast<const __nv_bfloat16*>(k_src),
+                            static_cast<__nv_bfloat16*>(q_dst), static_cast<__nv_bfloat16*>(k_dst), cos_t, sin_t,
+                            sin_sign);
+  return launch(dependent, rope_rows_kernel<float>, grid, 256, 0, st, cu_seqlens, num_seqs, T, hq, hkv, d,
+                          static_cast<const float*>(q_src), static_cast<const float*>(k_src),
+                          static_cast<float*>(q_dst), static_cast<float*>(k_dst), cos_t, sin_t, sin_sign);
 }
 
 }  // namespace ism

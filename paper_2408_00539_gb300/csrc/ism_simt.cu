@@ -232,11 +232,12 @@ __device__ __forceinline__ Tile own_rows(const Tile* tiles, const int32_t* order
 template <class C>
 __global__ void __launch_bounds__(C::TH) simt_fwd_kernel(const AttnArgs a) {
   using T = typename C::T;
+  pdl_wait();
+  advance_cache_len(a);
   extern __shared__ __align__(16) float sm[];
   float *own = sm, *kt = own + C::OWN, *vt = kt + C::TILE, *wt = vt + C::TILE;
   int h, row0;
   const Tile w = own_rows<C>(a.qtiles, a.q_order, a.hq, &h, &row0);
-  advance_cache_len(a);
   if (row0 >= w.q_len) return;
   const int g = h / (a.hq / a.hkv);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rw = warp % C::W, sw = warp / C::W;
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(C::TH) simt_fwd_kernel(const AttnArgs a) {
 template <class C>
 __global__ void __launch_bounds__(C::TH) simt_dq_kernel(const AttnArgs a) {
   using T = typename C::T;
+  pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *own_q = sm, *own_do = own_q + C::OWN, *kt = own_do + C::OWN, *vt = kt + C::TILE, *wt = vt + C::TILE;
   int h, row0;
@@ -437,6 +439,7 @@ __global__ void __launch_bounds__(C::TH) simt_dq_kernel(const AttnArgs a) {
 template <class C>
 __global__ void __launch_bounds__(C::TH) simt_dkdv_kernel(const AttnArgs a) {
   using T = typename C::T;
+  pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float *own_k = sm, *own_v = own_k + C::OWN, *qt = own_v + C::OWN, *dot = qt + C::TILE, *pt = dot + C::TILE,
         *dst = pt + C::WGT;
@@ -552,12 +555,11 @@ __global__ void __launch_bounds__(C::TH) simt_dkdv_kernel(const AttnArgs a) {
 
 // Launches `kern` over SUB blocks a (tile, head) with its shared memory.
 template <class C, class K>
-cudaError_t launch(K kern, int64_t tiles_heads, int floats, const AttnArgs& a, cudaStream_t st) {
+cudaError_t launch_cfg(K kern, int64_t tiles_heads, int floats, const AttnArgs& a, cudaStream_t st) {
   const int smem = floats * (int)sizeof(float);
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)(tiles_heads * C::SUB), C::TH, smem, st>>>(a);
-  return cudaGetLastError();
+  return ism::launch(a.dependent, kern, tiles_heads * C::SUB, C::TH, smem, st, a);
 }
 
 // 64 rows a block, or 16 with the streamed side split over four warps while
@@ -568,15 +570,15 @@ template <typename T, int D> using Small = Cfg<T, D, 4, 4, 4, 32>;
 
 template <class C>
 cudaError_t fwd_cfg(const AttnArgs& a, cudaStream_t st) {
-  return launch<C>(simt_fwd_kernel<C>, a.nq * a.hq, C::OWN + 2 * C::TILE + C::WGT, a, st);
+  return launch_cfg<C>(simt_fwd_kernel<C>, a.nq * a.hq, C::OWN + 2 * C::TILE + C::WGT, a, st);
 }
 template <class C>
 cudaError_t dq_cfg(const AttnArgs& a, cudaStream_t st) {
-  return launch<C>(simt_dq_kernel<C>, a.nq * a.hq, 2 * C::OWN + 2 * C::TILE + C::WGT, a, st);
+  return launch_cfg<C>(simt_dq_kernel<C>, a.nq * a.hq, 2 * C::OWN + 2 * C::TILE + C::WGT, a, st);
 }
 template <class C>
 cudaError_t dkdv_cfg(const AttnArgs& a, cudaStream_t st) {
-  return launch<C>(simt_dkdv_kernel<C>, a.nk * a.hkv, 2 * C::OWN + 2 * C::TILE + 2 * C::WGT, a, st);
+  return launch_cfg<C>(simt_dkdv_kernel<C>, a.nk * a.hkv, 2 * C::OWN + 2 * C::TILE + 2 * C::WGT, a, st);
 }
 
 template <typename T, int D>

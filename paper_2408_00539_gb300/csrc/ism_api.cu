@@ -580,6 +580,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     a.npairs = c.npairs;
   }
   a.work_counter = dynamic ? L.counters + kFwdCounter : nullptr;
+  a.bucketed = fwd_bucketed(a, a.npairs * a.hq);
   a.status = status;
   a.flags = tc_flags();
   timer_begin(ISM_KERNEL_FWD, st);

@@ -89,7 +89,7 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, int64_t item, Uni
     x.nkb0 = x.nkb1 = x.w0.a1;
   } else {
     int64_t ppos;
-    bucket_item(item, a.npairs, a.hq, ppos, x.h0, false);
+    bucket_item(item, a.npairs, a.hq, ppos, x.h0, a.bucketed);
     x.h1 = x.h0;
     const int gq = a.pair_order[ppos];
     x.w0 = a.qtiles[gq];

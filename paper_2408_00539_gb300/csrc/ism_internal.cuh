@@ -192,6 +192,7 @@ struct AttnArgs {
   // the next q-tile of its sequence, when there is one) in cost order.
   const int32_t* pair_order;
   int64_t npairs;
+  bool bucketed;  // their work list in buckets of neighbouring tiles, head by head (fwd_bucketed)
   // Work counter, at zero: of the persistent dK/dV kernel, or of the paired
   // forward on query-tile pairs.
   int32_t* work_counter;
@@ -243,6 +244,16 @@ inline bool dependent_pass(int64_t q_tiles, int heads) { return q_tiles * heads 
 // on many even ones (2 x 8192, 13 a CTA: 654 -> 662; one dialogue of 32768 4881
 // -> 4951).
 inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || items < 8 * (int64_t)sm_count(); }
+// Whether that list keeps its buckets (bucket_item) instead of the plain cost
+// order: with one query head per KV head, 32 KB tiles and many units, sharing
+// tiles in L2 saves more (power above all, in a loop of steps) than the order's
+// balance: 4 x 4096 of 32 heads 1767 us a step against 1786, although the forward
+// alone takes 396 against 387; six ragged dialogues 2684 and 2699.  Half-size
+// tiles and few units: e4m3 4 x 4096 333 and 318, head_dim 64 over 6001 tokens 318
+// and 302.
+inline bool fwd_bucketed(const AttnArgs& a, int64_t items) {
+  return a.hq == a.hkv && a.d == 128 && a.dtype == ISM_BF16 && items >= 8 * (int64_t)sm_count();
+}
 // Called by every thread of every block of a forward kernel.
 __device__ __forceinline__ void advance_cache_len(const AttnArgs& a) {
   if (a.adv_cache_len && blockIdx.x == 0)

@@ -56,8 +56,16 @@ __device__ __forceinline__ void mma_head_dim(uint32_t d, uint32_t sA, uint32_t s
 // head_dim 64 A also has a low part 32 columns on: P and dS keep 16 mantissa
 // bits there (hi = bf16(x), lo = bf16(x - hi)), because the results of that
 // head size are to be those of fp32 P and dS to within the output rounding.
+// half (head_dim 128): only over the first 64 rows of B, a last tile's that has
+// no more (24 dialogues of 32 heads, 16001 tokens: dK/dV 259 -> 254 us with the
+// stores of such tiles; at head_dim 64 the branch cost 115 -> 118).
 template <int kHD>
-__device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t sB, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t sB, uint32_t idesc, uint32_t acc,
+                                              bool half = false) {
+  if (kHD == 128 && half) {
+    ptx::mma4_bf16_ts_warp<8, 128>(d, tA, desc_mnmajor(sB, 0), idesc, acc);
+    return;
+  }
   ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(d, tA, desc_mnmajor(sB, 0), idesc, acc);
   if constexpr (kHD == 64)
     ptx::mma8_bf16_ts_warp<ptx::TmemPairsGap32, ptx::MnMajorSw128>(d, tA + 32, desc_mnmajor(sB, 0), idesc, 1u);
@@ -701,17 +709,18 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
     };
     // P^T (bf16, two queries per column) sits in the S^T columns and dS^T in the dP^T
     // columns: warpgroup wg's queries [64 wg, 64 wg + 64) at column 64 wg + [0, 32)
-    auto issue_dv = [&](uint32_t gi, bool first) {
+    // `half`: only the first 64 queries of the tile exist (P and dS of the others are zero)
+    auto issue_dv = [&](uint32_t gi, bool first, bool half) {
       const uint32_t s = gi & 1;
       const uint32_t sdO = ptx::smem_u32(smem + L::DO + s * L::TB);
-      mma_tile_rows<kHD>(tmem + TM_DV, tmem + TM_S, sdO, idesc_nn, first ? 0u : 1u);
+      mma_tile_rows<kHD>(tmem + TM_DV, tmem + TM_S, sdO, idesc_nn, first ? 0u : 1u, half);
       ptx::mma_commit_warp(&bar->do_empty[s]);
       ptx::mma_commit_warp(&bar->dv_done);
     };
-    auto issue_dk = [&](uint32_t gi, bool first) {
+    auto issue_dk = [&](uint32_t gi, bool first, bool half) {
       const uint32_t sq = gi % kQStages;
       const uint32_t sQ = ptx::smem_u32(smem + L::Q + sq * L::TB);
-      mma_tile_rows<kHD>(tmem + TM_DK, tmem + TM_DP, sQ, idesc_nn, first ? 0u : 1u);
+      mma_tile_rows<kHD>(tmem + TM_DK, tmem + TM_DP, sQ, idesc_nn, first ? 0u : 1u, half);
       ptx::mma_commit_warp(&bar->q_empty[sq]);
       ptx::mma_commit_warp(&bar->dk_done);
     };
@@ -719,6 +728,9 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
     for (uint32_t u = 0; ok; ++u) {
       if (!__all_sync(0xffffffffu, next_item(u, x))) break;
       const int n_it = x.n_it;
+      // the first iterations visit the last query tile: a short one when it
+      // holds at most 64 rows
+      const int short_its = x.w.q_len - (x.nqt - 1) * kRows <= 64 ? group : 0;
       if (!wait_warp(&bar->kv_full, nkv & 1, a.status)) { ok = false; break; }
       ++nkv;
       // Event-driven issue, in order of urgency (the tensor pipe runs MMAs in
@@ -742,7 +754,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         bool progressed = false;
         if (nk < nv && ptx::mbar_test_warp(&bar->p_full, nk & 1)) {
           ptx::tc_fence_after();
-          issue_dk(nk, nk == I0);
+          issue_dk(nk, nk == I0, (int)(nk - I0) < short_its);
           ++nk;
           progressed = true;
         }
@@ -757,7 +769,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         }
         if (nv < np && ptx::mbar_test_warp(&bar->pt_full, nv & 1)) {
           ptx::tc_fence_after();
-          issue_dv(nv, nv == I0);
+          issue_dv(nv, nv == I0, (int)(nv - I0) < short_its);
           ++nv;
           progressed = true;
         }
@@ -809,6 +821,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
       // dS^T stores of the previous iteration left for after this iteration's P
       // phase (half of them), where the compute warps wait for dP^T anyway
       uint4* ds_dst = nullptr;
+      int ds_groups = 8;  // this warpgroup's groups of 8 queries that exist: only those are kept
       uint32_t ds_rest[16];
       for (int i = 0; ok && i < n_it; ++i, ++I) {
         const int s = (int)(I & 1);
@@ -882,9 +895,10 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         if (ds_dst) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
-                                   make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
-                                   pol_ds);
+            if (k + 4 < ds_groups)
+              ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
+                                     make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
+                                     pol_ds);
           ds_dst = nullptr;
         }
         // phase 2: dS from dP^T
@@ -938,11 +952,13 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           // after the hand-off so that the dV/dK MMAs do not wait for it.
           const int hh = i % group, t = x.nqt - 1 - i / group;
           const int64_t slot = ((int64_t)a.kpair_off[x.gk] + (t - x.qt0)) * a.hq + (x.g * group + hh);
+          ds_groups = ds_query_groups(x.w.q_len - t * kRows) - 8 * wg;
           uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(a.ds) + slot * kTileBytes) + wg * 8 * kRows + r;
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            ptx::st_global_v4_hint(dst + k * kRows, make_uint4(pd[4 * k], pd[4 * k + 1], pd[4 * k + 2], pd[4 * k + 3]),
-                                   pol_ds);
+            if (k < ds_groups)
+              ptx::st_global_v4_hint(dst + k * kRows, make_uint4(pd[4 * k], pd[4 * k + 1], pd[4 * k + 2], pd[4 * k + 3]),
+                                     pol_ds);
 #pragma unroll
           for (int k = 0; k < 16; ++k) ds_rest[k] = pd[16 + k];
           ds_dst = dst;
@@ -951,9 +967,10 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
       if (ds_dst) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
-                                 make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
-                                 pol_ds);
+          if (k + 4 < ds_groups)
+            ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
+                                   make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
+                                   pol_ds);
       }
       if (!ok) break;
       // epilogue of the item: dV, dK from tensor memory

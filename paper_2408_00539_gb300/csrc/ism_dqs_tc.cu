@@ -98,6 +98,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t pol_ds = ptx::l2_policy_evict_first(), pol_k = ptx::l2_policy_evict_last();
     for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
       const Item x = decode(a, item);
+      // a sequence's last tile keeps only the query groups that exist (the rows
+      // of the accumulator past them are not stored): 24 dialogues of 32 heads,
+      // 16001 tokens 152 -> 147 us
+      const uint32_t ds_bytes = (uint32_t)ds_query_groups(x.w.q_len - x.t * kRows) * kIlvUnitRow;
       for (int c = 0; c < x.nkb; ++c, ++it) {
         const int s = (int)(it % kStages);
         if (__any_sync(0xffffffffu, aborted(&bar->abort))) { ok = false; break; }
@@ -111,9 +115,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int64_t slot = ((int64_t)a.kpair_off[gk] + (x.t - a.ktiles[gk].a0)) * a.hq + x.h;
           const int32_t yk = x.w.k_base + c * kRows;
           uint8_t* st = smem + s * kStageBytes;
-          ptx::mbar_expect_tx(&bar->full[s], kStageBytes);
-          ptx::bulk_load_hint(st, static_cast<const uint8_t*>(a.ds) + slot * kTileBytes, kTileBytes, &bar->full[s],
-                              pol_ds);
+          ptx::mbar_expect_tx(&bar->full[s], ds_bytes + kTileBytes);
+          ptx::bulk_load_hint(st, static_cast<const uint8_t*>(a.ds) + slot * kTileBytes, ds_bytes, &bar->full[s], pol_ds);
           ptx::tma_load_2d_hint(st + kTileBytes, &tmK, &bar->full[s], x.g * kD, yk, pol_k);
           ptx::tma_load_2d_hint(st + kTileBytes + kHalfBytes, &tmK, &bar->full[s], x.g * kD + 64, yk, pol_k);
         }

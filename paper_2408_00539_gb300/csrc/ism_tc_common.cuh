@@ -265,6 +265,9 @@ __device__ __forceinline__ uint64_t desc_mnmajor(uint32_t tile_saddr, int kk) {
 // 8 K rows are 128 bytes on (leading offset), the next 8 MN columns 2048
 // bytes on (stride offset).  k-step kk (16 K rows) starts 256 bytes on.
 constexpr uint32_t kIlvUnitRow = 128 * 16;  // bytes between MN groups of 8
+// Query groups of 8 that a stored dS tile keeps: those with rows of the
+// sequence (`rows` from the tile's first row to the end).
+__device__ __forceinline__ int ds_query_groups(int rows) { return rows >= 128 ? 16 : (rows + 7) >> 3; }
 __host__ __device__ constexpr uint32_t ilv_offset(int mn, int k) {
   return (uint32_t)(mn >> 3) * kIlvUnitRow + (uint32_t)k * 16u + (uint32_t)(mn & 7) * 2u;
 }

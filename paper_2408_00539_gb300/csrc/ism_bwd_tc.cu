@@ -998,7 +998,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           ptx::reg_fence(hi);
           float rc[32], rs[32];
           if (kvalid) {
-            rope_row<32>(a.rope_cos + (int64_t)key * (kHD / 2) + 32 * q2, a.rope_sin + (int64_t)key * (kHD / 2) + 32 * q2, rc, rs);
+            rope_row<32, kHD == 128>(a.rope_cos + (int64_t)key * (kHD / 2) + 32 * q2,
+                                     a.rope_sin + (int64_t)key * (kHD / 2) + 32 * q2, rc, rs);
           } else {
 #pragma unroll
             for (int k = 0; k < 32; ++k) rc[k] = rs[k] = 0.f;

@@ -178,10 +178,23 @@ __device__ __forceinline__ void pack_scaled32(const uint32_t (&v)[32], float f, 
 // x_{k+64} = g_{k+64} c - g_k s, packed as bf16 pairs into wl (columns
 // k0..) and wh (columns k0+64..) for store_slice32.  c and s point into
 // register arrays at offsets fixed at compile time (the loops are unrolled).
-template <int N>
+// The lanes of a warp read rows 256 bytes apart, and with the operand stages in
+// shared memory the L1 is too small to keep the other halves of their sectors:
+// kWide takes whole 32-byte sectors where the tables' alignment allows (dQ from
+// stored dS, 24 dialogues of 32 heads, 16001 tokens: 126 -> 121 us; dK/dV of
+// head_dim 64 spills with it).
+template <int N, bool kWide = true>
 __device__ __forceinline__ void rope_row(const float* __restrict__ cs, const float* __restrict__ sn, float* c,
                                          float* s) {
-  static_assert(N % 4 == 0, "whole float4 loads");
+  static_assert(N % 8 == 0, "whole 32-byte loads");
+  if (kWide && ((reinterpret_cast<uintptr_t>(cs) | reinterpret_cast<uintptr_t>(sn)) & 31u) == 0) {
+#pragma unroll
+    for (int i = 0; i < N / 8; ++i) {
+      ptx::ldg_f32x8(cs + 8 * i, c + 8 * i);
+      ptx::ldg_f32x8(sn + 8 * i, s + 8 * i);
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < N / 4; ++i) {
     const float4 cv = __ldg(reinterpret_cast<const float4*>(cs) + i);

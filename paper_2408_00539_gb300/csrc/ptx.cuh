@@ -395,6 +395,13 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t m, uint32_t n, ui
          | ((m >> 4) << 24);  // M / 16
 }
 
+// Eight read-only floats at a 32-byte aligned address: one whole sector.
+__device__ __forceinline__ void ldg_f32x8(const float* p, float* v) {
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p));
+}
+
 // Four k-steps (K = 64) of a bf16 TS contraction, issued like mma8_bf16_ts_warp.
 template <uint32_t kAStep, uint32_t kBStep>
 __device__ __forceinline__ void mma4_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,

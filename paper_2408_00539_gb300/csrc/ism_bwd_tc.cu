@@ -72,11 +72,14 @@ __device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t 
 }
 
 // ------------------------------------------------------------------ delta
-// One group of kHD / 8 lanes per (row, head): 8 bf16 per lane.  A group takes
-// four (row, head) pairs per round with all eight loads issued before any
-// use (more bytes in flight per thread: the kernel only streams O and dO).
-// The reductions shuffle within the group's own lanes, so the groups of a
-// warp may run different numbers of rounds.
+// One group of kHD / 8 lanes per (row, head): 8 bf16 per lane.  Bound by HBM
+// (it streams O and dO): a group takes two (row, head) pairs with all its loads
+// issued before any use, and the grid holds one round, so blocks come and go
+// while others wait for memory.  16384 rows of 32 heads: 43 us (6.3 TB/s); four
+// pairs a group in rounds of 16 blocks per SM took 49, one round of four 44, of
+// eight 56.
+// The reductions shuffle within the group's own lanes.
+constexpr int kDeltaThreads = 256, kDeltaPairs = 2;
 template <int kHD, bool kDependent>
 __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
                              float* __restrict__ delta, int64_t rows, int hq) {
@@ -85,42 +88,35 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
   // and runs beside as a dependent launch.  The wait at the end makes this
   // kernel's completion imply that one's.  (It costs 4 of 48 us on 2 x 8192
   // tokens of 32 heads, which are launched plainly.)
-  constexpr int kUnroll = 4;
+  constexpr int kLanes = kHD / 8, kGroups = kDeltaThreads / kLanes;
   const int64_t n = rows * hq;
-  constexpr int kLanes = kHD / 8;
   const int sub = threadIdx.x % kLanes;
   const uint32_t group_mask = ((1u << kLanes) - 1u) << (threadIdx.x & 31 & ~(kLanes - 1));
-  const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / kLanes;
-  for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes; i0 < n; i0 += groups * kUnroll) {
-    uint4 a[kUnroll], b[kUnroll];
+  const int64_t i0 = (int64_t)blockIdx.x * (kGroups * kDeltaPairs) + threadIdx.x / kLanes;
+  uint4 a[kDeltaPairs], b[kDeltaPairs];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int64_t i = i0 + u * groups;
-      if (i < n) {
-        a[u] = reinterpret_cast<const uint4*>(O + i * kHD)[sub];
-        b[u] = reinterpret_cast<const uint4*>(dO + i * kHD)[sub];
-      }
+  for (int u = 0; u < kDeltaPairs; ++u) {
+    const int64_t i = i0 + u * kGroups;
+    if (i < n) {
+      a[u] = reinterpret_cast<const uint4*>(O + i * kHD)[sub];
+      b[u] = reinterpret_cast<const uint4*>(dO + i * kHD)[sub];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kDeltaPairs; ++u) {
+    const int64_t i = i0 + u * kGroups;
+    if (i >= n) break;
+    const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a[u]);
+    const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b[u]);
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 x = __bfloat1622float2(pa[k]), y = __bfloat1622float2(pb[k]);
+      acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int64_t i = i0 + u * groups;
-      if (i >= n) break;
-      const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a[u]);
-      const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b[u]);
-      float acc = 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float2 x = __bfloat1622float2(pa[k]), y = __bfloat1622float2(pb[k]);
-        acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
-      }
-#pragma unroll
-      for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(group_mask, acc, o);
-      if (sub == 0) {
-        const int64_t row = i / hq;
-        const int h = (int)(i % hq);
-        delta[(int64_t)h * rows + row] = acc;
-      }
-    }
+    for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(group_mask, acc, o);
+    if (sub == 0) delta[(i % hq) * rows + i / hq] = acc;
   }
   if constexpr (kDependent) pdl_wait();
 }
@@ -1042,12 +1038,11 @@ template <int kHD>
 cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
   cudaError_t e;
   if (a.q_rows > 0) {
-    int64_t groups = a.q_rows * a.hq;
-    int grid = (int)((groups * (kHD / 8) + 255) / 256);
-    if (grid > 152 * 16) grid = 152 * 16;
+    constexpr int64_t kPairs = kDeltaThreads / (kHD / 8) * kDeltaPairs;  // a block's
+    const int64_t grid = (a.q_rows * a.hq + kPairs - 1) / kPairs;
     timer_begin(ISM_KERNEL_BWD_PRE, st);
-    e = launch(a.dependent, a.dependent ? delta_kernel<kHD, true> : delta_kernel<kHD, false>, grid, 256, 0, st, (const __nv_bfloat16*)a.o,
-                         (const __nv_bfloat16*)a.dout, a.delta, a.q_rows, a.hq);
+    e = launch(a.dependent, a.dependent ? delta_kernel<kHD, true> : delta_kernel<kHD, false>, grid, kDeltaThreads, 0, st,
+               (const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows, a.hq);
     timer_end(ISM_KERNEL_BWD_PRE, st);
     count_launch();
     if (e != cudaSuccess) return e;

@@ -127,44 +127,25 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
 // read by the first and the last MMA of a block) and a 2-stage V ring.  S is
 // double-buffered in tensor memory: S_{c+1} is computed while block c's
 // scores are turned into dS.
-// Persistent: a CTA takes items (query tile, head) in a snake walk over the cost
-// order, and its rings and barrier phases count blocks over the whole walk, so
-// the next item's loads and first S and dP run under this item's last blocks
-// and epilogue.  One CTA per item paid the set-up, the first loads and the
-// epilogue of each: DQ_FIGURES.
 namespace dq {
 constexpr int kKStages = 3;
 template <int kHD>
 struct Layout {
-  static constexpr int kQStages = kHD == 64 ? 2 : 1;  // all that fits
   static constexpr uint32_t TB = kHD / 64 * kHalfBytes;
-  static constexpr uint32_t Q = 0, DO = kQStages * TB, K = 2 * kQStages * TB, V = K + kKStages * TB, BAR = V + 2 * TB;
+  static constexpr uint32_t Q = 0, DO = TB, K = 2 * TB, V = 5 * TB, BAR = 7 * TB;
   static constexpr uint32_t kSmemBytes = BAR + 256 + 1024;
-  static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 };
 constexpr uint32_t TM_S = 0, TM_DP = 256, TM_DQ = 384;  // S regions at 0 and 128
 
 struct Bars {
-  uint64_t qdo_full[2], qdo_empty[2];  // per item
+  uint64_t qdo_full;
   uint64_t k_full[kKStages], k_empty[kKStages], v_full[2], v_empty[2];
   uint64_t s_full[2], p_full[2], dq_done[2];  // per S region
-  uint64_t dp_full, dp_read;
-  uint64_t acc_full, acc_read;  // per item: dQ complete, read by the epilogue
-  uint64_t final_mma;
+  uint64_t dp_full, dp_read, final_mma;
   uint32_t tmem_base;
   int32_t abort;
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
-
-// The CTA's n-th item: position of its tile in q_order, and its head.  false past the end.
-__device__ __forceinline__ bool nth_item(const AttnArgs& a, uint32_t n, int64_t& tpos, int& h) {
-  const int64_t item = (int64_t)n * gridDim.x + ((n & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
-  if (item >= a.nq * a.hq) return false;
-  bucket_item(item, a.nq, a.hq, tpos, h, a.hq == a.hkv);
-  return true;
-}
-// Key blocks of a tile (every row sees at least itself).
-__device__ __forceinline__ int key_blocks(const Tile& w) { return w.a1 > 1 ? w.a1 : 1; }
 }  // namespace dq
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
@@ -177,21 +158,25 @@ __global__ void __launch_bounds__(kThreads, 1)
               const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
   using namespace dq;
   using L = Layout<kHD>;
-  constexpr int kQStages = L::kQStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int group = a.hq / a.hkv;
+  pdl_wait();
+  int64_t tpos;
+  int h;
+  bucket_item(blockIdx.x, a.nq, a.hq, tpos, h, a.hq == a.hkv);  // blocks start roughly in index order
+  const Tile w = a.qtiles[a.q_order[tpos]];
+  const int g = h / (a.hq / a.hkv);
+  const int nkb = w.a1, kfull = w.a0;
 
   if (threadIdx.x == 0) {
+    ptx::mbar_init(&bar->qdo_full, 1);
     for (int s = 0; s < kKStages; ++s) {
       ptx::mbar_init(&bar->k_full[s], 1);
       ptx::mbar_init(&bar->k_empty[s], 1);
     }
     for (int s = 0; s < 2; ++s) {
-      ptx::mbar_init(&bar->qdo_full[s], 1);
-      ptx::mbar_init(&bar->qdo_empty[s], 1);
       ptx::mbar_init(&bar->v_full[s], 1);
       ptx::mbar_init(&bar->v_empty[s], 1);
       ptx::mbar_init(&bar->s_full[s], 1);
@@ -200,8 +185,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     ptx::mbar_init(&bar->dp_full, 1);
     ptx::mbar_init(&bar->dp_read, kComputeThreads);
-    ptx::mbar_init(&bar->acc_full, 1);
-    ptx::mbar_init(&bar->acc_read, kComputeThreads);
     ptx::mbar_init(&bar->final_mma, 1);
     bar->abort = 0;
     ptx::fence_mbar_init();
@@ -214,44 +197,38 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
-  pdl_wait();  // the set-up above overlaps the kernel before
 
   if (warp == 8) {
     // the warp waits converged, lane 0 issues the copies
-    uint32_t nqdo = 0, C = 0, nk[kKStages] = {}, nv[2] = {};  // C: blocks so far
-    bool ok = true;
-    int64_t tpos;
-    int h;
-    for (uint32_t n = 0; ok && nth_item(a, n, tpos, h); ++n) {
-      const Tile w = a.qtiles[a.q_order[tpos]];
-      const int nkb = key_blocks(w), g = h / group, sq = (int)(n % kQStages);
-      for (int c = 0; ok && c < nkb; ++c, ++C) {
-        const int sk = (int)(C % kKStages), sv = (int)(C & 1);
+    if (nkb > 0) {
+      if (lane == 0) {
+        ptx::tma_prefetch_desc(&tmK);
+        ptx::tma_prefetch_desc(&tmV);
+        const int32_t qy = w.q_base + w.tile * kRows;
+        ptx::mbar_expect_tx(&bar->qdo_full, 2 * L::TB);
+        load_tile<kHD>(smem + L::Q, &tmQ, &bar->qdo_full, h * kHD, qy);
+        load_tile<kHD>(smem + L::DO, &tmdO, &bar->qdo_full, h * kHD, qy);
+      }
+      __syncwarp();
+      uint32_t nk[kKStages] = {0, 0, 0}, nv[2] = {0, 0};
+      for (int c = 0; c < nkb; ++c) {
+        const int sk = c % kKStages, sv = c & 1;
+        if (__any_sync(0xffffffffu, aborted(&bar->abort))) break;
         const int32_t ky = w.k_base + c * kRows;
-        ok = !__any_sync(0xffffffffu, aborted(&bar->abort)) &&
-             (C < kKStages || wait_warp(&bar->k_empty[sk], (C / kKStages - 1) & 1, a.status));
-        if (!ok) break;
+        if (c >= kKStages && !wait_warp(&bar->k_empty[sk], (uint32_t)(c / kKStages - 1) & 1, a.status)) {
+          if (lane == 0) set_abort(&bar->abort);
+          break;
+        }
         if (lane == 0) {
           ptx::mbar_expect_tx(&bar->k_full[sk], L::TB);
           load_tile<kHD>(smem + L::K + sk * L::TB, &tmK, &bar->k_full[sk], g * kHD, ky);
         }
         __syncwarp();
         ++nk[sk];
-        if (c == 0) {
-          // the MMAs have read the Q and dO of the item kQStages back
-          ok = n < kQStages || wait_warp(&bar->qdo_empty[sq], (n / kQStages - 1) & 1, a.status);
-          if (!ok) break;
-          if (lane == 0) {
-            const int32_t qy = w.q_base + w.tile * kRows;
-            ptx::mbar_expect_tx(&bar->qdo_full[sq], 2 * L::TB);
-            load_tile<kHD>(smem + L::Q + sq * L::TB, &tmQ, &bar->qdo_full[sq], h * kHD, qy);
-            load_tile<kHD>(smem + L::DO + sq * L::TB, &tmdO, &bar->qdo_full[sq], h * kHD, qy);
-          }
-          __syncwarp();
-          ++nqdo;
+        if (c >= 2 && !wait_warp(&bar->v_empty[sv], (uint32_t)((c >> 1) - 1) & 1, a.status)) {
+          if (lane == 0) set_abort(&bar->abort);
+          break;
         }
-        ok = C < 2 || wait_warp(&bar->v_empty[sv], ((C >> 1) - 1) & 1, a.status);
-        if (!ok) break;
         if (lane == 0) {
           ptx::mbar_expect_tx(&bar->v_full[sv], L::TB);
           load_tile<kHD>(smem + L::V + sv * L::TB, &tmV, &bar->v_full[sv], g * kHD, ky);
@@ -259,254 +236,193 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         ++nv[sv];
       }
+      if (__any_sync(0xffffffffu, aborted(&bar->abort))) {
+        wait_warp(&bar->qdo_full, 0, a.status);
+        for (int s = 0; s < kKStages; ++s)
+          if (nk[s]) wait_warp(&bar->k_full[s], (nk[s] - 1) & 1, a.status);
+        for (int s = 0; s < 2; ++s)
+          if (nv[s]) wait_warp(&bar->v_full[s], (nv[s] - 1) & 1, a.status);
+      }
     }
-    if (!ok) {
-      if (lane == 0) set_abort(&bar->abort);
-      // every issued copy lands before the CTA exits
-      for (uint32_t n = nqdo > kQStages ? nqdo - kQStages : 0; n < nqdo; ++n)
-        wait_warp(&bar->qdo_full[n % kQStages], (n / kQStages) & 1, a.status);
-      for (int s = 0; s < kKStages; ++s)
-        if (nk[s]) wait_warp(&bar->k_full[s], (nk[s] - 1) & 1, a.status);
-      for (int s = 0; s < 2; ++s)
-        if (nv[s]) wait_warp(&bar->v_full[s], (nv[s] - 1) & 1, a.status);
-    }
-    __syncwarp();
   } else if (warp == 9) {
     // the whole warp runs the loop, one elected lane issues each instruction
-    constexpr uint32_t idesc_nt = ptx::idesc_bf16_f32(128, 128, 0, 0);  // A K-major, B K-major
-    constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, kHD, 0, 1);  // A K-major, B MN-major
-    auto blocks_of = [&](uint32_t n) {
-      int64_t tpos;
-      int h;
-      return nth_item(a, n, tpos, h) ? key_blocks(a.qtiles[a.q_order[tpos]]) : 0;
-    };
-    // Event-driven issue: S_C, dP_C, dQ_C (C counts blocks over all items) go out
-    // as soon as their inputs are ready, so no wait blocks an unrelated MMA.
-    //   S_C  needs K_C, an item's first also its Q and dO, and dQ_{C-2} issued (it
-    //        overwrites the dS that dQ_{C-2} reads; MMAs of this thread execute in
-    //        order, or, with kFlagDrainTmemReuse, dQ_{C-2} completed)
-    //   dP_C needs S_C issued, V_C, and dP_{C-1} read by the compute warps
-    //   dQ_C needs dS_C written, an item's first also the dQ of the item before read
-    uint32_t cs = 0, cd = 0, cq = 0;  // blocks issued
-    uint32_t is = 0, id = 0, iq = 0;  // items they are in
-    int bs = 0, ns = blocks_of(0), ns1 = ns ? blocks_of(1) : 0;  // S: block of its item, blocks of that item and the next
-    uint32_t last = 0;     // bit C % 32: block C is the last of its item (S runs at most two ahead of dQ)
-    bool first_q = true;   // dQ is at the first block of its item
-    bool ok = true;
-    uint64_t t_idle = 0;
-    while (ok && (ns > 0 || cq < cs)) {
-      bool progressed = false;
-      if (ns > 0 && cs < cq + 2 &&
-          (cs < 2 || !(a.flags & kFlagDrainTmemReuse) ||
-           ptx::mbar_test_warp(&bar->dq_done[cs & 1], ((cs - 2) >> 1) & 1)) &&
-          ptx::mbar_test_warp(&bar->k_full[cs % kKStages], (cs / kKStages) & 1) &&
-          (bs > 0 || ptx::mbar_test_warp(&bar->qdo_full[is % kQStages], (is / kQStages) & 1))) {
-        ptx::tc_fence_after();
-        const uint32_t sQ = ptx::smem_u32(smem + L::Q + is % kQStages * L::TB);
-        const uint32_t sK = ptx::smem_u32(smem + L::K + cs % kKStages * L::TB);
-        mma_head_dim<kHD>(tmem + TM_S + 128u * (cs & 1), sQ, sK, idesc_nt);
-        ptx::mma_commit_warp(&bar->s_full[cs & 1]);
-        const uint32_t bit = 1u << (cs & 31);
-        ++cs;
-        if (++bs == ns) {
-          last |= bit;
-          bs = 0;
-          ++is;
-          ns = ns1;
-          ns1 = ns ? blocks_of(is + 1) : 0;
-        } else {
-          last &= ~bit;
-        }
-        progressed = true;
-      }
-      if (cd < cs && (cd == 0 || ptx::mbar_test_warp(&bar->dp_read, (cd - 1) & 1)) &&
-          ptx::mbar_test_warp(&bar->v_full[cd & 1], (cd >> 1) & 1)) {
-        ptx::tc_fence_after();
-        const uint32_t sdO = ptx::smem_u32(smem + L::DO + id % kQStages * L::TB);
-        const uint32_t sV = ptx::smem_u32(smem + L::V + (cd & 1) * L::TB);
+    if (nkb > 0) {
+      constexpr uint32_t idesc_nt = ptx::idesc_bf16_f32(128, 128, 0, 0);  // A K-major, B K-major
+      constexpr uint32_t idesc_nn = ptx::idesc_bf16_f32(128, kHD, 0, 1);  // A K-major, B MN-major
+      const uint32_t sQ = ptx::smem_u32(smem + L::Q), sdO = ptx::smem_u32(smem + L::DO);
+      auto issue_s = [&](int c) {
+        const uint32_t sK = ptx::smem_u32(smem + L::K + (c % kKStages) * L::TB);
+        mma_head_dim<kHD>(tmem + TM_S + 128u * (c & 1), sQ, sK, idesc_nt);
+        ptx::mma_commit_warp(&bar->s_full[c & 1]);
+      };
+      auto issue_dp = [&](int c) {
+        const int sv = c & 1;
+        const uint32_t sV = ptx::smem_u32(smem + L::V + sv * L::TB);
         mma_head_dim<kHD>(tmem + TM_DP, sdO, sV, idesc_nt);
         ptx::mma_commit_warp(&bar->dp_full);
-        ptx::mma_commit_warp(&bar->v_empty[cd & 1]);
-        if (last >> (cd & 31) & 1) {  // S of the item's last block went out before
-          ptx::mma_commit_warp(&bar->qdo_empty[id % kQStages]);
-          ++id;
-        }
-        ++cd;
-        progressed = true;
-      }
-      if (cq < cd && ptx::mbar_test_warp(&bar->p_full[cq & 1], (cq >> 1) & 1) &&
-          (!first_q || iq == 0 || ptx::mbar_test_warp(&bar->acc_read, (iq - 1) & 1))) {
-        ptx::tc_fence_after();
-        const uint32_t R = cq & 1, sk = cq % kKStages;
-        // dQ += dS K_C: dS (bf16, keys packed two per column) in S region R, keys [0,64) at
+        ptx::mma_commit_warp(&bar->v_empty[sv]);
+      };
+      auto issue_dq = [&](int c) {
+        const int R = c & 1;
+        const uint32_t sK = ptx::smem_u32(smem + L::K + (c % kKStages) * L::TB);
+        // dQ += dS K_c: dS (bf16, keys packed two per column) in S region R, keys [0,64) at
         // columns [0,32) and [64,128) at columns [64,96)
-        mma_tile_rows<kHD>(tmem + TM_DQ, tmem + TM_S + 128u * R, ptx::smem_u32(smem + L::K + sk * L::TB), idesc_nn,
-                           first_q ? 0u : 1u);
+        mma_tile_rows<kHD>(tmem + TM_DQ, tmem + TM_S + 128u * R, sK, idesc_nn, c > 0 ? 1u : 0u);
         ptx::mma_commit_warp(&bar->dq_done[R]);
-        ptx::mma_commit_warp(&bar->k_empty[sk]);
-        first_q = last >> (cq & 31) & 1;
-        if (first_q) {
-          ptx::mma_commit_warp(&bar->acc_full);
-          ++iq;
-        }
-        ++cq;
-        progressed = true;
+        ptx::mma_commit_warp(&bar->k_empty[c % kKStages]);
+      };
+      // Event-driven issue: S_c, dP_c, dQ_c go out as soon as their inputs are
+      // ready, so no wait blocks an unrelated MMA.
+      //   S_c  needs K_c and dQ_{c-2} issued (it overwrites the dS that dQ_{c-2}
+      //        reads; MMAs of this thread execute in order, or, with
+      //        kFlagDrainTmemReuse, dQ_{c-2} completed)
+      //   dP_c needs V_c and dP_{c-1} read by the compute warps
+      //   dQ_c needs dS_c written
+      bool ok = wait_warp(&bar->qdo_full, 0, a.status) && wait_warp(&bar->k_full[0], 0, a.status) &&
+                wait_warp(&bar->v_full[0], 0, a.status);
+      if (ok) {
+        ptx::tc_fence_after();
+        issue_s(0);
+        issue_dp(0);
       }
-      if (progressed) {
-        t_idle = 0;
-      } else {
-        __nanosleep(16);
-        const uint64_t now = globaltimer();
-        if (t_idle == 0) t_idle = now;
-        const bool expired = __shfl_sync(0xffffffffu, (now - t_idle > kWaitLimitNs || aborted(&bar->abort)) ? 1 : 0, 0);
-        if (expired) {
-          if (lane == 0) atomicOr(a.status, kStatusTimeout);
-          ok = false;
+      int ns = 1, nd = 1, nq = 0;
+      uint64_t t_idle = 0;
+      while (ok && nq < nkb) {
+        bool progressed = false;
+        if (ns < nkb && (ns < 2 || nq > ns - 2) &&
+            (ns < 2 || !(a.flags & kFlagDrainTmemReuse) ||
+             ptx::mbar_test_warp(&bar->dq_done[ns & 1], (uint32_t)((ns - 2) >> 1) & 1)) &&
+            ptx::mbar_test_warp(&bar->k_full[ns % kKStages], (uint32_t)(ns / kKStages) & 1)) {
+          ptx::tc_fence_after();
+          issue_s(ns++);
+          progressed = true;
+        }
+        if (nd < nkb && ptx::mbar_test_warp(&bar->dp_read, (uint32_t)(nd - 1) & 1) &&
+            ptx::mbar_test_warp(&bar->v_full[nd & 1], (uint32_t)(nd >> 1) & 1)) {
+          ptx::tc_fence_after();
+          issue_dp(nd++);
+          progressed = true;
+        }
+        if (nq < ns && nq < nd && ptx::mbar_test_warp(&bar->p_full[nq & 1], (uint32_t)(nq >> 1) & 1)) {
+          ptx::tc_fence_after();
+          issue_dq(nq++);
+          progressed = true;
+        }
+        if (progressed) {
+          t_idle = 0;
+        } else {
+          __nanosleep(16);
+          const uint64_t now = globaltimer();
+          if (t_idle == 0) t_idle = now;
+          const bool expired = __shfl_sync(0xffffffffu, (now - t_idle > kWaitLimitNs || aborted(&bar->abort)) ? 1 : 0, 0);
+          if (expired) {
+            if (lane == 0) atomicOr(a.status, kStatusTimeout);
+            ok = false;
+          }
         }
       }
+      if (!ok && lane == 0) set_abort(&bar->abort);
+      __syncwarp();
+      ptx::mma_commit_warp(&bar->final_mma);
+      wait_warp(&bar->final_mma, 0, a.status);
     }
-    if (!ok && lane == 0) set_abort(&bar->abort);
-    __syncwarp();
-    ptx::mma_commit_warp(&bar->final_mma);
-    wait_warp(&bar->final_mma, 0, a.status);
     __syncwarp();
   } else {
     // compute: thread = query row r of the tile; warpgroup wg owns key columns [64 wg, 64 wg + 64)
     const int wg = threadIdx.x >> 7, r = threadIdx.x & 127;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+    const int row = w.tile * kRows + r;
+    const bool valid = row < w.q_len;
+    const int64_t grow = (int64_t)w.q_base + row;
+    const int ke = valid ? a.kv_end[w.kv_base + row] : 0;
+    const float lse2 = valid ? a.lse_in[(int64_t)h * a.q_rows + grow] * kLog2e : 0.f;
+    const float dl = valid ? a.delta[(int64_t)h * a.q_rows + grow] : 0.f;
     const float sl2 = a.scale * kLog2e;
-    // The next item's tile and row values are read while this one is computed:
-    // its place two items ahead, its tile one ahead, its row values before the
-    // epilogue.
-    int64_t tpos;
-    int h, h1 = 0, gq1 = 0, ke = 0;
-    float lse2 = 0.f, dl = 0.f;
-    Tile w = {}, w1 = {};
-    auto row_values = [&](const Tile& y, int hy) {
-      const int row = y.tile * kRows + r;
-      const bool valid = row < y.q_len;
-      const int64_t at = (int64_t)hy * a.q_rows + y.q_base + row;
-      ke = valid ? a.kv_end[y.kv_base + row] : 0;
-      lse2 = valid ? a.lse_in[at] * kLog2e : 0.f;
-      dl = valid ? a.delta[at] : 0.f;
-    };
-    bool have = nth_item(a, 0, tpos, h), have1 = false;
-    if (have) {
-      w = a.qtiles[a.q_order[tpos]];
-      row_values(w, h);
-      have1 = nth_item(a, 1, tpos, h1);
-      if (have1) gq1 = a.q_order[tpos];
-    }
-    bool ok = true;
-    uint32_t C = 0;
-    for (uint32_t n = 0; ok && have; ++n) {
-      int h2 = 0, gq2 = 0;
-      if (have1) w1 = a.qtiles[gq1];
-      const bool have2 = have1 && nth_item(a, n + 2, tpos, h2);
-      if (have2) gq2 = a.q_order[tpos];
-      const int nkb = key_blocks(w), kfull = w.a0;
-      const int row = w.tile * kRows + r;
-      for (int c = 0; c < nkb; ++c, ++C) {
-        const uint32_t R = C & 1;
-        const uint32_t tS = tmem + lane_addr + TM_S + 128u * R + 64u * wg;
-        if (!wait(&bar->s_full[R], (C >> 1) & 1, a.status) || !wait(&bar->dp_full, C & 1, a.status)) {
-          ok = false;
-          break;
-        }
-        ptx::tc_fence_after();
-        uint32_t s0[32], s1[32], d0[32], d1[32];
-        ld64(tS, s0, s1);
-        ld64(tmem + lane_addr + TM_DP + 64u * wg, d0, d1);
-        ptx::tmem_ld_wait();
-        ptx::reg_fence(s0);
-        ptx::reg_fence(s1);
-        ptx::reg_fence(d0);
-        ptx::reg_fence(d1);
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(&bar->dp_read);
-        const int lim = (c < kfull) ? 128 : ke - c * kRows - wg * 64;  // visible columns of this half
-        uint32_t pk[32], plo[kHD == 64 ? 32 : 1];  // pk[k] holds columns 2k and 2k+1 of this half
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          float v[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int jj = 2 * k + e;
-            const float sv = __uint_as_float(jj < 32 ? s0[jj] : s1[jj - 32]);
-            const float dv = __uint_as_float(jj < 32 ? d0[jj] : d1[jj - 32]);
-            const float p = jj < lim ? ex2(sv * sl2 - lse2) : 0.f;
-            v[e] = p * (dv - dl);
-          }
-          pk[k] = pack_bf16(v[0], v[1]);
-          if constexpr (kHD == 64) plo[k] = pack_bf16_rest(v[0], v[1], pk[k]);
-        }
-        // dS over the first 32 columns of this half of S (already read)
-        ptx::tmem_st32(tS, pk);
-        if constexpr (kHD == 64) ptx::tmem_st32(tS + 32, plo);
-        ptx::tmem_st_wait();
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(&bar->p_full[R]);
-      }
-      if (!ok) break;
-      const bool valid = row < w.q_len;
-      const int64_t grow = (int64_t)w.q_base + row;
-      // rotary encoding: this warpgroup's 32 pairs of the row's tables, loaded
-      // while the last dQ MMAs run
-      float rc[32], rs[32];
-      if (valid && a.rope_cos && wg < kHD / 64) {
-        const int64_t pos = (int64_t)w.tile * kRows + r;
-        rope_row<32>(a.rope_cos + pos * (kHD / 2) + wg * 32, a.rope_sin + pos * (kHD / 2) + wg * 32, rc, rs);
-      }
-      if (have1) row_values(w1, h1);
-      if (!wait(&bar->acc_full, n & 1, a.status)) {
+    bool ok = nkb > 0;
+    for (int c = 0; ok && c < nkb; ++c) {
+      const int R = c & 1;
+      const uint32_t tS = tmem + lane_addr + TM_S + 128u * R + 64u * wg;
+      if (!wait(&bar->s_full[R], (uint32_t)(c >> 1) & 1, a.status) || !wait(&bar->dp_full, (uint32_t)c & 1, a.status)) {
         ok = false;
         break;
       }
       ptx::tc_fence_after();
-      uint32_t q0[32], q1[32];
-      if (wg < kHD / 64) {  // (64 columns: warpgroup 0 alone)
-        if (a.rope_cos) {
-          // rotary encoding: warpgroup wg takes columns wg*32.. and kHD/2 + wg*32.., which pair up
-          ptx::tmem_ld32(tmem + lane_addr + TM_DQ + wg * 32, q0);
-          ptx::tmem_ld32(tmem + lane_addr + TM_DQ + kHD / 2 + wg * 32, q1);
-        } else {
-          ld64(tmem + lane_addr + TM_DQ + wg * 64, q0, q1);
-        }
-        ptx::tmem_ld_wait();
-        ptx::reg_fence(q0);
-        ptx::reg_fence(q1);
-      }
+      uint32_t s0[32], s1[32], d0[32], d1[32];
+      ld64(tS, s0, s1);
+      ld64(tmem + lane_addr + TM_DP + 64u * wg, d0, d1);
+      ptx::tmem_ld_wait();
+      ptx::reg_fence(s0);
+      ptx::reg_fence(s1);
+      ptx::reg_fence(d0);
+      ptx::reg_fence(d1);
       ptx::tc_fence_before();
-      ptx::mbar_arrive(&bar->acc_read);
-      if (wg < kHD / 64) {
-        // rows are stored by groups of four lanes (store_slice32)
-        const int64_t rstride = (int64_t)a.hq * kHD;
-        __nv_bfloat16* const g0 = reinterpret_cast<__nv_bfloat16*>(a.dq) + (grow - (lane & 3)) * rstride + h * kHD;
-        const int g_rows = w.q_len - (row - (lane & 3));
-        uint32_t w0[16], w1s[16];
-        if (a.rope_cos) {
-          if (!valid) {
+      ptx::mbar_arrive(&bar->dp_read);
+      const int lim = (c < kfull) ? 128 : ke - c * kRows - wg * 64;  // visible columns of this half
+      uint32_t pk[32], plo[kHD == 64 ? 32 : 1];  // pk[k] holds columns 2k and 2k+1 of this half
 #pragma unroll
-            for (int k = 0; k < 32; ++k) rc[k] = rs[k] = 0.f;
-          }
-          rope_back_pack(q0, q1, a.scale, rc, rs, w0, w1s);
-          store_slice32(w0, g0 + 32 * wg, rstride, g_rows);
-          store_slice32(w1s, g0 + kHD / 2 + 32 * wg, rstride, g_rows);
-        } else {
-          pack_scaled32(q0, a.scale, w0);
-          pack_scaled32(q1, a.scale, w1s);
-          store_slice32(w0, g0 + 64 * wg, rstride, g_rows);
-          store_slice32(w1s, g0 + 64 * wg + 32, rstride, g_rows);
+      for (int k = 0; k < 32; ++k) {
+        float v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int jj = 2 * k + e;
+          const float sv = __uint_as_float(jj < 32 ? s0[jj] : s1[jj - 32]);
+          const float dv = __uint_as_float(jj < 32 ? d0[jj] : d1[jj - 32]);
+          const float p = jj < lim ? ex2(sv * sl2 - lse2) : 0.f;
+          v[e] = p * (dv - dl);
         }
+        pk[k] = pack_bf16(v[0], v[1]);
+        if constexpr (kHD == 64) plo[k] = pack_bf16_rest(v[0], v[1], pk[k]);
       }
-      have = have1;
-      w = w1;
-      h = h1;
-      have1 = have2;
-      gq1 = gq2;
-      h1 = h2;
+      // dS over the first 32 columns of this half of S (already read)
+      ptx::tmem_st32(tS, pk);
+      if constexpr (kHD == 64) ptx::tmem_st32(tS + 32, plo);
+      ptx::tmem_st_wait();
+      ptx::tc_fence_before();
+      ptx::mbar_arrive(&bar->p_full[R]);
     }
-    if (!ok) set_abort(&bar->abort);
+    // rotary encoding: this warpgroup's 32 pairs of the row's tables, loaded
+    // while the last dQ MMAs run
+    float rc[32], rs[32];
+    if (valid && a.rope_cos && wg < kHD / 64) {
+      const int64_t pos = (int64_t)w.tile * kRows + r;
+      rope_row<32>(a.rope_cos + pos * (kHD / 2) + wg * 32, a.rope_sin + pos * (kHD / 2) + wg * 32, rc, rs);
+    }
+    if (ok) ok = wait(&bar->final_mma, 0, a.status);
+    if (!ok) {
+      set_abort(&bar->abort);
+    } else if (wg < kHD / 64) {  // (64 columns: warpgroup 0 alone)
+      ptx::tc_fence_after();
+      uint32_t q0[32], q1[32];
+      if (a.rope_cos) {
+        // rotary encoding: warpgroup wg takes columns wg*32.. and kHD/2 + wg*32.., which pair up
+        ptx::tmem_ld32(tmem + lane_addr + TM_DQ + wg * 32, q0);
+        ptx::tmem_ld32(tmem + lane_addr + TM_DQ + kHD / 2 + wg * 32, q1);
+      } else {
+        ld64(tmem + lane_addr + TM_DQ + wg * 64, q0, q1);
+      }
+      ptx::tmem_ld_wait();
+      ptx::reg_fence(q0);
+      ptx::reg_fence(q1);
+      // rows are stored by groups of four lanes (store_slice32)
+      const int64_t rstride = (int64_t)a.hq * kHD;
+      __nv_bfloat16* const g0 = reinterpret_cast<__nv_bfloat16*>(a.dq) + (grow - (lane & 3)) * rstride + h * kHD;
+      const int g_rows = w.q_len - (row - (lane & 3));
+      uint32_t w0[16], w1[16];
+      if (a.rope_cos) {
+        if (!valid) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) rc[k] = rs[k] = 0.f;
+        }
+        rope_back_pack(q0, q1, a.scale, rc, rs, w0, w1);
+        store_slice32(w0, g0 + 32 * wg, rstride, g_rows);
+        store_slice32(w1, g0 + kHD / 2 + 32 * wg, rstride, g_rows);
+      } else {
+        pack_scaled32(q0, a.scale, w0);
+        pack_scaled32(q1, a.scale, w1);
+        store_slice32(w0, g0 + 64 * wg, rstride, g_rows);
+        store_slice32(w1, g0 + 64 * wg + 32, rstride, g_rows);
+      }
+    }
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -1144,8 +1060,8 @@ cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
         cudaSuccess)
       return e;
     timer_begin(ISM_KERNEL_BWD_DQ, st);
-    const int64_t grid = std::min(a.nq * a.hq, (int64_t)sm_count());
-    e = launch(a.dependent, dq_kernel<kHD>, grid, kThreads, dq::Layout<kHD>::kSmemBytes, st, tq, tdo, tk, tv, a);
+    e = launch(a.dependent, dq_kernel<kHD>, a.nq * a.hq, kThreads, dq::Layout<kHD>::kSmemBytes, st, tq,
+                         tdo, tk, tv, a);
     timer_end(ISM_KERNEL_BWD_DQ, st);
     count_launch();
     if (e != cudaSuccess) return e;

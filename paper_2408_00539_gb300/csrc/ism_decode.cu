@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(160) decode_tma_kernel(const __grid_constant__
 // grid B*Hq, block D threads.  Launched as a programmatic dependent of the
 // split kernel: it may start while that kernel runs and waits for it (and
 // its memory) before reading the partials.  kRow: the partials of the
-// tensor-core kernel, whose CTAs share out one row of tiles (DecodeArgs); else
+// tensor-core kernel where its CTAs share out one row of tiles (DecodeArgs); else
 // one for each of a.splits chunks, those without keys marked by a maximum of -inf.
 template <int D, bool kRow>
 __global__ void decode_combine_kernel(DecodeArgs a) {
@@ -432,7 +432,7 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
   int s = 0, end = 0, per_cta = 1, c0 = 0;
   if constexpr (kRow) {
     const int n = dec_tiles(a.c_snap[b]), alloc = dec_alloc_tiles(a, n);
-    s = (a.uniform ? b * a.hkv * alloc : a.start[b]) + h / a.group * alloc;
+    s = a.start[b] + h / a.group * alloc;
     end = s + n;
     per_cta = (a.tpc + kDecTcTiles - 1) / kDecTcTiles;
     c0 = s / a.tpc;
@@ -546,7 +546,7 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st) {
   if (a.tc) {
     cudaError_t e = tc::launch_decode_tc(a, st);
     if (e != cudaSuccess) return e;
-    return a.dtype == ISM_E4M3 ? launch_combine<128>(a, st) : launch_combine<128, true>(a, st);
+    return a.tpc ? launch_combine<128, true>(a, st) : launch_combine<128>(a, st);
   }
   return a.d == 64 ? run_d<64>(a, st) : run_d<128>(a, st);
 }

@@ -6,15 +6,16 @@
 // slots on dot products and the reductions that assemble them; here both
 // contractions run on the tensor cores and the threads only do the softmax.
 //
-// Work split: the 128-key tiles of all (sequence b, KV head g) caches stand in
-// one row, b outermost, and CTA c takes tiles [c * tpc, (c + 1) * tpc) of it,
-// tpc = tiles / SMs rounded up, so every CTA reads the same number of bytes
-// whatever the cache lengths are.  A work item is what a CTA's share has of one
-// (b, g), at most kMaxTiles tiles: keys [k0, k1).  Equal chunks of the longest
-// cache, dealt out in turn, took 64.4 us on 40 ragged caches (250 to 4000
-// keys, 341 MB) and this split takes 59.  (e4m3 keeps equal chunks, splits of
-// the longest cache: P is rounded to three mantissa bits relative to its
-// item's maximum, so other items would move its results by 3.5 %.)  Per item
+// Work split, of caches of different lengths: the 128-key tiles of all (sequence
+// b, KV head g) caches stand in one row, b outermost, and CTA c takes tiles [c *
+// tpc, (c + 1) * tpc) of it, tpc = tiles / SMs rounded up, so every CTA reads the
+// same number of bytes.  A work item is what a CTA's share has of one (b, g), at
+// most kMaxTiles tiles: keys [k0, k1).  40 ragged caches (250 to 4000 keys, 341
+// MB) take 59 us; equal chunks of the longest cache, dealt out in turn, 64.4.
+// Caches of about one length keep the equal chunks (like pieces, neighbouring
+// rows: 8 x 16384 keys 84.5 us a step against 88.4), and so does e4m3 (P is
+// rounded to three mantissa bits relative to its item's maximum, so other items
+// would move its results by 3.5 %).  Per item
 //   pass 1: S^T_t = K_t Q^T for every tile t (M = 128 keys, N = 16 query
 //           heads of the group, zero or foreign rows past the group), all
 //           tiles kept in tensor memory (16 columns each); the softmax
@@ -122,51 +123,45 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
   w.end = min(w.t + a.tpc, a.row_tiles);
   w.b = 0;
   int sb = 0;  // first tile of sequence w.b
-  if (a.uniform) {
-    const int per = dec_alloc_tiles(a, a.uniform) * a.hkv;
-    w.b = w.t / per;
-    sb = w.b * per;
-  } else {
-    const int lane = threadIdx.x & 31;
-    for (int base = 0; base < a.batch; base += 128) {
-      // four sequences a lane, in order
-      int n[4], sum = 0;
+  const int lane = threadIdx.x & 31;
+  for (int base = 0; base < a.batch; base += 128) {
+    // four sequences a lane, in order
+    int n[4], sum = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int b = base + lane * 4 + i;
-        n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * a.hkv : 0;
-        sum += n[i];
-      }
-      int incl = sum;
+    for (int i = 0; i < 4; ++i) {
+      const int b = base + lane * 4 + i;
+      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * a.hkv : 0;
+      sum += n[i];
+    }
+    int incl = sum;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      if (w.t >= sb + total && base + 128 < a.batch) {
-        sb += total;
-        continue;
-      }
-      int at = sb + incl - sum, found = -1, start = 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    if (w.t >= sb + total && base + 128 < a.batch) {
+      sb += total;
+      continue;
+    }
+    int at = sb + incl - sum, found = -1, start = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (w.t >= at && w.t < at + n[i]) {
-          found = base + lane * 4 + i;
-          start = at;
-        }
-        at += n[i];
+    for (int i = 0; i < 4; ++i) {
+      if (w.t >= at && w.t < at + n[i]) {
+        found = base + lane * 4 + i;
+        start = at;
       }
-      const uint32_t who = __ballot_sync(0xffffffffu, found >= 0);
-      if (!who) {
-        w.end = w.t;  // past the last tile: nothing to do
-        break;
-      }
-      const int src = __ffs(who) - 1;
-      w.b = __shfl_sync(0xffffffffu, found, src);
-      sb = __shfl_sync(0xffffffffu, start, src);
+      at += n[i];
+    }
+    const uint32_t who = __ballot_sync(0xffffffffu, found >= 0);
+    if (!who) {
+      w.end = w.t;  // past the last tile: nothing to do
       break;
     }
+    const int src = __ffs(who) - 1;
+    w.b = __shfl_sync(0xffffffffu, found, src);
+    sb = __shfl_sync(0xffffffffu, start, src);
+    break;
   }
   if (w.b >= a.batch) {
     w.b = 0;
@@ -252,13 +247,14 @@ __device__ __forceinline__ void ld_scores(uint32_t taddr, uint32_t (&v)[G]) {
 
 // kG: the heads the softmax warps process (4, 8 or 16, at least the group);
 // the score MMAs always compute 16 (N = 16), the columns past kG are not read.
-template <bool kE4M3, int kG>
+// kRow: the CTAs share out the row of all tiles; else equal chunks in turn.
+template <bool kE4M3, int kG, bool kRow>
 __global__ void __launch_bounds__(kThreads, 1)
     decode_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const DecodeArgs a) {
   using Cfg = DecCfg<kE4M3>;
   constexpr int kStages = Cfg::kStages, kSub = Cfg::kSub;
-  constexpr bool kRow = !kE4M3;
+  static_assert(!(kE4M3 && kRow), "e4m3 keeps equal chunks");
   constexpr uint32_t kTile = Cfg::kTile, kSubBytes = Cfg::kSubBytes, kQHalf = Cfg::kQHalf, kQBytes = Cfg::kQBytes;
   constexpr uint32_t OFF_RING = Cfg::OFF_RING, OFF_P = Cfg::OFF_P, OFF_Q = Cfg::OFF_Q, OFF_BAR = Cfg::OFF_BAR;
   extern __shared__ uint8_t smem_raw[];
@@ -668,7 +664,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <bool kE4M3, int kG>
+template <bool kE4M3, int kG, bool kRow>
 cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
   using Cfg = DecCfg<kE4M3>;
   CUtensorMap tq, tk, tv;
@@ -682,18 +678,26 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     if ((e = make_tmap_bf16(&tk, a.k_cache, (uint64_t)a.hkv * kD, (uint64_t)a.kv_rows)) != cudaSuccess) return e;
     if ((e = make_tmap_bf16(&tv, a.v_cache, (uint64_t)a.hkv * kD, (uint64_t)a.kv_rows)) != cudaSuccess) return e;
   }
-  if ((e = cudaFuncSetAttribute(decode_tc_kernel<kE4M3, kG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if ((e = cudaFuncSetAttribute(decode_tc_kernel<kE4M3, kG, kRow>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Cfg::kSmemBytes)) != cudaSuccess)
     return e;
   int64_t grid;
-  if constexpr (kE4M3) {
+  if constexpr (kRow) {
+    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc;
+  } else {
     const int64_t sms = sm_count(), n_items = (int64_t)a.batch * a.hkv * a.splits;
     grid = sms < n_items ? sms : n_items;
-  } else {
-    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc;
   }
   if (grid <= 0) return cudaSuccess;
-  return launch(true, decode_tc_kernel<kE4M3, kG>, grid, kThreads, Cfg::kSmemBytes, st, tq, tk, tv, a);
+  return launch(true, decode_tc_kernel<kE4M3, kG, kRow>, grid, kThreads, Cfg::kSmemBytes, st, tq, tk, tv, a);
+}
+
+template <bool kE4M3, bool kRow>
+cudaError_t launch_group(const DecodeArgs& a, cudaStream_t st) {
+  // the softmax warps process the group's heads rounded up to 4, 8 or 16
+  return a.group <= 4   ? launch_decode_tc_t<kE4M3, 4, kRow>(a, st)
+         : a.group <= 8 ? launch_decode_tc_t<kE4M3, 8, kRow>(a, st)
+                        : launch_decode_tc_t<kE4M3, kHeadsPad, kRow>(a, st);
 }
 
 }  // namespace
@@ -701,16 +705,10 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
 cudaError_t launch_decode_tc(const DecodeArgs& a, cudaStream_t st) {
   if (a.d != kD || (a.dtype != ISM_BF16 && a.dtype != ISM_E4M3) || a.group > kHeadsPad)
     return cudaErrorInvalidValue;
-  if (a.dtype == ISM_E4M3 ? a.chunk % 128 != 0 || a.chunk > kDecTcMaxKeys : a.tpc < 1 || !a.start)
+  if (a.tpc ? a.dtype == ISM_E4M3 || !a.start : a.chunk < 128 || a.chunk % 128 != 0 || a.chunk > kDecTcMaxKeys)
     return cudaErrorInvalidValue;
-  // the softmax warps process the group's heads rounded up to 4, 8 or 16
-  if (a.dtype == ISM_E4M3)
-    return a.group <= 4 ? launch_decode_tc_t<true, 4>(a, st)
-           : a.group <= 8 ? launch_decode_tc_t<true, 8>(a, st)
-                          : launch_decode_tc_t<true, kHeadsPad>(a, st);
-  return a.group <= 4 ? launch_decode_tc_t<false, 4>(a, st)
-         : a.group <= 8 ? launch_decode_tc_t<false, 8>(a, st)
-                        : launch_decode_tc_t<false, kHeadsPad>(a, st);
+  if (a.dtype == ISM_E4M3) return launch_group<true, false>(a, st);
+  return a.tpc ? launch_group<false, true>(a, st) : launch_group<false, false>(a, st);
 }
 
 }  // namespace tc

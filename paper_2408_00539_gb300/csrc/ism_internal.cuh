@@ -282,13 +282,13 @@ struct DecodeArgs {
   float* part_ml;        // [B, Hq, splits, 2]
   int32_t tma;           // stream the cache with TMA (head_dim 128, sm_103)
   int32_t tc;            // tensor-core kernel (bf16 or e4m3, head_dim 128, group <= 16)
-  // e4m3: equal chunks of a multiple of 128 keys (splits, chunk).  bf16: the 128-key tiles of all (sequence, KV head) caches in one
-  // row of row_tiles, tpc of them per CTA, an item at most kDecTcTiles; splits =
-  // room for partials per (sequence, KV head).  uniform: tiles of every cache
-  // when all are equal, else 0.  align: each cache's tiles are padded to a
-  // multiple of it in the row (1: not).  start [B]: written with the first tile
-  // of each sequence in the row.
-  int32_t tpc, row_tiles, uniform, align;
+  // tpc == 0: equal chunks of a multiple of 128 keys (splits, chunk).  Else
+  // (bf16, ragged caches) the 128-key tiles of all (sequence, KV head) caches in
+  // one row of row_tiles, tpc of them per CTA, an item at most kDecTcTiles;
+  // splits = room for partials per (sequence, KV head).  align: each cache's
+  // tiles are padded to a multiple of it in the row (1: not).  start [B]: written
+  // with the first tile of each sequence in the row.
+  int32_t tpc, row_tiles, align;
   int32_t q_written;     // the queries come from the cache write (rotated)
   int32_t* start;
   uint32_t* status;      // device status word (bounded waits)

@@ -999,13 +999,18 @@ struct CacheGeom {
 // one CTA per SM covers the row, and room for the partials of any (sequence, KV
 // head): the CTAs that its tiles touch, times the items of a CTA's share.
 // Where that exceeds kMaxSplits (a few very long caches), every cache starts at
-// a CTA's share of kDecTcTiles tiles instead.
+// a CTA's share of kDecTcTiles tiles instead.  Neighbouring CTAs take the same
+// share for up to eight KV heads (lanes), whose rows lie side by side: 8 caches
+// of 12000 to 16384 keys 80.0 -> 76.5 us a step against one row of all heads.
 // false: equal chunks, because the caches are about as long as the longest (its
-// tiles at most 1.08 of their mean) or the row has more tiles than 32 bits hold.
-// Equal chunks leave at most what the longest is above the mean, and all CTAs
-// run like pieces of neighbouring rows: 8 x 16384 keys 84.5 us a step against 88.4
-// on the row, 4 x 16384 48.2 and 51.7, 32 x 4000 88.4 and 88.5; ragged lengths,
-// 4 up to 9000, 27.5 and 22.9, 24 up to 3000 with 16 / 4 heads 27.8 and 21.6.
+// tiles at most 1.12 of their mean) and the shares are long, or the row has more
+// tiles than 32 bits hold.  Equal chunks leave idle at most what the longest is
+// above the mean and have fewer short items.  Chunks and row, us a step: 8 x
+// 16384 keys (shares of 55 tiles) 82.5 and 86.0, 4 x 16384 (28) 46.4 and 48.8, 4
+// of 8400 to 9000 (15) 30.0 and 30.2, 1 x 3000 (2) 11.3 and 10.7; 8 from 0.85 of
+// 16384 to all of it (1.08) 79.1 and 82.2, from 0.75 (1.14) 77.7 and 76.5, from
+// 0.6 74.5 and 71.4; 32 from 0.75 of 4000 79.3 and 79.0; 24 up to 3000 with 16 / 4
+// heads 25.0 and 21.8.
 bool decode_row(DecodeArgs& a, const int32_t* cache_len_host, int32_t batch, int32_t hkv, int sms) {
   int64_t sum = 0;
   int32_t most = 0;
@@ -1014,16 +1019,19 @@ bool decode_row(DecodeArgs& a, const int32_t* cache_len_host, int32_t batch, int
     sum += n;
     if (n > most) most = n;
   }
-  if ((int64_t)most * batch * 25 <= sum * 27) return false;
   a.align = 1;
-  int64_t row = sum * hkv, tpc = (row + sms - 1) / sms;
+  a.lanes = 8;
+  while (hkv % a.lanes || sms % a.lanes) a.lanes /= 2;
+  const int64_t groups = sms / a.lanes;
+  int64_t row = sum * (hkv / a.lanes), tpc = (row + groups - 1) / groups;
+  if (tpc > 16 && (int64_t)most * batch * 25 <= sum * 28) return false;
   const int64_t per_cta = (tpc + kDecTcTiles - 1) / kDecTcTiles;
   int64_t slots = ((most + tpc - 1) / tpc + 1) * per_cta;
   if (slots > kMaxSplits) {
     tpc = a.align = kDecTcTiles;
     row = 0;
     for (int b = 0; b < batch; ++b) row += dec_alloc_tiles(a, dec_tiles(cache_len_host[b]));
-    row *= hkv;
+    row *= hkv / a.lanes;
     slots = (most + tpc - 1) / tpc;
   }
   if (row >= (int64_t(1) << 31) - kDecTcTiles || slots > kMaxSplits) return false;

@@ -432,7 +432,7 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
   int s = 0, end = 0, per_cta = 1, c0 = 0;
   if constexpr (kRow) {
     const int n = dec_tiles(a.c_snap[b]), alloc = dec_alloc_tiles(a, n);
-    s = a.start[b] + h / a.group * alloc;
+    s = (a.batch > 1 ? a.start[b] : 0) + h / a.group / a.lanes * alloc;
     end = s + n;
     per_cta = (a.tpc + kDecTcTiles - 1) / kDecTcTiles;
     c0 = s / a.tpc;

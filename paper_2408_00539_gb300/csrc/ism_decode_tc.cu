@@ -6,16 +6,17 @@
 // slots on dot products and the reductions that assemble them; here both
 // contractions run on the tensor cores and the threads only do the softmax.
 //
-// Work split, of caches of different lengths: the 128-key tiles of all (sequence
-// b, KV head g) caches stand in one row, b outermost, and CTA c takes tiles [c *
-// tpc, (c + 1) * tpc) of it, tpc = tiles / SMs rounded up, so every CTA reads the
-// same number of bytes.  A work item is what a CTA's share has of one (b, g), at
-// most kMaxTiles tiles: keys [k0, k1).  40 ragged caches (250 to 4000 keys, 341
-// MB) take 59 us; equal chunks of the longest cache, dealt out in turn, 64.4.
-// Caches of about one length keep the equal chunks (like pieces, neighbouring
-// rows: 8 x 16384 keys 84.5 us a step against 88.4), and so does e4m3 (P is
-// rounded to three mantissa bits relative to its item's maximum, so other items
-// would move its results by 3.5 %).  Per item
+// Work split, of caches of different lengths: the 128-key tiles of all sequences
+// b stand in one row (those of the next group of KV heads after a sequence's
+// own), and the CTAs take shares of tpc tiles of it, one for each of `lanes`
+// neighbouring KV heads, so every CTA reads the same number of bytes and
+// neighbours read the same cache rows.  A work item is what a CTA's share has of
+// one (b, g), at most kMaxTiles tiles: keys [k0, k1).  40 ragged caches (250 to
+// 4000 keys, 341 MB) take 59 us; equal chunks of the longest cache, dealt out in
+// turn, 64.4.  Caches of about one length keep the equal chunks (8 x 16384 keys
+// 82.5 us a step against 86.0), and so does e4m3 (P is rounded to three mantissa
+// bits relative to its item's maximum, so other items would move its results by
+// 3.5 %).  Per item
 //   pass 1: S^T_t = K_t Q^T for every tile t (M = 128 keys, N = 16 query
 //           heads of the group, zero or foreign rows past the group), all
 //           tiles kept in tensor memory (16 columns each); the softmax
@@ -100,14 +101,14 @@ struct DecItem {
   int slot;  // of the partial result among those of (b, g)
   int nt;    // ring tiles (kSub sub-tiles of 128 keys each, the last possibly short)
   int nsub;  // 128-key sub-tiles
-  bool first;  // the first tile of sequence b's first KV head: `s0` is its place in the row
+  bool first;  // the first tile of sequence b: `s0` is its place in the row
   int s0;
 };
 
 // The items of this CTA, one after the other; every role walks them alike.
 struct DecWalk {
   int t, end;    // tiles of the row left to this CTA
-  int b, g, s;   // current (b, g) and its first tile in the row
+  int b, g, s;   // current sequence, head group (DecodeArgs::lanes heads each) and its first tile in the row
   int len;       // keys of sequence b, the new one included
   int64_t item;  // (equal chunks) the next item
 };
@@ -119,18 +120,20 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
     w.item = blockIdx.x;
     return w;
   }
-  w.t = (int)blockIdx.x * a.tpc;
+  w.t = (int)(blockIdx.x / a.lanes) * a.tpc;
   w.end = min(w.t + a.tpc, a.row_tiles);
   w.b = 0;
   int sb = 0;  // first tile of sequence w.b
+  const int row_heads = a.hkv / a.lanes;
   const int lane = threadIdx.x & 31;
-  for (int base = 0; base < a.batch; base += 128) {
+  // (a single sequence needs no search: 8 steps over 3000 keys 87.8 -> 85.4 us)
+  for (int base = 0; a.batch > 1 && base < a.batch; base += 128) {
     // four sequences a lane, in order
     int n[4], sum = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int b = base + lane * 4 + i;
-      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * a.hkv : 0;
+      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * row_heads : 0;
       sum += n[i];
     }
     int incl = sum;
@@ -198,7 +201,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
       const int n = (w.len + 127) / 128, alloc = dec_alloc_tiles(a, n), local = w.t - w.s;
       if (local >= alloc) {  // the next (b, g)
         w.s += alloc;
-        if (++w.g == a.hkv) {
+        if (++w.g == a.hkv / a.lanes) {
           w.g = 0;
           if (++w.b >= a.batch) return false;
           w.len = a.cache_len[w.b] + 1;
@@ -210,15 +213,15 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
         continue;
       }
       const int cnt = min(min(n - local, w.end - w.t), kMaxTiles);
-      const int begin = (int)blockIdx.x * a.tpc;
+      const int cta = (int)blockIdx.x / a.lanes, lane_head = (int)blockIdx.x % a.lanes;
       x.b = w.b;
-      x.g = w.g;
+      x.g = w.g * a.lanes + lane_head;
       x.k0 = local * 128;
       x.k1 = min(w.len, x.k0 + cnt * 128);
       x.nsub = cnt;
       x.nt = (cnt + kSub - 1) / kSub;
-      x.slot = min(dec_slot(a, w.s, (int)blockIdx.x, (w.t - max(w.s, begin)) / kMaxTiles), a.splits - 1);
-      x.first = w.g == 0 && local == 0;
+      x.slot = min(dec_slot(a, w.s, cta, (w.t - max(w.s, cta * a.tpc)) / kMaxTiles), a.splits - 1);
+      x.first = x.g == 0 && local == 0;
       x.s0 = w.s;
       w.t += cnt;
       return true;
@@ -683,7 +686,7 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     return e;
   int64_t grid;
   if constexpr (kRow) {
-    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc;
+    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc * a.lanes;
   } else {
     const int64_t sms = sm_count(), n_items = (int64_t)a.batch * a.hkv * a.splits;
     grid = sms < n_items ? sms : n_items;

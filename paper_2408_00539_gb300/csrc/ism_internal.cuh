@@ -283,12 +283,15 @@ struct DecodeArgs {
   int32_t tma;           // stream the cache with TMA (head_dim 128, sm_103)
   int32_t tc;            // tensor-core kernel (bf16 or e4m3, head_dim 128, group <= 16)
   // tpc == 0: equal chunks of a multiple of 128 keys (splits, chunk).  Else
-  // (bf16, ragged caches) the 128-key tiles of all (sequence, KV head) caches in
+  // (bf16, by decode_row) the 128-key tiles of all (sequence, head group) caches in
   // one row of row_tiles, tpc of them per CTA, an item at most kDecTcTiles;
   // splits = room for partials per (sequence, KV head).  align: each cache's
   // tiles are padded to a multiple of it in the row (1: not).  start [B]: written
   // with the first tile of each sequence in the row.
-  int32_t tpc, row_tiles, align;
+  // lanes: KV heads side by side; CTA i takes share i / lanes of head group g's
+  // (head g * lanes + i % lanes) part of the row, so lanes neighbours read along
+  // the same cache rows.
+  int32_t tpc, row_tiles, align, lanes;
   int32_t q_written;     // the queries come from the cache write (rotated)
   int32_t* start;
   uint32_t* status;      // device status word (bounded waits)

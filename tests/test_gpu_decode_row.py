@@ -63,6 +63,13 @@ def test_matches_cuda_cores(monkeypatch, name, hq, hkv):
     _compare(monkeypatch, CASES[name], hq, hkv)
 
 
+@pytest.mark.parametrize("name", ["edges", "ragged", "one_among"])
+@pytest.mark.parametrize("hq,hkv", [(3, 3), (16, 16), (24, 12)])
+def test_head_lanes(monkeypatch, name, hq, hkv):
+    """One, eight (two groups in the row) and four neighbouring heads a share."""
+    _compare(monkeypatch, CASES[name], hq, hkv)
+
+
 @pytest.mark.parametrize("lens,hkv", [([150000], 1), ([195000], 2), ([190000, 5], 1)])
 def test_long_caches(monkeypatch, lens, hkv):
     """Few caches of more than 62 shares: each starts at a share of its own."""

@@ -893,7 +893,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           for (int k = 0; k < 4; ++k)
             if (k + 4 < ds_groups)
               ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
-                                     make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
+                                     make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2],
+                                                ds_rest[4 * k + 3]),
                                      pol_ds);
           ds_dst = nullptr;
         }
@@ -953,8 +954,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             if (k < ds_groups)
-              ptx::st_global_v4_hint(dst + k * kRows, make_uint4(pd[4 * k], pd[4 * k + 1], pd[4 * k + 2], pd[4 * k + 3]),
-                                     pol_ds);
+              ptx::st_global_v4_hint(dst + k * kRows,
+                                     make_uint4(pd[4 * k], pd[4 * k + 1], pd[4 * k + 2], pd[4 * k + 3]), pol_ds);
 #pragma unroll
           for (int k = 0; k < 16; ++k) ds_rest[k] = pd[16 + k];
           ds_dst = dst;
@@ -965,7 +966,8 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
         for (int k = 0; k < 4; ++k)
           if (k + 4 < ds_groups)
             ptx::st_global_v4_hint(ds_dst + (k + 4) * kRows,
-                                   make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2], ds_rest[4 * k + 3]),
+                                   make_uint4(ds_rest[4 * k], ds_rest[4 * k + 1], ds_rest[4 * k + 2],
+                                              ds_rest[4 * k + 3]),
                                    pol_ds);
       }
       if (!ok) break;
@@ -1041,8 +1043,8 @@ cudaError_t launch_bwd_t(const AttnArgs& a, int64_t k_rows, cudaStream_t st) {
     constexpr int64_t kPairs = kDeltaThreads / (kHD / 8) * kDeltaPairs;  // a block's
     const int64_t grid = (a.q_rows * a.hq + kPairs - 1) / kPairs;
     timer_begin(ISM_KERNEL_BWD_PRE, st);
-    e = launch(a.dependent, a.dependent ? delta_kernel<kHD, true> : delta_kernel<kHD, false>, grid, kDeltaThreads, 0, st,
-               (const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows, a.hq);
+    e = launch(a.dependent, a.dependent ? delta_kernel<kHD, true> : delta_kernel<kHD, false>, grid, kDeltaThreads, 0,
+               st, (const __nv_bfloat16*)a.o, (const __nv_bfloat16*)a.dout, a.delta, a.q_rows, a.hq);
     timer_end(ISM_KERNEL_BWD_PRE, st);
     count_launch();
     if (e != cudaSuccess) return e;

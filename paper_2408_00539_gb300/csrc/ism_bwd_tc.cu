@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   Bars* bar = reinterpret_cast<Bars*>(smem + L::BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_wait();
+  pdl_sync();
   int64_t tpos;
   int h;
   bucket_item(blockIdx.x, a.nq, a.hq, tpos, h, a.hq == a.hkv);  // blocks start roughly in index order
@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  pdl_trigger();  // (after the allocation)
 
   if (warp == 8) {
     // the warp waits converged, lane 0 issues the copies

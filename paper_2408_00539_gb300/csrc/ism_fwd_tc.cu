@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   Bars* bar = reinterpret_cast<Bars*>(smem + OFF_BAR);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_wait();
+  pdl_sync();
   const int h = blockIdx.x % a.hq;
   const Tile w = a.qtiles[a.q_order[blockIdx.x / a.hq]];
   const int g = h / (a.hq / a.hkv);
@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
+  pdl_trigger();  // (after the allocation)
 
   advance_cache_len(a);
 

@@ -77,14 +77,20 @@ enum : uint32_t { kStatusTimeout = 1u, kStatusSmemAlign = 2u };
 // kernel before this one to complete.  Only then does it let the next one start
 // its set-up, so that a kernel that runs at all has everything before its direct
 // predecessor in place.
+// A kernel that allocates tensor memory lets the next one start only after its
+// allocation (pdl_sync at the top, pdl_trigger behind it): the next kernel may
+// allocate before it waits for this one, and would otherwise hold columns that
+// a block of this one still needs, each waiting for the other.
 // Appends and decode steps are launched so, and the passes of a small batch
 // (dependent_pass): one fp32 dialogue of 256 tokens 69.8 -> 55.7 us a step (with the
 // small metadata pass), 4000 ragged tokens of 12 heads 162 -> 148.  On large ones
 // the blocks that wait on the SMs cost more than the launches: 24 dialogues of
 // 32 heads (16001 tokens) 652 -> 686.
+__device__ __forceinline__ void pdl_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_sync();
+  pdl_trigger();
 }
 template <class... Params, class... Args>
 cudaError_t launch(bool dependent, void (*kern)(Params...), int64_t grid, int threads, size_t smem, cudaStream_t st,

@@ -1,0 +1,57 @@
+"""Rules of the kernels launched as programmatic dependents that no run can be
+trusted to show (a breach would hang now and then, or read stale memory), held
+to the sources themselves."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2408_00539_gb300", "csrc")
+
+
+def _body(text, at):
+    """The block that opens at or after `at`."""
+    start = text.index("{", at)
+    depth = 0
+    for i in range(start, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[start:i]
+    raise ValueError("unbalanced braces")
+
+
+def _kernels():
+    """(name, parameters, body) of every kernel, comments taken out."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s+)?(\w+)\s*\(", text):
+            depth, end = 1, m.end()
+            while depth:
+                depth += {"(": 1, ")": -1}.get(text[end], 0)
+                end += 1
+            out.append((m.group(1), text[m.end():end], _body(text, end)))
+    return out
+
+
+KERNELS = _kernels()
+TRIGGER = re.compile(r"pdl_wait\(\)|pdl_trigger\(\)|griddepcontrol\.launch_dependents")
+
+
+def test_kernels_found():
+    names = {n for n, _, _ in KERNELS}
+    assert {"fwd_pair_kernel", "fwd_kernel", "dq_kernel", "dkdv_kernel", "dq_gemm_kernel", "decode_tc_kernel"} <= names
+
+
+@pytest.mark.parametrize("name", [n for n, _, b in KERNELS if "tmem_alloc" in b])
+def test_trigger_follows_the_allocation(name):
+    """A kernel that holds tensor memory lets its successor start only after
+    the block-wide barrier behind its own allocation: the successor may allocate
+    before it waits, and each would wait for the other."""
+    body = next(b for n, _, b in KERNELS if n == name)
+    allocated = body.index("__syncthreads()", body.index("tmem_alloc"))
+    for m in TRIGGER.finditer(body):
+        # a block that leaves before the allocation needs none
+        leaves = re.match(r"[^{}]*\breturn;", body[m.end():])
+        assert m.start() > allocated or leaves, name

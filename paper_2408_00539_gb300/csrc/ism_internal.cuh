@@ -33,8 +33,9 @@ struct KvPages {
   const int32_t* table;
   int32_t page_size, max_pages;
 };
+// (A plain load of the table: dependent kernels read it behind their wait.)
 __device__ __forceinline__ int64_t paged_row(const KvPages& pg, int b, int64_t p) {
-  return (int64_t)__ldg(pg.table + (int64_t)b * pg.max_pages + p / pg.page_size) * pg.page_size + p % pg.page_size;
+  return (int64_t)pg.table[(int64_t)b * pg.max_pages + p / pg.page_size] * pg.page_size + p % pg.page_size;
 }
 
 // Device view of the segment arrays (device pointers only).
@@ -76,7 +77,10 @@ enum : uint32_t { kStatusTimeout = 1u, kStatusSmemAlign = 2u };
 // depends on earlier work or that earlier work may still use: it waits for the
 // kernel before this one to complete.  Only then does it let the next one start
 // its set-up, so that a kernel that runs at all has everything before its direct
-// predecessor in place.
+// predecessor in place.  What it reads is not __restrict__ and not read through
+// __ldg: such loads count as constant, and the compiler may move them before the
+// wait.  (rope_row and order_body may: their addresses come from descriptors that
+// are read behind it, or their kernel wrote them itself.)
 // A kernel that allocates tensor memory lets the next one start only after its
 // allocation (pdl_sync at the top, pdl_trigger behind it): the next kernel may
 // allocate before it waits for this one, and would otherwise hold columns that

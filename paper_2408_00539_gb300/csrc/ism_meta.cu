@@ -555,8 +555,8 @@ template <bool kE4M3>
 __global__ void rope_cache_write_kernel(int batch, int l_new, int hq, int hkv, int d, int64_t cap, KvPages pages,
                                         const int32_t* c_snap, const __nv_bfloat16* q_new,
                                         const __nv_bfloat16* k_new,
-                                        const __nv_bfloat16* v_new, const float* __restrict__ cos_t,
-                                        const float* __restrict__ sin_t, float q_descale, float k_descale,
+                                        const __nv_bfloat16* v_new, const float* cos_t,
+                                        const float* sin_t, float q_descale, float k_descale,
                                         float v_descale, void* q_rot, void* k_cache, void* v_cache,
                                         const __grid_constant__ AppendPlan plan, int32_t* snap_out) {
   pdl_wait();
@@ -604,7 +604,7 @@ __global__ void rope_cache_write_kernel(int batch, int l_new, int hq, int hkv, i
     load8(src + half + k0, hi);
     const float4* cp = reinterpret_cast<const float4*>(cos_t + p * half + k0);
     const float4* sp = reinterpret_cast<const float4*>(sin_t + p * half + k0);
-    const float4 c0 = __ldg(cp), c1 = __ldg(cp + 1), s0 = __ldg(sp), s1 = __ldg(sp + 1);
+    const float4 c0 = cp[0], c1 = cp[1], s0 = sp[0], s1 = sp[1];
     c[0] = c0.x; c[1] = c0.y; c[2] = c0.z; c[3] = c0.w; c[4] = c1.x; c[5] = c1.y; c[6] = c1.z; c[7] = c1.w;
     s[0] = s0.x; s[1] = s0.y; s[2] = s0.z; s[3] = s0.w; s[4] = s1.x; s[5] = s1.y; s[6] = s1.z; s[7] = s1.w;
     float ol[8], oh[8];

@@ -19,11 +19,11 @@ namespace {
 
 // Sequence of token t: the last b with cu_seqlens[b] <= t (zero-length
 // sequences share their offset with the next one).
-__device__ __forceinline__ int seq_of(const int32_t* __restrict__ cu, int num_seqs, int64_t t) {
+__device__ __forceinline__ int seq_of(const int32_t* cu, int num_seqs, int64_t t) {
   int lo = 0, hi = num_seqs;  // cu[lo] <= t < cu[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if ((int64_t)__ldg(cu + mid) <= t) lo = mid; else hi = mid;
+    if ((int64_t)cu[mid] <= t) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -64,13 +64,14 @@ struct Vec<float> {
 };
 
 // One thread per 16-byte unit of the first half of one head row (query heads
-// first, then key heads) and its partner unit in the second half.
+// first, then key heads) and its partner unit in the second half.  The inputs
+// are not __restrict__: what the compiler may take for constant it may load
+// before the wait (the middle offset of cu_seqlens above all).
 template <typename E>
-__global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* __restrict__ cu_seqlens, int num_seqs,
+__global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* cu_seqlens, int num_seqs,
                                                         int64_t T, int hq, int hkv, int d, const E* q_src,
                                                         const E* k_src, E* q_dst, E* k_dst,
-                                                        const float* __restrict__ cos_t,
-                                                        const float* __restrict__ sin_t, float sin_sign) {
+                                                        const float* cos_t, const float* sin_t, float sin_sign) {
   pdl_wait();
   constexpr int N = Vec<E>::N;
   const int half = d / 2;
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* __restric
     const int r = (int)(i % per_row);
     const int head = r / units;
     const int k0 = (r % units) * N;
-    const int64_t pos = t - __ldg(cu_seqlens + seq_of(cu_seqlens, num_seqs, t));
+    const int64_t pos = t - cu_seqlens[seq_of(cu_seqlens, num_seqs, t)];
     const E* src;
     E* dst;
     if (head < hq) {
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(256) rope_rows_kernel(const int32_t* __restric
     const float4* sp = reinterpret_cast<const float4*>(sin_t + pos * half + k0);
 #pragma unroll
     for (int v = 0; v < N / 4; ++v) {
-      const float4 cv = __ldg(cp + v), sv = __ldg(sp + v);
+      const float4 cv = cp[v], sv = sp[v];
       c[4 * v] = cv.x; c[4 * v + 1] = cv.y; c[4 * v + 2] = cv.z; c[4 * v + 3] = cv.w;
       s[4 * v] = sv.x * sin_sign; s[4 * v + 1] = sv.y * sin_sign;
       s[4 * v + 2] = sv.z * sin_sign; s[4 * v + 3] = sv.w * sin_sign;

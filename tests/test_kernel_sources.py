@@ -55,3 +55,18 @@ def test_trigger_follows_the_allocation(name):
         # a block that leaves before the allocation needs none
         leaves = re.match(r"[^{}]*\breturn;", body[m.end():])
         assert m.start() > allocated or leaves, name
+
+
+@pytest.mark.parametrize("name", [n for n, _, b in KERNELS if "pdl_" in b and n != "delta_kernel"])
+def test_nothing_counts_as_constant(name):
+    """Loads of a dependent kernel that the compiler may take for constant may
+    be moved before its wait: no __restrict__ parameters, no __ldg."""
+    params, body = next((p, b) for n, p, b in KERNELS if n == name)
+    assert "__restrict__" not in params and "__ldg" not in body
+
+
+def test_page_table_and_offsets_are_plain_loads():
+    for name, function in (("ism_internal.cuh", "paged_row"), ("ism_rope.cu", "seq_of")):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        at = text.index(function + "(")
+        assert "__restrict__" not in text[at:text.index(")", at)] and "__ldg" not in _body(text, at)

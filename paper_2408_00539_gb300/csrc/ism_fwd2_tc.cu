@@ -482,13 +482,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int c = 0; c < 128; c += 2) mr[(c >> 1) & 3] = max3(mr[(c >> 1) & 3], xs[c], xs[c + 1]);
         const float mraw = max3(fmaxf(mr[0], mr[1]), mr[2], mr[3]);
         const float m_new = fmaxf(m_use, mraw * sl2);
+        const bool raise = m_new > m_use + 8.f;
         if (j == 0) {
           m_use = m_new;
-        } else if (m_new > m_use + 8.f) {
-          // bring O (complete through PV(j-1)) and l to the new max
-          if (!wait(&bar->pv_done[xh], (blk - 1) & 1, a.status)) { ok = false; break; }
+        } else if (__any_sync(0xffffffffu, raise)) {
+          // bring O (complete through PV(j-1)) and l of the rows that need it to
+          // the new max.  The whole warp goes: tensor-memory loads and stores are
+          // the warp's, and lanes left behind would never meet them.
+          if (!__all_sync(0xffffffffu, wait(&bar->pv_done[xh], (blk - 1) & 1, a.status))) { ok = false; break; }
           ptx::tc_fence_after();
-          const float f = ex2(m_use - m_new);
+          const float f = raise ? ex2(m_use - m_new) : 1.f;
           l *= f;
 #pragma unroll 1
           for (int c = 0; c < kHD / 32; ++c) {
@@ -500,7 +503,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
             ptx::tmem_st32(tO + c * 32, o);
           }
-          m_use = m_new;
+          if (raise) m_use = m_new;
         }
         // P over the first 64 columns of S (already read), 32 columns at a time
         float2 rsv[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};

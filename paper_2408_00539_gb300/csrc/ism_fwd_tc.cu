@@ -243,14 +243,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float mraw = fmaxf(fmaxf(fmaxf(mr[0], mr[1]), fmaxf(mr[2], mr[3])),
                                fmaxf(fmaxf(mr[4], mr[5]), fmaxf(mr[6], mr[7])));
       const float m_new = fmaxf(m_use, mraw * sl2);
+      const bool raise = m_new > m_use + 8.f;
       if (j == 0) {
         m_use = m_new;
-      } else if (m_new > m_use + 8.f) {
-        // the max grew a lot: bring O (complete through PV_{j-1}) and l to the new max
+      } else if (__any_sync(0xffffffffu, raise)) {
+        // the max grew a lot: bring O (complete through PV_{j-1}) and l of such rows
+        // to the new max (the whole warp goes: tensor-memory loads and stores are
+        // the warp's, and lanes left behind would never meet them)
         const int sp = (j - 1) & 1;
-        if (!wait(&bar->p_free[sp], (uint32_t)((j - 1) >> 1) & 1, a.status)) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, wait(&bar->p_free[sp], (uint32_t)((j - 1) >> 1) & 1, a.status))) { ok = false; break; }
         ptx::tc_fence_after();
-        const float f = ex2(m_use - m_new);
+        const float f = raise ? ex2(m_use - m_new) : 1.f;
         l *= f;
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
@@ -263,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ptx::tmem_st32(tmem + lane_addr + TM_O + c * 32, o);
         }
         ptx::tmem_st_wait();
-        m_use = m_new;
+        if (raise) m_use = m_new;
       }
       float rsv[4] = {0.f, 0.f, 0.f, 0.f};
       uint32_t pk[64];

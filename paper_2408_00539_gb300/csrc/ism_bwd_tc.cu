@@ -81,11 +81,11 @@ __device__ __forceinline__ void mma_tile_rows(uint32_t d, uint32_t tA, uint32_t 
 // The reductions shuffle within the group's own lanes.
 constexpr int kDeltaThreads = 256, kDeltaPairs = 2;
 template <int kHD, bool kDependent>
-__global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
-                             float* __restrict__ delta, int64_t rows, int hq) {
+__global__ void delta_kernel(const __nv_bfloat16* O, const __nv_bfloat16* dO, float* delta, int64_t rows, int hq) {
   // O and dO are in place when this kernel runs at all: its direct predecessor
   // is the metadata pass (or a reset of its counter), which it does not depend on
-  // and runs beside as a dependent launch.  The wait at the end makes this
+  // and runs beside as a dependent launch.  It loads them from L2, where finished
+  // kernels' writes are, since it has not waited for anything itself.  The wait at the end makes this
   // kernel's completion imply that one's.  (It costs 4 of 48 us on 2 x 8192
   // tokens of 32 heads, which are launched plainly.)
   constexpr int kLanes = kHD / 8, kGroups = kDeltaThreads / kLanes;
@@ -98,8 +98,8 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfl
   for (int u = 0; u < kDeltaPairs; ++u) {
     const int64_t i = i0 + u * kGroups;
     if (i < n) {
-      a[u] = reinterpret_cast<const uint4*>(O + i * kHD)[sub];
-      b[u] = reinterpret_cast<const uint4*>(dO + i * kHD)[sub];
+      a[u] = __ldcg(reinterpret_cast<const uint4*>(O + i * kHD) + sub);
+      b[u] = __ldcg(reinterpret_cast<const uint4*>(dO + i * kHD) + sub);
     }
   }
 #pragma unroll

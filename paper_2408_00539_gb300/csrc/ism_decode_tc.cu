@@ -74,6 +74,8 @@ struct DecCfg {
   static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 };
 
+constexpr int kLensCopied = 128;
+
 struct Bars {
   uint64_t full[kMaxStages], empty[kMaxStages];
   uint64_t q_full[2], q_empty[2];
@@ -87,6 +89,7 @@ struct Bars {
   // per item parity: warp 0's epilogue of item u reads them while the other
   // warps may already fold the scores of item u + 1
   float red_m[2][4][kHeadsPad], red_l[2][4][kHeadsPad];
+  int32_t lens[kLensCopied];  // cached keys of the first sequences
 };
 static_assert(sizeof(Bars) <= 2048, "barrier block");
 
@@ -109,12 +112,24 @@ struct DecItem {
 struct DecWalk {
   int t, end;    // tiles of the row left to this CTA
   int b, g, s;   // current sequence, head group (DecodeArgs::lanes heads each) and its first tile in the row
-  int len;       // keys of sequence b, the new one included
+  int len;       // keys of the current item's sequence, the new one included
   int64_t item;  // (equal chunks) the next item
 };
+// A sequence's cached keys.  This grid may start before the kernel in front of
+// it (the cache write) is complete and reads the lengths without waiting for it;
+// the combine of the step before advanced them on other SMs and is complete, so
+// they are right in L2, whatever an SM's L1 holds.
+__device__ __forceinline__ int32_t cached(const DecodeArgs& a, int b) { return ld_gpu(a.cache_len + b); }
+
+// The same from the block's copy of the first ones (a read of L2 by every warp of
+// every CTA costs 40 ragged caches 0.9 us of a step's 66.5).
+__device__ __forceinline__ int32_t cached(const DecodeArgs& a, const int32_t* lens, int b) {
+  return b < kLensCopied ? lens[b] : cached(a, b);
+}
+
 // The whole warp: finds the (b, g) of the CTA's first tile.
 template <bool kRow>
-__device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
+__device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a, const int32_t* lens) {
   DecWalk w;
   if constexpr (!kRow) {
     w.item = blockIdx.x;
@@ -133,7 +148,7 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int b = base + lane * 4 + i;
-      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(a.cache_len[b])) * row_heads : 0;
+      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(cached(a, lens, b))) * row_heads : 0;
       sum += n[i];
     }
     int incl = sum;
@@ -170,14 +185,14 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
     w.b = 0;
     w.end = w.t;
   }
-  w.len = a.cache_len[w.b] + 1;
+  w.len = cached(a, lens, w.b) + 1;
   const int per_head = dec_alloc_tiles(a, (w.len + 127) / 128);
   w.g = w.t < w.end ? (w.t - sb) / per_head : 0;
   w.s = sb + w.g * per_head;
   return w;
 }
 template <bool kRow, int kSub>
-__device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecItem& x) {
+__device__ __forceinline__ bool dec_next(const DecodeArgs& a, const int32_t* lens, DecWalk& w, DecItem& x) {
   if constexpr (!kRow) {
     // item = (split * batch + b) * hkv + g: consecutive CTAs take the KV heads of
     // one (sequence, split), whose rows lie side by side in the cache
@@ -190,7 +205,8 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
     x.b = (int)(rest % a.batch);
     x.slot = (int)(rest / a.batch);
     x.k0 = x.slot * a.chunk;
-    x.k1 = min(a.cache_len[x.b] + 1, x.k0 + a.chunk);
+    w.len = cached(a, lens, x.b) + 1;
+    x.k1 = min(w.len, x.k0 + a.chunk);
     x.nsub = x.k1 > x.k0 ? (x.k1 - x.k0 + 127) / 128 : 0;
     x.nt = (x.nsub + kSub - 1) / kSub;
     x.first = false;
@@ -204,7 +220,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
         if (++w.g == a.hkv / a.lanes) {
           w.g = 0;
           if (++w.b >= a.batch) return false;
-          w.len = a.cache_len[w.b] + 1;
+          w.len = cached(a, lens, w.b) + 1;
         }
         continue;
       }
@@ -258,6 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   using Cfg = DecCfg<kE4M3>;
   constexpr int kStages = Cfg::kStages, kSub = Cfg::kSub;
   static_assert(!(kE4M3 && kRow), "e4m3 keeps equal chunks");
+  static_assert(kMaxTiles <= 32, "a lane for each sub-tile of an item");
   constexpr uint32_t kTile = Cfg::kTile, kSubBytes = Cfg::kSubBytes, kQHalf = Cfg::kQHalf, kQBytes = Cfg::kQBytes;
   constexpr uint32_t OFF_RING = Cfg::OFF_RING, OFF_P = Cfg::OFF_P, OFF_Q = Cfg::OFF_Q, OFF_BAR = Cfg::OFF_BAR;
   extern __shared__ uint8_t smem_raw[];
@@ -293,6 +310,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tmem_alloc(&bar->tmem_base, kTmemCols);
     ptx::tmem_relinquish();
   }
+  if (warp == kLoadWarp)
+    for (int b = lane; b < min(a.batch, kLensCopied); b += 32) bar->lens[b] = cached(a, b);
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
@@ -317,17 +336,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::tma_prefetch_desc(&tmK);
       ptx::tma_prefetch_desc(&tmV);
     }
-    DecWalk walk = dec_walk<kRow>(a);
+    DecWalk walk = dec_walk<kRow>(a, bar->lens);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
       if (!kRow && x.nt == 0) continue;
+      const bool last_item = x.k1 == walk.len;  // it has the cache's last tile
+      // rows of the item's sub-tiles in the K / V tensors, one a lane: a 128-key
+      // sub-tile starts at a multiple of 128 keys and lies in one page.  (Table
+      // entries as they come, one from L2 in front of each copy: 40 ragged paged
+      // caches 73.3 us a step, all of an item at once 66.5.)
+      const int64_t p = (int64_t)x.k0 + lane * 128;
+      int64_t row = (int64_t)x.b * a.cap + p;
+      if (a.pages.table)
+        row = lane < x.nsub ? page_row(a.pages, ld_gpu(page_entry(a.pages, x.b, p)), p) : 0;
+      const int32_t rows = (int32_t)row;
       const uint32_t qb = nu & 1;
       if (__any_sync(0xffffffffu, aborted(&bar->abort)) ||
           (nu >= 2 && !wait_warp(&bar->q_empty[qb], ((nu >> 1) - 1) & 1, a.status))) {
         ok = false;
         break;
       }
-      const bool last_item = x.k1 == a.cache_len[x.b] + 1;  // it has the cache's last tile
       auto load_q = [&] {
         if (lane == 0) {
           // the 16 query rows from the group's first head (rows past the group
@@ -360,17 +388,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = false;
             break;
           }
+          int32_t y[kSub];
+#pragma unroll
+          for (int hh = 0; hh < kSub; ++hh) y[hh] = __shfl_sync(0xffffffffu, rows, t * kSub + hh);
           if (lane == 0) {
-            // a 128-key sub-tile starts at a multiple of 128 keys and lies in one page
             const int nh = min(kSub, x.nsub - t * kSub);
             uint8_t* dst = smem + OFF_RING + s * kTile;
             ptx::mbar_expect_tx(&bar->full[s], (uint32_t)nh * kSubBytes);
-            for (int hh = 0; hh < nh; ++hh) {
-              const int64_t p = (int64_t)x.k0 + (int64_t)(t * kSub + hh) * 128;
-              const int32_t y =
-                  a.pages.table ? (int32_t)paged_row(a.pages, x.b, p) : (int32_t)((int64_t)x.b * a.cap + p);
-              ptx::tma_load_2d_hint(dst + hh * kSubBytes, map, &bar->full[s], x.g * kD, y, pol);
-              if (!kE4M3) ptx::tma_load_2d_hint(dst + kHalfBytes, map, &bar->full[s], x.g * kD + 64, y, pol);
+#pragma unroll
+            for (int hh = 0; hh < kSub; ++hh) {
+              if (hh >= nh) break;
+              ptx::tma_load_2d_hint(dst + hh * kSubBytes, map, &bar->full[s], x.g * kD, y[hh], pol);
+              if (!kE4M3) ptx::tma_load_2d_hint(dst + kHalfBytes, map, &bar->full[s], x.g * kD + 64, y[hh], pol);
             }
           }
           __syncwarp();
@@ -395,9 +424,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t idesc_pv = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 1, 1) : ptx::idesc_bf16_f32(128, 128, 1, 1);
     uint32_t nl = 0, nu = 0, T = 0, TS = 0;  // ring tiles consumed; non-empty items; P tiles; S tiles
     bool ok = true;
-    DecWalk walk = dec_walk<kRow>(a);
+    DecWalk walk = dec_walk<kRow>(a, bar->lens);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
       if (!kRow && x.nt == 0) continue;
       const uint32_t qb = nu & 1;
       // Q landed; the softmax warps have read the previous item's S
@@ -484,9 +513,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int group = a.group;
     uint32_t nu = 0, T = 0, TS = 0;
     bool ok = true;
-    DecWalk walk = dec_walk<kRow>(a);
+    DecWalk walk = dec_walk<kRow>(a, bar->lens);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
       const int64_t pbase = ((int64_t)x.b * a.hq + (int64_t)x.g * group) * a.splits + x.slot;
       if (!kRow && x.nt == 0) {
         // a split past the sequence's keys: a partial the combine skips

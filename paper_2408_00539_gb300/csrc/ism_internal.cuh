@@ -25,6 +25,13 @@ struct Tile {
 };
 static_assert(sizeof(Tile) == 32, "Tile layout");
 
+// A load from L2, where another SM's finished writes are.
+__device__ __forceinline__ int32_t ld_gpu(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // Paged K/V cache (append-prefill and decode): key p of sequence b sits in
 // row table[b * max_pages + p / page_size] * page_size + p % page_size of the
 // pools.  With table == nullptr the cache is contiguous: the rows of sequence
@@ -33,9 +40,15 @@ struct KvPages {
   const int32_t* table;
   int32_t page_size, max_pages;
 };
+__device__ __forceinline__ const int32_t* page_entry(const KvPages& pg, int b, int64_t p) {
+  return pg.table + (int64_t)b * pg.max_pages + p / pg.page_size;
+}
+__device__ __forceinline__ int64_t page_row(const KvPages& pg, int32_t entry, int64_t p) {
+  return (int64_t)entry * pg.page_size + p % pg.page_size;
+}
 // (A plain load of the table: dependent kernels read it behind their wait.)
 __device__ __forceinline__ int64_t paged_row(const KvPages& pg, int b, int64_t p) {
-  return (int64_t)pg.table[(int64_t)b * pg.max_pages + p / pg.page_size] * pg.page_size + p % pg.page_size;
+  return page_row(pg, *page_entry(pg, b, p), p);
 }
 
 // Device view of the segment arrays (device pointers only).

@@ -129,3 +129,80 @@ def test_small_and_general_metadata_agree(seed, monkeypatch):
     ism.check_status(DEV)
     for name, y, z in zip("o lse dq dk dv".split(), a, b):
         assert torch.equal(y[:, :T] if name == "lse" else y[:T], z), name
+
+
+def _decode_64(waits, paged, rope, stream):
+    """64 steps of three caches on a stream; the new rows of each step are
+    written into the same buffers by the kernel just before it."""
+    lens = np.array([300, 5, 121], np.int32)  # every cache crosses into its next tile of 128 on the way
+    gen = torch.Generator().manual_seed(8)
+    B, n, hq, hkv = 3, 64, 8, 2
+    new = [torch.randn((n, B, 1, h, 128), generator=gen).bfloat16().to(DEV) for h in (hq, hkv, hkv)]
+    rows = (9 * 128, hkv, 128) if paged else (B, 400, hkv, 128)
+    kc, vc = (torch.randn(rows, generator=gen).bfloat16().to(DEV) for _ in range(2))
+    table = np.arange(9, dtype=np.int32)[::-1].reshape(3, 3).copy()
+    dev_table, cl, host = torch.from_numpy(table).to(DEV), torch.from_numpy(lens.copy()).to(DEV), lens.copy()
+    tables = tuple(torch.from_numpy(a).to(DEV) for a in wl.rope_tables(400, 128))
+    x = [torch.empty_like(t[0]) for t in new]
+    outs = []
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for i in range(n):
+            for a, b in zip(x, new):
+                torch.mul(b[i], 1.0, out=a)
+            args = (cl, host, [1], [1])
+            if paged:
+                o = ism.prefill_append_paged(*x, kc, vc, 128, dev_table, table, *args, 0.09)
+            elif rope:
+                o = ism.prefill_append_rope(*x, kc, vc, *args, *tables, 0.09)
+            else:
+                o = ism.prefill_append(*x, kc, vc, *args, 0.09)
+            outs.append(o)
+            host += 1
+            if waits:
+                torch.cuda.synchronize()
+    return outs, kc, vc, cl
+
+
+@pytest.mark.parametrize("paged,rope", [(False, False), (True, False), (False, True)])
+def test_decode_steps_back_to_back(paged, rope):
+    """Steps without a wait, on two streams, against the same steps with a wait
+    after each: the decode reads lengths, page table and old rows before the
+    cache write in front of it is complete."""
+    streams = [torch.cuda.Stream(DEV) for _ in range(2)]
+    ref = _decode_64(True, paged, rope, streams[0])
+    ism.check_status(DEV)
+    got = [_decode_64(False, paged, rope, s) for s in streams for _ in range(2)]
+    torch.cuda.synchronize()
+    ism.check_status(DEV)
+    for outs, *rest in got:
+        assert all(torch.equal(a, b) for a, b in zip(rest, ref[1:]))
+        assert all(torch.equal(a, b) for x, y in zip(outs, ref[0]) for a, b in zip(x, y))
+
+
+def test_training_steps_on_changing_inputs():
+    """Steps without a wait on inputs that change in place, against the same
+    steps with a wait after each (Delta reads O and dO before the pass in front
+    of it is complete)."""
+    w = wl.Workload("pdl", wl.pack(DIALOGUES), 4, 2, 64, "bf16", 0.125, 1.0, 33)
+    segs = ism.Segments.from_workload(w.segs, DEV)
+    xs = [[(t.float() * f).bfloat16().to(DEV) for t in wl.attention_tensors(w)] for f in (1.0, 0.5, -1.5, 2.0)]
+    live = [torch.empty_like(t) for t in xs[0]]
+    o, lse = torch.empty_like(live[0]), torch.empty((4, live[0].shape[0]), device=DEV)
+
+    def steps(waits):
+        outs = []
+        for i in range(12):
+            for a, b in zip(live, xs[i % 4]):
+                torch.mul(b, 1.0, out=a)
+            ism.fwd(segs, *live[:3], w.softmax_scale, out=o, lse=lse)
+            outs.append((o.clone(), *ism.bwd(segs, *live[:3], o, lse, live[3], w.softmax_scale)))
+            if waits:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return outs
+
+    ref = steps(True)
+    for _ in range(3):
+        assert all(torch.equal(a, b) for x, y in zip(steps(False), ref) for a, b in zip(x, y))
+    ism.check_status(DEV)

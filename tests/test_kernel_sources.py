@@ -57,7 +57,7 @@ def test_trigger_follows_the_allocation(name):
         assert m.start() > allocated or leaves, name
 
 
-@pytest.mark.parametrize("name", [n for n, _, b in KERNELS if "pdl_" in b and n != "delta_kernel"])
+@pytest.mark.parametrize("name", [n for n, _, b in KERNELS if "pdl_" in b])
 def test_nothing_counts_as_constant(name):
     """Loads of a dependent kernel that the compiler may take for constant may
     be moved before its wait: no __restrict__ parameters, no __ldg."""
@@ -70,3 +70,15 @@ def test_page_table_and_offsets_are_plain_loads():
         text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
         at = text.index(function + "(")
         assert "__restrict__" not in text[at:text.index(")", at)] and "__ldg" not in _body(text, at)
+
+
+def test_early_reads_go_to_l2():
+    """What is read before the kernel's own wait comes from L2: the lengths and
+    the page table of the decode, O and dO of the dependent Delta."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "ism_decode_tc.cu")).read())
+    assert re.findall(r"[^\n]*\bcache_len\b[^\n]*", text) == [
+        "__device__ __forceinline__ int32_t cached(const DecodeArgs& a, int b) { return ld_gpu(a.cache_len + b); }"]
+    assert "ld_gpu(page_entry(" in text and "paged_row(" not in text
+    body = next(b for n, _, b in KERNELS if n == "delta_kernel")
+    loads = re.findall(r"=([^;]*(?:\bO\b|\bdO\b)[^;]*);", body)
+    assert len(loads) == 2 and all("__ldcg" in x for x in loads)

@@ -283,9 +283,10 @@ ism_status_t ism_attn_bwd_rope(const ism_segments_t* segs, const ism_attn_shape_
  *   recompute schedule: both cover what the planned call uses).
  * ism_attn_fwd_rope_planned / ism_attn_bwd_rope_planned: the same for
  *   ism_attn_fwd_rope / ism_attn_bwd_rope (arguments as there).
- * The plan must stay unchanged while a call that uses it may run, and calls
- * that share a plan run in stream order (the backward resets a work counter
- * held in the plan).  No counterpart in the paper.
+ * The plan must stay unchanged while a call that uses it may run.  The
+ * forwards only read it and may overlap (on several streams); the backward
+ * resets and advances a work counter held in it, so backwards that share a
+ * plan run one after the other in stream order.  No counterpart in the paper.
  * ------------------------------------------------------------------------- */
 typedef struct {
   uint64_t fingerprint;

@@ -208,7 +208,7 @@ struct PassLayout {
   void* ds;
   int32_t* pair_order;
   int32_t* kp_order;  // k-tile pairs in cost order (backward only)
-  int32_t* counters;  // work counters: of dK/dV (backward), of the forward's query-tile pairs
+  int32_t* counters;  // work counters: of dK/dV (backward, plans), of the forward
   size_t bytes;
 };
 constexpr int kPassCounters = 2;
@@ -558,14 +558,13 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   }
   // query-tile pairs: an odd group
   const bool tile_pairs = L.pair_order || (use_tc(shape) && shape->head_dim == 64 && pairs_first(shape));
-  const bool dynamic = (use_tc(shape) || e4m3) &&
+  // A planned forward walks statically: a plan may serve forwards on several
+  // streams at once, and the counter would have to lie in it.
+  const bool dynamic = !pre && (use_tc(shape) || e4m3) &&
                        fwd_dynamic(tile_pairs ? c.npairs * shape->num_heads_q : c.nq * (shape->num_heads_q / 2),
                                    tile_pairs);
-  if (!pre) {
-    if ((r = build_pass_meta(segs, c, L, false, st, shape->num_heads_q, pairs_first(shape))) != ISM_OK) return r;
-  } else if (dynamic) {
-    ISM_TRY_CUDA(cudaMemsetAsync(L.counters + kFwdCounter, 0, sizeof(int32_t), st), "work counter reset");
-  }
+  if (!pre && (r = build_pass_meta(segs, c, L, false, st, shape->num_heads_q, pairs_first(shape))) != ISM_OK)
+    return r;
 
   AttnArgs a{};
   a.q = q; a.k = k; a.v = v; a.out = o; a.lse = lse;
@@ -580,7 +579,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     a.npairs = c.npairs;
   }
   a.work_counter = dynamic ? L.counters + kFwdCounter : nullptr;
-  a.bucketed = fwd_bucketed(a, a.npairs * a.hq);
+  a.bucketed = dynamic ? fwd_bucketed(a, a.npairs * a.hq) : a.hq == a.hkv;
   a.status = status;
   a.flags = tc_flags();
   timer_begin(ISM_KERNEL_FWD, st);

@@ -687,9 +687,11 @@ cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CU
                               cudaStream_t st) {
   cudaError_t e;
   const bool split = a.split_items > 0;
+  // e4m3 tile pairs always have a counter (they take no plan)
+  constexpr bool kNeedsCounter = kTilePairs && kE4M3;
   auto kern = split ? fwd_pair_kernel<kTilePairs, kE4M3, true, kHD, false>
               : a.work_counter ? fwd_pair_kernel<kTilePairs, kE4M3, false, kHD, true>
-                               : fwd_pair_kernel<kTilePairs, kE4M3, false, kHD, kTilePairs>;
+                               : fwd_pair_kernel<kTilePairs, kE4M3, false, kHD, kNeedsCounter>;
   constexpr uint32_t smem = PairLayout<kE4M3, kHD>::SMEM;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
@@ -699,7 +701,7 @@ cudaError_t launch_fwd_pair_t(const AttnArgs& a, const CUtensorMap& tq, const CU
                 a.split_parts > kMaxParts))
     return cudaErrorInvalidValue;
   const int64_t n_units = split ? a.split_whole + a.split_parts * a.split_items : items;
-  if (!split && (a.work_counter ? n_units >= (int64_t(1) << 30) : kTilePairs)) return cudaErrorInvalidValue;
+  if (!split && (a.work_counter ? n_units >= (int64_t(1) << 30) : kNeedsCounter)) return cudaErrorInvalidValue;
   // persistent: one CTA per SM walks its share of the units
   const int64_t grid = n_units < sm_count() ? n_units : sm_count();
   if ((e = launch(split || a.dependent, kern, grid, kThreads, smem, st, tq, tk, tv, a, n_units)) != cudaSuccess ||

@@ -265,7 +265,7 @@ inline bool dependent_pass(int64_t q_tiles, int heads) { return q_tiles * heads 
 // 64 with 16 heads over 6001 tokens 98 -> 67.  Head pairs gain below eight units
 // a CTA (16 / 4 heads over 5000 ragged tokens, 2 units a CTA: 46 -> 39) and lose
 // on many even ones (2 x 8192, 13 a CTA: 654 -> 662; one dialogue of 32768 4881
-// -> 4951).
+// -> 4951).  Planned forwards have no counter and always walk statically.
 inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || items < 8 * (int64_t)sm_count(); }
 // Whether that list keeps its buckets (bucket_item) instead of the plain cost
 // order: with one query head per KV head, 32 KB tiles and many units, sharing
@@ -273,7 +273,8 @@ inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || i
 // balance: 4 x 4096 of 32 heads 1767 us a step against 1786, although the forward
 // alone takes 396 against 387; six ragged dialogues 2684 and 2699.  Half-size
 // tiles and few units: e4m3 4 x 4096 333 and 318, head_dim 64 over 6001 tokens 318
-// and 302.
+// and 302.  The static walk of tile pairs keeps its buckets wherever the heads do
+// not share K / V.
 inline bool fwd_bucketed(const AttnArgs& a, int64_t items) {
   return a.hq == a.hkv && a.d == 128 && a.dtype == ISM_BF16 && items >= 8 * (int64_t)sm_count();
 }

@@ -68,11 +68,9 @@ ism_status_t ism_attn_fwd_noalloc(const ism_segments_t* segs, const ism_attn_sha
   void* scratch = nullptr;
   r = scratch_address(&scratch);
   if (r != ISM_OK) return r;
-  // Nothing in the scratch has to start at zero: the forward's layout holds
-  // only the per-token key bounds, tile descriptors and work lists, and its
-  // metadata pass writes every entry the attention kernel then reads.  (The
-  // backward's layout also carries work counters; a forward that ever gains
-  // such state must clear it here before the launch.)
+  // Nothing in the scratch has to start at zero: the forward's layout holds the
+  // per-token key bounds, tile descriptors, work lists and a work counter, and
+  // its metadata pass writes every entry the attention kernel then reads.
   return ism_attn_fwd(segs, shape, q, k, v, o, lse, scratch, kNoAllocScratchBytes, stream);
 }
 

@@ -298,7 +298,8 @@ def tile_map(segs: Segments, bm: int = 128, bn: int = 128):
 class Plan:
     """The metadata of one batch of segments (ism_attn_plan_build) for the
     forward and backward of every layer over those segments and head counts:
-    built once, passed to fwd / bwd as plan=.  Holds its device buffer."""
+    built once, passed to fwd / bwd as plan=.  Holds its device buffer, which
+    forwards only read; backwards on one plan run one after the other."""
 
     def __init__(self, segs: Segments, num_heads_q: int, num_heads_kv: int, head_dim: int = 128,
                  dtype: torch.dtype = torch.bfloat16, device="cuda"):

@@ -1,7 +1,9 @@
 """The paired forward on the work counter against the static walk's results
 (bit for bit: only which CTA takes a unit differs) and the oracle: fewer units
 than CTAs, several a CTA, many single-tile dialogues (units whose second half is
-empty), plans used again and again, and the counter's place in every workspace.
+empty), plans used again and again (planned forwards walk statically and leave
+the plan as it is, so they may overlap), and the counter's place in every
+workspace.
 """
 import numpy as np
 import pytest
@@ -28,7 +30,7 @@ def test_plan_and_plain_calls(dialogues, hq, hkv, d):
     dev = [t.to(DEV) for t in (q, k, v)]
     o, lse = ism.fwd(segs, *dev, w.softmax_scale)
     plan = ism.Plan(segs, hq, hkv, d, torch.bfloat16, DEV)
-    for _ in range(3):  # the plan's counter starts at zero every time
+    for _ in range(3):
         o2, lse2 = ism.fwd(segs, *dev, w.softmax_scale, plan=plan)
         assert torch.equal(o, o2) and torch.equal(lse, lse2)
     ism.check_status(DEV)
@@ -51,3 +53,31 @@ def test_head_pairs_match_the_static_walk():
     for i in range(copies):
         assert torch.equal(many[0][i * T:(i + 1) * T], few[0])
         assert torch.equal(many[1][:, i * T:(i + 1) * T], few[1])
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(8, 2, 128), (3, 3, 128), (6, 2, 64)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_planned_forwards_leave_the_plan_alone(hq, hkv, d, rope):
+    """Forwards on one plan from two streams at once: the plan's bytes stay what
+    the build wrote, and every result is the plain call's."""
+    w = wl.Workload("dyn", wl.pack(RAGGED * 6), hq, hkv, d, "bf16", d ** -0.5, 1.0, 23)
+    x = [t.to(DEV) for t in wl.attention_tensors(w, with_dout=False)]
+    segs = ism.Segments.from_workload(w.segs, DEV)
+    tables = tuple(torch.from_numpy(t).to(DEV) for t in wl.rope_tables(900, d)) if rope else ()
+    call = ism.fwd_rope if rope else ism.fwd
+    ref = call(segs, *x, *tables, w.softmax_scale)
+    plan = ism.Plan(segs, hq, hkv, d, torch.bfloat16, DEV)
+    torch.cuda.synchronize()
+    before = plan.buffer.clone()
+    streams = [torch.cuda.Stream(DEV) for _ in range(2)]
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(20):
+        for s in streams:
+            with torch.cuda.stream(s):
+                outs.append(call(segs, *x, *tables, w.softmax_scale, plan=plan))
+    torch.cuda.synchronize()
+    ism.check_status(DEV)
+    assert torch.equal(plan.buffer, before)
+    for out in outs:
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))

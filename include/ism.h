@@ -85,10 +85,13 @@ typedef struct {
  * workspace queries.  The tensor-core kernels serve bf16 at head_dim 64 and
  * 128 and e4m3 at head_dim 128; fp32 runs the CUDA-core kernels, and so does a
  * single-token step at head_dim 64.  At head_dim 64 P and dS are kept to 16
- * mantissa bits (two bf16 parts), at 128 to bf16.  As at head_dim 128, a key
- * tile of 128 rows is read whole: NaN or Inf in K, V, Q or dO rows of a tile
- * reaches the results of other rows of that tile.  softmax_scale multiplies q.k before the softmax (the paper omits
- * the factor, Section 2.1; 1/sqrt(head_dim) is the usual choice). */
+ * mantissa bits (two bf16 parts), at 128 to bf16.  At head_dim 64, and for fp32,
+ * a NaN or Inf in Q, K, V or dO reaches only the results of rows that see it (or
+ * that it sees); the bf16 and e4m3 kernels of head_dim 128 read whole tiles of
+ * 128 rows, and it reaches the other rows of its tile too, those of the next
+ * dialogue in the buffer included.  softmax_scale multiplies q.k before the
+ * softmax (the paper omits the factor, Section 2.1; 1/sqrt(head_dim) is the
+ * usual choice). */
 typedef struct {
   int32_t num_heads_q;
   int32_t num_heads_kv;

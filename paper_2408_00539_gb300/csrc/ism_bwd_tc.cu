@@ -19,6 +19,7 @@
 // Warp roles in both MMA kernels: warps 0..7 compute (two warpgroups, each
 // owning 64 of the 128 columns of a tile; thread = TMEM lane = tile row),
 // warp 8 loads (TMA), warp 9 owns TMEM and issues the MMAs.
+#include "ism_rows64.cuh"
 #include "ism_tc_common.cuh"
 
 namespace ism {
@@ -155,7 +156,8 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 template <int kHD>
 __global__ void __launch_bounds__(kThreads, 1)
     dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
-              const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
+              const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+              const __grid_constant__ AttnArgs a) {
   using namespace dq;
   using L = Layout<kHD>;
   extern __shared__ uint8_t smem_raw[];
@@ -423,6 +425,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         store_slice32(w0, g0 + 64 * wg, rstride, g_rows);
         store_slice32(w1, g0 + 64 * wg + 32, rstride, g_rows);
       }
+      if constexpr (kHD == 64) {
+        float bad = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) bad = rows64::not_finite(q1[k], rows64::not_finite(q0[k], bad));
+        uint32_t rows = __ballot_sync(0xffffffffu, valid && bad != 0.f);
+        if (rows) __syncwarp();  // (a row's first store may be another lane's)
+        for (; rows; rows &= rows - 1) {
+          const int t = __ffs(rows) - 1;
+          const int32_t q_row = (int32_t)grow - lane + t;
+          float2 x = rows64::dq_row(a, q_row, w.k_base, h, __shfl_sync(0xffffffffu, ke, t),
+                                    __shfl_sync(0xffffffffu, lse2, t), __shfl_sync(0xffffffffu, dl, t));
+          x = make_float2(x.x * a.scale, x.y * a.scale);
+          __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.dq) + q_row * rstride + h * kHD;
+          if (a.rope_cos) rows64::store_row_back(dst, x, a, row - lane + t);
+          else rows64::store_row(dst, x);
+        }
+      }
     }
   }
   ptx::tc_fence_before();
@@ -472,7 +491,8 @@ static_assert(Layout<128>::kSmemBytes <= 232448, "shared memory per CTA");
 template <int kHD>
 __global__ void __launch_bounds__(dkv::kThreads, 1)
     dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
-                const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
+                const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+              const __grid_constant__ AttnArgs a) {
   using namespace dkv;
   using L = Layout<kHD>;
   extern __shared__ uint8_t smem_raw[];
@@ -986,6 +1006,7 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
       const int g_rows = x.w.k_len - (key - (lane & 3));
       __nv_bfloat16* const dvg = reinterpret_cast<__nv_bfloat16*>(a.dv) + grow * rstride + x.g * kHD;
       __nv_bfloat16* const dkg = reinterpret_cast<__nv_bfloat16*>(a.dk) + grow * rstride + x.g * kHD;
+      float bad = 0.f;  // NaN where an accumulator of the row is not finite (head_dim 64)
       if (wg == 1 && a.rope_cos) {
 #pragma unroll 1
         for (int q2 = 0; q2 < kHD / 64; ++q2) {
@@ -995,6 +1016,9 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           ptx::tmem_ld_wait();
           ptx::reg_fence(lo);
           ptx::reg_fence(hi);
+          if constexpr (kHD == 64)
+#pragma unroll
+            for (int k = 0; k < 32; ++k) bad = rows64::not_finite(hi[k], rows64::not_finite(lo[k], bad));
           float rc[32], rs[32];
           if (kvalid) {
             rope_row<32, kHD == 128>(a.rope_cos + (int64_t)key * (kHD / 2) + 32 * q2,
@@ -1008,20 +1032,38 @@ __global__ void __launch_bounds__(dkv::kThreads, 1)
           store_slice32(wl, dkg + q2 * 32, rstride, g_rows);
           store_slice32(wh, dkg + kHD / 2 + q2 * 32, rstride, g_rows);
         }
-        ptx::tc_fence_before();
-        continue;
-      }
-      // warpgroup 0 writes dV, warpgroup 1 writes dK (scaled)
+      } else {
+        // warpgroup 0 writes dV, warpgroup 1 writes dK (scaled)
 #pragma unroll 1
-      for (int q4 = 0; q4 < kHD / 32; ++q4) {
-        uint32_t v[32], w[16];
-        ptx::tmem_ld32(tmem + lane_addr + (wg == 0 ? TM_DV : TM_DK) + 32 * q4, v);
-        ptx::tmem_ld_wait();
-        ptx::reg_fence(v);
-        pack_scaled32(v, wg == 0 ? 1.f : a.scale, w);
-        store_slice32(w, (wg == 0 ? dvg : dkg) + 32 * q4, rstride, g_rows);
+        for (int q4 = 0; q4 < kHD / 32; ++q4) {
+          uint32_t v[32], w[16];
+          ptx::tmem_ld32(tmem + lane_addr + (wg == 0 ? TM_DV : TM_DK) + 32 * q4, v);
+          ptx::tmem_ld_wait();
+          ptx::reg_fence(v);
+          if constexpr (kHD == 64)
+#pragma unroll
+            for (int k = 0; k < 32; ++k) bad = rows64::not_finite(v[k], bad);
+          pack_scaled32(v, wg == 0 ? 1.f : a.scale, w);
+          store_slice32(w, (wg == 0 ? dvg : dkg) + 32 * q4, rstride, g_rows);
+        }
       }
       ptx::tc_fence_before();
+      if constexpr (kHD == 64) {
+        uint32_t rows = __ballot_sync(0xffffffffu, kvalid && bad != 0.f);
+        if (rows) __syncwarp();  // (a row's first store may be another lane's)
+        for (; rows; rows &= rows - 1) {
+          const int krow = key - lane + __ffs(rows) - 1;
+          float2 g = rows64::dkdv_row(a, x.w.q_base, x.w.q_len, x.w.k_base, x.w.kv_base, x.g, krow, wg == 1);
+          const int64_t off = ((int64_t)x.w.k_base + krow) * rstride + x.g * kHD;
+          if (wg == 0) {
+            rows64::store_row(static_cast<__nv_bfloat16*>(a.dv) + off, g);
+            continue;
+          }
+          g = make_float2(g.x * a.scale, g.y * a.scale);
+          if (a.rope_cos) rows64::store_row_back(static_cast<__nv_bfloat16*>(a.dk) + off, g, a, krow);
+          else rows64::store_row(static_cast<__nv_bfloat16*>(a.dk) + off, g);
+        }
+      }
     }
     if (!ok) set_abort(&bar->abort);
   }

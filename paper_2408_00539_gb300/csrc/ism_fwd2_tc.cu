@@ -19,6 +19,7 @@
 // kernel (Eq. e_ISM with the bound of Eq. fj; full tiles unmasked).
 #include <cfloat>
 
+#include "ism_rows64.cuh"
 #include "ism_tc_common.cuh"
 
 namespace ism {
@@ -159,7 +160,7 @@ __device__ __forceinline__ int64_t unit_of(int64_t k, int64_t n_units) {
 template <bool kTilePairs, bool kE4M3, bool kSplit, int kHD, bool kDyn>
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                    const __grid_constant__ CUtensorMap tmV, const AttnArgs a, int64_t n_units) {
+                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AttnArgs a, int64_t n_units) {
   static_assert(kHD == 128 || (kHD == 64 && !kE4M3), "head sizes of the paired forward");
   static_assert(!(kSplit && kDyn), "split launches walk statically");
   using L = PairLayout<kE4M3, kHD>;
@@ -582,17 +583,33 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (nkbm > 0) {
           const float f = kE4M3 ? a.v_descale : 1.f;
           float4* dst = reinterpret_cast<float4*>(a.part_o + pu * kHD);
+          float bad = 0.f;
 #pragma unroll 1
           for (int c = 0; c < kHD / 32; ++c) {
             uint32_t o[32];
             ptx::tmem_ld32(tO + c * 32, o);
             ptx::tmem_ld_wait();
             ptx::reg_fence(o);
+            if constexpr (kHD == 64)
+#pragma unroll
+              for (int i = 0; i < 32; ++i) bad = rows64::not_finite(o[i], bad);
             if (valid)
 #pragma unroll
               for (int i = 0; i < 8; ++i)
                 dst[c * 8 + i] = make_float4(__uint_as_float(o[4 * i]) * f, __uint_as_float(o[4 * i + 1]) * f,
                                              __uint_as_float(o[4 * i + 2]) * f, __uint_as_float(o[4 * i + 3]) * f);
+          }
+          if constexpr (kHD == 64) {
+            uint32_t rows = __ballot_sync(0xffffffffu, valid && bad != 0.f);
+            for (; rows; rows &= rows - 1) {
+              const int t = __ffs(rows) - 1;
+              const int k1 = min(__shfl_sync(0xffffffffu, ke, t), nkbm * kRows), k0 = x.jb * kRows;
+              const float2 acc = rows64::out_row(a, wm.q_base + row - lane + t, wm.k_base, h, k0, k0 + k1,
+                                                 __shfl_sync(0xffffffffu, m_use, t));
+              float* p = a.part_o + __shfl_sync(0xffffffffu, pu, t) * kHD + lane;
+              p[0] = acc.x;
+              p[32] = acc.y;
+            }
           }
         }
       } else if (nkbm > 0) {
@@ -602,14 +619,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int li = r & 3;
         const int64_t rstride = (int64_t)a.hq * kHD;
         __nv_bfloat16* const g0 = reinterpret_cast<__nv_bfloat16*>(a.out) + (orow - li) * rstride + h * kHD;
+        float bad = 0.f;
 #pragma unroll 1
         for (int c = 0; c < kHD / 32; ++c) {
           uint32_t o[32], w[16];
           ptx::tmem_ld32(tO + c * 32, o);
           ptx::tmem_ld_wait();
           ptx::reg_fence(o);
+          if constexpr (kHD == 64)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) bad = rows64::not_finite(o[i], bad);
           pack_scaled32(o, inv, w);
           store_slice32(w, g0 + 32 * c, rstride, wm.q_len - (row - li));
+        }
+        if constexpr (kHD == 64) {
+          uint32_t rows = __ballot_sync(0xffffffffu, valid && bad != 0.f);
+          if (rows) __syncwarp();  // (a row's first store may be another lane's)
+          for (; rows; rows &= rows - 1) {
+            const int t = __ffs(rows) - 1;
+            const int32_t q_row = (int32_t)orow - lane + t;
+            const float f = __shfl_sync(0xffffffffu, inv, t);
+            const float2 acc = rows64::out_row(a, q_row, wm.k_base, h, 0, __shfl_sync(0xffffffffu, ke, t),
+                                               __shfl_sync(0xffffffffu, m_use, t));
+            rows64::store_row(static_cast<__nv_bfloat16*>(a.out) + (int64_t)q_row * rstride + h * kHD,
+                              make_float2(acc.x * f, acc.y * f));
+          }
         }
         if (valid && a.lse) a.lse[(int64_t)h * a.q_rows + orow] = (m_use + log2f(l)) * kLn2;
       }

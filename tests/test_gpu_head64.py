@@ -103,3 +103,78 @@ def test_append(hq, hkv, ln):
         qf = torch.cat([torch.zeros((int(c), hq, D), dtype=torch.bfloat16), q[b]])
         ref = orc.attn_fwd(qf, *full, whole, D ** -0.5)[0][c:]
         assert _rel(o[b], ref) <= REL
+
+
+def _cuda_cores(monkeypatch, call):
+    monkeypatch.setenv("ISM_FORCE_CUDA_CORES", "1")
+    ism.load().ism_debug_reload_env()
+    try:
+        return call()
+    finally:
+        monkeypatch.delenv("ISM_FORCE_CUDA_CORES")
+        ism.load().ism_debug_reload_env()
+
+
+def _same_reach(got, ref, rel=2 * REL):
+    """NaN and Inf in the same places, and the finite values those of the
+    reference to within both roundings."""
+    a, b = (t.double().cpu().numpy() for t in (got, ref))
+    assert np.array_equal(np.isnan(a), np.isnan(b))
+    inf = np.isinf(a)
+    assert np.array_equal(inf, np.isinf(b)) and np.array_equal(a[inf], b[inf])
+    ok = np.isfinite(a)
+    assert np.linalg.norm(a[ok] - b[ok]) <= rel * np.linalg.norm(b[ok])
+    return ok.mean()
+
+
+BAD = [("q", "nan"), ("k", "nan"), ("v", "nan"), ("do", "nan"), ("v", "inf"), ("do", "inf"), ("k", "-inf")]
+
+
+@pytest.mark.parametrize("name,value", BAD)
+@pytest.mark.parametrize("hq,hkv,rope", [(4, 2, False), (3, 1, False), (4, 2, True)])
+def test_reach_of_nan_and_inf(monkeypatch, name, value, hq, hkv, rope):
+    """A NaN or Inf in one row reaches what the mask lets it reach and nothing
+    beside it, neither in its own dialogue nor in its neighbours'.  Reference:
+    the CUDA-core kernels, which read visible rows only."""
+    w = wl.Workload("d64", wl.pack([([50], [1]), ([30, 400], [0, 1]), ([50], [0]), ([260], [1])]), hq, hkv, D, "bf16",
+                    D ** -0.5, 1.0, 14)
+    x = dict(zip(("q", "k", "v", "do"), wl.attention_tensors(w)))
+    x[name][50 + 150, 0] = float(value)
+    segs = ism.Segments.from_workload(w.segs, DEV)
+    q, k, v, do = (t.to(DEV) for t in x.values())
+    tables = tuple(torch.from_numpy(t).to(DEV) for t in wl.rope_tables(500, D))
+
+    def step():
+        if rope:
+            o, lse, qr, kr = ism.fwd_rope(segs, q, k, v, *tables, w.softmax_scale)
+            out = (o, lse, *ism.bwd_rope(segs, qr, kr, v, o, lse, do, *tables, w.softmax_scale))
+        else:
+            o, lse = ism.fwd(segs, q, k, v, w.softmax_scale)
+            out = (o, lse, *ism.bwd(segs, q, k, v, o, lse, do, w.softmax_scale))
+        ism.check_status(DEV)
+        return out
+
+    got, ref = step(), _cuda_cores(monkeypatch, step)
+    finite = [_same_reach(a, b, 1e-5 if i == 1 else 2 * REL) for i, (a, b) in enumerate(zip(got, ref))]
+    assert 0.4 < min(finite) < 1.0
+
+
+@pytest.mark.parametrize("hq,hkv,cached", [(4, 2, 3000), (4, 2, 10), (3, 1, 1000)])
+@pytest.mark.parametrize("value", ["nan", "inf"])
+def test_reach_in_an_append(monkeypatch, hq, hkv, cached, value):
+    """A bad value row among the new ones: earlier rows of the chunk do not see it."""
+    ln, lens = 150, np.array([cached], np.int32)
+    gen = torch.Generator().manual_seed(7)
+    new = [torch.randn((1, ln, h, D), generator=gen).bfloat16() for h in (hq, hkv, hkv)]
+    caches = [torch.randn((1, cached + ln, hkv, D), generator=gen).bfloat16() for _ in range(2)]
+    new[2][0, 60, 0] = float(value)
+
+    def call():
+        o, lse = ism.prefill_append(*(t.to(DEV) for t in new + caches), torch.from_numpy(lens.copy()).to(DEV), lens,
+                                    [ln], [1], D ** -0.5)
+        ism.check_status(DEV)
+        return o, lse
+
+    got, ref = call(), _cuda_cores(monkeypatch, call)
+    assert 0.3 < _same_reach(got[0], ref[0]) < 1.0
+    assert _same_reach(got[1], ref[1], 1e-5) == 1.0

@@ -74,8 +74,6 @@ struct DecCfg {
   static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 };
 
-constexpr int kLensCopied = 128;
-
 struct Bars {
   uint64_t full[kMaxStages], empty[kMaxStages];
   uint64_t q_full[2], q_empty[2];
@@ -89,7 +87,6 @@ struct Bars {
   // per item parity: warp 0's epilogue of item u reads them while the other
   // warps may already fold the scores of item u + 1
   float red_m[2][4][kHeadsPad], red_l[2][4][kHeadsPad];
-  int32_t lens[kLensCopied];  // cached keys of the first sequences
 };
 static_assert(sizeof(Bars) <= 2048, "barrier block");
 
@@ -121,18 +118,13 @@ struct DecWalk {
 // they are right in L2, whatever an SM's L1 holds.
 __device__ __forceinline__ int32_t cached(const DecodeArgs& a, int b) { return ld_gpu(a.cache_len + b); }
 
-// The same from the block's copy of the first ones (a read of L2 by every warp of
-// every CTA costs 40 ragged caches 0.9 us of a step's 66.5).
-__device__ __forceinline__ int32_t cached(const DecodeArgs& a, const int32_t* lens, int b) {
-  return b < kLensCopied ? lens[b] : cached(a, b);
-}
-
 // The whole warp: finds the (b, g) of the CTA's first tile.
 template <bool kRow>
-__device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a, const int32_t* lens) {
+__device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
   DecWalk w;
   if constexpr (!kRow) {
     w.item = blockIdx.x;
+    w.b = -1;
     return w;
   }
   w.t = (int)(blockIdx.x / a.lanes) * a.tpc;
@@ -142,57 +134,45 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a, const int32_t* 
   const int row_heads = a.hkv / a.lanes;
   const int lane = threadIdx.x & 31;
   // (a single sequence needs no search: 8 steps over 3000 keys 87.8 -> 85.4 us)
-  for (int base = 0; a.batch > 1 && base < a.batch; base += 128) {
-    // four sequences a lane, in order
-    int n[4], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int b = base + lane * 4 + i;
-      n[i] = b < a.batch ? dec_alloc_tiles(a, dec_tiles(cached(a, lens, b))) * row_heads : 0;
-      sum += n[i];
-    }
-    int incl = sum;
+  for (int base = 0; a.batch > 1 && base < a.batch; base += 32) {
+    // a sequence a lane (every warp of every CTA reads the same few lines of L2:
+    // with four a lane, in order, 40 ragged caches took 0.7 us a step more)
+    const int b = base + lane;
+    const int n = b < a.batch ? dec_alloc_tiles(a, dec_tiles(cached(a, b))) * row_heads : 0;
+    int incl = n;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int x = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += x;
     }
     const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (w.t >= sb + total && base + 128 < a.batch) {
+    if (w.t >= sb + total && base + 32 < a.batch) {
       sb += total;
       continue;
     }
-    int at = sb + incl - sum, found = -1, start = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (w.t >= at && w.t < at + n[i]) {
-        found = base + lane * 4 + i;
-        start = at;
-      }
-      at += n[i];
-    }
-    const uint32_t who = __ballot_sync(0xffffffffu, found >= 0);
+    const int at = sb + incl - n;
+    const uint32_t who = __ballot_sync(0xffffffffu, w.t >= at && w.t < at + n);
     if (!who) {
       w.end = w.t;  // past the last tile: nothing to do
       break;
     }
     const int src = __ffs(who) - 1;
-    w.b = __shfl_sync(0xffffffffu, found, src);
-    sb = __shfl_sync(0xffffffffu, start, src);
+    w.b = base + src;
+    sb = __shfl_sync(0xffffffffu, at, src);
     break;
   }
   if (w.b >= a.batch) {
     w.b = 0;
     w.end = w.t;
   }
-  w.len = cached(a, lens, w.b) + 1;
+  w.len = cached(a, w.b) + 1;
   const int per_head = dec_alloc_tiles(a, (w.len + 127) / 128);
   w.g = w.t < w.end ? (w.t - sb) / per_head : 0;
   w.s = sb + w.g * per_head;
   return w;
 }
 template <bool kRow, int kSub>
-__device__ __forceinline__ bool dec_next(const DecodeArgs& a, const int32_t* lens, DecWalk& w, DecItem& x) {
+__device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecItem& x) {
   if constexpr (!kRow) {
     // item = (split * batch + b) * hkv + g: consecutive CTAs take the KV heads of
     // one (sequence, split), whose rows lie side by side in the cache
@@ -205,7 +185,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, const int32_t* len
     x.b = (int)(rest % a.batch);
     x.slot = (int)(rest / a.batch);
     x.k0 = x.slot * a.chunk;
-    w.len = cached(a, lens, x.b) + 1;
+    if (x.b != w.b) w.len = cached(a, w.b = x.b) + 1;
     x.k1 = min(w.len, x.k0 + a.chunk);
     x.nsub = x.k1 > x.k0 ? (x.k1 - x.k0 + 127) / 128 : 0;
     x.nt = (x.nsub + kSub - 1) / kSub;
@@ -220,7 +200,7 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, const int32_t* len
         if (++w.g == a.hkv / a.lanes) {
           w.g = 0;
           if (++w.b >= a.batch) return false;
-          w.len = cached(a, lens, w.b) + 1;
+          w.len = cached(a, w.b) + 1;
         }
         continue;
       }
@@ -310,8 +290,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tmem_alloc(&bar->tmem_base, kTmemCols);
     ptx::tmem_relinquish();
   }
-  if (warp == kLoadWarp)
-    for (int b = lane; b < min(a.batch, kLensCopied); b += 32) bar->lens[b] = cached(a, b);
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
@@ -336,15 +314,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       ptx::tma_prefetch_desc(&tmK);
       ptx::tma_prefetch_desc(&tmV);
     }
-    DecWalk walk = dec_walk<kRow>(a, bar->lens);
+    DecWalk walk = dec_walk<kRow>(a);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
       if (!kRow && x.nt == 0) continue;
       const bool last_item = x.k1 == walk.len;  // it has the cache's last tile
       // rows of the item's sub-tiles in the K / V tensors, one a lane: a 128-key
       // sub-tile starts at a multiple of 128 keys and lies in one page.  (Table
       // entries as they come, one from L2 in front of each copy: 40 ragged paged
-      // caches 73.3 us a step, all of an item at once 66.5.)
+      // caches 73.3 us a step, all of an item at once 66.)
       const int64_t p = (int64_t)x.k0 + lane * 128;
       int64_t row = (int64_t)x.b * a.cap + p;
       if (a.pages.table)
@@ -424,9 +402,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t idesc_pv = kE4M3 ? ptx::idesc_e4m3_f32(128, 128, 1, 1) : ptx::idesc_bf16_f32(128, 128, 1, 1);
     uint32_t nl = 0, nu = 0, T = 0, TS = 0;  // ring tiles consumed; non-empty items; P tiles; S tiles
     bool ok = true;
-    DecWalk walk = dec_walk<kRow>(a, bar->lens);
+    DecWalk walk = dec_walk<kRow>(a);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
       if (!kRow && x.nt == 0) continue;
       const uint32_t qb = nu & 1;
       // Q landed; the softmax warps have read the previous item's S
@@ -513,9 +491,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int group = a.group;
     uint32_t nu = 0, T = 0, TS = 0;
     bool ok = true;
-    DecWalk walk = dec_walk<kRow>(a, bar->lens);
+    DecWalk walk = dec_walk<kRow>(a);
     DecItem x;
-    while (ok && dec_next<kRow, kSub>(a, bar->lens, walk, x)) {
+    while (ok && dec_next<kRow, kSub>(a, walk, x)) {
       const int64_t pbase = ((int64_t)x.b * a.hq + (int64_t)x.g * group) * a.splits + x.slot;
       if (!kRow && x.nt == 0) {
         // a split past the sequence's keys: a partial the combine skips

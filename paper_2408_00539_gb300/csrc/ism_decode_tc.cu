@@ -96,6 +96,10 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 __device__ __forceinline__ bool aborted(const int32_t* f) { return *reinterpret_cast<const volatile int32_t*>(f) != 0; }
 __device__ __forceinline__ void set_abort(int32_t* f) { *reinterpret_cast<volatile int32_t*>(f) = 1; }
 
+// Floats of a row of O in shared memory: the 16-byte stores of eight lanes, a
+// row each, hit all banks.
+constexpr int kOutRow = kD + 4;
+
 struct DecItem {
   int b, g, k0, k1;
   int slot;  // of the partial result among those of (b, g)
@@ -228,9 +232,15 @@ __device__ __forceinline__ bool dec_next(const DecodeArgs& a, DecWalk& w, DecIte
 
 // The P operand is stored MN-major (128-byte swizzled rows = keys, the heads
 // contiguous along a row, as the V tile stores dimensions): the thread of key
-// k writes its 16 heads as whole 16-byte chunks (bf16: chunks 0 and 1 of the
-// row, e4m3: chunk 0), swizzled by k & 7.  Heads past 16 (M up to 128) are
-// never written; they only feed output rows that are not read.
+// k writes its rows as whole 16-byte chunks of the 128 (eight heads in bf16, 16 in
+// e4m3), swizzled by k & 7.  Rows past the last (M up to 128) are never written;
+// they only feed output rows that are not read.
+// In the row split P goes in two parts, hi = bf16(p) of head h in row h and
+// bf16(p - hi) in row kG + h: which of a cache's keys share an item, and with it
+// the maximum that P is rounded against, is up to the lengths of all caches there,
+// and with P to 16 bits that choice no longer shows in the result.  The MMAs are
+// the same (M = 128 either way): 40 ragged caches 66.5 -> 66.7 us a step, one of
+// 3000 keys 10.8 -> 11.0.
 __device__ __forceinline__ uint32_t p_chunk(uint32_t k, uint32_t c) { return k * 128u + ((c ^ (k & 7u)) << 4); }
 
 // The scores of the first G heads of a 128-key sub-tile (thread = key).
@@ -253,6 +263,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                      const __grid_constant__ CUtensorMap tmV, const DecodeArgs a) {
   using Cfg = DecCfg<kE4M3>;
   constexpr int kStages = Cfg::kStages, kSub = Cfg::kSub;
+  constexpr int kParts = kRow ? 2 : 1;  // of P (bf16)
+  static_assert(kParts * kG <= 32, "the epilogue's warp reads 32 rows of O");
+  constexpr uint32_t OFF_O = Cfg::OFF_BAR + 2048;  // the rows of O on their way out (row split)
   static_assert(!(kE4M3 && kRow), "e4m3 keeps equal chunks");
   static_assert(kMaxTiles <= 32, "a lane for each sub-tile of an item");
   constexpr uint32_t kTile = Cfg::kTile, kSubBytes = Cfg::kSubBytes, kQHalf = Cfg::kQHalf, kQBytes = Cfg::kQBytes;
@@ -592,19 +605,28 @@ __global__ void __launch_bounds__(kThreads, 1)
           ptx::tmem_ld_wait();
           ptx::reg_fence(v);
           const bool valid = x.k0 + t * 128 + r < x.k1;
-          uint32_t pk[kHeadsPad / 2] = {};  // heads past kG: zero
+          uint32_t pk[kParts * kG / 2];
 #pragma unroll
           for (int h = 0; h < kG; h += 2) {
             const float p0 = (valid && h < group) ? ex2(__uint_as_float(v[h]) * c2 - m2[h]) : 0.f;
             const float p1 = (valid && h + 1 < group) ? ex2(__uint_as_float(v[h + 1]) * c2 - m2[h + 1]) : 0.f;
             pk[h >> 1] = pack_bf16(p0, p1);
-            l[h] += __uint_as_float(pk[h >> 1] << 16);  // the sum of the P that enters P V
-            l[h + 1] += __uint_as_float(pk[h >> 1] & 0xFFFF0000u);
+            if constexpr (kParts == 2) {
+              pk[(kG + h) >> 1] = pack_bf16_rest(p0, p1, pk[h >> 1]);
+              l[h] += p0;
+              l[h + 1] += p1;
+            } else {
+              l[h] += __uint_as_float(pk[h >> 1] << 16);  // the sum of the P that enters P V
+              l[h + 1] += __uint_as_float(pk[h >> 1] & 0xFFFF0000u);
+            }
           }
-          *reinterpret_cast<uint4*>(P + p_chunk((uint32_t)r, 0u)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          // heads 8-15 feed only output rows that are not read when kG is 8 or less
-          if constexpr (kG > 8)
-            *reinterpret_cast<uint4*>(P + p_chunk((uint32_t)r, 1u)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          // eight rows a chunk; those past kParts * kG feed only output rows that are not read
+#pragma unroll
+          for (int c = 0; c < (kParts * kG + 7) / 8; ++c) {
+            const bool all = 8 * c + 8 <= kParts * kG;
+            *reinterpret_cast<uint4*>(P + p_chunk((uint32_t)r, (uint32_t)c)) =
+                make_uint4(pk[4 * c], pk[4 * c + 1], all ? pk[4 * c + 2] : 0u, all ? pk[4 * c + 3] : 0u);
+          }
         }
         ptx::fence_proxy_async_smem();
         ptx::mbar_arrive(&bar->p_ready[pb]);
@@ -627,27 +649,63 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       if (warp == 0) {
-        // epilogue: lane h holds row h of O = the unnormalised output of head h
+        // epilogue: lane h holds row h of O = the unnormalised output of head h (lane
+        // kG + h what the low part of its P adds)
         if (!wait(&bar->o_full, nu & 1, a.status)) {
           ok = false;
           break;
         }
         ptx::tc_fence_after();
         const bool mine = lane < group;
-        float* dst = a.part_o + (pbase + (int64_t)(mine ? lane : 0) * a.splits) * kD;
+        if constexpr (kParts == 2) {
+          // through shared memory: the two parts of a head's row are added and
+          // stored a whole row an instruction.  A low part that is not finite is left
+          // out: an Inf in V has its sign from the high part.
+          auto add = [](float hi, float lo) { return fabsf(lo) < INFINITY ? hi + lo : hi; };
+          float* rows = reinterpret_cast<float*>(smem + OFF_O);
 #pragma unroll 1
-        for (int q4 = 0; q4 < 4; ++q4) {
-          uint32_t o[32];
-          ptx::tmem_ld32(tmem + TM_O + 32u * q4, o);
-          ptx::tmem_ld_wait();
-          ptx::reg_fence(o);
-          if (mine) {
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t o[32];
+            ptx::tmem_ld32(tmem + TM_O + 32u * q4, o);
+            ptx::tmem_ld_wait();
+            ptx::reg_fence(o);
+            if (lane < 2 * kG) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              reinterpret_cast<float4*>(dst + 32 * q4)[i] =
-                  make_float4(__uint_as_float(o[4 * i]) * o_scale, __uint_as_float(o[4 * i + 1]) * o_scale,
-                              __uint_as_float(o[4 * i + 2]) * o_scale, __uint_as_float(o[4 * i + 3]) * o_scale);
+              for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<uint4*>(rows + lane * kOutRow + 32 * q4 + 4 * i) =
+                    make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+            }
           }
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(&bar->o_free);
+          __syncwarp();
+#pragma unroll
+          for (int h = 0; h < kG; ++h)
+            if (h < group) {
+              const float4 x = *reinterpret_cast<const float4*>(rows + h * kOutRow + 4 * lane);
+              const float4 y = *reinterpret_cast<const float4*>(rows + (kG + h) * kOutRow + 4 * lane);
+              reinterpret_cast<float4*>(a.part_o + (pbase + (int64_t)h * a.splits) * kD)[lane] =
+                  make_float4(add(x.x, y.x), add(x.y, y.y), add(x.z, y.z), add(x.w, y.w));
+            }
+          __syncwarp();
+        } else {
+          float* dst = a.part_o + (pbase + (int64_t)(mine ? lane : 0) * a.splits) * kD;
+#pragma unroll 1
+          for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t o[32];
+            ptx::tmem_ld32(tmem + TM_O + 32u * q4, o);
+            ptx::tmem_ld_wait();
+            ptx::reg_fence(o);
+            if (mine) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                reinterpret_cast<float4*>(dst + 32 * q4)[i] =
+                    make_float4(__uint_as_float(o[4 * i]) * o_scale, __uint_as_float(o[4 * i + 1]) * o_scale,
+                                __uint_as_float(o[4 * i + 2]) * o_scale, __uint_as_float(o[4 * i + 3]) * o_scale);
+            }
+          }
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(&bar->o_free);
         }
         if (mine) {
           float mh = -INFINITY, lh = 0.f;
@@ -659,8 +717,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           a.part_ml[(pbase + (int64_t)lane * a.splits) * 2] = mh * c2;
           a.part_ml[(pbase + (int64_t)lane * a.splits) * 2 + 1] = lh;
         }
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(&bar->o_free);
       }
       ++nu;
     }
@@ -688,8 +744,10 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     if ((e = make_tmap_bf16(&tk, a.k_cache, (uint64_t)a.hkv * kD, (uint64_t)a.kv_rows)) != cudaSuccess) return e;
     if ((e = make_tmap_bf16(&tv, a.v_cache, (uint64_t)a.hkv * kD, (uint64_t)a.kv_rows)) != cudaSuccess) return e;
   }
+  constexpr uint32_t smem = Cfg::kSmemBytes + (kRow ? 2 * kG * kOutRow * 4 : 0);
+  static_assert(smem <= 232448, "shared memory per CTA");
   if ((e = cudaFuncSetAttribute(decode_tc_kernel<kE4M3, kG, kRow>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Cfg::kSmemBytes)) != cudaSuccess)
+                                (int)smem)) != cudaSuccess)
     return e;
   int64_t grid;
   if constexpr (kRow) {
@@ -699,7 +757,7 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     grid = sms < n_items ? sms : n_items;
   }
   if (grid <= 0) return cudaSuccess;
-  return launch(true, decode_tc_kernel<kE4M3, kG, kRow>, grid, kThreads, Cfg::kSmemBytes, st, tq, tk, tv, a);
+  return launch(true, decode_tc_kernel<kE4M3, kG, kRow>, grid, kThreads, smem, st, tq, tk, tv, a);
 }
 
 template <bool kE4M3, bool kRow>

@@ -4,9 +4,10 @@ at once, shares of one tile and of several items, caches at tile edges, and few
 long caches (each starting at a CTA's share).  Reference: the CUDA-core decode
 of the same step (ISM_DECODE_NO_TC=1, fp32 P) and the oracle for one of them.
 
-Tolerance: P is rounded to bf16 for P V (2^-9 of independent terms) and the
-output to bf16 (2^-9), the reference rounds its output (2^-9): 3 * 2^-9 in the
-2-norm; LSE 2^-9, as its sum is of the rounded P (each term off by at most 2^-9).
+Tolerance: in equal chunks P is rounded to bf16 for P V (2^-9 of independent
+terms) and the output to bf16 (2^-9), the reference rounds its output (2^-9):
+3 * 2^-9 in the 2-norm; LSE 2^-9, as its sum is of the rounded P (each term off by
+at most 2^-9).  The row split keeps P to 16 bits.
 """
 import numpy as np
 import pytest
@@ -96,3 +97,26 @@ def test_paged_matches_contiguous(page):
                                  torch.from_numpy(lens.copy()).to(DEV), lens, [1], [1], 0.09)
     ism.check_status(DEV)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("hq,hkv", [(8, 2), (16, 2), (32, 2)])
+@pytest.mark.parametrize("value", [None, "inf", "nan"])
+def test_values_to_16_bits(monkeypatch, hq, hkv, value):
+    """The row split keeps P to 16 bits: against the CUDA-core decode (fp32 P)
+    only output roundings differ where the two sums fall on either side of a
+    boundary, so the 2-norm of the difference stays far below one rounding
+    (2^-12; a bf16 P gives 1.5e-3).  An Inf or NaN among the values comes out
+    as there."""
+    lens = [700, 3000, 130, 1900]
+    gen = torch.Generator(device=DEV).manual_seed(11)
+    q, k, v = (torch.randn((4, 1, h, 128), generator=gen, device=DEV).bfloat16() for h in (hq, hkv, hkv))
+    kc, vc = (torch.randn((4, 3001, hkv, 128), generator=gen, device=DEV).bfloat16() for _ in range(2))
+    if value:
+        vc[1, 1500, 0, 7] = vc[3, 40, 1, 100] = float(value)
+    got, ref = (_step(monkeypatch, no_tc, lens, q, k, v, kc, vc) for no_tc in (False, True))
+    a, b = got[0].double(), ref[0].double()
+    ok = torch.isfinite(b)
+    assert torch.equal(torch.isnan(a), torch.isnan(b)) and torch.equal(torch.isinf(a), torch.isinf(b))
+    assert int((~ok).sum()) == (2 * (hq // hkv) if value else 0)
+    assert float((a - b)[ok].norm() / b[ok].norm()) <= 2.0 ** -12
+    assert float((got[1] - ref[1]).abs().max()) <= 1e-5

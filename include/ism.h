@@ -334,7 +334,12 @@ ism_status_t ism_attn_bwd_rope_planned(const ism_segments_t* segs, const ism_att
  *     the same for every sequence, last end == l_new, n_new_segs <= 256
  *   k_cache/v_cache [B, cache_capacity, Hkv, D] (dtype, in/out)
  *   cache_len [B] int32 device (in/out), cache_len_host [B] its host mirror;
- *     cache_len_host[b] + l_new <= cache_capacity is required.
+ *     cache_len_host[b] + l_new <= cache_capacity is required.  The launch is laid
+ *     out from the mirror, so it must hold the lengths that the kernels find: a
+ *     captured call replayed after the lengths have moved on is not supported
+ *     (only the bf16 single-token step at head_dim 128 whose caches differ in
+ *     length or are short covers all keys then; others stop where the mirror's
+ *     last chunk or part ends).
  *   o_new [B, l_new, Hq, D] (dtype, written); lse_new [Hq, B, l_new] fp32 or NULL.
  * If a cache ends inside a query segment its old rows would differ from a
  * full pass once the segment grows; the new rows are still exact.

@@ -1039,8 +1039,8 @@ bool decode_row(DecodeArgs& a, const int32_t* cache_len_host, int32_t batch, int
   }
   if (row >= (int64_t(1) << 31) - kDecTcTiles || slots > kMaxSplits) return false;
   a.tpc = (int32_t)tpc;
-  a.row_tiles = (int32_t)row;
-  a.splits = (int32_t)slots;
+  a.shares = (int32_t)((row + tpc - 1) / tpc);
+  a.splits = kMaxSplits;
   a.chunk = 0;
   return true;
 }

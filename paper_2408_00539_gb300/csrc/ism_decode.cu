@@ -435,15 +435,18 @@ __global__ void decode_combine_kernel(DecodeArgs a) {
     s = (a.batch > 1 ? a.start[b] : 0) + h / a.group / a.lanes * alloc;
     end = s + n;
     per_cta = (a.tpc + kDecTcTiles - 1) / kDecTcTiles;
-    c0 = s / a.tpc;
-    n_slots = min(((end - 1) / a.tpc - c0 + 1) * per_cta, a.splits);
+    c0 = dec_share(a, s);
+    const int c1 = dec_share(a, end - 1);
+    // (the last share has no end: as many items as it takes)
+    const int last = c1 < a.shares - 1 ? per_cta : (end - max(s, c1 * a.tpc) + kDecTcTiles - 1) / kDecTcTiles;
+    n_slots = min((c1 - c0) * per_cta + last, a.splits);
   }
-  // whether CTA c0 + slot / per_cta has a (slot % per_cta)-th item here
+  // whether share c0 + slot / per_cta (the last one: of the slots left) has such an item here
   auto used = [&](int slot) -> bool {
     if (slot >= n_slots) return false;
     if (!kRow || per_cta == 1) return true;
-    const int c = c0 + slot / per_cta;
-    return max(s, c * a.tpc) + slot % per_cta * kDecTcTiles < min(end, (c + 1) * a.tpc);
+    const int c = min(c0 + slot / per_cta, a.shares - 1);
+    return c == a.shares - 1 || max(s, c * a.tpc) + slot % per_cta * kDecTcTiles < min(end, (c + 1) * a.tpc);
   };
   const float* pml = a.part_ml + (int64_t)bh * a.splits * 2;
   // slots in chunks of eight with every load of a chunk issued before any use

@@ -131,8 +131,9 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
     w.b = -1;
     return w;
   }
-  w.t = (int)(blockIdx.x / a.lanes) * a.tpc;
-  w.end = min(w.t + a.tpc, a.row_tiles);
+  const int cta = (int)(blockIdx.x / a.lanes);
+  w.t = cta * a.tpc;
+  w.end = cta < a.shares - 1 ? w.t + a.tpc : INT32_MAX;  // (the last one to the end of the row)
   w.b = 0;
   int sb = 0;  // first tile of sequence w.b
   const int row_heads = a.hkv / a.lanes;
@@ -171,6 +172,7 @@ __device__ __forceinline__ DecWalk dec_walk(const DecodeArgs& a) {
   }
   w.len = cached(a, w.b) + 1;
   const int per_head = dec_alloc_tiles(a, (w.len + 127) / 128);
+  if (w.t >= sb + row_heads * per_head) w.end = w.t;
   w.g = w.t < w.end ? (w.t - sb) / per_head : 0;
   w.s = sb + w.g * per_head;
   return w;
@@ -751,7 +753,7 @@ cudaError_t launch_decode_tc_t(const DecodeArgs& a, cudaStream_t st) {
     return e;
   int64_t grid;
   if constexpr (kRow) {
-    grid = ((int64_t)a.row_tiles + a.tpc - 1) / a.tpc * a.lanes;
+    grid = (int64_t)a.shares * a.lanes;
   } else {
     const int64_t sms = sm_count(), n_items = (int64_t)a.batch * a.hkv * a.splits;
     grid = sms < n_items ? sms : n_items;

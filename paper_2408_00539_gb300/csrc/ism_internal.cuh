@@ -308,14 +308,16 @@ struct DecodeArgs {
   int32_t tc;            // tensor-core kernel (bf16 or e4m3, head_dim 128, group <= 16)
   // tpc == 0: equal chunks of a multiple of 128 keys (splits, chunk).  Else
   // (bf16, by decode_row) the 128-key tiles of all (sequence, head group) caches in
-  // one row of row_tiles, tpc of them per CTA, an item at most kDecTcTiles;
-  // splits = room for partials per (sequence, KV head).  align: each cache's
+  // one row of `shares` shares of tpc tiles, an item at most kDecTcTiles; splits =
+  // room for partials per (sequence, KV head).  The row is walked by the device's
+  // lengths, and the last share has no end: where they have outgrown the host's
+  // copy (a captured step replayed), it takes what the copy did not count.  align: each cache's
   // tiles are padded to a multiple of it in the row (1: not).  start [B]: written
   // with the first tile of each sequence in the row.
   // lanes: KV heads side by side; CTA i takes share i / lanes of head group g's
   // (head g * lanes + i % lanes) part of the row, so lanes neighbours read along
   // the same cache rows.
-  int32_t tpc, row_tiles, align, lanes;
+  int32_t tpc, shares, align, lanes;
   int32_t q_written;     // the queries come from the cache write (rotated)
   int32_t* start;
   uint32_t* status;      // device status word (bounded waits)
@@ -329,9 +331,14 @@ __host__ __device__ __forceinline__ int32_t dec_tiles(int32_t cached) { return (
 __host__ __device__ __forceinline__ int32_t dec_alloc_tiles(const DecodeArgs& a, int32_t tiles) {
   return a.align == 1 ? tiles : (tiles + a.align - 1) / a.align * a.align;
 }
-// Slot of the j-th item that CTA c has of the (sequence, KV head) whose tiles start at s.
+// The share that a tile of the row belongs to.
+__host__ __device__ __forceinline__ int32_t dec_share(const DecodeArgs& a, int32_t tile) {
+  const int32_t c = tile / a.tpc;
+  return c < a.shares ? c : a.shares - 1;
+}
+// Slot of the j-th item that share c has of the (sequence, KV head) whose tiles start at s.
 __host__ __device__ __forceinline__ int32_t dec_slot(const DecodeArgs& a, int32_t s, int32_t c, int32_t j) {
-  return (c - s / a.tpc) * ((a.tpc + kDecTcTiles - 1) / kDecTcTiles) + j;
+  return (c - dec_share(a, s)) * ((a.tpc + kDecTcTiles - 1) / kDecTcTiles) + j;
 }
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st);
 

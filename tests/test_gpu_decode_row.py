@@ -120,3 +120,29 @@ def test_values_to_16_bits(monkeypatch, hq, hkv, value):
     assert int((~ok).sum()) == (2 * (hq // hkv) if value else 0)
     assert float((a - b)[ok].norm() / b[ok].norm()) <= 2.0 ** -12
     assert float((got[1] - ref[1]).abs().max()) <= 1e-5
+
+
+@pytest.mark.parametrize("name", ["one_long", "ragged", "many_short", "edges"])
+@pytest.mark.parametrize("off", [-1000, -130, -1, 500])
+def test_host_lengths_that_lag(name, off):
+    """Lengths on the device that the host's copy does not know (a captured step
+    replayed): the keys past what the launch was laid out for go to the last
+    share, in place of being left out; a copy ahead of the device leaves shares
+    without keys.  Reference: the same step with the right copy, which shares
+    the tiles out otherwise (output roundings on either side of a boundary)."""
+    lens = np.array(CASES[name], np.int32)
+    gen = torch.Generator(device=DEV).manual_seed(3)
+    B, cap, hq, hkv = len(lens), int(lens.max()) + 600, 8, 2
+    x = [torch.randn((B, 1, h, 128), generator=gen, device=DEV).bfloat16() for h in (hq, hkv, hkv)]
+    caches = [torch.randn((B, cap, hkv, 128), generator=gen, device=DEV).bfloat16() for _ in range(2)]
+    out = []
+    for host in (lens, np.maximum(lens + off, 0)):
+        cl = torch.from_numpy(lens.copy()).to(DEV)
+        out.append(ism.prefill_append(*x, *(c.clone() for c in caches), cl, host, [1], [1], 128 ** -0.5))
+        ism.check_status(DEV)
+        assert np.array_equal(cl.cpu().numpy(), lens + 1)
+    a, b = out[1][0].double(), out[0][0].double()
+    err = (a - b).flatten(1).norm(dim=1) / b.flatten(1).norm(dim=1)
+    assert torch.isfinite(a).all() and float(err.max()) <= 2.0 ** -9
+    assert float((a - b).norm() / b.norm()) <= 2.0 ** -12
+    assert float((out[1][1] - out[0][1]).abs().max()) <= 1e-5

@@ -423,8 +423,8 @@ __global__ void __launch_bounds__(160) decode_tma_kernel(const __grid_constant__
 template <int D, bool kRow>
 __global__ void decode_combine_kernel(DecodeArgs a) {
   // the next step's cache write, which waits for this kernel, may be launched at once
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_trigger();
+  pdl_sync();
   const int bh = blockIdx.x;
   const int d = threadIdx.x;
   const int b = bh / a.hq, h = bh % a.hq;

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // row, and the values zeroed after it) and of rotated queries wait for the
   // write (every cache has a last tile, so this grid does not end before it).
   // The combine after this grid may start early and waits for it in turn.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_trigger();
 
   if (warp == kLoadWarp) {
     // ------------------------------------------------ TMA loads (the warp waits converged, lane 0 issues)
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t s = nl % kStages;
           const bool needs_q = pass == 0 && t == q_after;
           if (!written && ((last_item && t == x.nt - 1) || (needs_q && a.q_written))) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+            pdl_sync();
             written = true;
           }
           if (needs_q) load_q();

@@ -200,10 +200,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   ptx::tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
   // the set-up above overlaps the kernel before (a split launch lets the merge
-  // start only once every CTA is done: its blocks would take issue slots and
-  // registers of the running ones)
+  // start only once every warp of every CTA is done, at the end: its blocks
+  // would take issue slots and registers of the running ones)
   if constexpr (kSplit)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_sync();
   else
     pdl_wait();
   advance_cache_len(a);
@@ -650,9 +650,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!ok) set_abort(&bar->abort);
   }
-  if constexpr (kSplit) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   ptx::tc_fence_before();
   __syncthreads();
+  if constexpr (kSplit) pdl_trigger();  // (the first warp to do so speaks for the CTA)
   if (warp == 9) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, kTmemCols);

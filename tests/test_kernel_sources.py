@@ -82,3 +82,10 @@ def test_early_reads_go_to_l2():
     body = next(b for n, _, b in KERNELS if n == "delta_kernel")
     loads = re.findall(r"=([^;]*(?:\bO\b|\bdO\b)[^;]*);", body)
     assert len(loads) == 2 and all("__ldcg" in x for x in loads)
+
+
+def test_split_forward_triggers_behind_its_last_barrier():
+    """The merge behind a split forward starts when every warp is done: the
+    first thread of a block to trigger does so for the block."""
+    body = next(b for n, _, b in KERNELS if n == "fwd_pair_kernel")
+    assert body.rindex("pdl_trigger()") > body.rindex("__syncthreads()")

@@ -294,13 +294,17 @@ bool fwd_tile_pairs(const ism_attn_shape_t* sh) {
   return !knobs().fwd_one_head;
 }
 
-// Whether the metadata pass puts the query-tile pair heads at the front of
-// q_order: an odd group without a pair list of its own.  The head_dim 64
-// forward pairs tiles from there, so its workspaces and plans are those of the
-// CUDA-core kernels (which take any order), in size and in use: a plan built
-// for fp32 or under ISM_FORCE_CUDA_CORES=1 serves it and the other way round.
-bool pairs_first(const ism_attn_shape_t* sh) {
+// Whether a plan has the query-tile pair heads at the front of q_order: that of
+// an odd group without a pair list of its own.  The head_dim 64 forward pairs
+// tiles from there, so its plans are those of the CUDA-core kernels, in size and
+// in use: a plan built for fp32 or under ISM_FORCE_CUDA_CORES=1 serves it and the
+// other way round (the kernels that want the cost order read it by q_tile_at).
+bool plan_pairs_first(const ism_attn_shape_t* sh) {
   return (sh->num_heads_q / sh->num_heads_kv) % 2 != 0 && !fwd_tile_pairs(sh);
+}
+// The same of a forward's own metadata pass: only where that forward pairs.
+bool pairs_first(const ism_attn_shape_t* sh) {
+  return plan_pairs_first(sh) && use_tc(sh) && sh->head_dim == 64;
 }
 
 // dS tile slots of the stored-dS backward (pairs x query heads), or 0 where
@@ -557,7 +561,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
     k = k_rot;
   }
   // query-tile pairs: an odd group
-  const bool tile_pairs = L.pair_order || (use_tc(shape) && shape->head_dim == 64 && pairs_first(shape));
+  const bool tile_pairs = L.pair_order || pairs_first(shape);
   // A planned forward walks statically: a plan may serve forwards on several
   // streams at once, and the counter would have to lie in it.
   const bool dynamic = !pre && (use_tc(shape) || e4m3) &&
@@ -573,6 +577,7 @@ ism_status_t fwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.dependent = dependent_pass(c.nq, shape->num_heads_q);
   a.qk_descale = qk_descale; a.v_descale = v_descale;
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
+  a.order_pairs = pre && plan_pairs_first(shape) ? c.npairs : 0;
   a.pair_order = L.pair_order; a.npairs = L.pair_order ? c.npairs : 0;
   if (tile_pairs && !a.pair_order) {
     a.pair_order = L.q_order;
@@ -690,6 +695,7 @@ ism_status_t bwd_impl(const ism_segments_t* segs, const ism_attn_shape_t* shape,
   a.q_rows = info.total_tokens; a.scale = shape->softmax_scale;
   a.dependent = dependent_pass(c.nq, shape->num_heads_q);
   a.kv_end = L.kv_end; a.qtiles = L.qtiles; a.q_order = L.q_order; a.nq = c.nq;
+  a.order_pairs = pre && plan_pairs_first(shape) ? c.npairs : 0;
   a.ktiles = L.ktiles; a.k_order = L.k_order; a.nk = c.nk;
   a.ds = L.ds; a.kpair_off = L.kpair_off; a.ds_slots = L.ds ? slots : 0;
   a.work_counter = L.counters + kBwdCounter;
@@ -765,7 +771,7 @@ ism_status_t ism_attn_plan_build(const ism_segments_t* segs, const ism_attn_shap
   if ((r = check_ws(plan, plan_bytes, L.bytes)) != ISM_OK) return r;
   if (info.total_tokens > 0) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if ((r = build_pass_meta(segs, c, L, true, st, shape->num_heads_q, pairs_first(shape))) != ISM_OK) return r;
+    if ((r = build_pass_meta(segs, c, L, true, st, shape->num_heads_q, plan_pairs_first(shape))) != ISM_OK) return r;
   }
   plan_info->fingerprint = plan_fingerprint(segs, shape, tile_pairs);
   plan_info->bytes = L.bytes;

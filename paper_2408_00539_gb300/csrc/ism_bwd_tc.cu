@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int64_t tpos;
   int h;
   bucket_item(blockIdx.x, a.nq, a.hq, tpos, h, a.hq == a.hkv);  // blocks start roughly in index order
-  const Tile w = a.qtiles[a.q_order[tpos]];
+  const Tile w = a.qtiles[q_tile_at(a, tpos)];
   const int g = h / (a.hq / a.hkv);
   const int nkb = w.a1, kfull = w.a0;
 

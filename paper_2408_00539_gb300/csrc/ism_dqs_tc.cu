@@ -59,7 +59,7 @@ __device__ __forceinline__ Item decode(const AttnArgs& a, int64_t item) {
   Item it;
   int64_t tpos;
   bucket_item(item, a.nq, a.hq, tpos, it.h, a.hq == a.hkv);  // bucketed only when no two heads share K
-  const int gq = a.q_order[tpos];
+  const int gq = q_tile_at(a, tpos);
   it.w = a.qtiles[gq];
   it.g = it.h / (a.hq / a.hkv);
   it.nkb = it.w.a1;

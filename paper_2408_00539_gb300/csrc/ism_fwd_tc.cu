@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_sync();
   const int h = blockIdx.x % a.hq;
-  const Tile w = a.qtiles[a.q_order[blockIdx.x / a.hq]];
+  const Tile w = a.qtiles[q_tile_at(a, blockIdx.x / a.hq)];
   const int g = h / (a.hq / a.hkv);
   const int nkb = w.a1, kfull = w.a0;
   const uint32_t sQ = ptx::smem_u32(smem + OFF_Q);

@@ -201,6 +201,9 @@ struct AttnArgs {
   float scale;
   const int32_t* kv_end;
   const Tile* qtiles; const int32_t* q_order; int64_t nq;
+  // 0: q_order is in cost order.  Else a plan's whose first order_pairs entries
+  // are the even-indexed q-tiles and whose others are the odd ones (q_tile_at).
+  int64_t order_pairs;
   const Tile* ktiles; const int32_t* k_order; int64_t nk;
   uint32_t* status;
   // Stored-dS backward: when ds is set, dK/dV also writes each bf16 dS tile
@@ -277,6 +280,16 @@ inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || i
 // not share K / V.
 inline bool fwd_bucketed(const AttnArgs& a, int64_t items) {
   return a.hq == a.hkv && a.d == 128 && a.dtype == ISM_BF16 && items >= 8 * (int64_t)sm_count();
+}
+// The q-tile at position `pos` of the cost order.  Where the even and the odd
+// tiles stand apart, each half most expensive first, they alternate: the i-th pair
+// head goes with a tile of about its cost.
+__device__ __forceinline__ int32_t q_tile_at(const AttnArgs& a, int64_t pos) {
+  if (a.order_pairs) {
+    const int64_t odd = a.nq - a.order_pairs;
+    pos = pos >= 2 * odd ? pos - odd : pos & 1 ? a.order_pairs + pos / 2 : pos / 2;
+  }
+  return a.q_order[pos];
 }
 // Called by every thread of every block of a forward kernel.
 __device__ __forceinline__ void advance_cache_len(const AttnArgs& a) {

@@ -218,13 +218,13 @@ __device__ __forceinline__ void add_parts(float* red, float (&acc)[C::R][C::DPL]
 }
 
 // The rows of block `b` of a launch over n_heads x tiles x SUB: the head is
-// the fastest index, the tiles come in cost order.
-template <class C>
-__device__ __forceinline__ Tile own_rows(const Tile* tiles, const int32_t* order, int n_heads, int* head, int* row0) {
+// the fastest index, the tiles come in cost order (tile_at).
+template <class C, class At>
+__device__ __forceinline__ Tile own_rows(const Tile* tiles, At tile_at, int n_heads, int* head, int* row0) {
   const int64_t b = blockIdx.x;
   *head = (int)(b % n_heads);
   const int64_t t = b / n_heads;
-  const Tile w = tiles[order[t / C::SUB]];
+  const Tile w = tiles[tile_at(t / C::SUB)];
   *row0 = w.tile * kTileRows + (int)(t % C::SUB) * C::ROWS;
   return w;
 }
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(C::TH) simt_fwd_kernel(const AttnArgs a) {
   extern __shared__ __align__(16) float sm[];
   float *own = sm, *kt = own + C::OWN, *vt = kt + C::TILE, *wt = vt + C::TILE;
   int h, row0;
-  const Tile w = own_rows<C>(a.qtiles, a.q_order, a.hq, &h, &row0);
+  const Tile w = own_rows<C>(a.qtiles, [&](int64_t p) { return q_tile_at(a, p); }, a.hq, &h, &row0);
   if (row0 >= w.q_len) return;
   const int g = h / (a.hq / a.hkv);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rw = warp % C::W, sw = warp / C::W;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(C::TH) simt_dq_kernel(const AttnArgs a) {
   extern __shared__ __align__(16) float sm[];
   float *own_q = sm, *own_do = own_q + C::OWN, *kt = own_do + C::OWN, *vt = kt + C::TILE, *wt = vt + C::TILE;
   int h, row0;
-  const Tile w = own_rows<C>(a.qtiles, a.q_order, a.hq, &h, &row0);
+  const Tile w = own_rows<C>(a.qtiles, [&](int64_t p) { return q_tile_at(a, p); }, a.hq, &h, &row0);
   if (row0 >= w.q_len) return;
   const int g = h / (a.hq / a.hkv);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rw = warp % C::W, sw = warp / C::W;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(C::TH) simt_dkdv_kernel(const AttnArgs a) {
   float *own_k = sm, *own_v = own_k + C::OWN, *qt = own_v + C::OWN, *dot = qt + C::TILE, *pt = dot + C::TILE,
         *dst = pt + C::WGT;
   int g, key0;
-  const Tile w = own_rows<C>(a.ktiles, a.k_order, a.hkv, &g, &key0);
+  const Tile w = own_rows<C>(a.ktiles, [&](int64_t p) { return a.k_order[p]; }, a.hkv, &g, &key0);
   if (key0 >= w.k_len) return;
   const int group = a.hq / a.hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rw = warp % C::W, sw = warp / C::W;

@@ -77,3 +77,41 @@ def test_bf16_forced(d, monkeypatch):
     ref = (*orc.attn_fwd(*x[:3], w.segs, w.softmax_scale), *orc.attn_bwd(*x, w.segs, w.softmax_scale))
     for a, b in zip(got, ref):  # the bf16 output rounding (and Delta from the bf16 O)
         assert _rel(a, b) <= 2.0 ** -9 + 2.0 ** -12
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(3, 1, 64), (3, 3, 128), (4, 2, 64)])
+@pytest.mark.parametrize("copies", [2, 40])  # the small metadata pass and the general one
+def test_query_tiles_in_cost_order(hq, hkv, d, copies):
+    """The fp32 forward takes the most expensive query tiles first, whatever the
+    group; a plan of an odd group has the even-indexed tiles in front and each
+    half in order, and gives the same results."""
+    segs = wl.pack([([70, 150, 170, 700], [0, 1, 0, 1]), ([129], [0]), ([400], [1]), ([1], [1])] * copies)
+    w = wl.Workload("order", segs, hq, hkv, d, "fp32", d ** -0.5, 1.0, 8)
+    q, k, v, do = (t.to(DEV) for t in wl.attention_tensors(w))
+    s = ism.Segments.from_workload(segs, DEV)
+    T, nq = w.total_tokens, sum(-(-segs.seq(b)[1] // 128) for b in range(segs.num_seqs))
+    up = lambda n: (n + 255) // 256 * 256
+
+    def lists(buffer):  # (tile index in its dialogue, key tiles) along q_order
+        words = buffer.cpu().numpy().view(np.int32)
+        tiles = words[up(4 * T) // 4:][:8 * nq].reshape(nq, 8)
+        order = words[(up(4 * T) + up(32 * nq)) // 4:][:nq]
+        assert sorted(order) == list(range(nq))
+        return tiles[order, 4], tiles[order, 6]
+
+    ws = ism._workspace(64 << 20, DEV)
+    o, lse = ism.fwd(s, q, k, v, w.softmax_scale, workspace=ws)
+    grads = ism.bwd(s, q, k, v, o, lse, do, w.softmax_scale)
+    cost = lists(ws)[1]
+    assert (np.diff(cost) <= 0).all()
+    plan = ism.Plan(s, hq, hkv, d, torch.float32, DEV)
+    index, cost = lists(plan.buffer)
+    if (hq // hkv) % 2:
+        heads = int((index % 2 == 0).sum())
+        assert (index[:heads] % 2 == 0).all() and (np.diff(cost[heads:]) <= 0).all()
+    else:
+        assert (np.diff(cost) <= 0).all()
+    o2, lse2 = ism.fwd(s, q, k, v, w.softmax_scale, plan=plan)
+    for a, b in zip((o, lse, *grads), (o2, lse2, *ism.bwd(s, q, k, v, o, lse, do, w.softmax_scale, plan=plan))):
+        assert torch.equal(a, b)
+    ism.check_status(DEV)

@@ -244,8 +244,8 @@ ism_status_t ism_attn_bwd(const ism_segments_t* segs, const ism_attn_shape_t* sh
  * forward), v, o, lse, dout, except that dq and dk are the gradients with
  * respect to the UNROTATED q and k: the gradients of the rotated rows go back
  * through the transposed rotation (the rotation by the opposite angle).  On
- * the tensor cores (bf16, head_dim 128) that happens in the dQ and dK
- * epilogues; otherwise one more pass rotates dq and dk in place.
+ * the tensor cores (bf16) that happens in the dQ and dK epilogues; otherwise
+ * (fp32) one more pass rotates dq and dk in place.
  * Workspaces: ism_attn_fwd_workspace_size / ism_attn_bwd_workspace_size (or
  * _min) of the same segments and shape.  Errors as ism_attn_fwd /
  * ism_attn_bwd, plus ISM_ERR_INVALID_ARG for a missing or misaligned table,

@@ -135,9 +135,6 @@ constexpr int kMaxSeqs = 8192;
 cudaError_t launch_tiles(const SegsDev& s, int bm, int bn, const int32_t* kv_end, int64_t nq, int64_t nk,
                          Tile* qtiles, Tile* ktiles, uint8_t* tile_class, int32_t* kt_full_end,
                          int32_t* kt_end, int32_t* qt_begin, cudaStream_t st);
-cudaError_t launch_order(const Tile* qtiles, int64_t nq, const Tile* ktiles, int64_t nk, int max_cost,
-                         int32_t* q_order, int32_t* k_order, cudaStream_t st, int32_t* pair_order = nullptr);
-cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_off, cudaStream_t st);
 // kv_end, tiles, work lists (and pair offsets when kpair_off is set, the
 // k-tile pair list when kp_order is set) in one launch.  pairs_first: q_order
 // starts with the even-indexed q-tiles (pair heads, in the pair list's order).
@@ -187,10 +184,11 @@ cudaError_t launch_rope_rows(const int32_t* cu_seqlens, int num_seqs, int64_t T,
                              const void* q_src, const void* k_src, void* q_dst, void* k_dst, const float* cos_t,
                              const float* sin_t, float sin_sign, cudaStream_t st, bool dependent);
 
-// CUDA-core attention (ism_simt.cu), fp32 or bf16 storage, fp32 math.
 // Multiprocessor count of the current device (looked up once per device).
 int sm_count();
 
+// Arguments of the attention kernels: the CUDA-core ones (ism_simt.cu; fp32 or
+// bf16 storage, fp32 math) and the tensor-core ones.
 struct AttnArgs {
   const void* q; const void* k; const void* v; const void* o; const void* dout;
   void* out; float* lse; const float* lse_in;
@@ -247,7 +245,7 @@ struct AttnArgs {
   // Rotary encoding (tensor-core backward only): when rope_cos is set, the dQ
   // and dK epilogues store the gradients of the unrotated queries and keys,
   // applying the transposed rotation of the row's position in its sequence
-  // (tables [rows, 64] fp32, the angle of pair k of position p at p * 64 + k).
+  // (tables [rows, d / 2] fp32, the angle of pair k of position p at p * d / 2 + k).
   const float* rope_cos;
   const float* rope_sin;
   bool dependent;  // launch as programmatic dependents (dependent_pass)

@@ -240,12 +240,6 @@ __device__ void order_body(const Tile* __restrict__ qtiles, int64_t nq, const Ti
   }
 }
 
-__global__ void order_kernel(const Tile* __restrict__ qtiles, int64_t nq, const Tile* __restrict__ ktiles,
-                             int64_t nk, int max_cost, int32_t* q_order, int32_t* k_order, int32_t* pair_order) {
-  extern __shared__ int32_t hist[];  // [max_cost + 1]
-  order_body(qtiles, nq, ktiles, nk, max_cost, q_order, k_order, pair_order, hist);
-}
-
 // Exclusive prefix over k-tiles of their non-empty q-tile counts (a1 - a0):
 // the first (k-tile, q-tile) pair slot of each k-tile.  One block, chunks of
 // blockDim.x with a running carry.
@@ -263,10 +257,6 @@ __device__ void pair_offsets_body(const Tile* __restrict__ ktiles, int64_t nk, i
     if (i < nk) kpair_off[i] = carry + incl - v;
     carry += tot;
   }
-}
-
-__global__ void pair_offsets_kernel(const Tile* __restrict__ ktiles, int64_t nk, int32_t* kpair_off) {
-  pair_offsets_body(ktiles, nk, kpair_off);
 }
 
 // All metadata of one attention pass in a single block: kv_end per token
@@ -645,17 +635,6 @@ cudaError_t launch_tiles(const SegsDev& s, int bm, int bn, const int32_t* kv_end
   return cudaGetLastError();
 }
 
-cudaError_t launch_order(const Tile* qtiles, int64_t nq, const Tile* ktiles, int64_t nk, int max_cost,
-                         int32_t* q_order, int32_t* k_order, cudaStream_t st, int32_t* pair_order) {
-  size_t smem = sizeof(int32_t) * (size_t)(max_cost + 1);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  order_kernel<<<1, 1024, smem, st>>>(qtiles, nq, ktiles, nk, max_cost, q_order, k_order, pair_order);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, int64_t nq, int64_t nk,
                              Tile* qtiles, Tile* ktiles, int max_cost, int32_t* q_order, int32_t* k_order,
                              int32_t* pair_order, int32_t* kpair_off, int32_t* counters, int n_counters,
@@ -677,18 +656,13 @@ cudaError_t launch_pass_meta(const SegsDev& s, int32_t* kv_end, int bm, int bn, 
                           q_order, k_order, pair_order, kpair_off, counters, n_counters, kp_order, pairs_first);
 }
 
-cudaError_t launch_pair_offsets(const Tile* ktiles, int64_t nk, int32_t* kpair_off, cudaStream_t st) {
-  if (nk == 0) return cudaSuccess;
-  pair_offsets_kernel<<<1, 1024, 0, st>>>(ktiles, nk, kpair_off);
-  return cudaGetLastError();
-}
-
 namespace {
 // A cache-write kernel over `total` threads.
 template <class... Params, class... Args>
 cudaError_t launch_write(void (*kern)(Params...), int64_t total, cudaStream_t st, Args... args) {
   int64_t grid = (total + 255) / 256;
-  if (grid > 152 * 16) grid = 152 * 16;
+  const int64_t top = (int64_t)sm_count() * 16;
+  if (grid > top) grid = top;
   return launch(true, kern, grid, 256, 0, st, args...);
 }
 }  // namespace

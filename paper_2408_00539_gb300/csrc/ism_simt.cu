@@ -92,8 +92,8 @@ struct Stage {
 
 // The warp's own rows [first, first + R) into shared memory (lanes over columns), zero past n_rows.
 template <class C>
-__device__ __forceinline__ void load_own(float* dst, const typename C::T* base, int64_t stride, int first, int n_rows,
-                                         float mul = 1.f) {
+__device__ __forceinline__ void load_own(float* dst, const typename C::T* base, int64_t stride, int first,
+                                         int n_rows) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int i = 0; i < C::R * C::D / 128; ++i) {

@@ -1,6 +1,6 @@
 """Key-range split of the append forward: every number of parts the rule takes
-(head pairs, query-tile pairs of odd groups, paged, e4m3, head_dim 64), parts
-without key tiles, workspaces of the required size only, and the cache lengths
+(head pairs, query-tile pairs of odd groups, paged, head_dim 64), the halves of
+e4m3, parts without key tiles, workspaces of the required size only, and the cache lengths
 after each call.  Reference: the same call unsplit (ISM_PREFILL_SPLIT=0).
 
 Tolerance, in the 2-norm against the whole item's result: at head_dim 128 P is
@@ -137,3 +137,45 @@ def test_split_e4m3_and_paged(monkeypatch, hq, hkv):
     _same((b[2], b[3], b[4], b[5]), (a[2], a[3], a[4], a[5]))
     contiguous = _call(monkeypatch, None, x, lens, [ln], [0], d ** -0.5)
     assert torch.equal(contiguous[0], b[2]) and torch.equal(contiguous[1], b[3])
+
+
+@pytest.mark.parametrize("hq,hkv,batch,cached,split", [(8, 2, 2, 1500, "8"), (3, 3, 2, 1500, "6"), (32, 8, 10, 8200, None)])
+def test_e4m3_halves(monkeypatch, hq, hkv, batch, cached, split):
+    """e4m3 in two halves of the key range, forced on all items (an even and an
+    odd group) and by its own rule (items past a whole round, long caches).  Both
+    results are off the exact one by their roundings of P, and differ from each
+    other: the split was taken."""
+    ln, d, f = 60, 128, 0.01
+    gen = torch.Generator(device=DEV).manual_seed(4)
+
+    def e8(*shape):
+        x = torch.randn(shape, generator=gen, device=DEV, dtype=torch.bfloat16)
+        return (x.float() / f).clamp(-448, 448).to(torch.float8_e4m3fn)
+
+    x = [e8(batch, ln, h, d) for h in (hq, hkv, hkv)] + [e8(batch, cached + ln, hkv, d) for _ in range(2)]
+    lens = np.full((batch,), cached, np.int32)
+    out = []
+    for n in ("0", split):
+        if n is None:
+            monkeypatch.delenv("ISM_PREFILL_SPLIT", raising=False)
+        else:
+            monkeypatch.setenv("ISM_PREFILL_SPLIT", n)
+        ism.load().ism_debug_reload_env()
+        try:
+            out.append(ism.prefill_append_e4m3(*x, torch.from_numpy(lens.copy()).to(DEV), lens, [ln], [0], f, f, f,
+                                               d ** -0.5))
+            ism.check_status(DEV)
+        finally:
+            monkeypatch.delenv("ISM_PREFILL_SPLIT", raising=False)
+            ism.load().ism_debug_reload_env()
+    whole, got = (o.double() for o, _ in out)
+    assert torch.isfinite(got).all() and not torch.equal(whole, got)
+    assert float((whole - got).norm() / whole.norm()) <= 4e-2
+    assert float((out[0][1] - out[1][1]).abs().max()) <= 2e-5
+    # the last sequence against 64 bits (the rule splits the last items)
+    kv = [(torch.cat([c[-1, :cached], n[-1]]).double() * f) for c, n in ((x[3], x[1]), (x[4], x[2]))]
+    q = x[0][-1].double() * f
+    for h in range(0, hq, max(1, hq // 4)):
+        k, v = (t[:, h // (hq // hkv)] for t in kv)
+        exact = torch.softmax(q[:, h] @ k.T * d ** -0.5, dim=1) @ v
+        assert float((got[-1, :, h] - exact).norm() / exact.norm()) <= 4e-2

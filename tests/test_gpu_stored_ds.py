@@ -53,7 +53,8 @@ def test_head_units(hq, hkv, rope):
             room[4 if rope == 16 else 0:][:t.size] = torch.from_numpy(t).to(DEV).flatten()
             tables.append(room[4 if rope == 16 else 0:][:t.size].view(t.shape))
     few = _step(ism.Segments.from_workload(w.segs, DEV), x, w.softmax_scale, tables)
-    copies = 152 * 10 // (12 * hq) + 2  # 12 query tiles a copy: above ten items an SM
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    copies = sms * 10 // (12 * hq) + 2  # 12 query tiles a copy: above ten items an SM
     many = _step(ism.Segments.from_workload(wl.pack(RAGGED * copies), DEV), [t.repeat(copies, 1, 1) for t in x],
                  w.softmax_scale, tables)
     ism.check_status(DEV)

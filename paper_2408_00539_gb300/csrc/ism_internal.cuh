@@ -92,8 +92,8 @@ enum : uint32_t { kStatusTimeout = 1u, kStatusSmemAlign = 2u };
 // its set-up, so that a kernel that runs at all has everything before its direct
 // predecessor in place.  What it reads is not __restrict__ and not read through
 // __ldg: such loads count as constant, and the compiler may move them before the
-// wait.  (rope_row and order_body may: their addresses come from descriptors that
-// are read behind it, or their kernel wrote them itself.)
+// wait.  (rope_row may: its addresses come from descriptors that are read behind
+// it.)
 // A kernel that allocates tensor memory lets the next one start only after its
 // allocation (pdl_sync at the top, pdl_trigger behind it): the next kernel may
 // allocate before it waits for this one, and would otherwise hold columns that

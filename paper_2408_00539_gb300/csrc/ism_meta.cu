@@ -101,7 +101,7 @@ __global__ void kv_end_kernel(SegsDev s, int32_t* kv_end) {
 // non-empty tiles; k-tile c is first reached by the q-tile holding the first
 // row whose kv_end exceeds c*bn.
 // `dyn` holds the per-sequence offsets ((num_seqs + 1) * 16 bytes).
-__device__ void tiles_body(const SegsDev& s, int bm, int bn, const int32_t* __restrict__ kv_end, int64_t nq,
+__device__ void tiles_body(const SegsDev& s, int bm, int bn, const int32_t* kv_end, int64_t nq,
                            int64_t nk, Tile* qtiles, Tile* ktiles, uint8_t* tile_class, int32_t* kt_full_end,
                            int32_t* kt_end, int32_t* qt_begin, unsigned char* dyn) {
   int64_t* toff = reinterpret_cast<int64_t*>(dyn);
@@ -157,7 +157,7 @@ __device__ void tiles_body(const SegsDev& s, int bm, int bn, const int32_t* __re
   }
 }
 
-__global__ void __launch_bounds__(256) tiles_kernel(SegsDev s, int bm, int bn, const int32_t* __restrict__ kv_end,
+__global__ void __launch_bounds__(256) tiles_kernel(SegsDev s, int bm, int bn, const int32_t* kv_end,
                              int64_t nq, int64_t nk, Tile* qtiles, Tile* ktiles, uint8_t* tile_class,
                              int32_t* kt_full_end, int32_t* kt_end, int32_t* qt_begin) {
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -188,7 +188,7 @@ __device__ __forceinline__ bool pair_head(const Tile* qtiles, int64_t nq, int64_
 // pairs_first: q_order lists the pair heads of the third list first (in its
 // order), then the odd-indexed q-tiles; the forward of an odd group at
 // head_dim 64 reads its pairs from there.
-__device__ void order_body(const Tile* __restrict__ qtiles, int64_t nq, const Tile* __restrict__ ktiles, int64_t nk,
+__device__ void order_body(const Tile* qtiles, int64_t nq, const Tile* ktiles, int64_t nk,
                            int max_cost, int32_t* q_order, int32_t* k_order, int32_t* pair_order, int32_t* hist,
                            int32_t* kp_order = nullptr, bool pairs_first = false) {
   int32_t heads = 0;  // pair heads listed at the front of q_order (pairs_first)
@@ -243,7 +243,7 @@ __device__ void order_body(const Tile* __restrict__ qtiles, int64_t nq, const Ti
 // Exclusive prefix over k-tiles of their non-empty q-tile counts (a1 - a0):
 // the first (k-tile, q-tile) pair slot of each k-tile.  One block, chunks of
 // blockDim.x with a running carry.
-__device__ void pair_offsets_body(const Tile* __restrict__ ktiles, int64_t nk, int32_t* kpair_off) {
+__device__ void pair_offsets_body(const Tile* ktiles, int64_t nk, int32_t* kpair_off) {
   int32_t carry = 0;  // the same in every thread
   for (int64_t base = 0; base < nk; base += blockDim.x) {
     const int64_t i = base + threadIdx.x;

@@ -89,3 +89,10 @@ def test_split_forward_triggers_behind_its_last_barrier():
     first thread of a block to trigger does so for the block."""
     body = next(b for n, _, b in KERNELS if n == "fwd_pair_kernel")
     assert body.rindex("pdl_trigger()") > body.rindex("__syncthreads()")
+
+
+def test_metadata_is_read_as_it_was_written():
+    """The metadata kernels read tiles and bounds that they wrote themselves:
+    nothing of theirs counts as constant."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "ism_meta.cu")).read())
+    assert "__restrict__" not in text and "__ldg" not in text

@@ -515,7 +515,7 @@ enum {
   ISM_KERNEL_FWD = 1,        /* one-pass forward (and append-prefill over a chunk) */
   ISM_KERNEL_BWD_DKDV = 2,   /* backward dK/dV */
   ISM_KERNEL_BWD_DQ = 3,     /* backward dQ */
-  ISM_KERNEL_BWD_PRE = 4,    /* backward preprocessing (Delta) */
+  ISM_KERNEL_BWD_PRE = 4,    /* backward preprocessing (Delta; bf16: the CUDA-core dQ kernel computes its own) */
   ISM_KERNEL_DECODE = 5,     /* single-token append (split-KV + merge) */
   ISM_KERNEL_META = 6,       /* tile map / work lists */
   ISM_KERNEL_ROPE = 7        /* rotary encoding pass of the one-pass forward (and CUDA-core backward) */

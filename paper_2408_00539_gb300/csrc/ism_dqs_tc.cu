@@ -11,7 +11,8 @@
 // Bound by HBM (the dS stream) on long sequences, by the L2 reads beside it on
 // short ones.  Units of two query heads of one KV head read their K tile, and
 // their rows of the rotary tables, once for both: 2 x 8192 tokens of 32 / 8
-// heads 690 -> 663 us (6.6 TB/s), 24 rotary dialogues of 16001 tokens 142 -> 120.
+// heads 702 -> 681 us (6.7 TB/s), 24 rotary dialogues of 16001 tokens 147 -> 124
+// (events around the kernel, L2 flushed before each pass).
 // A dS tile is stored 8-interleaved (16-byte units of 8 consecutive queries
 // of one key, the 128 keys of a query group adjacent), which is the no-swizzle
 // MN-major operand layout: one contiguous bulk copy moves it into shared

@@ -218,7 +218,7 @@ struct AttnArgs {
   int64_t npairs;
   bool bucketed;  // their work list in buckets of neighbouring tiles, head by head (fwd_bucketed)
   // Work counter, at zero: of the persistent dK/dV kernel, or of the paired
-  // forward on query-tile pairs.
+  // forward (fwd_dynamic).
   int32_t* work_counter;
   // dK/dV on CTA pairs: kp_order lists the even-indexed k-tiles (each with the
   // next k-tile of its sequence, when there is one) in cost order; nkp of them.
@@ -270,9 +270,10 @@ inline bool dependent_pass(int64_t q_tiles, int heads) { return q_tiles * heads 
 inline bool fwd_dynamic(int64_t items, bool tile_pairs) { return tile_pairs || items < 8 * (int64_t)sm_count(); }
 // Whether that list keeps its buckets (bucket_item) instead of the plain cost
 // order: with one query head per KV head, 32 KB tiles and many units, sharing
-// tiles in L2 saves more (power above all, in a loop of steps) than the order's
-// balance: 4 x 4096 of 32 heads 1767 us a step against 1786, although the forward
-// alone takes 396 against 387; six ragged dialogues 2684 and 2699.  Half-size
+// tiles in L2 saves about as much (power above all, in a loop of steps) as the
+// order's balance gives: 4 x 4096 of 32 heads 1767 us a step against 1786 (the
+// forward alone 396 and 387), six ragged dialogues 2684 and 2699, little more than
+// two runs differ by.  Half-size
 // tiles and few units: e4m3 4 x 4096 333 and 318, head_dim 64 over 6001 tokens 318
 // and 302.  The static walk of tile pairs keeps its buckets wherever the heads do
 // not share K / V.
